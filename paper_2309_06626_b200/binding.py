@@ -7,7 +7,9 @@ from typing import Tuple
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "libasx.so")
+_EXT_PATH = os.path.join(_PKG, "_asx_torch.so")
 _lib = None
+_fast = None
 
 ACT_RELU, RECOMPACT, IMPL_NAIVE, OUT_COMPACT, IN_COMPACT, ACT_SILU, F32, IMPL_ROW_GATHER, IMPL_WINDOW_PATCH = 1, 2, 4, 8, 16, 32, 64, 128, 256
 
@@ -75,6 +77,21 @@ def lib():
     return _lib
 
 
+def _native():
+    """The calls made once per layer and step, from torch tensors to the C ABI without Python in between
+    (csrc/torch_binding.cpp).  Each returns its result or an int: a status code of the library, or -1 when
+    the arguments do not fit, upon which the caller goes through the checks below, which say why."""
+    global _fast
+    if _fast is None:
+        lib()
+        import torch  # noqa: F401  (its libraries must be loaded before the extension)
+        if not os.path.exists(_EXT_PATH):
+            raise RuntimeError(f"{_EXT_PATH} is missing: build it with `python -m paper_2309_06626_b200.build`")
+        from . import _asx_torch
+        _fast = _asx_torch
+    return _fast
+
+
 def _check(code: int, what: str) -> None:
     if code != 0:
         raise AsxError(code, what)
@@ -94,6 +111,7 @@ class MaskedConvLayer:
         _check(lib().asx_create_layer(C_in, C_out, kh, kw, stride, pad, ctypes.byref(self._h)),
                "asx_create_layer")
         self.C_in, self.C_out, self.kh, self.kw, self.stride, self.pad = C_in, C_out, kh, kw, stride, pad
+        self._geometry = (self._h.value, C_in, C_out, kh, kw, stride, pad)
 
     def out_hw(self, H: int, W: int) -> Tuple[int, int]:
         return ((H + 2 * self.pad - self.kh) // self.stride + 1,
@@ -101,6 +119,10 @@ class MaskedConvLayer:
 
     def set_mask(self, mask, stream=None) -> None:
         """mask: uint8 torch tensor (CPU or CUDA) or numpy array, 1 = keep, 0 = drop."""
+        rc = (_fast or _native()).set_mask(self._geometry[0], mask, None if stream is None else stream.cuda_stream)
+        if rc >= 0:
+            _check(rc, "asx_set_mask")
+            return
         import numpy as np
         import torch
         if isinstance(mask, torch.Tensor):
@@ -162,6 +184,11 @@ class MaskedConvLayer:
         """x: CUDA bf16 [Nb][H][W][C_in]; w: CUDA bf16 [C_out][kh][kw][C_in]; bias: CUDA fp32 or
         None.  Returns the CUDA bf16 output [Nb][Ho][Wo][C_out] (allocated by torch unless
         `out` is given).  With the F32 flag x, w and the output are float32 instead."""
+        y = (_fast or _native()).run(self._geometry, x, w, bias, out, flags, None if stream is None else stream.cuda_stream)
+        if type(y) is not int:
+            return y
+        if y > 0:
+            raise AsxError(y, "asx_run")
         import torch
         dt = torch.float32 if flags & F32 else torch.bfloat16
         if x.dtype != dt or w.dtype != dt:
@@ -213,6 +240,7 @@ class MaskedConvLayer:
         if getattr(self, "_h", None) is not None and self._h:
             lib().asx_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._geometry = (0,) + self._geometry[1:]
 
     def __del__(self):
         try:
@@ -234,6 +262,11 @@ def mask_from_scores(score, Ho: int, Wo: int, sparsity: float):
 def mask_from_activation(x_dev, stream=None):
     """mask[r] = 1 iff a channel of row r of the CUDA bf16 tensor x_dev [..., C] is positive; returns a
     CUDA uint8 tensor with one entry per row (allocated by torch)."""
+    m = (_fast or _native()).mask_from_activation(x_dev, None if stream is None else stream.cuda_stream)
+    if type(m) is not int:
+        return m
+    if m > 0:
+        raise AsxError(m, "asx_mask_from_activation")
     import torch
     if x_dev.dtype != torch.bfloat16 or not x_dev.is_cuda or not x_dev.is_contiguous():
         raise ValueError("x must be a contiguous CUDA bfloat16 tensor")
@@ -249,6 +282,11 @@ def compact_mask(mask_dev, stream=None):
     """Stand-alone S1 on a CUDA uint8 tensor: returns (kept int32 tensor of mask.numel()
     entries, count int32 tensor of one entry, scratch tensor).  Only the first `count`
     entries of `kept` are defined."""
+    all3 = (_fast or _native()).compact_mask(mask_dev, None if stream is None else stream.cuda_stream)
+    if type(all3) is not int:
+        return all3
+    if all3 > 0:
+        raise AsxError(all3, "asx_compact")
     import torch
     rows = mask_dev.numel()
     kept = torch.empty(max(rows, 1), dtype=torch.int32, device=mask_dev.device)

@@ -1,14 +1,18 @@
-"""Builds the C-ABI shared library (libasx.so) in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI shared library (libasx.so) in-tree with nvcc for sm_100a, and the torch side of the
+binding (_asx_torch.so, a CPython extension linked against it) with the host compiler."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import tempfile
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libasx.so")
+EXT = os.path.join(PKG, "_asx_torch.so")
+EXT_SRC = os.path.join(CSRC, "torch_binding.cpp")
 
 
 def sources():
@@ -27,21 +31,55 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _deps())
 
 
+def _ext_is_stale() -> bool:
+    if not os.path.exists(EXT):
+        return True
+    t = os.path.getmtime(EXT)
+    return any(os.path.getmtime(f) > t for f in [EXT_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h")))
+
+
+def _build_ext() -> None:
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    tmp = EXT + f".tmp{os.getpid()}"
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    libs = cpp_extension.library_paths()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include")]
+    for d in cpp_extension.include_paths():
+        cmd += ["-isystem", d]
+    cmd += ["-o", tmp, EXT_SRC, "-L", PKG, "-Wl,-rpath,$ORIGIN", "-lasx"]
+    for d in libs:
+        cmd += ["-L", d]
+    subprocess.check_call(cmd + ["-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    os.replace(tmp, EXT)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source of the library into libasx.so (the CUDA runtime is linked
     statically and the driver is reached through the runtime, so the library loads on a
-    machine without a GPU driver)."""
-    if not force and not is_stale():
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-shared", "-Xcompiler", "-fPIC", "-cudart", "static",
-           "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp] + sources()
-    if verbose:
-        cmd.insert(1, "-Xptxas=-v")
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    machine without a GPU driver), one nvcc process per source, and then the torch extension."""
+    stale = force or is_stale()
+    if stale:
+        nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+        arch = ["-gencode", "arch=compute_100a,code=sm_100a"]
+        flags = arch + ["-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC,-O3", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+        if verbose:
+            flags.insert(0, "-Xptxas=-v")
+        with tempfile.TemporaryDirectory() as tmpdir:
+            jobs = []
+            for src in sources():
+                obj = os.path.join(tmpdir, os.path.basename(src) + ".o")
+                jobs.append((obj, subprocess.Popen([nvcc] + flags + ["-c", "-o", obj, src])))
+            failed = [obj for obj, p in jobs if p.wait() != 0]
+            if failed:
+                raise RuntimeError("nvcc failed on " + ", ".join(os.path.basename(f) for f in failed))
+            tmp = LIB + f".tmp{os.getpid()}"
+            subprocess.check_call([nvcc] + arch + ["-shared", "-cudart", "static", "-o", tmp] + [obj for obj, _ in jobs])
+        os.replace(tmp, LIB)
+    if force or _ext_is_stale():
+        _build_ext()
     return LIB
 
 
