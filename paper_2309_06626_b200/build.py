@@ -16,7 +16,7 @@ EXT_SRC = os.path.join(CSRC, "torch_binding.cpp")
 
 
 def sources():
-    return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+    return sorted(glob.glob(os.path.join(CSRC, "*.cu"))) + [os.path.join(CSRC, "mask_from_scores.cpp")]
 
 
 def _deps():

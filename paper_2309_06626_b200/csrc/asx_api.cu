@@ -132,6 +132,20 @@ asx_status run_compaction(asx_layer* L, cudaStream_t st)
     return from_cuda(launch_compact(L->d_mask, L->rows, L->d_kept, L->d_small, L->d_scratch, st, true));
 }
 
+int64_t count_nonzero(const uint8_t* mask, int64_t rows)
+{
+    int64_t kept = 0;
+    for (int64_t i = 0; i < rows;) {                              // byte counters first: sums of up to 255 vectorise
+        const int64_t end = std::min<int64_t>(rows, i + 255 * 64);
+        uint8_t part[64] = {0};
+        for (; i + 64 <= end; i += 64)
+            for (int l = 0; l < 64; ++l) part[l] = (uint8_t)(part[l] + (mask[i + l] != 0));
+        for (int l = 0; l < 64; ++l) kept += part[l];
+        for (; i < end; ++i) kept += mask[i] != 0;
+    }
+    return kept;
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw: "Parallel random numbers: as easy as 1, 2, 3", 2011).
 void philox4x32_10(const uint32_t ctr[4], const uint32_t key[2], uint32_t out[4])
 {
@@ -232,10 +246,11 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
     s = ensure_mask_buffers(L, rows);
     if (s != ASX_OK) return s;
     cudaPointerAttributes attr;
-    bool on_device = false;
-    if (cudaPointerGetAttributes(&attr, mask) == cudaSuccess)
+    bool on_device = false, pinned = true;
+    if (cudaPointerGetAttributes(&attr, mask) == cudaSuccess) {
         on_device = (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged);
-    else
+        pinned = attr.type != cudaMemoryTypeUnregistered;
+    } else
         cudaGetLastError();
     cudaError_t e;
     if (on_device) {
@@ -243,9 +258,7 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
         L->host_kept = -1;
         L->host_mask.clear();
     } else {
-        int64_t kept = 0;                                         // only sizes the tiles (a launch heuristic)
-        for (int64_t i = 0; i < rows; ++i) kept += mask[i] != 0;
-        L->host_kept = kept;
+        L->host_kept = count_nonzero(mask, rows);                 // only sizes the tiles (a launch heuristic)
         L->host_mask.clear();
         if (rows <= (1ll << 24)) {
             try {
@@ -254,8 +267,10 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
                 L->host_mask.clear();                              // only costs the choice of kernel form
             }
         }
+        // The caller may free a host mask on return.  A copy from pageable memory returns once the source has been
+        // staged; only a page-locked one is read in place, behind the call's back.
         e = cudaMemcpyAsync(L->d_mask, mask, (size_t)rows, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);      // the caller may free a host mask on return
+        if (e == cudaSuccess && pinned) e = cudaStreamSynchronize(st);
     }
     if (e != cudaSuccess) return from_cuda(e);
     L->rows = rows;
@@ -298,37 +313,6 @@ asx_status asx_set_mask_random(asx_layer* L, int64_t rows, double sparsity, int 
         std::memset(mask.data() + lo, 0, (size_t)(hi - lo));
     }
     return asx_set_mask(L, mask.data(), rows, cuda_stream);
-}
-
-asx_status asx_mask_from_scores(const float* score, int H0, int W0, int Ho, int Wo, double sparsity,
-                                uint8_t* mask_out)
-{
-    if (score == nullptr || mask_out == nullptr || H0 < 1 || W0 < 1 || Ho < 1 || Wo < 1 || Ho > H0 || Wo > W0 ||
-        !(sparsity >= 0.0 && sparsity <= 1.0) || (int64_t)Ho * Wo >= (1ll << 31))
-        return ASX_ERR_INVALID_ARG;
-    const int rh = H0 / Ho, rw = W0 / Wo;                 // ratio = input_res // layer.res
-    const int64_t P = (int64_t)Ho * Wo;
-    std::vector<std::pair<double, int64_t>> ranked;       // (pooled score, position): ordered by score, then position
-    try {
-        ranked.resize((size_t)P);
-    } catch (const std::bad_alloc&) {
-        return ASX_ERR_OOM;
-    }
-    for (int i = 0; i < Ho; ++i)
-        for (int j = 0; j < Wo; ++j) {
-            double acc = 0.0;                              // window sum in fp64, raster order of the window
-            const float* win = score + (size_t)i * rh * W0 + (size_t)j * rw;
-            for (int a2 = 0; a2 < rh; ++a2)
-                for (int b2 = 0; b2 < rw; ++b2) acc += (double)win[(size_t)a2 * W0 + b2];
-            const int64_t p = (int64_t)i * Wo + j;
-            ranked[(size_t)p] = {acc / (double)(rh * rw), p};
-        }
-    int64_t n_drop = (int64_t)std::floor(sparsity * (double)P + 0.5);
-    if (n_drop > P) n_drop = P;
-    if (n_drop > 0 && n_drop < P) std::nth_element(ranked.begin(), ranked.begin() + (n_drop - 1), ranked.end());
-    std::memset(mask_out, 1, (size_t)P);
-    for (int64_t k = 0; k < n_drop; ++k) mask_out[(size_t)ranked[(size_t)k].second] = 0;
-    return ASX_OK;
 }
 
 asx_status asx_set_mask_from_scores(asx_layer* L, const float* score, int H0, int W0, int Ho, int Wo,
