@@ -396,8 +396,8 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 {
     if (L == nullptr || x == nullptr || w == nullptr || y == nullptr) return ASX_ERR_INVALID_ARG;
     if (Nb < 1 || H < 1 || W < 1) return ASX_ERR_INVALID_ARG;
-    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH)) return ASX_ERR_INVALID_ARG;
-    if ((flags & ASX_IMPL_ROW_GATHER) && (flags & ASX_IMPL_WINDOW_PATCH)) return ASX_ERR_INVALID_ARG;
+    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT)) return ASX_ERR_INVALID_ARG;
+    if (((flags & ASX_IMPL_ROW_GATHER) != 0) + ((flags & ASX_IMPL_WINDOW_PATCH) != 0) + ((flags & ASX_IMPL_DIRECT) != 0) > 1) return ASX_ERR_INVALID_ARG;
     const bool f32 = (flags & ASX_F32) != 0;
     const int ES = f32 ? 4 : 2;                 // bytes per element of x, w and y
     const int EPC = 16 / ES;                    // elements per 16-byte chunk
@@ -453,12 +453,26 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     // shared memory as 16-bit positions); the reference kernel and large masks take the stand-alone compaction
     // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
     // leaves the plan its pipeline stages (decided below, once the geometry the kernel sees is known).
+    const int relu = (flags & ASX_ACT_SILU) ? 2 : (flags & ASX_ACT_RELU) ? 1 : 0;      // activation code: 0 identity, 1 ReLU, 2 SiLU
+    // Small filter matrices take the direct form, which needs no list and rebuilds it beside the convolution when asked to.
+    DirectPlan dplan;
+    const int impl = flags & (ASX_IMPL_NAIVE | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT);
+    if (!in_compact && !out_compact && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) &&
+        (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, L->host_kept < 0 ? M : L->rows == P ? L->host_kept * Nb : L->host_kept))) {
+        const bool list = (flags & ASX_RECOMPACT) && L->rows <= DIRECT_LIST_MAX_ROWS;
+        if ((flags & ASX_RECOMPACT) && !list) {
+            s = run_compaction(L, st);
+            if (s != ASX_OK) return s;
+        }
+        L->last_form = ASX_FORM_DIRECT;
+        return from_cuda(launch_direct(g, dplan, x, w, bias, y, L->d_mask, list ? L->d_kept : nullptr, list ? L->d_small : nullptr, relu, L->residual,
+                                       f32 ? 1 : 0, L->num_sms, st));
+    }
     bool fuse_compact = (flags & ASX_RECOMPACT) && !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS;
     if ((flags & ASX_RECOMPACT) && !fuse_compact) {
         s = run_compaction(L, st);
         if (s != ASX_OK) return s;
     }
-    const int relu = (flags & ASX_ACT_SILU) ? 2 : (flags & ASX_ACT_RELU) ? 1 : 0;      // activation code: 0 identity, 1 ReLU, 2 SiLU
     int32_t* d_count = L->d_small;
     int* d_status = reinterpret_cast<int*>(L->d_small + 1);
 

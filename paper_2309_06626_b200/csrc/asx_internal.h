@@ -105,6 +105,21 @@ cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtenso
                          int relu, int* dev_status, int num_sms, int fuse_compact, long long host_kept,
                          const void* residual, const void* tiles, int n_mtiles, long long kept_rows, int out_compact,
                          int wait_limit_kcycles, cudaStream_t st);
+// ---- the direct form (masked_conv_direct.cu): small filter matrices, dense input and output
+struct DirectPlan {
+    int KQ;                // 16-byte chunks of a window in groups of four, or (words > 0) its words in groups of sixteen
+    int words, shift;      // C_in that is no whole number of 16-byte chunks: 4-byte words per filter row, leading padding
+    int NG, n_tiles;       // 32-column groups per block, blocks side by side
+    int smem_bytes;
+};
+// false: this geometry does not take the direct form
+bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan);
+constexpr int64_t DIRECT_LIST_MAX_ROWS = 1 << 17;       // longest list it rebuilds itself
+// whether a layer with `kept_rows` kept lowered rows is faster here than in the tensor-memory forms
+bool direct_pays(const DirectPlan& plan, int num_sms, int64_t kept_rows);
+// kept_out, count_out: where the kept-row list is rebuilt beside the convolution, or null
+cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
+                          int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32, int num_sms, cudaStream_t st);
 // src[rows][C] -> dst[rows][Cp] with zero channels added (Cp = 4 or a multiple of 8; rows*Cp % 8 == 0)
 cudaError_t launch_pad_channels(const void* src, void* dst, long long rows, int C, int Cp, cudaStream_t st);
 // filters for the pixel-pair form: w[C_out][kh][kw][C] -> w2[C_out][kh][kw2][2][4], where pair kxx,

@@ -194,11 +194,15 @@ __device__ __forceinline__ void load_residual8(const __nv_bfloat16* residual, lo
     }
 }
 
-// z * sigmoid(z) with the fast exponential and division (relative error about 1e-6, far below the
-// bf16 rounding of the result); exp(-z) = inf for very negative z gives -0.
+// z * sigmoid(z) in five instructions: the approximate exponential and reciprocal as they are, without the range
+// handling that __expf and __fdividef put around them (relative error about 1e-6, far below the bf16 rounding of
+// the result).  exp(-z) = inf for very negative z gives -0, a flushed exp(-z) gives z.
 __device__ __forceinline__ float silu(float z)
 {
-    return __fdividef(z, 1.f + __expf(-z));
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(z * -1.4426950408889634f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
+    return z * r;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)

@@ -1,0 +1,560 @@
+// S1 - S4 for layers with a small filter matrix: the direct form of the masked convolution.
+//
+// The two tensor-memory forms pay 2000-3000 clocks of hand-overs per 128-row tile (row coordinates, gather, MMA
+// issue, accumulator, epilogue, each behind a barrier) however little a tile computes: on a 1x1 layer of 64 -> 32
+// channels at 160 x 160 the tensor core works 64 of those clocks, and 245 760 kept rows took 28 us for 57 MB.  Here
+// nothing is handed over.  A warp gathers its rows' window values from global memory straight into the
+// operand registers of mma.sync, multiplies and stores:
+//
+//   A  lane (g, t) of a warp holds rows g and g + 8 of a 16-row tile; for every 32 K-elements (64 bytes of bf16) of
+//      a row its four lanes load 16 bytes each.  Any order of k serves as long as both operands use it, so a
+//      lane's 16 bytes are simply the k values that the fragment layout wants from that lane, and fp32 works
+//      the same way with 16 K-elements.
+//   B  the filters lie in shared memory in that order, 512 consecutive bytes per (32 K-elements, 8 columns).
+//   D  the columns of an 8-column tile are chosen so that a lane ends up with 8 consecutive output channels.
+//
+// The legacy tensor path runs at a quarter of the tcgen05 rate (1017 of 4096 multiply-adds per clock and SM,
+// measured), which is why only small filter matrices come here; the warps are independent, so 16 to 24 of them
+// per SM hide each other's latencies.
+//
+// There is no kept-row list: a warp walks over 64 output rows at a time, reads their mask bytes, writes the zeros of
+// the dropped ones and queues the kept ones; whenever 16 or 32 rows are queued it computes them.  With ASX_RECOMPACT
+// a few extra blocks write the list to global memory beside the others.
+#include <atomic>
+#include <cuda_bf16.h>
+#include "asx_internal.h"
+#include "ptx_sm100.cuh"
+#include "conv_common.cuh"
+
+namespace asx {
+
+namespace {
+
+constexpr int THREADS = 256, WARPS = THREADS / 32;
+constexpr int CHUNK = 32;               // output rows a warp scans at a time
+constexpr int QUEUE = 48;               // row queue of a warp: up to 15 left over and 32 new ones
+
+struct DirectArgs {
+    FastDiv fdP, fdWo, fdUnits;         // divisions by P, Wo and the 16-byte units of a row's column range
+    FastDiv fdChunks, fdCin, fdkw, fdWords;   // by the chunks (words) of a window, C_in, kw, words
+    const void* x;
+    const void* w;
+    const float* bias;
+    void* y;
+    const uint8_t* mask;
+    const void* residual;
+    int32_t* kept_out;                  // non-null: the first list_blocks blocks write the kept-row list and its count
+    int list_blocks;
+    int32_t* count_out;
+    int relu;
+    int KQ;                             // groups of four 16-byte chunks (word form: of sixteen words) of a window
+    int words;                          // word form: 4-byte words per filter row, else 0
+    int shift;                          // word form: K-elements in front of a filter row's first (0 or 1)
+    int block_rows;                     // output rows per block
+    int unit_shift;
+    int lanes_per_row;                  // the 16-byte units of a row's column range are a power of two up to 32
+};
+
+__device__ __forceinline__ uint4 ld_x4(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_x1(const void* p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+template <bool F32>
+__device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    if (F32)      // the tensor core ignores the lower 13 mantissa bits of either operand
+        asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                     : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    else
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                     : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// The list for asx_get_kept (S1): block `part` writes the positions of mask bytes 4096 part .. 4096 part + 4095, for which
+// it first counts the kept rows in front of them.  (One block for the whole list was the last to finish: 14 us for a
+// mask of 25 600 rows.)
+constexpr int LIST_ROWS = THREADS * 16;
+__device__ void write_kept_list(const uint8_t* __restrict__ mask, int rows, int part, int32_t* kept, int32_t* count)
+{
+    __shared__ int s_total[2][WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int first = part * LIST_ROWS + tid * 16;
+    const unsigned f = first < rows ? mask_flags16(mask, rows, first) : 0u;
+    int before = 0;
+#pragma unroll 4
+    for (int i = 0; i < part; ++i) before += __popc(mask_flags16(mask, rows, i * LIST_ROWS + tid * 16));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+    const int mine = __popc(f);
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += u;
+    }
+    if (lane == 31) {
+        s_total[0][warp] = before;
+        s_total[1][warp] = incl;
+    }
+    __syncthreads();
+    int at = incl - mine, all = 0;
+#pragma unroll
+    for (int i = 0; i < WARPS; ++i) {
+        at += s_total[0][i] + (i < warp ? s_total[1][i] : 0);
+        all += s_total[0][i] + s_total[1][i];
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+        if ((f >> q) & 1u) kept[at + __popc(f & ((1u << q) - 1u))] = first + q;
+    if (tid == 0 && (part + 1) * (long long)LIST_ROWS >= rows) *count = all;
+}
+
+// Shared memory: the filters in fragment order, the bias, one entry per chunk (or word) of a window, the warps' row
+// queues.
+struct Tables {
+    uint4* b;          // [KQ][2][MTL][32]
+    float* bias;       // [16 MTL]
+    int2* pos;         // [KQ * 4] or [KQ * 16]: element offset from the window's corner, ky << 16 | kx (word form: the word's element)
+    int4* queue;       // [WARPS][QUEUE]
+};
+
+// What depends on the geometry alone.
+template <bool F32, bool WORDS>
+__device__ __forceinline__ void fill_positions(const Tables& s, const ConvGeom& g, const DirectArgs& a)
+{
+    constexpr int EPC = F32 ? 4 : 8;
+    for (int c = threadIdx.x; c < a.KQ * (WORDS ? 16 : 4); c += THREADS) {
+        int2 e = make_int2(WORDS ? -a.shift : 0, 0x7fff0000);  // past the window: no row has it inside the image (its filter entries are zero)
+        if (WORDS) {
+            const int ky = (int)fd_div((uint32_t)c, a.fdWords), i = c - ky * a.words;
+            const int el = F32 ? i : 2 * i - a.shift;
+            if (ky < g.kh) e = make_int2(ky * g.W * g.C_in + el, (ky << 16) | (el & 0xffff));
+        } else if (c * EPC < g.K) {
+            const int tap = (int)fd_div((uint32_t)(c * EPC), a.fdCin), ci = c * EPC - tap * g.C_in;
+            const int ky = (int)fd_div((uint32_t)tap, a.fdkw), kx = tap - ky * g.kw;
+            e = make_int2((ky * g.W + kx) * g.C_in + ci, (ky << 16) | kx);
+        }
+        s.pos[c] = e;
+    }
+}
+
+// Filters and bias.  Fragment (q, h, j): the 16 channels of tile j against half h of operand group q (16 K-elements of
+// bf16); lane (g, t) of it holds the words {channel a, word 2 h} {channel b, 2 h} {a, 2 h + 1} {b, 2 h + 1} of 16-byte
+// chunk 4 q + t, where a and b are its channels 2 MTL g + 2 j and + 1 (after all tiles a lane then holds 2 MTL
+// consecutive channels).
+template <int MTL>
+__device__ __forceinline__ int fragment_word(int ch, int q, int t, int word)
+{
+    const int gn = ch / (2 * MTL), j = (ch >> 1) % MTL;
+    return ((((q * 2 + (word >> 1)) * MTL + j) * 32) + gn * 4 + t) * 4 + (word & 1) * 2 + (ch & 1);
+}
+template <bool F32, bool WORDS, int MTL>
+__device__ __forceinline__ void load_filters(const Tables& s, const ConvGeom& g, const DirectArgs& a, int n0)
+{
+    constexpr int EPC = F32 ? 4 : 8, ES = F32 ? 4 : 2;
+    const int tid = threadIdx.x;
+    uint32_t* const frag = reinterpret_cast<uint32_t*>(s.b);
+    if (tid < 16 * MTL) s.bias[tid] = (a.bias != nullptr && n0 + tid < g.C_out) ? __ldg(a.bias + n0 + tid) : 0.f;
+    if (!WORDS) {
+        const int cpr = 4 * a.KQ, total = cpr * 16 * MTL;
+#pragma unroll 4
+        for (int i = tid; i < total; i += THREADS) {
+            const int ch = (int)fd_div((uint32_t)i, a.fdChunks), c = i - ch * cpr;
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (n0 + ch < g.C_out && c * EPC < g.K)
+                v = __ldcg(reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(a.w) + ((size_t)(n0 + ch) * g.K + (size_t)c * EPC) * ES));
+            frag[fragment_word<MTL>(ch, c >> 2, c & 3, 0)] = v.x;
+            frag[fragment_word<MTL>(ch, c >> 2, c & 3, 1)] = v.y;
+            frag[fragment_word<MTL>(ch, c >> 2, c & 3, 2)] = v.z;
+            frag[fragment_word<MTL>(ch, c >> 2, c & 3, 3)] = v.w;
+        }
+    } else {
+        // word k of the chunk of lane t is word 16 q + 4 k + t of the window: word i of filter row ky holds its elements
+        // 2 i - shift, + 1 (fp32: i)
+        const int wpr = 16 * a.KQ, total = wpr * 16 * MTL, run = g.kw * g.C_in;
+#pragma unroll 4
+        for (int i = tid; i < total; i += THREADS) {
+            const int ch = (int)fd_div((uint32_t)i, a.fdChunks), wd = i - ch * wpr;
+            const int ky = (int)fd_div((uint32_t)wd, a.fdWords), i2 = wd - ky * a.words;
+            const size_t row = ((size_t)(n0 + ch) * g.kh + ky) * run;
+            const bool in = n0 + ch < g.C_out && ky < g.kh;
+            uint32_t v;
+            if (F32) {
+                v = in ? __ldcg(static_cast<const uint32_t*>(a.w) + row + i2) : 0u;
+            } else {
+                const int e = 2 * i2 - a.shift;
+                const unsigned short* wp = static_cast<const unsigned short*>(a.w) + row;
+                const uint32_t lo = (in && e >= 0 && e < run) ? __ldcg(wp + e) : 0u, hi = (in && e + 1 < run) ? __ldcg(wp + e + 1) : 0u;
+                v = lo | (hi << 16);
+            }
+            frag[fragment_word<MTL>(ch, wd >> 4, wd & 3, (wd >> 2) & 3)] = v;
+        }
+    }
+}
+
+// A queued row: x its output row, y the element index of its window's corner, z the corner's coordinates (iy0 << 16 | ix0,
+// word form: ix0 * C_in), w 1 when every word or chunk the window's filter rows touch lies inside the image.
+using Row = int4;
+
+// One group of operand loads: chunk 4 q + t (or four words) of the two rows of this lane.  CHECK: some window of the tile
+// reaches over the image's edge.
+template <bool F32, bool WORDS, bool CHECK>
+__device__ __forceinline__ void load_group(uint4 (&v)[2], int q, int t, const int2 (&row)[2], const Tables& s, const ConvGeom& g,
+                                           const uint8_t* __restrict__ xb)
+{
+    constexpr int ES = F32 ? 4 : 2;
+    const int xlim = WORDS ? g.W * g.C_in : g.W;
+    if (CHECK) v[0] = v[1] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int k = 0; k < (WORDS ? 4 : 1); ++k) {
+        const int2 e = s.pos[WORDS ? 16 * q + 4 * k + t : 4 * q + t];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            bool in = true;
+            if (CHECK) {
+                const int iy = (row[r].y >> 16) + (e.y >> 16), ix = (int)(short)row[r].y + (int)(short)e.y;
+                in = (unsigned)iy < (unsigned)g.H && (unsigned)ix < (unsigned)xlim;
+            }
+            if (in) {
+                const uint8_t* src = xb + (long long)(row[r].x + e.x) * ES;
+                if (WORDS) (&v[r].x)[k] = ld_x1(src);
+                else v[r] = ld_x4(src);
+            }
+        }
+    }
+}
+
+// acc += the group whose two rows' values lie in v, against the filters at aq.
+template <bool F32, int MTL>
+__device__ __forceinline__ void multiply_group(float (&acc)[2][MTL][4], const uint4 (&v)[2], const uint4* aq)
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < MTL; ++j) {
+            const uint4 w = aq[(h * MTL + j) * 32];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) mma<F32>(acc[r][j], w.x, w.y, w.z, w.w, h ? v[r].z : v[r].x, h ? v[r].w : v[r].y);
+        }
+}
+
+// KQT: the number of operand groups where it is 1 or 2 (all loads first, nothing loops), else 0.
+template <bool F32, bool WORDS, bool CHECK, int MTL, int KQT>
+__device__ __forceinline__ void multiply(float (&acc)[2][MTL][4], const int2 (&row)[2], const Tables& s, const ConvGeom& g, int KQ,
+                                         const uint8_t* __restrict__ xb, int lane)
+{
+    constexpr int STEP = 2 * MTL * 32;
+    const int t = lane & 3;
+    const uint4* aq = s.b + lane;
+    uint4 v[2], next[2];
+    load_group<F32, WORDS, CHECK>(v, 0, t, row, s, g, xb);
+    if (KQT == 1) {
+        multiply_group<F32, MTL>(acc, v, aq);
+    } else if (KQT == 2) {
+        load_group<F32, WORDS, CHECK>(next, 1, t, row, s, g, xb);
+        multiply_group<F32, MTL>(acc, v, aq);
+        multiply_group<F32, MTL>(acc, next, aq + STEP);
+    } else {
+        // two groups a turn, each loaded while the other is used (with an exit in the middle of the turn the compiler
+        // copied every accumulator once per product)
+#pragma unroll 1
+        for (int q = 1; q < KQ; q += 2, aq += 2 * STEP) {
+            load_group<F32, WORDS, CHECK>(next, q, t, row, s, g, xb);
+            multiply_group<F32, MTL>(acc, v, aq);
+            if (q + 1 < KQ) load_group<F32, WORDS, CHECK>(v, q + 1, t, row, s, g, xb);
+            multiply_group<F32, MTL>(acc, next, aq + STEP);
+        }
+        if (KQ & 1) multiply_group<F32, MTL>(acc, v, aq);
+    }
+}
+
+// Bias is in the sums already.  Accumulator (r, j): rows 8 r + 2 t, + 1 of channels CH gr + 2 j (values 0, 1) and + 1
+// (values 2, 3); the first `n` rows are valid.
+template <bool F32, int MTL, bool RESIDUAL, bool SILU>
+__device__ __forceinline__ void store_rows(const float (&acc)[2][MTL][4], const Row* queue, int n, const ConvGeom& g, const DirectArgs& a,
+                                           int n0, int lane)
+{
+    constexpr int CH = 2 * MTL;                  // consecutive channels of a lane
+    const int t = lane & 3, gr = lane >> 2, N = g.C_out;
+    if (n0 + CH * gr >= N) return;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = 8 * (r >> 1) + 2 * t + (r & 1);
+        if (i >= n) continue;
+        const long long yoff = (long long)queue[i].x * N + n0 + CH * gr;
+        float f[CH];
+#pragma unroll
+        for (int c = 0; c < CH; ++c) f[c] = acc[r >> 1][c >> 1][(c & 1) * 2 + (r & 1)];
+        if (RESIDUAL) {
+            const __nv_bfloat16* rs = static_cast<const __nv_bfloat16*>(a.residual) + yoff;
+#pragma unroll
+            for (int c = 0; c < CH; c += 4) {
+                const uint2 q = __ldcg(reinterpret_cast<const uint2*>(rs + c));
+                f[c] += __uint_as_float(q.x << 16);
+                f[c + 1] += __uint_as_float(q.x & 0xffff0000u);
+                f[c + 2] += __uint_as_float(q.y << 16);
+                f[c + 3] += __uint_as_float(q.y & 0xffff0000u);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < CH; ++c) f[c] = SILU ? silu(f[c]) : a.relu ? fmaxf(f[c], 0.f) : f[c];
+        if (F32) {
+            float* yf = static_cast<float*>(a.y) + yoff;
+#pragma unroll
+            for (int c = 0; c < CH; c += 4)
+                if (n0 + CH * gr + c < N) *reinterpret_cast<float4*>(yf + c) = make_float4(f[c], f[c + 1], f[c + 2], f[c + 3]);
+        } else if (CH == 8) {
+            *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.y) + yoff) =
+                make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+        } else {
+            *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(a.y) + yoff) = make_uint2(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]));
+        }
+    }
+}
+
+// The first `n` (1 .. 16) queued rows.  Rows past them repeat the last one; they are not stored.
+template <bool F32, bool WORDS, int MTL, int KQT, bool RESIDUAL, bool SILU>
+__device__ __forceinline__ void compute_rows(const Row* queue, int n, const Tables& s, const ConvGeom& g, const DirectArgs& a, int n0, int lane)
+{
+    const int gr = lane >> 2;
+    float acc[2][MTL][4];
+#pragma unroll
+    for (int j = 0; j < MTL; ++j) {              // the sums start from the bias
+        const float2 b2 = *reinterpret_cast<const float2*>(s.bias + 2 * MTL * gr + 2 * j);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            acc[r][j][0] = acc[r][j][1] = b2.x;
+            acc[r][j][2] = acc[r][j][3] = b2.y;
+        }
+    }
+    const Row r0 = queue[gr < n ? gr : n - 1], r1 = queue[gr + 8 < n ? gr + 8 : n - 1];
+    const int2 row[2] = {make_int2(r0.y, r0.z), make_int2(r1.y, r1.z)};
+    const uint8_t* xb = static_cast<const uint8_t*>(a.x);
+    if (__all_sync(0xffffffffu, r0.w & r1.w)) multiply<F32, WORDS, false, MTL, KQT>(acc, row, s, g, a.KQ, xb, lane);
+    else multiply<F32, WORDS, true, MTL, KQT>(acc, row, s, g, a.KQ, xb, lane);
+    store_rows<F32, MTL, RESIDUAL, SILU>(acc, queue, n, g, a, n0, lane);
+}
+
+// Zeros for the dropped rows among row0 .. row0 + 31 (bit i of `drop`: row row0 + i), this block's columns.
+template <bool F32>
+__device__ __forceinline__ void zero_rows(unsigned drop, int row0, const ConvGeom& g, const DirectArgs& a, int n0, int ncols, int lane)
+{
+    constexpr int ES = F32 ? 4 : 2, EPC = 16 / ES;
+    uint8_t* yb = static_cast<uint8_t*>(a.y) + ((long long)row0 * g.C_out + n0) * ES;
+    const int units = (int)a.fdUnits.d;                     // 16-byte units of a row
+    if (a.lanes_per_row) {                                  // a power of two up to 32: every lane keeps its column
+        const int r0 = lane >> a.unit_shift, rows = 32 >> a.unit_shift;
+        yb += (long long)(r0 * g.C_out * ES + (lane & (units - 1)) * 16);
+        const int step = rows * g.C_out * ES;
+        drop >>= r0;
+#pragma unroll 4
+        for (int i = 0; i < units; ++i, yb += step, drop = rows < 32 ? drop >> rows : 0u)
+            if (drop & 1u) *reinterpret_cast<uint4*>(yb) = make_uint4(0, 0, 0, 0);
+        return;
+    }
+    for (int u = lane; u < 32 * units; u += 32) {
+        const int r = (int)fd_div((uint32_t)u, a.fdUnits), c = (u - r * units) * EPC;
+        if (((drop >> r) & 1u) && c < ncols) *reinterpret_cast<uint4*>(yb + ((long long)r * g.C_out + c) * ES) = make_uint4(0, 0, 0, 0);
+    }
+}
+
+template <bool F32, bool WORDS, int MTL, int KQT, bool RESIDUAL, bool SILU, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(const ConvGeom g, const DirectArgs a)
+{
+    extern __shared__ uint4 smem_v[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ptx::grid_launch_dependents();
+    int block = blockIdx.x;
+    if (a.kept_out != nullptr) {
+        if (block < a.list_blocks) {
+            if (blockIdx.y != 0) return;
+            ptx::grid_dependency_wait();           // an earlier kernel may still read the list
+            write_kept_list(a.mask, g.rows, block, a.kept_out, a.count_out);
+            return;
+        }
+        block -= a.list_blocks;
+    }
+    const int n0 = blockIdx.y * 16 * MTL;
+    const int ncols = g.C_out - n0 < 16 * MTL ? g.C_out - n0 : 16 * MTL;
+    Tables s;
+    s.b = smem_v;
+    s.bias = reinterpret_cast<float*>(s.b + (size_t)a.KQ * 2 * MTL * 32);
+    s.queue = reinterpret_cast<Row*>(s.bias + 16 * MTL);
+    s.pos = reinterpret_cast<int2*>(s.queue + WARPS * QUEUE);
+    fill_positions<F32, WORDS>(s, g, a);
+
+    const int first = block * a.block_rows, end = g.M - first < a.block_rows ? g.M : first + a.block_rows;
+    auto read_mask = [&](int row0) -> unsigned {            // masks are written by copies, never by a kernel
+        int p = row0 + lane;
+        if (p >= end) return 0;
+        if (g.rows == g.P) p -= (int)fd_div((uint32_t)p, a.fdP) * g.P;
+        return __ldg(a.mask + p);
+    };
+    int row0 = first + warp * CHUNK;
+    unsigned next = read_mask(row0);
+    ptx::grid_dependency_wait();
+    // The input is read through L1 (neighbouring windows overlap).  This block may have been launched while the
+    // kernel that wrote it was running; the fence drops whatever this SM's L1 still holds from before.
+    __threadfence();
+    load_filters<F32, WORDS, MTL>(s, g, a, n0);
+    __syncthreads();
+
+    Row* const queue = s.queue + warp * QUEUE;
+    int queued = 0;
+#pragma unroll 1
+    for (;; row0 += WARPS * CHUNK) {
+        const bool scan = row0 < end;
+        if (scan) {
+            const bool keep = next != 0;
+            next = read_mask(row0 + WARPS * CHUNK);         // in flight while this chunk is worked on
+            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+            const unsigned all = end - row0 < 32 ? (1u << (end - row0)) - 1u : 0xffffffffu;
+            if (keep) {
+                const int rw = row0 + lane;
+                const int img = (int)fd_div((uint32_t)rw, a.fdP), p = rw - img * g.P;
+                const int oy = (int)fd_div((uint32_t)p, a.fdWo), ox = p - oy * g.Wo;
+                const int iy0 = oy * g.stride - g.pad, ix0 = ox * g.stride - g.pad;
+                const int slack = WORDS ? 1 : 0;            // a filter row's first and last word may reach into the pixels beside it
+                const bool inner = iy0 >= 0 && iy0 + g.kh <= g.H && ix0 >= slack && ix0 + g.kw + slack <= g.W;
+                queue[queued + __popc(kept & ((1u << lane) - 1u))] =
+                    make_int4(rw, ((img * g.H + iy0) * g.W + ix0) * g.C_in, (iy0 << 16) | ((WORDS ? ix0 * g.C_in : ix0) & 0xffff), inner ? 1 : 0);
+            }
+            queued += __popc(kept);
+            if (all & ~kept) zero_rows<F32>(all & ~kept, row0, g, a, n0, ncols, lane);
+            __syncwarp();
+        }
+        // whole tiles, and behind the last chunk what is left
+        int done = 0;
+#pragma unroll 1
+        while (queued - done >= (scan ? 16 : 1)) {
+            const int n = queued - done < 16 ? queued - done : 16;
+            compute_rows<F32, WORDS, MTL, KQT, RESIDUAL, SILU>(queue + done, n, s, g, a, n0, lane);
+            done += n;
+        }
+        if (!scan) break;
+        if (done) {
+            queued -= done;                                 // fewer than a tile: to the front
+            const Row v = queue[done + (lane < queued ? lane : 0)];
+            __syncwarp();
+            if (lane < queued) queue[lane] = v;
+        }
+        __syncwarp();
+    }
+}
+
+}  // namespace
+
+bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan)
+{
+    const int epc = 16 / elem_bytes;
+    if (g.C_out % epc != 0) return false;                // 16-byte stores
+    plan->words = 0;
+    plan->shift = 0;
+    if (g.C_in % epc == 0) {
+        plan->KQ = (g.K + 4 * epc - 1) / (4 * epc);
+    } else {
+        // 4-byte words of a filter row: in bf16 the windows' rows must all start at the same parity of elements
+        if (elem_bytes == 2 && ((g.stride * g.C_in) % 2 != 0 || (g.W * g.C_in) % 2 != 0)) return false;
+        if (g.W * g.C_in > 32000 || g.kw * g.C_in > 1000) return false;
+        plan->shift = elem_bytes == 2 ? (g.pad * g.C_in) & 1 : 0;
+        plan->words = elem_bytes == 2 ? (g.kw * g.C_in + plan->shift + 1) / 2 : g.kw * g.C_in;
+        plan->KQ = (g.kh * plan->words + 15) / 16;
+    }
+    plan->NG = g.C_out <= 32 ? 1 : 2;
+    plan->n_tiles = (g.C_out + 32 * plan->NG - 1) / (32 * plan->NG);
+    plan->smem_bytes = plan->KQ * plan->NG * 2048 + 128 * plan->NG + plan->KQ * (plan->words ? 16 : 4) * 8 + WARPS * QUEUE * 16;
+    return plan->smem_bytes <= 112 * 1024 && plan->n_tiles < 65536;
+}
+
+// Measured against the tensor-memory forms on 147 layers (networks' layers and random ones, bf16 and fp32).  The k loop
+// here costs 35 clocks per operand group (32 K-elements of bf16) and 16 rows at up to 32 output channels, 80 at 64, the
+// hand-overs of the other forms about 2000 per 128 rows: up to four groups this form was 1.0-3.5 times as fast on all
+// layers, with up to 32 output channels also up to nine (1.0-1.6).  Channel counts that are no whole number of 16-byte chunks cost the
+// other forms a padded copy of the input, which moves the line: 1.1-4.3 times as fast up to ten groups once every SM has
+// some tiles to work on (0.91-1.02 below that).
+bool direct_pays(const DirectPlan& plan, int num_sms, int64_t kept_rows)
+{
+    if (plan.words == 0) return plan.KQ <= 4 || (plan.KQ <= 9 && plan.NG == 1);
+    return plan.KQ <= 4 || (plan.KQ <= 10 && kept_rows / 16 * plan.n_tiles >= 10ll * num_sms);
+}
+
+cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
+                          int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32, int num_sms, cudaStream_t st)
+{
+    DirectArgs a;
+    const int es = f32 ? 4 : 2, epc = 16 / es;
+    a.fdP = make_fastdiv((uint32_t)g.P);
+    a.fdWo = make_fastdiv((uint32_t)g.Wo);
+    const int cols = g.C_out < 32 * plan.NG ? g.C_out : 32 * plan.NG;
+    a.fdUnits = make_fastdiv((uint32_t)((cols + epc - 1) / epc));
+    a.fdChunks = make_fastdiv((uint32_t)((plan.words > 0 ? 16 : 4) * plan.KQ));
+    a.fdCin = make_fastdiv((uint32_t)g.C_in);
+    a.fdkw = make_fastdiv((uint32_t)g.kw);
+    a.fdWords = make_fastdiv((uint32_t)(plan.words > 0 ? plan.words : 1));
+    const int units = (int)a.fdUnits.d;
+    a.lanes_per_row = (units <= 32 && (units & (units - 1)) == 0 && g.C_out % (32 * plan.NG) == 0) || (plan.n_tiles == 1 && units <= 32 && (units & (units - 1)) == 0);
+    a.x = x;
+    a.w = w;
+    a.bias = bias;
+    a.y = y;
+    a.mask = mask;
+    a.residual = residual;
+    a.kept_out = kept_out;
+    a.list_blocks = kept_out != nullptr ? (g.rows + LIST_ROWS - 1) / LIST_ROWS : 0;
+    a.count_out = count_out;
+    a.relu = relu == 1 ? 1 : 0;
+    a.KQ = plan.KQ;
+    a.unit_shift = 0;
+    while ((1 << a.unit_shift) < units) ++a.unit_shift;
+    a.words = plan.words;
+    a.shift = plan.shift;
+
+    using Kern = void (*)(const ConvGeom, const DirectArgs);
+    // blocks per SM as the accumulators leave registers for: 85 a thread for three, 128 for two
+    const bool wd = plan.words != 0;
+    Kern kern;
+    int per_sm;
+    const bool res = residual != nullptr, is_silu = relu == 2;
+#define ASX_PICK3(F32, WD, MTL, KQT, BLOCKS)                                                                        \
+    (F32 || !res ? (is_silu ? masked_conv_direct_kernel<F32, WD, MTL, KQT, false, true, BLOCKS>                         \
+                            : masked_conv_direct_kernel<F32, WD, MTL, KQT, false, false, BLOCKS>)                       \
+                 : (is_silu ? masked_conv_direct_kernel<F32, WD, MTL, KQT, !F32, true, BLOCKS> : masked_conv_direct_kernel<F32, WD, MTL, KQT, !F32, false, BLOCKS>))
+#define ASX_PICK2(F32, WD, MTL, BLOCKS) \
+    (plan.KQ == 1 ? ASX_PICK3(F32, WD, MTL, 1, BLOCKS) : plan.KQ == 2 ? ASX_PICK3(F32, WD, MTL, 2, BLOCKS) : ASX_PICK3(F32, WD, MTL, 0, BLOCKS))
+#define ASX_PICK(MTL, BLOCKS)                                                                       \
+    per_sm = BLOCKS;                                                                                \
+    kern = f32 ? (wd ? ASX_PICK2(true, true, MTL, BLOCKS) : ASX_PICK2(true, false, MTL, BLOCKS))    \
+               : (wd ? ASX_PICK2(false, true, MTL, BLOCKS) : ASX_PICK2(false, false, MTL, BLOCKS))
+    if (plan.NG == 1) { ASX_PICK(2, 3); }
+    else { ASX_PICK(4, 2); }
+#undef ASX_PICK
+#undef ASX_PICK2
+#undef ASX_PICK3
+    const int fit = 226 * 1024 / (plan.smem_bytes + 1024);
+    if (fit < per_sm) per_sm = fit;
+    const long long chunks = ((long long)g.M + CHUNK - 1) / CHUNK;
+    long long slots = (long long)num_sms * per_sm / plan.n_tiles;
+    if (slots < 1) slots = 1;
+    const long long per = (chunks + slots - 1) / slots;
+    a.block_rows = (int)per * CHUNK;
+    const int grid = (int)((chunks + per - 1) / per) + a.list_blocks;
+    static std::atomic<int> smem_set[96];                // largest dynamic shared memory size enabled so far, per instance
+    const int vi = ((plan.KQ <= 2 ? plan.KQ : 0) * 2 + (plan.NG - 1)) * 16 + (f32 ? 8 : 0) + (wd ? 4 : 0) + (res ? 2 : 0) + (is_silu ? 1 : 0);
+    if (plan.smem_bytes > smem_set[vi].load(std::memory_order_relaxed)) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
+        if (e != cudaSuccess) return e;
+        smem_set[vi].store(plan.smem_bytes, std::memory_order_relaxed);
+    }
+    return launch_pdl(kern, dim3(grid, plan.n_tiles), dim3(THREADS), (size_t)plan.smem_bytes, st, g, a);
+}
+
+}  // namespace asx

@@ -1,0 +1,106 @@
+"""The direct form of the fused layer (operands gathered into registers, no kept-row list) against the CPU
+oracle at the sizes where it can go wrong: channel counts that are whole 16-byte chunks and words of four bytes,
+windows that reach over every edge, column ranges that end inside a 32- or 64-channel block, row counts around the
+16-row tiles, lists rebuilt by several blocks."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2309_06626_b200 as asx
+import workloads as wl
+from gpu_util import check_against_oracle, make_problem, to_dev_bf16
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # C_in, C_out, k, stride, pad, H, W, Nb, pct, block
+    (8, 8, 1, 1, 0, 9, 7, 2, 30, 1),            # one chunk of a group of four
+    (64, 32, 1, 1, 0, 16, 16, 2, 40, 2),        # two groups, all loaded first
+    (96, 40, 1, 2, 0, 15, 17, 3, 50, 4),        # three groups, columns end inside the block
+    (128, 136, 1, 1, 0, 12, 11, 2, 25, 1),      # four groups, three blocks of columns
+    (32, 32, 3, 1, 1, 14, 15, 2, 30, 1),        # nine groups, odd count
+    (24, 56, 3, 2, 1, 13, 12, 2, 50, 2),        # taps change inside a group
+    (3, 64, 7, 2, 3, 32, 30, 2, 50, 4),         # words, leading half word
+    (3, 32, 3, 2, 1, 18, 20, 1, 40, 2),
+    (4, 24, 5, 2, 2, 14, 16, 2, 30, 1),         # words without a leading half
+    (6, 16, 3, 1, 1, 10, 9, 2, 20, 1),
+    (2, 48, 4, 2, 1, 18, 22, 2, 25, 4),
+    (1, 8, 2, 2, 0, 16, 16, 3, 50, 1),
+]
+
+
+def _spec(c, seed=0):
+    cin, cout, k, s, p, H, W, Nb, pct, blk = c
+    return wl.LayerSpec("direct", cin, cout, k, k, s, p, H, W, Nb, pct, blk, "relu", wl.BASE_SEED + 8800 + seed)
+
+
+@pytest.mark.parametrize("per_row", [False, True])
+@pytest.mark.parametrize("case", CASES, ids=["-".join(map(str, c)) for c in CASES])
+def test_against_the_oracle(case, per_row):
+    spec = _spec(case)
+    x, w, b, mask = make_problem(spec, per_row=per_row)
+    for flags in (asx.ACT_RELU, asx.ACT_SILU | asx.RECOMPACT):
+        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT)
+    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT)
+
+
+@pytest.mark.parametrize("kept", [0, 1, 15, 16, 17, 33, "all"])
+def test_row_counts_around_a_tile(kept):
+    spec = _spec((32, 32, 3, 1, 1, 19, 21, 1, 0, 1))
+    x, w, b, _ = make_problem(spec)
+    mask = np.zeros(spec.P, np.uint8)
+    if kept == "all":
+        mask[:] = 1
+    else:
+        mask[np.random.default_rng(kept).permutation(spec.P)[:kept]] = 1
+    check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | asx.RECOMPACT | asx.IMPL_DIRECT)
+
+
+@pytest.mark.parametrize("cin,cout,k,s,p", [(3, 64, 7, 2, 3), (5, 12, 3, 1, 1), (32, 36, 1, 1, 0), (8, 32, 3, 1, 1)])
+def test_fp32_storage(cin, cout, k, s, p):
+    spec = _spec((cin, cout, k, s, p, 17, 19, 2, 40, 2), 1)
+    x, w = oracle.tf32_operand(wl.make_x(spec)), oracle.tf32_operand(wl.make_w(spec))
+    b, mask = wl.make_b(spec), wl.make_layer_mask(spec)
+    layer = asx.MaskedConvLayer(cin, cout, k, k, s, p)
+    layer.set_mask(mask)
+    y = layer.run(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda(),
+                  flags=asx.ACT_RELU | asx.F32 | asx.IMPL_DIRECT)
+    torch.cuda.synchronize()
+    assert layer.last_run_form() == asx.FORM_DIRECT
+    layer.close()
+    ref = oracle.masked_conv(x, w, b, mask, s, p, True, storage="fp32")
+    got = y.cpu().numpy().astype(np.float64).reshape(ref.shape)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 2e-4
+    assert not got.reshape(spec.M, -1)[np.tile(mask, spec.Nb) == 0].any()
+
+
+@pytest.mark.parametrize("rows_hw", [(64, 64), (65, 64), (130, 127)])
+def test_list_rebuilt_beside_the_convolution(rows_hw):
+    """Masks of one block, one row more and several blocks of the list."""
+    spec = _spec((8, 16, 1, 1, 0, *rows_hw, 1, 45, 1), 2)
+    x, w, b, mask = make_problem(spec)
+    layer = asx.MaskedConvLayer(8, 16, 1, 1, 1, 0)
+    layer.set_mask(mask)
+    layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.RECOMPACT)
+    assert layer.last_run_form() == asx.FORM_DIRECT                    # the library's own choice
+    assert np.array_equal(layer.kept(), oracle.kept_list(mask))
+    layer.close()
+
+
+def test_residual():
+    spec = _spec((64, 72, 1, 1, 0, 11, 13, 2, 30, 1), 3)
+    x, w, b, mask = make_problem(spec)
+    res = np.random.default_rng(3).standard_normal((spec.Nb, spec.Ho, spec.Wo, 72)).astype(np.float32)
+    rd = to_dev_bf16(res)
+    layer = asx.MaskedConvLayer(64, 72, 1, 1, 1, 0)
+    layer.set_mask(mask)
+    layer.set_residual(rd)
+    y = layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU)
+    torch.cuda.synchronize()
+    assert layer.last_run_form() == asx.FORM_DIRECT
+    layer.close()
+    ref = oracle.masked_conv(x, w, b, mask, 1, 0, False).reshape(spec.M, -1) + rd.float().cpu().numpy().reshape(spec.M, -1)
+    ref = np.maximum(ref, 0) * np.tile(mask, spec.Nb)[:, None]
+    got = y.float().cpu().numpy().reshape(spec.M, -1)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 5e-3
