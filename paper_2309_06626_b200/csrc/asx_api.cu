@@ -31,9 +31,7 @@ struct asx_layer {
     // staging copies with zero-padded channels, for C_in not a multiple of 8
     void* d_wpack = nullptr;
     size_t wpack_bytes = 0;
-    void* d_ws = nullptr;              // split-K workspace: fp32 partial tiles, then the tile counters
-    size_t ws_bytes = 0;
-    int* d_wscnt = nullptr;
+    int* d_wscnt = nullptr;            // shared k-blocks: two ints per output tile, zero unless a test sets one
     size_t wscnt_ints = 0;
     void* d_xpad = nullptr;
     size_t xpad_bytes = 0;
@@ -468,8 +466,11 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         return from_cuda(launch_direct(g, dplan, x, w, bias, y, L->d_mask, list ? L->d_kept : nullptr, list ? L->d_small : nullptr, relu, L->residual,
                                        f32 ? 1 : 0, L->num_sms, st));
     }
-    bool fuse_compact = (flags & ASX_RECOMPACT) && !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS;
-    if ((flags & ASX_RECOMPACT) && !fuse_compact) {
+    // Also without ASX_RECOMPACT: the list in global memory is behind the dependency wait (an earlier kernel may have
+    // written it), the mask is not.
+    const bool recompact = (flags & ASX_RECOMPACT) != 0;
+    bool fuse_compact = !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS;
+    if (recompact && !fuse_compact) {
         s = run_compaction(L, st);
         if (s != ASX_OK) return s;
     }
@@ -618,13 +619,15 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     if (L->host_kept >= 0) est_rows = (L->rows == P) ? L->host_kept * Nb : L->host_kept;
     // Sharing a tile's k-blocks between blocks needs the exact tile count (to size the workspace)
     // and 16-byte output stores.
-    const bool allow_split = !f32 && L->host_kept >= 0 && L->C_out % 8 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
+    const bool allow_split = L->host_kept >= 0 && L->C_out % 8 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
     if (!plan_fast(g, L->num_sms, est_rows, fuse_compact ? (int)L->rows : 0, allow_split, ES, &plan)) {
         if (!(fuse_compact && L->rows > COMPACT_SMALL_MAX_ROWS)) return ASX_ERR_UNSUPPORTED;
         // no room for the list beside the pipeline stages: the stand-alone compaction, and the list in global memory
         fuse_compact = false;
-        s = run_compaction(L, st);
-        if (s != ASX_OK) return s;
+        if (recompact) {
+            s = run_compaction(L, st);
+            if (s != ASX_OK) return s;
+        }
         if (!plan_fast(g, L->num_sms, est_rows, 0, allow_split, ES, &plan)) return ASX_ERR_UNSUPPORTED;
     }
     // Stride-1 layers with several filter taps and whole 64-channel slices take the window-patch form
@@ -681,14 +684,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         }
     }
     if (plan.ksplit > 1 && !use_patch) {
-        const size_t need = (size_t)plan.ws_items * 128 * (size_t)plan.BN * sizeof(float);
-        if (need > L->ws_bytes) {
-            cudaFree(L->d_ws);
-            L->d_ws = nullptr; L->ws_bytes = 0;
-            if (cudaMalloc(&L->d_ws, need) != cudaSuccess) return ASX_ERR_OOM;
-            L->ws_bytes = need;
-        }
-        const size_t ints = 2 * (size_t)(plan.ws_items / plan.ksplit);
+        const size_t ints = 2 * (size_t)(plan.items / plan.ksplit);
         if (ints > L->wscnt_ints) {
             cudaFree(L->d_wscnt);
             L->d_wscnt = nullptr; L->wscnt_ints = 0;
@@ -735,7 +731,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         }
         L->last_form = ASX_FORM_WINDOW_PATCH;
         return from_cuda(launch_patch(gp, pplan, L->tmap, L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
-                                      fuse_compact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
+                                      fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
                                       out_compact ? 1 : 0, L->wait_limit_kcycles, st));
     }
     if (plan.vec == 2) {
@@ -757,7 +753,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     L->last_form = plan.vec == 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
     return from_cuda(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
-                                 L->num_sms, fuse_compact ? 1 : 0, L->host_kept, static_cast<float*>(L->d_ws), L->d_wscnt,
+                                 L->num_sms, fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->d_wscnt,
                                  out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles, st));
 }
 
@@ -850,7 +846,7 @@ asx_status asx_destroy(asx_layer* L)
     if (L->device >= 0) {
         cudaStreamSynchronize(L->last_stream);
         cudaFree(L->d_mask); cudaFree(L->d_kept); cudaFree(L->d_scratch);
-        cudaFree(L->d_small); cudaFree(L->d_wpack); cudaFree(L->d_xpad); cudaFree(L->d_ws); cudaFree(L->d_wscnt); cudaFree(L->d_in_rank); cudaFree(L->d_tiles);
+        cudaFree(L->d_small); cudaFree(L->d_wpack); cudaFree(L->d_xpad); cudaFree(L->d_wscnt); cudaFree(L->d_in_rank); cudaFree(L->d_tiles);
     }
     delete L;
     return ASX_OK;

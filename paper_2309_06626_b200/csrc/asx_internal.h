@@ -21,24 +21,36 @@ struct ConvGeom {
 // Device status word values (bit flags), reported as ASX_ERR_TIMEOUT.
 enum : int { DEV_OK = 0, DEV_TIMEOUT_PIPE = 2, DEV_BAD_INDEX = 4 };
 
+// Set while this host thread launches kernels that read a layer's mask before their dependency wait although a kernel wrote
+// it (asx_set_mask with a device mask): the launch then waits for everything before it in the stream.
+inline thread_local bool launch_in_stream_order = false;
+
 // Launch with the programmatic-stream-serialization attribute: the kernel may begin while its
 // predecessor in the stream is still running and must execute griddepcontrol.wait before it
 // touches anything an earlier kernel produced (and before it writes anything one may still read).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args... args)
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st,
+                                      Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = launch_in_stream_order ? 0 : 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    return launch_pdl_cluster(kernel, grid, block, 1, smem, st, args...);
 }
 
 // ---- S1: mask compaction (compact.cu)
@@ -66,8 +78,9 @@ struct FastPlan {
     int smem_bytes;
     int vec;          // gather mode: 1 cp.async 16 B (a pixel's channels are whole 16-byte chunks), 2 TMA row
                       // gather (they are whole 128-byte runs)
-    int ksplit;       // work items per output tile (shares of the k-blocks); > 1 needs the workspace
-    long long ws_items;   // m_tiles * n_tiles * ksplit for the estimated kept rows
+    int ksplit;       // work items per output tile (shares of the k-blocks), the blocks of a cluster
+    long long items;  // m_tiles * n_tiles * ksplit for the estimated kept rows
+    int list_bytes;   // shared memory set aside for the fused compaction's list
     double est_cost_us;   // the planner's estimate of the launch's duration
 };
 // elem_bytes: 2 (bf16 storage) or 4 (fp32 storage, TF32 contraction)
@@ -76,7 +89,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
 cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorMap& tmap_w,
                         const CUtensorMap& tmap_x, const void* x, const float* bias, void* y, const uint8_t* mask,
                         const int32_t* kept, const int32_t* count, int relu, int* dev_status,
-                        int num_sms, int fuse_compact, long long host_kept, float* ws_partial, int* ws_counters,
+                        int num_sms, int fuse_compact, int write_list, long long host_kept, int* split_hook,
                         int out_compact, const int32_t* in_rank, int in_kept, const void* residual, int f32, int wait_limit_kcycles,
                         cudaStream_t st);
 // ---- the window-patch form of the tensor-core path (masked_conv_patch_sm100.cu): stride-1 layers with
@@ -102,7 +115,7 @@ void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, PatchPl
 // W counts units of four blocks (64 values)
 cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x4,
                          const float* bias, void* y, const uint8_t* mask, const int32_t* kept, const int32_t* count,
-                         int relu, int* dev_status, int num_sms, int fuse_compact, long long host_kept,
+                         int relu, int* dev_status, int num_sms, int fuse_compact, int write_list, long long host_kept,
                          const void* residual, const void* tiles, int n_mtiles, long long kept_rows, int out_compact,
                          int wait_limit_kcycles, cudaStream_t st);
 // ---- the direct form (masked_conv_direct.cu): small filter matrices, dense input and output

@@ -83,7 +83,8 @@ struct PatchArgs {
                         // row's box has, Wp8 the row pitch in blocks (a multiple of 32: rows start 1024-byte aligned)
     int slices;         // C_in / 64
     int G;              // filter taps per pipeline stage (a chunk); chunks = ceil(kh*kw / G) per slice
-    int fuse_compact;   // rebuild the kept-row list from the mask inside this kernel (small masks)
+    int fuse_compact;   // build the kept-row list from the mask inside this kernel (small masks)
+    int write_list;     // and write it to global memory
     int32_t* kept_out;
     int32_t* count_out;
     const __nv_bfloat16* residual;
@@ -341,7 +342,7 @@ masked_conv_patch_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const
     }
     if (a.fuse_compact) {
         ptx::grid_dependency_wait();
-        if (blockIdx.x == 0) {      // the list in global memory, for asx_get_kept and later runs
+        if (a.write_list && blockIdx.x == 0) {      // the list in global memory, for asx_get_kept and later runs
             for (int i = tid; i < cnt; i += WORK_THREADS) a.kept_out[i] = (int32_t)kept_s[i];
             if (tid == 0) *a.count_out = cnt;
         }
@@ -680,7 +681,7 @@ void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, PatchPl
 
 cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x4,
                          const float* bias, void* y, const uint8_t* mask, const int32_t* kept, const int32_t* count,
-                         int relu, int* dev_status, int num_sms, int fuse_compact, long long host_kept,
+                         int relu, int* dev_status, int num_sms, int fuse_compact, int write_list, long long host_kept,
                          const void* residual, const void* tiles, int n_mtiles, long long kept_rows, int out_compact,
                          int wait_limit_kcycles, cudaStream_t st)
 {
@@ -714,6 +715,7 @@ cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtenso
     a.epi8 = plan.epi8;
     a.slices = g.C_in / 64;
     a.fuse_compact = fuse_compact;
+    a.write_list = write_list;
     a.kept_out = const_cast<int32_t*>(kept);
     a.count_out = const_cast<int32_t*>(count);
     a.residual = static_cast<const __nv_bfloat16*>(residual);

@@ -22,6 +22,8 @@
 // in); either way the host never has to know the count.  Layers with few kept rows and a long
 // reduction may share a tile's k-blocks between blocks (split K with a fixed-order exchange).
 // All waits are bounded: a wait that runs out sets the status word and every role leaves.
+#include <algorithm>
+#include <atomic>
 #include <cuda_bf16.h>
 #include "asx_internal.h"
 #include "ptx_sm100.cuh"
@@ -50,6 +52,7 @@ struct FastArgs {
     FastDiv fdP, fdWo;           // divisions by P and Wo
     FastDiv fdNt;                // division by n_tiles
     FastDiv fdKs;                // division by ksplit
+    FastDiv fdGps;               // ksplit > 1: division by the 8-column groups per share
     FastDiv fdCin, fdkw, fdS;    // divisions by C_in, kw and the number of stages (cp.async gather)
     FastDiv fdcnt_host;          // division by the kept count when the host knows it (d = 0: it does not)
     const __nv_bfloat16* x;
@@ -63,7 +66,8 @@ struct FastArgs {
     int BN, n_tiles, stages, tmem_cols;
     int vec_out;        // C_out % 8 == 0 and y 16-byte aligned: 16-byte stores
     int st32;           // bf16, C_out % 16 == 0, y 32-byte aligned and the layer is paced by its stores: 32-byte epilogue stores
-    int fuse_compact;   // rebuild the kept-row list from the mask inside this kernel (small masks)
+    int fuse_compact;   // build the kept-row list from the mask inside this kernel (small masks)
+    int write_list;     // and write it to global memory
     int32_t* kept_out;  // where the fused compaction writes the list and its count
     int32_t* count_out;
     const __nv_bfloat16* residual;   // non-null: added to acc + bias before the activation, same layout as y
@@ -72,9 +76,10 @@ struct FastArgs {
                               // pos within its image's in_kept rows, or -1 for a dropped position (read as zeros)
     int in_kept;        // kept input positions per image
     int ksplit;         // work items per output tile: each takes a contiguous share of the k-blocks
-    float* ws_partial;  // ksplit > 1: [item][128][BN] fp32 partial tiles
-    int* ws_counters;   // ksplit > 1: per output tile {partials written, slices reduced}, zero between launches
-    int ws_items;       // capacity of ws_partial in items
+    int* split_hook;    // ksplit > 1: two ints per output tile, zero; a test makes a share wait for a partial sum that never comes
+                        // by setting the first
+    int split_items;    // ksplit > 1: the items the grid was sized for, one per block
+    int list_bytes;     // shared memory set aside for the fused compaction's list; the partial sums of the other shares follow
     int wait_limit_kcycles;   // bound of every wait in the kernel, in units of 1024 clock cycles
 };
 
@@ -87,6 +92,7 @@ struct alignas(16) Shared {           // lives after the operand stages
     unsigned long long empty[MAX_STAGES];
     unsigned long long acc_full[2];
     unsigned long long acc_empty[2];
+    unsigned long long partials;   // ksplit > 1: the other shares' partial sums have arrived
     unsigned int tmem_base;
     WaitCtl ctl;          // abort flag and the wait limit of this launch
     int scan_total[32];   // fused compaction: kept rows per warp
@@ -100,10 +106,11 @@ enum : int { GATHER_CPASYNC = 1, GATHER_TMA = 2 };
 struct Item {
     int tile, ks, m_tile, n_tile, kb_lo, kb_hi;
 };
+template <bool SPLIT>
 __device__ __forceinline__ Item item_of(int t, int KB, const FastArgs& a)
 {
     Item it;
-    if (a.ksplit == 1) {
+    if (!SPLIT) {
         it.tile = t;
         it.ks = 0;
         it.kb_lo = 0;
@@ -117,6 +124,14 @@ __device__ __forceinline__ Item item_of(int t, int KB, const FastArgs& a)
     it.m_tile = (int)fd_div((uint32_t)it.tile, a.fdNt);
     it.n_tile = it.tile - it.m_tile * a.n_tiles;
     return it;
+}
+
+// Rows of a tile that the TMA row gather fetches: the tile's kept rows in fours.  The rest of a last tile's stage keeps
+// what was there; a row of the product depends on its own row of the stage alone, and those are not stored.
+__device__ __forceinline__ int gathered_rows(int Mk, int m_tile)
+{
+    const int left = Mk - m_tile * BM;
+    return left < BM ? (left + 3) & ~3 : BM;
 }
 
 // What the gather warps need to know about the rk-th kept lowered row: the pixel index of its
@@ -150,7 +165,8 @@ __device__ __forceinline__ int2 row_info_of(int rk, int Mk, const FastDiv& fdcnt
 // (an instance of its own, like RESIDUAL: the plain path pays for every extra branch in the epilogue).
 // F32: x, w and y are fp32 (the storage type of Appendix A); a pipeline stage is still 128 rows of
 // 128 bytes, i.e. 32 K-elements, and the tensor core reads the operands as TF32.
-template <int MODE, bool IN_COMPACT, bool RESIDUAL, bool SILU, bool F32>
+// SPLIT: a.ksplit > 1 (an instance of its own as well: with the exchange in the plain one every launch took 0.8 us longer).
+template <int MODE, bool IN_COMPACT, bool RESIDUAL, bool SILU, bool F32, bool SPLIT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                          const ConvGeom g, const FastArgs a)
@@ -200,6 +216,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             ptx::mbar_init(ptx::smem_u32(bar), count);
             ptx::fence_mbar_init();
         }
+        if (SPLIT && tid == 32 * WARP_INFO) {
+            ptx::mbar_init(ptx::smem_u32(&sh->partials), 1);
+            ptx::fence_mbar_init();
+        }
         if (tid == 0) {
             sh->ctl.abort = 0;
             sh->ctl.limit_kcycles = a.wait_limit_kcycles;
@@ -217,6 +237,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = sh->tmem_base;
+    if (SPLIT) ptx::cluster_arrive();        // this block's barrier can take the others' partial sums
 
     int cnt = 0;
     KeptList kept_list{a.kept, nullptr};
@@ -235,8 +256,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     // With every position dropped there are no tiles; the zero warps then write the whole output
     // (Algorithm 2, mask == 0 branch).
     const int m_tiles = (Mk + BM - 1) / BM;
-    int total_tiles = m_tiles * a.n_tiles * a.ksplit;     // work items
-    if (a.ksplit > 1 && total_tiles > a.ws_items) {       // cannot happen when the host sized the workspace from this mask
+    int total_tiles = m_tiles * a.n_tiles * (SPLIT ? a.ksplit : 1);     // work items
+    if (SPLIT && total_tiles > a.split_items) {       // cannot happen when the host sized the grid from this mask
         if (tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);
         total_tiles = 0;
     }
@@ -250,16 +271,17 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             const int jj = idx / BM, rr = idx - jj * BM;
             const long long t = blockIdx.x + (long long)jj * gridDim.x;
             if (t < total_tiles)
-                sh->rowinfo[jj][rr] = row_info_of(item_of((int)t, KB, a).m_tile * BM + rr, Mk, fdcnt, g, a, kept_list);
+                sh->rowinfo[jj][rr] = row_info_of(item_of<SPLIT>((int)t, KB, a).m_tile * BM + rr, Mk, fdcnt, g, a, kept_list);
         }
         __syncthreads();
         if (tid < INFO_RING && blockIdx.x + (long long)tid * gridDim.x < total_tiles) ptx::mbar_arrive(ptx::smem_u32(&sh->info_full[tid]));
     }
+    if (SPLIT) ptx::cluster_wait();
     // From here on the kernel reads what earlier kernels wrote (the input, the filters) and writes
     // the output and the list, so it waits for them to have finished.
     if (a.fuse_compact) {
         ptx::grid_dependency_wait();
-        if (blockIdx.x == 0) {      // the list in global memory, for asx_get_kept and later runs
+        if (a.write_list && blockIdx.x == 0) {      // the list in global memory, for asx_get_kept and later runs
             for (int i = tid; i < cnt; i += NUM_THREADS) a.kept_out[i] = (int32_t)kept_s[i];
             if (tid == 0) *a.count_out = cnt;
         }
@@ -272,12 +294,13 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             uint32_t ph = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-                const Item item = item_of(t, KB, a);
+                const Item item = item_of<SPLIT>(t, KB, a);
                 const int n_tile = item.n_tile;
+                const int row_bytes = gathered_rows(Mk, item.m_tile) * BK * 2;
                 for (int kb = item.kb_lo; kb < item.kb_hi; ++kb) {
                     if (!wait_bar<40>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
                     const uint32_t full = ptx::smem_u32(&sh->full[s]);
-                    ptx::mbar_arrive_expect_tx(full, (uint32_t)(BN * BK * 2 + (MODE == GATHER_TMA ? A_STAGE_BYTES : 0)));
+                    ptx::mbar_arrive_expect_tx(full, (uint32_t)(BN * BK * 2 + (MODE == GATHER_TMA ? row_bytes : 0)));
                     ptx::tma_load_2d(smem_base + s * stage_bytes + A_STAGE_BYTES, &tmap_w, full, kb * BKE, n_tile * BN);
                     if (++s == S) { s = 0; ph ^= 1u; }
                 }
@@ -298,7 +321,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 good = wait_bar<200>(ptx::smem_u32(&sh->info_empty[r]), ((uint32_t)(j / INFO_RING) & 1u) ^ 1u, abort_flag, a.dev_status) ? 1 : 0;
             good = __shfl_sync(0xffffffffu, good, 0);
             if (!good) break;
-            const int m_tile = item_of((int)t, KB, a).m_tile;
+            const int m_tile = item_of<SPLIT>((int)t, KB, a).m_tile;
             // the four list entries first (with the list in global memory each is a trip to L2: one after the other
             // they were 2.7 us per tile, which paced every layer with one k-block per tile and a mask too large for
             // the fused compaction), then the arithmetic
@@ -330,7 +353,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             if (!ok) break;
             ptx::tc_fence_after_sync();
             const uint32_t d = tmem_base + (uint32_t)(buf * BN);
-            const Item item = item_of(t, KB, a);
+            const Item item = item_of<SPLIT>(t, KB, a);
             for (int kb = item.kb_lo; kb < item.kb_hi; ++kb) {
                 ok = warp_wait_bar<0>(ptx::smem_u32(&sh->full[s]), ph, abort_flag, a.dev_status);
                 if (!ok) break;
@@ -368,7 +391,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         int ti = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++ti) {
-            const Item item = item_of(t, KB, a);
+            const Item item = item_of<SPLIT>(t, KB, a);
             const int m_tile = item.m_tile, n_tile = item.n_tile;
             const int n0 = n_tile * BN;
             // kept rows from the accumulator
@@ -388,90 +411,76 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             if (!warp_wait_bar<100>(ptx::smem_u32(&sh->acc_full[buf]), use, abort_flag, a.dev_status)) { ok = false; break; }
             ptx::tc_fence_after_sync();
             const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            if (!F32 && a.ksplit > 1) {
-                // ---- split K: this item holds a partial sum.  Every share writes its partial tile
-                // to the workspace; when all shares of the tile are there, each share adds up the
-                // partials of its slice of the tile's rows, always in share order (so the result
-                // does not depend on which block finished first), and writes that slice of y.
-                const int et = (warp - WARP_EPI0) * 32 + lane;
-                // A partial tile is stored as [BN / 4 column groups][128 rows] float4, so that the
-                // warps (one row per lane) write and read whole consecutive lines.
-                float4* mine = reinterpret_cast<float4*>(a.ws_partial) + (size_t)t * (BN >> 2) * BM + (q * 32 + lane);
-                for (int c0 = 0; c0 < BN; c0 += 32) {
-                    uint32_t r[32];
-                    if (c0 + 32 <= BN) {
-                        ptx::tmem_ld_32(tacc + (uint32_t)c0, r);
-                    } else {
-                        uint32_t r16[16];
-                        ptx::tmem_ld_16(tacc + (uint32_t)c0, r16);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) { r[j] = r16[j]; r[16 + j] = 0; }
-                    }
-                    ptx::tmem_ld_wait();
-#pragma unroll
-                    for (int h = 0; h < 8; ++h)
-                        if (c0 + 4 * h < BN)
-                            __stcg(mine + (size_t)((c0 >> 2) + h) * BM,
-                                   make_float4(__uint_as_float(r[4 * h]), __uint_as_float(r[4 * h + 1]),
-                                               __uint_as_float(r[4 * h + 2]), __uint_as_float(r[4 * h + 3])));
+            if (SPLIT) {
+                // ---- split K: this item holds a partial sum.  The shares of a tile are the blocks of a cluster; share k
+                // finishes 8-column groups gps k .. gps k + gps - 1 of the tile (gps = ceil(groups / ksplit)).  Every share
+                // sends each other one its partial sums of that one's columns straight from its registers to that block's
+                // shared memory ([share][group][half][R rows] 16 bytes, R the tile's rows rounded up to whole warps; a bulk copy
+                // by the TMA unit from a staging area took 1.4 us to arrive, these stores 0.3), then adds what it received in
+                // share order (the result does not depend on which block finished first) and writes its columns of y.
+                const int KS = a.ksplit, gps = (int)a.fdGps.d, trow = q * 32 + lane;
+                const int left = Mk - m_tile * BM, R = left < BM ? (left + 31) & ~31 : BM;
+                const uint32_t recv = ptx::smem_u32(sh + 1) + (uint32_t)a.list_bytes;
+                const uint32_t recv_bar = ptx::smem_u32(&sh->partials);
+                const uint32_t half = (uint32_t)R * 16, slot = (uint32_t)gps * 2 * half;     // bytes of a half group and of a share's slice
+                if (warp == WARP_EPI0 && lane == 0) {
+                    // a test's hook makes this wait for more than is sent
+                    const int never = *reinterpret_cast<volatile int*>(a.split_hook + 2 * item.tile) != 0 ? 16 : 0;
+                    const int groups = (BN >> 3) - item.ks * gps < gps ? (BN >> 3) - item.ks * gps : gps;
+                    ptx::mbar_arrive_expect_tx(recv_bar, (uint32_t)((KS - 1) * groups) * 2 * half + (uint32_t)never);
                 }
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->acc_empty[buf]));     // the accumulator is free again
-                int* counters = a.ws_counters + 2 * item.tile;
-                __threadfence();
-                asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
-                if (et == 0) {
-                    atomicAdd(counters, 1);
-                    const long long t0 = clock64();
-                    while (*reinterpret_cast<volatile int*>(counters) < a.ksplit) {
-                        if (abort_flag->abort) break;
-                        if (clock64() - t0 > ((long long)abort_flag->limit_kcycles << 10)) {
-                            abort_flag->abort = 1;
-                            atomicOr(a.dev_status, DEV_TIMEOUT_PIPE);
-                            break;
+                if (q * 32 < R) {
+                    const uint32_t mine = recv + (uint32_t)item.ks * slot + (uint32_t)trow * 16;
+                    for (int c0 = 0; c0 < BN; c0 += 32) {
+                        uint32_t r[32];
+                        if (c0 + 32 <= BN) {
+                            ptx::tmem_ld_32(tacc + (uint32_t)c0, r);
+                        } else {
+                            uint32_t r16[16];
+                            ptx::tmem_ld_16(tacc + (uint32_t)c0, r16);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) { r[j] = r16[j]; r[16 + j] = 0; }
                         }
-                        __nanosleep(64);
-                    }
-                    __threadfence();
-                }
-                asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
-                if (abort_flag->abort) { ok = false; break; }
-                // this share's slice: 8-column groups [g_lo, g_hi) of all 128 rows, one row per lane
-                const int G = BN >> 3;
-                const int g_lo = item.ks * G / a.ksplit, g_hi = (item.ks + 1) * G / a.ksplit;
-                const float4* __restrict__ tile_ws = reinterpret_cast<const float4*>(a.ws_partial) + (size_t)item.tile * a.ksplit * (BN >> 2) * BM;
-                uint4* __restrict__ yv = reinterpret_cast<uint4*>(a.y);
-                const int rk2 = m_tile * BM + et;              // NUM_EPI_WARPS * 32 == BM: thread et owns row et
-                const long long yrow = rk2 < Mk ? (long long)(a.out_compact ? rk2 : out_row_of(rk2, fdcnt, g, kept_list)) * N : -1;
-#pragma unroll 2
-                for (int gq = g_lo; gq < g_hi; ++gq) {
-                    if (yrow < 0 || n0 + gq * 8 >= N) continue;
-                    float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
-                    for (int sp0 = 0; sp0 < a.ksplit; sp0 += 4) {
-                        float4 pl[4], phh[4];
+                        ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int d2 = 0; d2 < 4; ++d2) {
-                            const int sp = sp0 + d2;
-                            if (sp < a.ksplit) {
-                                const float4* src = tile_ws + ((size_t)sp * (BN >> 2) + 2 * gq) * BM + et;
-                                pl[d2] = __ldcg(src);
-                                phh[d2] = __ldcg(src + BM);
+                        for (int h = 0; h < 4; ++h) {
+                            const int gq = (c0 >> 3) + h;
+                            if (c0 + 8 * h >= BN) break;
+                            const int dst = (int)fd_div((uint32_t)gq, a.fdGps);
+                            const uint32_t at = mine + (uint32_t)(gq - dst * gps) * 2 * half;
+                            if (dst == item.ks) {
+                                ptx::st_shared_v4(at, r[8 * h], r[8 * h + 1], r[8 * h + 2], r[8 * h + 3]);
+                                ptx::st_shared_v4(at + half, r[8 * h + 4], r[8 * h + 5], r[8 * h + 6], r[8 * h + 7]);
                             } else {
-                                pl[d2] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                phh[d2] = pl[d2];
+                                const uint32_t to = ptx::cluster_map(at, (uint32_t)dst), to_bar = ptx::cluster_map(recv_bar, (uint32_t)dst);
+                                ptx::st_cluster_v4(to, to_bar, r[8 * h], r[8 * h + 1], r[8 * h + 2], r[8 * h + 3]);
+                                ptx::st_cluster_v4(to + half, to_bar, r[8 * h + 4], r[8 * h + 5], r[8 * h + 6], r[8 * h + 7]);
                             }
                         }
-#pragma unroll
-                        for (int d2 = 0; d2 < 4; ++d2) {          // always in share order
-                            lo4.x += pl[d2].x; lo4.y += pl[d2].y; lo4.z += pl[d2].z; lo4.w += pl[d2].w;
-                            hi4.x += phh[d2].x; hi4.y += phh[d2].y; hi4.z += phh[d2].z; hi4.w += phh[d2].w;
-                        }
                     }
-                    float v[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
+                }
+                ptx::tc_fence_before_sync();
+                if (!warp_wait_bar<20>(recv_bar, 0u, abort_flag, a.dev_status)) { ok = false; break; }
+                ptx::fence_cluster();
+                if (!valid) continue;
+                for (int gl = 0; gl < gps; ++gl) {
+                    const int gq = item.ks * gps + gl;
+                    if (gq * 8 >= BN || n0 + gq * 8 >= N) break;
+                    float v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = 0.f;
+                    uint32_t src = recv + (uint32_t)gl * 2 * half + (uint32_t)trow * 16;
+#pragma unroll 4
+                    for (int sp = 0; sp < KS; ++sp, src += slot) {                   // always in share order
+                        uint32_t p[8];
+                        ptx::ld_shared_v4(src, p[0], p[1], p[2], p[3]);
+                        ptx::ld_shared_v4(src + half, p[4], p[5], p[6], p[7]);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(p[j]);
+                    }
                     if (RESIDUAL) {
                         float res[8];
-                        load_residual8(a.residual, yrow + n0 + gq * 8, 8, 1, res);
+                        load_residual8(a.residual, yoff + n0 + gq * 8, 8, 1, res);
 #pragma unroll
                         for (int j = 0; j < 8; ++j) v[j] += res[j];
                     }
@@ -480,22 +489,16 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                         const float f = v[j] + sbias[gq * 8 + j];
                         v[j] = SILU ? silu(f) : a.relu ? fmaxf(f, 0.f) : f;
                     }
-                    uint4 o;
-                    o.x = pack_bf16(v[0], v[1]);
-                    o.y = pack_bf16(v[2], v[3]);
-                    o.z = pack_bf16(v[4], v[5]);
-                    o.w = pack_bf16(v[6], v[7]);
-                    yv[(yrow + n0 + gq * 8) >> 3] = o;
-                }
-                asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
-                if (et == 0) {
-                    // the last share to finish its slice puts the tile's counters back to zero
-                    if (atomicAdd(counters + 1, 1) == a.ksplit - 1) {
-                        atomicExch(counters, 0);
-                        atomicExch(counters + 1, 0);
+                    if (F32) {
+                        float4* yv = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.y) + yoff + n0 + gq * 8);
+                        yv[0] = make_float4(v[0], v[1], v[2], v[3]);
+                        yv[1] = make_float4(v[4], v[5], v[6], v[7]);
+                    } else {
+                        *reinterpret_cast<uint4*>(y2 + yoff + n0 + gq * 8) =
+                            make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
                     }
                 }
-                continue;
+                continue;                                         // one item per block: nobody waits for the accumulator
             }
             for (int c0 = 0; c0 < BN; c0 += 32) {
                 const int col0 = n0 + c0;
@@ -603,7 +606,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                     const int pix[4] = {ra.x, ra.z, rb.x, rb.z}, yx[4] = {ra.y, ra.w, rb.y, rb.w};
                     __syncwarp(0xfu);
                     if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->info_empty[r]));    // the ring slot is in registers now
-                    const Item item = item_of(t, KB, a);
+                    const Item item = item_of<SPLIT>(t, KB, a);
+                    const bool fetch = 16 * pwg + 4 * lane < gathered_rows(Mk, item.m_tile);
                     int ky = 0, kx = 0, ci = 0;
                     if (item.kb_lo != 0) {                 // a later k share starts inside the window
                         const int tap = item.kb_lo * BKE / g.C_in;
@@ -646,7 +650,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                                 }
                             }
                             if (!wait_bar<20>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
-                            ptx::tma_gather4_2d(smem_base + s * stage_bytes + (uint32_t)(16 * pwg + 4 * lane) * 128u, &tmap_x,
+                            if (fetch) ptx::tma_gather4_2d(smem_base + s * stage_bytes + (uint32_t)(16 * pwg + 4 * lane) * 128u, &tmap_x,
                                                 ptx::smem_u32(&sh->full[s]), ci, idx[0], idx[1], idx[2], idx[3]);
                             if (IN_COMPACT && kb + 2 < item.kb_hi) request_ranks(kb + 2);
                         }
@@ -687,7 +691,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->info_empty[r]));    // the ring slot is in registers now
 
-                const Item item = item_of(t, KB, a);
+                const Item item = item_of<SPLIT>(t, KB, a);
                 const int kb0 = item.kb_lo + (int)((it0 ^ (uint32_t)grp) & 1u);          // this group's first k-block of the tile
                 // window position (filter tap, channel) of this lane's chunk in k-block kb0
                 int tap, ci;
@@ -735,6 +739,12 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         __syncwarp();
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
+    }
+    // Another share may still send to this block's shared memory when this one has given up a wait.  Every block gets
+    // here, because every wait is bounded.
+    if (SPLIT) {
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait();
     }
 }
 
@@ -886,6 +896,43 @@ __global__ void __launch_bounds__(128) stage_blocks2x2_kernel(const unsigned sho
 
 }  // namespace
 
+namespace {
+// Sharing k-blocks: fewest k-blocks of a tile, and what the exchange costs beside the bytes.
+constexpr int SPLIT_MIN_KB = 12;
+constexpr double SPLIT_US = 2.5;
+// Blocks in clusters of KS (one block per SM) that find a place on the device at a time; asked once per size.
+int cluster_room(int KS)
+{
+    static std::atomic<int> known[9];
+    int room = known[KS].load(std::memory_order_relaxed);
+    if (room == 0) {
+        constexpr int bytes = 200 * 1024;
+        auto kern = masked_conv_sm100_kernel<GATHER_TMA, false, false, false, false, true>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(KS * 64));
+        cfg.blockDim = dim3(NUM_THREADS);
+        cfg.dynamicSmemBytes = bytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)KS;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            clusters = 148 / KS * 3 / 4;
+        }
+        room = clusters * KS;
+        known[KS].store(room, std::memory_order_relaxed);
+    }
+    return room;
+}
+// Shared memory for the partial sums that a share receives.
+int split_bytes(int BN, int KS) { return KS > 1 ? KS * ((BN / 8 + KS - 1) / KS) * 2 * BM * 16 : 0; }
+}  // namespace
+
 bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fused_list_rows, bool allow_split, int elem_bytes,
                FastPlan* plan)
 {
@@ -893,50 +940,61 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const int bke = 128 / elem_bytes;             // K elements per stage: 64 bf16 or 32 fp32
     const int KB = (g.K + bke - 1) / bke;
     const long long m_tiles = (est_kept_rows + BM - 1) / BM > 0 ? (est_kept_rows + BM - 1) / BM : 1;
+    if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
+    const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
+    const int fixed = 1024 + (int)sizeof(Shared) + list_bytes;
     // Tile width and k shares.  A wider tile does more work per gathered byte, a narrower one
-    // gives more tiles when a layer has few kept rows, and sharing a tile's k-blocks between
-    // blocks gives more work items still, at the price of exchanging fp32 partial tiles.  Pick
+    // gives more tiles when a layer has few kept rows, and sharing a tile's k-blocks between the blocks of a
+    // cluster gives more work items still, at the price of exchanging fp32 partial tiles.  Pick
     // the pair with the lowest estimated time, from figures measured on B200: a 64-wide k-block
     // of a 128 x BN tile takes about 0.30 + 0.001 BN microseconds (the loop is bound by the TMA
     // requests and bytes one SM can pull from L2: 16 KB of gathered rows in 32 requests of about
     // 13 clocks, plus the BN x 128-byte filter slab), the last tile's epilogue about 0.012 BN,
-    // and the exchange of partial tiles about 7 + 0.025 BN (a chain of write, fence, counter and
-    // read latencies).  Sharing pays where there are far fewer tiles than SMs and K is long.
+    // and the exchange SPLIT_US (cluster barriers, BN x 512 bytes through distributed shared memory in and out).
+    // A shared tile is its block's only one.  Clusters have an even size: SMs come in pairs (144 blocks in clusters of
+    // three ran in two waves).
     int best_BN = 0, best_KS = 1;
     double best_cost = 0.0;
-    for (int n_tiles = (N + 255) / 256; ; n_tiles *= 2) {
+    const double fill = std::min(1.0, (double)est_kept_rows / (double)(m_tiles * BM));       // rows gathered of a tile's 128
+    int halving = (N + 255) / 256;                // tile widths of whole tiles: 256 or less, then halves
+    for (int n_tiles = halving; ; ++n_tiles) {
         const int per = (N + n_tiles - 1) / n_tiles;
         const int BN = ((per + 15) / 16) * 16;
         const int nt = (N + BN - 1) / BN;
-        const double t_kb = 0.30 + 0.001 * BN;                                // microseconds
-        for (int KS = 1; KS <= (allow_split ? 8 : 1); ++KS) {
-            if (KS > 1 && KB / KS < 4) break;
+        const double t_kb = 0.12 + 0.18 * fill + 0.001 * BN;                  // microseconds
+        const bool whole = n_tiles == halving;
+        if (whole) halving *= 2;
+        for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); KS += KS == 1 ? 1 : 2) {
+            const int gps = (BN / 8 + KS - 1) / KS;
+            if (KS > 1 && (KB / KS < 2 || (KS - 1) * gps >= BN / 8)) continue;       // every share finishes some columns
+            if (227 * 1024 - fixed - split_bytes(BN, KS) < MIN_STAGES * (A_STAGE_BYTES + BN * BK * 2)) continue;
             const long long items = m_tiles * nt * KS;
-            const long long waves = (items + num_sms - 1) / num_sms;
+            const int room = KS == 1 ? num_sms : cluster_room(KS);
+            if (KS > 1 && items > room) continue;
+            const long long waves = (items + room - 1) / room;
             const int kbi = (KB + KS - 1) / KS;
-            const double cost = (double)waves * (kbi * t_kb + 0.3) + 0.012 * BN + (KS > 1 ? 7.0 + 0.025 * BN : 0.0);
+            // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
+            const double cost = (double)waves * (kbi * t_kb + 0.3) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
             if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_cost = cost; }
         }
-        if (BN <= 64) break;
+        if (BN <= 64 && whole) break;
     }
+    if (best_BN == 0) return false;
     const int BN = best_BN;
     const int n_tiles = (N + BN - 1) / BN;
     const int stage_bytes = A_STAGE_BYTES + BN * BK * 2;
-    const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
-    const int budget = 227 * 1024 - 1024 - (int)sizeof(Shared) - list_bytes;
-    int S = budget / stage_bytes;
+    int S = (227 * 1024 - fixed - split_bytes(BN, best_KS)) / stage_bytes;
     if (S > MAX_STAGES) S = MAX_STAGES;
-    if (S < MIN_STAGES) return false;
     plan->BN = BN;
     plan->n_tiles = n_tiles;
     plan->ksplit = best_KS;
     plan->est_cost_us = best_cost;
-    plan->ws_items = (long long)m_tiles * n_tiles * best_KS;
+    plan->items = (long long)m_tiles * n_tiles * best_KS;
     plan->stages = S;
-    int smem = 1024 + S * stage_bytes + (int)sizeof(Shared) + list_bytes;
+    plan->list_bytes = list_bytes;
+    int smem = fixed + S * stage_bytes + split_bytes(BN, best_KS);
     if (smem < 120 * 1024) smem = 120 * 1024;      // one block per SM: tensor memory is not shared out
     plan->smem_bytes = smem;
-    if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
     plan->vec = (g.C_in % bke == 0) ? GATHER_TMA : GATHER_CPASYNC;
     return true;
 }
@@ -944,11 +1002,11 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
 cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorMap& tmap_w,
                         const CUtensorMap& tmap_x, const void* x, const float* bias, void* y, const uint8_t* mask,
                         const int32_t* kept, const int32_t* count, int relu, int* dev_status,
-                        int num_sms, int fuse_compact, long long host_kept, float* ws_partial, int* ws_counters,
+                        int num_sms, int fuse_compact, int write_list, long long host_kept, int* split_hook,
                         int out_compact, const int32_t* in_rank, int in_kept, const void* residual, int f32, int wait_limit_kcycles,
                         cudaStream_t st)
 {
-    if (f32 && (in_rank != nullptr || residual != nullptr || plan.ksplit != 1)) return cudaErrorInvalidValue;
+    if (f32 && (in_rank != nullptr || residual != nullptr)) return cudaErrorInvalidValue;
     FastArgs a;
     a.fdcnt_host = make_fastdiv((uint32_t)(host_kept > 0 && host_kept < (1ll << 31) ? host_kept : 1));
     if (!(host_kept > 0 && host_kept < (1ll << 31))) a.fdcnt_host.d = 0;
@@ -977,9 +1035,11 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
     a.fdkw = make_fastdiv((uint32_t)g.kw);
     a.fdS = make_fastdiv((uint32_t)plan.stages);
     a.fdKs = make_fastdiv((uint32_t)plan.ksplit);
-    a.ws_partial = ws_partial;
-    a.ws_counters = ws_counters;
-    a.ws_items = (int)plan.ws_items;
+    a.fdGps = make_fastdiv((uint32_t)((plan.BN / 8 + plan.ksplit - 1) / plan.ksplit));
+    a.split_hook = split_hook;
+    a.split_items = (int)plan.items;
+    a.list_bytes = plan.list_bytes;
+    a.write_list = write_list;
     a.wait_limit_kcycles = wait_limit_kcycles > 0 ? wait_limit_kcycles : WAIT_LIMIT_KCYCLES_DEFAULT;
     a.stages = plan.stages;
     int cols = 32;
@@ -991,33 +1051,40 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
     a.st32 = (!f32 && a.vec_out && g.C_out % 16 == 0 && plan.BN % 16 == 0 && (reinterpret_cast<uintptr_t>(y) & 31) == 0 &&
               plan.ksplit == 1 && out_compact == 0) ? 1 : 0;
 
-    long long tiles = ((long long)g.M + BM - 1) / BM * plan.n_tiles * plan.ksplit;
-    int grid = (int)(tiles < num_sms ? tiles : num_sms);
+    // Shared k-blocks: one item per block (the host knows the count).  Else as many resident blocks as there may be items.
+    const bool split = plan.ksplit > 1;
+    long long tiles = split ? plan.items : ((long long)g.M + BM - 1) / BM * plan.n_tiles;
+    int grid = (int)(split || tiles < num_sms ? tiles : num_sms);
     if (grid < 1) grid = 1;
     const int variant = plan.vec + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
     const bool has_res = residual != nullptr, is_silu = relu == 2;
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const FastArgs);
     Kern kern = nullptr;
-#define ASX_PICK(MODE, IC)                                                                                          \
-    kern = has_res ? (is_silu ? masked_conv_sm100_kernel<MODE, IC, true, true, false> : masked_conv_sm100_kernel<MODE, IC, true, false, false>) \
-                   : (is_silu ? masked_conv_sm100_kernel<MODE, IC, false, true, false> : masked_conv_sm100_kernel<MODE, IC, false, false, false>)
+#define ASX_PICK2(MODE, IC, SPLIT)                                                                                              \
+    (has_res ? (is_silu ? masked_conv_sm100_kernel<MODE, IC, true, true, false, SPLIT> : masked_conv_sm100_kernel<MODE, IC, true, false, false, SPLIT>) \
+             : (is_silu ? masked_conv_sm100_kernel<MODE, IC, false, true, false, SPLIT> : masked_conv_sm100_kernel<MODE, IC, false, false, false, SPLIT>))
+#define ASX_PICK_F32(MODE, SPLIT) \
+    (is_silu ? masked_conv_sm100_kernel<MODE, false, false, true, true, SPLIT> : masked_conv_sm100_kernel<MODE, false, false, false, true, SPLIT>)
+#define ASX_PICK(WHICH, ...) kern = split ? WHICH(__VA_ARGS__, true) : WHICH(__VA_ARGS__, false)
     if (f32) {      // fp32 storage: dense input, no residual
-        if (variant == 2) kern = is_silu ? masked_conv_sm100_kernel<GATHER_TMA, false, false, true, true> : masked_conv_sm100_kernel<GATHER_TMA, false, false, false, true>;
-        else kern = is_silu ? masked_conv_sm100_kernel<GATHER_CPASYNC, false, false, true, true> : masked_conv_sm100_kernel<GATHER_CPASYNC, false, false, false, true>;
+        if (variant == 2) { ASX_PICK(ASX_PICK_F32, GATHER_TMA); }
+        else { ASX_PICK(ASX_PICK_F32, GATHER_CPASYNC); }
     }
-    else if (variant == 2) { ASX_PICK(GATHER_TMA, false); }
-    else if (variant == 1) { ASX_PICK(GATHER_CPASYNC, false); }
-    else if (variant == 4) { ASX_PICK(GATHER_TMA, true); }
-    else { ASX_PICK(GATHER_CPASYNC, true); }
+    else if (variant == 2) { ASX_PICK(ASX_PICK2, GATHER_TMA, false); }
+    else if (variant == 1) { ASX_PICK(ASX_PICK2, GATHER_CPASYNC, false); }
+    else if (variant == 4) { ASX_PICK(ASX_PICK2, GATHER_TMA, true); }
+    else { ASX_PICK(ASX_PICK2, GATHER_CPASYNC, true); }
+#undef ASX_PICK2
+#undef ASX_PICK_F32
 #undef ASX_PICK
-    static int smem_set_all[40] = {0};          // largest dynamic shared memory size enabled so far, per instance
-    int* smem_set = smem_set_all + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0);
+    static int smem_set_all[80] = {0};          // largest dynamic shared memory size enabled so far, per instance
+    int* smem_set = smem_set_all + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0) + (split ? 40 : 0);
     if (plan.smem_bytes > smem_set[variant]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
         if (e != cudaSuccess) return e;
         smem_set[variant] = plan.smem_bytes;
     }
-    return launch_pdl(kern, dim3(grid), dim3(NUM_THREADS), (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
+    return launch_pdl_cluster(kern, dim3(grid), dim3(NUM_THREADS), plan.ksplit, (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
 }
 
 cudaError_t launch_pad_channels(const void* src, void* dst, long long rows, int C, int Cp, cudaStream_t st)
