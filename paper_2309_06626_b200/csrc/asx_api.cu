@@ -394,8 +394,8 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 {
     if (L == nullptr || x == nullptr || w == nullptr || y == nullptr) return ASX_ERR_INVALID_ARG;
     if (Nb < 1 || H < 1 || W < 1) return ASX_ERR_INVALID_ARG;
-    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT)) return ASX_ERR_INVALID_ARG;
-    if (((flags & ASX_IMPL_ROW_GATHER) != 0) + ((flags & ASX_IMPL_WINDOW_PATCH) != 0) + ((flags & ASX_IMPL_DIRECT) != 0) > 1) return ASX_ERR_INVALID_ARG;
+    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K)) return ASX_ERR_INVALID_ARG;
+    if (((flags & ASX_IMPL_ROW_GATHER) != 0) + ((flags & ASX_IMPL_WINDOW_PATCH) != 0) + ((flags & ASX_IMPL_DIRECT) != 0) + ((flags & ASX_IMPL_DIRECT_K) != 0) > 1) return ASX_ERR_INVALID_ARG;
     const bool f32 = (flags & ASX_F32) != 0;
     const int ES = f32 ? 4 : 2;                 // bytes per element of x, w and y
     const int EPC = 16 / ES;                    // elements per 16-byte chunk
@@ -452,13 +452,41 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
     // leaves the plan its pipeline stages (decided below, once the geometry the kernel sees is known).
     const int relu = (flags & ASX_ACT_SILU) ? 2 : (flags & ASX_ACT_RELU) ? 1 : 0;      // activation code: 0 identity, 1 ReLU, 2 SiLU
-    // Small filter matrices take the direct form, which needs no list and rebuilds it beside the convolution when asked to.
+    // Small filter matrices take the direct form, which needs no list and rebuilds it beside the convolution when asked to;
+    // few kept rows the direct form whose warps share the k range.
+    const int impl = flags & (ASX_IMPL_NAIVE | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K);
+    const int64_t known_rows = L->host_kept < 0 ? -1 : L->rows == P ? L->host_kept * Nb : L->host_kept;      // kept lowered rows, when the host knows
+    const bool recompact = (flags & ASX_RECOMPACT) != 0, dense = !in_compact && !out_compact;
     DirectPlan dplan;
-    const int impl = flags & (ASX_IMPL_NAIVE | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT);
-    if (!in_compact && !out_compact && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) &&
-        (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, L->host_kept < 0 ? M : L->rows == P ? L->host_kept * Nb : L->host_kept))) {
-        const bool list = (flags & ASX_RECOMPACT) && L->rows <= DIRECT_LIST_MAX_ROWS;
-        if ((flags & ASX_RECOMPACT) && !list) {
+    DirectKPlan kplan;
+    const bool direct = dense && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) &&
+                        (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, known_rows < 0 ? M : known_rows));
+    bool direct_k = dense && (impl == 0 || impl == ASX_IMPL_DIRECT_K) && plan_direct_k(g, ES, known_rows, L->num_sms, &kplan);
+    if (direct_k && impl == 0) {
+        // against what would run else: the estimates of a tensor-memory form leave out 4.5 us of a launch's set-up and ends
+        double other;
+        if (direct) {
+            other = direct_est_us(dplan, L->num_sms, known_rows, ES);
+        } else {
+            FastPlan fp;
+            PatchPlan pp;
+            other = plan_fast(g, L->num_sms, known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp) ? fp.est_cost_us : 1e9;
+            if (!f32 && plan_patch(g, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
+                plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, &pp);
+                other = std::min(other, pp.est_cost_us);
+            }
+            other += 4.5;
+        }
+        direct_k = kplan.est_us < 0.95 * other;
+    }
+    if (direct_k) {
+        L->last_form = ASX_FORM_DIRECT_K;
+        return from_cuda(launch_direct_k(g, kplan, x, w, bias, y, L->d_mask, recompact ? L->d_kept : nullptr, L->d_small, L->host_kept, relu, L->residual,
+                                         f32 ? 1 : 0, reinterpret_cast<int*>(L->d_small + 1), st));
+    }
+    if (direct) {
+        const bool list = recompact && L->rows <= DIRECT_LIST_MAX_ROWS;
+        if (recompact && !list) {
             s = run_compaction(L, st);
             if (s != ASX_OK) return s;
         }
@@ -468,7 +496,6 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     // Also without ASX_RECOMPACT: the list in global memory is behind the dependency wait (an earlier kernel may have
     // written it), the mask is not.
-    const bool recompact = (flags & ASX_RECOMPACT) != 0;
     bool fuse_compact = !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS;
     if (recompact && !fuse_compact) {
         s = run_compaction(L, st);

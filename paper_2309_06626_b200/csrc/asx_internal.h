@@ -130,9 +130,21 @@ bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan);
 constexpr int64_t DIRECT_LIST_MAX_ROWS = 1 << 17;       // longest list it rebuilds itself
 // whether a layer with `kept_rows` kept lowered rows is faster here than in the tensor-memory forms
 bool direct_pays(const DirectPlan& plan, int num_sms, int64_t kept_rows);
+double direct_est_us(const DirectPlan& plan, int num_sms, int64_t kept_rows, int elem_bytes);      // of a launch among others
 // kept_out, count_out: where the kept-row list is rebuilt beside the convolution, or null
 cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
                           int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32, int num_sms, cudaStream_t st);
+// ---- the direct form for few kept rows (masked_conv_direct.cu): a small tile's k range shared by the warps of a block
+struct DirectKPlan {
+    int KQ;                // 16-byte chunks of a window in groups of four
+    int NT, MTL;           // a tile is 8 NT rows x 16 MTL channels
+    int grid_x, grid_y, smem_bytes;
+    double est_us;         // estimated duration of a launch among others
+};
+bool plan_direct_k(const ConvGeom& g, int elem_bytes, int64_t kept_rows, int num_sms, DirectKPlan* plan);
+cudaError_t launch_direct_k(const ConvGeom& g, const DirectKPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
+                            int32_t* kept_out, int32_t* count_out, int64_t host_kept, int relu, const void* residual, int f32, int* dev_status,
+                            cudaStream_t st);
 // src[rows][C] -> dst[rows][Cp] with zero channels added (Cp = 4 or a multiple of 8; rows*Cp % 8 == 0)
 cudaError_t launch_pad_channels(const void* src, void* dst, long long rows, int C, int Cp, cudaStream_t st);
 // filters for the pixel-pair form: w[C_out][kh][kw][C] -> w2[C_out][kh][kw2][2][4], where pair kxx,

@@ -20,6 +20,7 @@
 // There is no kept-row list: a warp walks over 64 output rows at a time, reads their mask bytes, writes the zeros of
 // the dropped ones and queues the kept ones; whenever 16 or 32 rows are queued it computes them.  With ASX_RECOMPACT
 // a few extra blocks write the list to global memory beside the others.
+#include <algorithm>
 #include <atomic>
 #include <cuda_bf16.h>
 #include "asx_internal.h"
@@ -34,8 +35,26 @@ constexpr int THREADS = 256, WARPS = THREADS / 32;
 constexpr int CHUNK = 32;               // output rows a warp scans at a time
 constexpr int QUEUE = 48;               // row queue of a warp: up to 15 left over and 32 new ones
 
+// How the zeros of dropped rows are written: the 16-byte units of a row's column range, and whether they are a power of
+// two up to 32 (1 << shift), so that every lane keeps its column.
+struct ZeroShape {
+    FastDiv fdUnits;
+    int pow2, shift;
+};
+ZeroShape zero_shape(int cols, int elem_bytes, bool whole)
+{
+    ZeroShape z;
+    const int epc = 16 / elem_bytes, units = (cols + epc - 1) / epc;
+    z.fdUnits = make_fastdiv((uint32_t)units);
+    z.pow2 = (whole && units <= 32 && (units & (units - 1)) == 0) ? 1 : 0;
+    z.shift = 0;
+    while ((1 << z.shift) < units) ++z.shift;
+    return z;
+}
+
 struct DirectArgs {
-    FastDiv fdP, fdWo, fdUnits;         // divisions by P, Wo and the 16-byte units of a row's column range
+    FastDiv fdP, fdWo;                  // divisions by P and Wo
+    ZeroShape zero;
     FastDiv fdChunks, fdCin, fdkw, fdWords;   // by the chunks (words) of a window, C_in, kw, words
     const void* x;
     const void* w;
@@ -51,8 +70,6 @@ struct DirectArgs {
     int words;                          // word form: 4-byte words per filter row, else 0
     int shift;                          // word form: K-elements in front of a filter row's first (0 or 1)
     int block_rows;                     // output rows per block
-    int unit_shift;
-    int lanes_per_row;                  // the 16-byte units of a row's column range are a power of two up to 32
 };
 
 __device__ __forceinline__ uint4 ld_x4(const void* p)
@@ -346,13 +363,13 @@ __device__ __forceinline__ void compute_rows(const Row* queue, int n, const Tabl
 
 // Zeros for the dropped rows among row0 .. row0 + 31 (bit i of `drop`: row row0 + i), this block's columns.
 template <bool F32>
-__device__ __forceinline__ void zero_rows(unsigned drop, int row0, const ConvGeom& g, const DirectArgs& a, int n0, int ncols, int lane)
+__device__ __forceinline__ void zero_rows(unsigned drop, int row0, const ConvGeom& g, void* y, const ZeroShape& z, int n0, int ncols, int lane)
 {
     constexpr int ES = F32 ? 4 : 2, EPC = 16 / ES;
-    uint8_t* yb = static_cast<uint8_t*>(a.y) + ((long long)row0 * g.C_out + n0) * ES;
-    const int units = (int)a.fdUnits.d;                     // 16-byte units of a row
-    if (a.lanes_per_row) {                                  // a power of two up to 32: every lane keeps its column
-        const int r0 = lane >> a.unit_shift, rows = 32 >> a.unit_shift;
+    uint8_t* yb = static_cast<uint8_t*>(y) + ((long long)row0 * g.C_out + n0) * ES;
+    const int units = (int)z.fdUnits.d;
+    if (z.pow2) {
+        const int r0 = lane >> z.shift, rows = 32 >> z.shift;
         yb += (long long)(r0 * g.C_out * ES + (lane & (units - 1)) * 16);
         const int step = rows * g.C_out * ES;
         drop >>= r0;
@@ -362,7 +379,7 @@ __device__ __forceinline__ void zero_rows(unsigned drop, int row0, const ConvGeo
         return;
     }
     for (int u = lane; u < 32 * units; u += 32) {
-        const int r = (int)fd_div((uint32_t)u, a.fdUnits), c = (u - r * units) * EPC;
+        const int r = (int)fd_div((uint32_t)u, z.fdUnits), c = (u - r * units) * EPC;
         if (((drop >> r) & 1u) && c < ncols) *reinterpret_cast<uint4*>(yb + ((long long)r * g.C_out + c) * ES) = make_uint4(0, 0, 0, 0);
     }
 }
@@ -429,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
                     make_int4(rw, ((img * g.H + iy0) * g.W + ix0) * g.C_in, (iy0 << 16) | ((WORDS ? ix0 * g.C_in : ix0) & 0xffff), inner ? 1 : 0);
             }
             queued += __popc(kept);
-            if (all & ~kept) zero_rows<F32>(all & ~kept, row0, g, a, n0, ncols, lane);
+            if (all & ~kept) zero_rows<F32>(all & ~kept, row0, g, a.y, a.zero, n0, ncols, lane);
             __syncwarp();
         }
         // whole tiles, and behind the last chunk what is left
@@ -448,6 +465,195 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
             if (lane < queued) queue[lane] = v;
         }
         __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// The direct form for few kept rows and any filter matrix: the warps of a block share the k range of one small tile
+// (8 NT rows x 16 MTL channels) and meet once, in shared memory.
+//
+// At batch 1 a layer is all latency.  In the tensor-memory forms a launch with 18 to 72 k-blocks spends 1.8 us until the first
+// gathered stage, 3-6 us in a k loop that runs on 14 to 64 blocks one 64-wide k-block after another, 1-2 us in the epilogue or
+// the exchange of shared tiles, most of it in instructions that are executed once and come cold from L2: 7-13 us a
+// layer of ResNet-18, against 2.3-7.0 us here.  The tile is small, so that all SMs have one, its k range is spread over
+// eight warps, and both operands come straight from global memory: a filter value is used by one block once, so there
+// is nothing to stage.
+constexpr int KWARPS = 8, KZERO = 2, KTHREADS = 32 * (KWARPS + KZERO);
+
+struct DirectKArgs {
+    FastDiv fdP, fdWo, fdCin, fdkw, fdcnt;
+    const void* x;
+    const void* w;
+    const float* bias;
+    void* y;
+    const uint8_t* mask;
+    const void* residual;
+    int32_t* kept_out;                  // non-null: block 0 writes the kept-row list and its count
+    int32_t* count_out;
+    int* dev_status;
+    int relu;
+    int KQ;
+    int Mk;                             // kept lowered rows, as the host counts them
+    ZeroShape zero;
+};
+
+template <bool F32, int NT, int MTL, bool RESIDUAL, bool SILU>
+__global__ void __launch_bounds__(KTHREADS) masked_conv_direct_k_kernel(const ConvGeom g, const DirectKArgs a)
+{
+    constexpr int EPC = F32 ? 4 : 8, ES = F32 ? 4 : 2, ROWS = 8 * NT, CH = 16 * MTL;
+    extern __shared__ uint4 smem_v[];
+    __shared__ int scan_total[32];
+    __shared__ int4 rowinfo[ROWS];      // output row (-1: none), element index of the window's corner, its coordinates
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ptx::grid_launch_dependents();
+    float* const red = reinterpret_cast<float*>(smem_v);                                     // [KWARPS][4 NT MTL][32]
+    int2* const pos = reinterpret_cast<int2*>(red + KWARPS * 4 * NT * MTL * 32);             // [4 KQ]
+    unsigned short* const list = reinterpret_cast<unsigned short*>(pos + 4 * a.KQ);          // kept positions
+    // Everything up to the dependency wait needs the mask and the geometry only.
+    for (int c = tid; c < 4 * a.KQ; c += KTHREADS) {
+        int2 e = make_int2(0, 0x7fff0000);
+        if (c * EPC < g.K) {
+            const int tap = (int)fd_div((uint32_t)(c * EPC), a.fdCin), ci = c * EPC - tap * g.C_in;
+            const int ky = (int)fd_div((uint32_t)tap, a.fdkw), kx = tap - ky * g.kw;
+            e = make_int2((ky * g.W + kx) * g.C_in + ci, (ky << 16) | kx);
+        }
+        pos[c] = e;
+    }
+    const int cnt = block_compact(a.mask, g.rows, make_uint4(0, 0, 0, 0), false, list, scan_total, KTHREADS);
+    const int Mk = (g.rows == g.P) ? g.Nb * cnt : cnt;
+    if (Mk != a.Mk && tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);                      // the grid was sized for another mask
+    const int r_first = blockIdx.x * ROWS, n0 = blockIdx.y * CH;
+    if (tid < ROWS) {
+        const int rk = r_first + tid;
+        int4 e = make_int4(-1, 0, (int)0x80000000u, 0);
+        if (rk < Mk) {
+            int row = 0;
+            if (g.rows == g.P) {
+                const int n = (int)fd_div((uint32_t)rk, a.fdcnt);
+                row = n * g.P + list[rk - n * (int)a.fdcnt.d];
+            } else {
+                row = list[rk];
+            }
+            const int n = (int)fd_div((uint32_t)row, a.fdP), p = row - n * g.P;
+            const int oy = (int)fd_div((uint32_t)p, a.fdWo), ox = p - oy * g.Wo;
+            const int iy0 = oy * g.stride - g.pad, ix0 = ox * g.stride - g.pad;
+            e = make_int4(row, ((n * g.H + iy0) * g.W + ix0) * g.C_in, (iy0 << 16) | (ix0 & 0xffff), 0);
+        }
+        rowinfo[tid] = e;
+    }
+    __syncthreads();
+    ptx::grid_dependency_wait();
+    if (warp < KWARPS) {
+        __threadfence();                // the input is read through L1: drop what it holds from before (see above)
+        const int t = lane & 3, gr = lane >> 2;
+        const uint8_t* const xb = static_cast<const uint8_t*>(a.x);
+        int base[NT], yx[NT];
+#pragma unroll
+        for (int r = 0; r < NT; ++r) {
+            const int4 e = rowinfo[8 * r + gr];
+            base[r] = e.y;
+            yx[r] = e.z;
+        }
+        const uint8_t* wp[2 * MTL];     // this lane's channels: 2 MTL gr + i
+        bool have[2 * MTL];
+#pragma unroll
+        for (int i = 0; i < 2 * MTL; ++i) {
+            const int ch = n0 + 2 * MTL * gr + i;
+            have[i] = ch < g.C_out;
+            wp[i] = static_cast<const uint8_t*>(a.w) + (size_t)(have[i] ? ch : 0) * g.K * ES;
+        }
+        float acc[NT][MTL][4];
+#pragma unroll
+        for (int r = 0; r < NT; ++r)
+#pragma unroll
+            for (int j = 0; j < MTL; ++j)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[r][j][v] = 0.f;
+        auto load = [&](int q, uint4 (&xv)[NT], uint4 (&wv)[2 * MTL]) {
+            const int c = 4 * q + t;
+            const int2 e = pos[c];
+#pragma unroll
+            for (int i = 0; i < 2 * MTL; ++i) {
+                wv[i] = make_uint4(0, 0, 0, 0);
+                if (have[i] && c * EPC < g.K) wv[i] = ld_x4(wp[i] + (size_t)c * 16);
+            }
+#pragma unroll
+            for (int r = 0; r < NT; ++r) {
+                xv[r] = make_uint4(0, 0, 0, 0);
+                const int iy = (yx[r] >> 16) + (e.y >> 16), ix = (int)(short)yx[r] + (e.y & 0xffff);
+                if ((unsigned)iy < (unsigned)g.H && (unsigned)ix < (unsigned)g.W) xv[r] = ld_x4(xb + (long long)(base[r] + e.x) * ES);
+            }
+        };
+        auto multiply = [&](const uint4 (&xv)[NT], const uint4 (&wv)[2 * MTL]) {
+#pragma unroll
+            for (int j = 0; j < MTL; ++j)
+#pragma unroll
+                for (int r = 0; r < NT; ++r) {
+                    mma<F32>(acc[r][j], wv[2 * j].x, wv[2 * j + 1].x, wv[2 * j].y, wv[2 * j + 1].y, xv[r].x, xv[r].y);
+                    mma<F32>(acc[r][j], wv[2 * j].z, wv[2 * j + 1].z, wv[2 * j].w, wv[2 * j + 1].w, xv[r].z, xv[r].w);
+                }
+        };
+        uint4 x0[NT], x1[NT], w0[2 * MTL], w1[2 * MTL];
+        int q = warp;
+        if (q < a.KQ) load(q, x0, w0);
+#pragma unroll 1
+        for (; q + KWARPS < a.KQ; q += 2 * KWARPS) {          // two groups a turn, each loaded while the other is used
+            load(q + KWARPS, x1, w1);
+            multiply(x0, w0);
+            if (q + 2 * KWARPS < a.KQ) load(q + 2 * KWARPS, x0, w0);
+            multiply(x1, w1);
+        }
+        if (q < a.KQ) multiply(x0, w0);
+        float* const mine = red + warp * (4 * NT * MTL * 32) + lane;
+#pragma unroll
+        for (int r = 0; r < NT; ++r)
+#pragma unroll
+            for (int j = 0; j < MTL; ++j)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) mine[((r * MTL + j) * 4 + v) * 32] = acc[r][j][v];
+    } else {
+        if (a.kept_out != nullptr && blockIdx.x == 0 && blockIdx.y == 0) {
+            for (int i = tid - 32 * KWARPS; i < cnt; i += 32 * KZERO) a.kept_out[i] = (int32_t)list[i];
+            if (tid == 32 * KWARPS) *a.count_out = cnt;
+        }
+        // the zeros of the dropped rows, 32 rows of the output at a time, spread over all blocks
+        const int nb = (int)(gridDim.x * gridDim.y), first = (int)(blockIdx.y * gridDim.x + blockIdx.x) * KZERO + warp - KWARPS;
+        for (long long row0 = 32ll * first; row0 < g.M; row0 += 32ll * KZERO * nb) {
+            const int row = (int)row0 + lane;
+            bool drop = false;
+            if (row < g.M) drop = __ldg(a.mask + (g.rows == g.P ? row - (int)fd_div((uint32_t)row, a.fdP) * g.P : row)) == 0;
+            const unsigned d = __ballot_sync(0xffffffffu, drop);
+            if (d) zero_rows<F32>(d, (int)row0, g, a.y, a.zero, 0, g.C_out, lane);
+        }
+    }
+    __syncthreads();
+    // two neighbouring channels of a row per thread; the warps' sums are added in warp order
+#pragma unroll 1
+    for (int i = tid; i < ROWS * CH / 2; i += KTHREADS) {
+        const int row = i / (CH / 2), pr = i % (CH / 2), gn = pr / MTL, j = pr % MTL;
+        const int out = rowinfo[row].x, col = n0 + 2 * pr;
+        if (out < 0 || col >= g.C_out) continue;
+        const float* src = red + (((row >> 3) * MTL + j) * 4 + (row & 1)) * 32 + gn * 4 + ((row & 7) >> 1);
+        float v0 = 0.f, v1 = 0.f;
+#pragma unroll
+        for (int wq = 0; wq < KWARPS; ++wq) {
+            v0 += src[wq * (4 * NT * MTL * 32)];
+            v1 += src[wq * (4 * NT * MTL * 32) + 64];
+        }
+        if (a.bias != nullptr) {
+            v0 += __ldg(a.bias + col);
+            v1 += __ldg(a.bias + col + 1);
+        }
+        const long long at = (long long)out * g.C_out + col;
+        if (RESIDUAL) {
+            const uint32_t r2 = __ldcg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(a.residual) + at));
+            v0 += __uint_as_float(r2 << 16);
+            v1 += __uint_as_float(r2 & 0xffff0000u);
+        }
+        v0 = SILU ? silu(v0) : a.relu ? fmaxf(v0, 0.f) : v0;
+        v1 = SILU ? silu(v1) : a.relu ? fmaxf(v1, 0.f) : v1;
+        if (F32) *reinterpret_cast<float2*>(static_cast<float*>(a.y) + at) = make_float2(v0, v1);
+        else *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(a.y) + at) = pack_bf16(v0, v1);
     }
 }
 
@@ -487,21 +693,24 @@ bool direct_pays(const DirectPlan& plan, int num_sms, int64_t kept_rows)
     return plan.KQ <= 4 || (plan.KQ <= 10 && kept_rows / 16 * plan.n_tiles >= 10ll * num_sms);
 }
 
+double direct_est_us(const DirectPlan& plan, int num_sms, int64_t kept_rows, int elem_bytes)
+{
+    const double clocks = (plan.NG == 1 ? 150 + 35 * plan.KQ : 220 + 82 * plan.KQ) * (elem_bytes == 4 ? 1.5 : 1.0);      // per 16 rows
+    return 4.0 + 0.12 * plan.KQ + (double)kept_rows / 16 * plan.n_tiles / num_sms * clocks / 1900.0;
+}
+
 cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
                           int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32, int num_sms, cudaStream_t st)
 {
     DirectArgs a;
-    const int es = f32 ? 4 : 2, epc = 16 / es;
+    const int es = f32 ? 4 : 2;
     a.fdP = make_fastdiv((uint32_t)g.P);
     a.fdWo = make_fastdiv((uint32_t)g.Wo);
-    const int cols = g.C_out < 32 * plan.NG ? g.C_out : 32 * plan.NG;
-    a.fdUnits = make_fastdiv((uint32_t)((cols + epc - 1) / epc));
+    a.zero = zero_shape(g.C_out < 32 * plan.NG ? g.C_out : 32 * plan.NG, es, plan.n_tiles == 1 || g.C_out % (32 * plan.NG) == 0);
     a.fdChunks = make_fastdiv((uint32_t)((plan.words > 0 ? 16 : 4) * plan.KQ));
     a.fdCin = make_fastdiv((uint32_t)g.C_in);
     a.fdkw = make_fastdiv((uint32_t)g.kw);
     a.fdWords = make_fastdiv((uint32_t)(plan.words > 0 ? plan.words : 1));
-    const int units = (int)a.fdUnits.d;
-    a.lanes_per_row = (units <= 32 && (units & (units - 1)) == 0 && g.C_out % (32 * plan.NG) == 0) || (plan.n_tiles == 1 && units <= 32 && (units & (units - 1)) == 0);
     a.x = x;
     a.w = w;
     a.bias = bias;
@@ -513,8 +722,6 @@ cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void*
     a.count_out = count_out;
     a.relu = relu == 1 ? 1 : 0;
     a.KQ = plan.KQ;
-    a.unit_shift = 0;
-    while ((1 << a.unit_shift) < units) ++a.unit_shift;
     a.words = plan.words;
     a.shift = plan.shift;
 
@@ -555,6 +762,76 @@ cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void*
         smem_set[vi].store(plan.smem_bytes, std::memory_order_relaxed);
     }
     return launch_pdl(kern, dim3(grid, plan.n_tiles), dim3(THREADS), (size_t)plan.smem_bytes, st, g, a);
+}
+
+// The tile sizes and the estimate come from 197 layers (networks' layers at batch 1 to 16, random ones): a block costs about
+// 1.5 us of its SM (mask, row coordinates, reduction) and 16-38 ns per operand group, a launch 1-1.5 us and the longest
+// warp's groups.  Median error 8 %.
+bool plan_direct_k(const ConvGeom& g, int elem_bytes, int64_t kept_rows, int num_sms, DirectKPlan* plan)
+{
+    const int epc = 16 / elem_bytes;
+    if (g.C_in % epc != 0 || g.C_out % epc != 0 || kept_rows < 1 || g.rows > COMPACT_SMALL_MAX_ROWS) return false;
+    plan->KQ = (g.K + 4 * epc - 1) / (4 * epc);
+    plan->est_us = 0.0;
+    struct Shape { int NT, MTL; double base, chain, group, block; };
+    for (const Shape& t : {Shape{2, 1, 1.05, 0.213, 0.0163, 1.52}, Shape{4, 1, 1.40, 0.290, 0.0215, 1.65}, Shape{4, 2, 1.53, 0.430, 0.0383, 3.74}}) {
+        const int64_t gx = (kept_rows + 8 * t.NT - 1) / (8 * t.NT);
+        const int gy = (g.C_out + 16 * t.MTL - 1) / (16 * t.MTL);
+        const double est = t.base + t.chain * plan->KQ / KWARPS + (double)gx * gy / num_sms * (t.group * plan->KQ + t.block);
+        if (plan->est_us > 0.0 && est >= plan->est_us) continue;
+        plan->est_us = est;
+        plan->NT = t.NT;
+        plan->MTL = t.MTL;
+        plan->grid_x = (int)std::min<int64_t>(gx, 1 << 30);
+        plan->grid_y = gy;
+    }
+    plan->smem_bytes = KWARPS * 4 * plan->NT * plan->MTL * 128 + plan->KQ * 32 + (g.rows * 2 + 15) / 16 * 16;
+    return plan->smem_bytes <= 100 * 1024 && plan->grid_y < 65536;
+}
+
+cudaError_t launch_direct_k(const ConvGeom& g, const DirectKPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
+                            int32_t* kept_out, int32_t* count_out, int64_t host_kept, int relu, const void* residual, int f32, int* dev_status,
+                            cudaStream_t st)
+{
+    DirectKArgs a;
+    a.fdP = make_fastdiv((uint32_t)g.P);
+    a.fdWo = make_fastdiv((uint32_t)g.Wo);
+    a.fdCin = make_fastdiv((uint32_t)g.C_in);
+    a.fdkw = make_fastdiv((uint32_t)g.kw);
+    a.fdcnt = make_fastdiv((uint32_t)host_kept);
+    a.x = x;
+    a.w = w;
+    a.bias = bias;
+    a.y = y;
+    a.mask = mask;
+    a.residual = residual;
+    a.kept_out = kept_out;
+    a.count_out = count_out;
+    a.dev_status = dev_status;
+    a.relu = relu == 1 ? 1 : 0;
+    a.KQ = plan.KQ;
+    a.zero = zero_shape(g.C_out, f32 ? 4 : 2, true);
+    a.Mk = (int)(g.rows == g.P ? host_kept * g.Nb : host_kept);
+    using Kern = void (*)(const ConvGeom, const DirectKArgs);
+    const bool res = residual != nullptr, is_silu = relu == 2;
+    Kern kern;
+#define ASX_PICK2(F32, NT, MTL)                                                                                                             \
+    (F32 || !res ? (is_silu ? masked_conv_direct_k_kernel<F32, NT, MTL, false, true> : masked_conv_direct_k_kernel<F32, NT, MTL, false, false>) \
+                 : (is_silu ? masked_conv_direct_k_kernel<F32, NT, MTL, !F32, true> : masked_conv_direct_k_kernel<F32, NT, MTL, !F32, false>))
+#define ASX_PICK(NT, MTL) kern = f32 ? ASX_PICK2(true, NT, MTL) : ASX_PICK2(false, NT, MTL)
+    if (plan.NT == 2) { ASX_PICK(2, 1); }
+    else if (plan.MTL == 1) { ASX_PICK(4, 1); }
+    else { ASX_PICK(4, 2); }
+#undef ASX_PICK
+#undef ASX_PICK2
+    static std::atomic<int> smem_set[24];                // largest dynamic shared memory size enabled so far, per instance
+    const int vi = (plan.NT == 2 ? 0 : plan.MTL) * 8 + (f32 ? 4 : 0) + (res ? 2 : 0) + (is_silu ? 1 : 0);
+    if (plan.smem_bytes > smem_set[vi].load(std::memory_order_relaxed)) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
+        if (e != cudaSuccess) return e;
+        smem_set[vi].store(plan.smem_bytes, std::memory_order_relaxed);
+    }
+    return launch_pdl(kern, dim3(plan.grid_x, plan.grid_y), dim3(KTHREADS), (size_t)plan.smem_bytes, st, g, a);
 }
 
 }  // namespace asx

@@ -1,4 +1,4 @@
-"""The direct form of the fused layer (operands gathered into registers, no kept-row list) against the CPU
+"""The two direct forms of the fused layer (operands gathered into registers; small filter matrices, few rows) against the CPU
 oracle at the sizes where it can go wrong: channel counts that are whole 16-byte chunks and words of four bytes,
 windows that reach over every edge, column ranges that end inside a 32- or 64-channel block, row counts around the
 16-row tiles, lists rebuilt by several blocks."""
@@ -45,8 +45,31 @@ def test_against_the_oracle(case, per_row):
     check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT)
 
 
+K_CASES = [
+    # few rows, the k range shared by eight warps: fewer groups than warps, one more, several turns
+    (8, 8, 1, 1, 0, 9, 7, 2, 30, 1),
+    (24, 56, 3, 2, 1, 13, 12, 2, 50, 2),
+    (32, 40, 3, 1, 1, 7, 5, 1, 20, 1),
+    (64, 72, 3, 1, 1, 9, 10, 1, 90, 4),
+    (136, 64, 3, 2, 1, 8, 9, 3, 30, 1),
+    (256, 48, 1, 1, 0, 11, 11, 2, 0, 1),
+    (512, 32, 3, 1, 1, 6, 6, 1, 50, 4),
+]
+
+
+@pytest.mark.parametrize("per_row", [False, True])
+@pytest.mark.parametrize("case", K_CASES, ids=["-".join(map(str, c)) for c in K_CASES])
+def test_shared_k_range(case, per_row):
+    spec = _spec(case, 4)
+    x, w, b, mask = make_problem(spec, per_row=per_row)
+    for flags in (asx.ACT_RELU | asx.RECOMPACT, asx.ACT_SILU):
+        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT_K)
+    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT_K)
+
+
+@pytest.mark.parametrize("impl", [asx.IMPL_DIRECT, asx.IMPL_DIRECT_K], ids=["direct", "direct_k"])
 @pytest.mark.parametrize("kept", [0, 1, 15, 16, 17, 33, "all"])
-def test_row_counts_around_a_tile(kept):
+def test_row_counts_around_a_tile(kept, impl):
     spec = _spec((32, 32, 3, 1, 1, 19, 21, 1, 0, 1))
     x, w, b, _ = make_problem(spec)
     mask = np.zeros(spec.P, np.uint8)
@@ -54,20 +77,23 @@ def test_row_counts_around_a_tile(kept):
         mask[:] = 1
     else:
         mask[np.random.default_rng(kept).permutation(spec.P)[:kept]] = 1
-    check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | asx.RECOMPACT | asx.IMPL_DIRECT)
+    check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | asx.RECOMPACT | impl)
 
 
-@pytest.mark.parametrize("cin,cout,k,s,p", [(3, 64, 7, 2, 3), (5, 12, 3, 1, 1), (32, 36, 1, 1, 0), (8, 32, 3, 1, 1)])
-def test_fp32_storage(cin, cout, k, s, p):
+@pytest.mark.parametrize("cin,cout,k,s,p,impl,form", [
+    (3, 64, 7, 2, 3, asx.IMPL_DIRECT, asx.FORM_DIRECT), (5, 12, 3, 1, 1, asx.IMPL_DIRECT, asx.FORM_DIRECT),
+    (32, 36, 1, 1, 0, asx.IMPL_DIRECT, asx.FORM_DIRECT), (8, 32, 3, 1, 1, asx.IMPL_DIRECT, asx.FORM_DIRECT),
+    (36, 20, 3, 2, 1, asx.IMPL_DIRECT_K, asx.FORM_DIRECT_K), (128, 64, 3, 1, 1, asx.IMPL_DIRECT_K, asx.FORM_DIRECT_K)])
+def test_fp32_storage(cin, cout, k, s, p, impl, form):
     spec = _spec((cin, cout, k, s, p, 17, 19, 2, 40, 2), 1)
     x, w = oracle.tf32_operand(wl.make_x(spec)), oracle.tf32_operand(wl.make_w(spec))
     b, mask = wl.make_b(spec), wl.make_layer_mask(spec)
     layer = asx.MaskedConvLayer(cin, cout, k, k, s, p)
     layer.set_mask(mask)
     y = layer.run(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda(),
-                  flags=asx.ACT_RELU | asx.F32 | asx.IMPL_DIRECT)
+                  flags=asx.ACT_RELU | asx.F32 | impl)
     torch.cuda.synchronize()
-    assert layer.last_run_form() == asx.FORM_DIRECT
+    assert layer.last_run_form() == form
     layer.close()
     ref = oracle.masked_conv(x, w, b, mask, s, p, True, storage="fp32")
     got = y.cpu().numpy().astype(np.float64).reshape(ref.shape)
@@ -82,13 +108,14 @@ def test_list_rebuilt_beside_the_convolution(rows_hw):
     x, w, b, mask = make_problem(spec)
     layer = asx.MaskedConvLayer(8, 16, 1, 1, 1, 0)
     layer.set_mask(mask)
-    layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.RECOMPACT)
-    assert layer.last_run_form() == asx.FORM_DIRECT                    # the library's own choice
+    layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.RECOMPACT | asx.IMPL_DIRECT)
+    assert layer.last_run_form() == asx.FORM_DIRECT
     assert np.array_equal(layer.kept(), oracle.kept_list(mask))
     layer.close()
 
 
-def test_residual():
+@pytest.mark.parametrize("impl,form", [(asx.IMPL_DIRECT, asx.FORM_DIRECT), (asx.IMPL_DIRECT_K, asx.FORM_DIRECT_K)], ids=["direct", "direct_k"])
+def test_residual(impl, form):
     spec = _spec((64, 72, 1, 1, 0, 11, 13, 2, 30, 1), 3)
     x, w, b, mask = make_problem(spec)
     res = np.random.default_rng(3).standard_normal((spec.Nb, spec.Ho, spec.Wo, 72)).astype(np.float32)
@@ -96,9 +123,9 @@ def test_residual():
     layer = asx.MaskedConvLayer(64, 72, 1, 1, 1, 0)
     layer.set_mask(mask)
     layer.set_residual(rd)
-    y = layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU)
+    y = layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU | impl)
     torch.cuda.synchronize()
-    assert layer.last_run_form() == asx.FORM_DIRECT
+    assert layer.last_run_form() == form
     layer.close()
     ref = oracle.masked_conv(x, w, b, mask, 1, 0, False).reshape(spec.M, -1) + rd.float().cpu().numpy().reshape(spec.M, -1)
     ref = np.maximum(ref, 0) * np.tile(mask, spec.Nb)[:, None]
