@@ -23,6 +23,7 @@ struct asx_layer {
     void* d_scratch = nullptr;
     int32_t* d_small = nullptr;        // [0] kept count, [1] status word
     bool has_mask = false;
+    bool mask_from_kernel = false;     // a kernel wrote d_mask, and nothing that reads it was launched in stream order since
     int64_t host_kept = -1;            // kept entries of the mask when it came from the host, else -1
     const void* residual = nullptr;    // caller-owned shortcut tensor added in the epilogue, or null
     int32_t* d_in_rank = nullptr;      // compact input: row of each input position within its image, -1 = dropped
@@ -127,7 +128,7 @@ asx_status ensure_mask_buffers(asx_layer* L, int64_t rows)
 
 asx_status run_compaction(asx_layer* L, cudaStream_t st)
 {
-    return from_cuda(launch_compact(L->d_mask, L->rows, L->d_kept, L->d_small, L->d_scratch, st, true));
+    return from_cuda(launch_compact(L->d_mask, L->rows, L->d_kept, L->d_small, L->d_scratch, st, !L->mask_from_kernel, nullptr));
 }
 
 int64_t count_nonzero(const uint8_t* mask, int64_t rows)
@@ -252,10 +253,15 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
         cudaGetLastError();
     cudaError_t e;
     if (on_device) {
-        e = cudaMemcpyAsync(L->d_mask, mask, (size_t)rows, cudaMemcpyDeviceToDevice, st);
+        // one pass copies the mask and counts, or for a small one does everything; memory of another device is copied by
+        // the runtime (it may not be mapped here)
+        L->mask_from_kernel = attr.device == L->device;
+        e = L->mask_from_kernel ? launch_compact(mask, rows, L->d_kept, L->d_small, L->d_scratch, st, false, L->d_mask)
+                                : cudaMemcpyAsync(L->d_mask, mask, (size_t)rows, cudaMemcpyDeviceToDevice, st);
         L->host_kept = -1;
         L->host_mask.clear();
     } else {
+        L->mask_from_kernel = false;
         L->host_kept = count_nonzero(mask, rows);                 // only sizes the tiles (a launch heuristic)
         L->host_mask.clear();
         if (rows <= (1ll << 24)) {
@@ -274,7 +280,7 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
     L->rows = rows;
     L->last_stream = st;
     ++L->mask_epoch;
-    s = run_compaction(L, st);
+    s = L->mask_from_kernel ? ASX_OK : run_compaction(L, st);
     L->has_mask = (s == ASX_OK);
     return s;
 }
@@ -447,6 +453,13 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     L->last_stream = st;
+    // The kernels below read the mask through L1, some before their dependency wait: right after a kernel wrote it they
+    // start in stream order.
+    struct InOrder {
+        explicit InOrder(bool on) { launch_in_stream_order = on; }
+        ~InOrder() { launch_in_stream_order = false; }
+    } in_order(L->mask_from_kernel);
+    L->mask_from_kernel = false;
     // Small masks are compacted inside the fused kernel itself (no launches of its own, and the list stays in
     // shared memory as 16-bit positions); the reference kernel and large masks take the stand-alone compaction
     // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
@@ -472,7 +485,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             PatchPlan pp;
             other = plan_fast(g, L->num_sms, known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp) ? fp.est_cost_us : 1e9;
             if (!f32 && plan_patch(g, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
-                plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, &pp);
+                plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, false, &pp);
                 other = std::min(other, pp.est_cost_us);
             }
             other += 4.5;
@@ -659,7 +672,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     // Stride-1 layers with several filter taps and whole 64-channel slices take the window-patch form
     // when the host knows the mask, every tile's windows fit the patch buffers and the planner's
-    // estimate favours it; compact inputs and fp32 storage stay with the row gather.
+    // estimate favours it; fp32 storage stays with the row gather.
     PatchPlan pplan;
     bool use_patch = false;
     // The window-patch kernel sees the input as [Nb][H][W] pixels of C_in channels.  In the 2x2-block form a
@@ -668,7 +681,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     // are ever read.
     ConvGeom gp = g;
     if (blocks2x2) gp.H = g.Ho + g.kh - 1;
-    if (!f32 && !in_compact && !(flags & ASX_IMPL_ROW_GATHER) && !L->host_mask.empty() &&
+    if (!f32 && !(flags & ASX_IMPL_ROW_GATHER) && !L->host_mask.empty() &&
         (reinterpret_cast<uintptr_t>(y) & 15) == 0 && plan_patch(gp, fuse_compact ? (int)L->rows : 0, blocks2x2 ? 1 : 0, &pplan)) {
         if (L->tiles_epoch != L->mask_epoch || L->tiles_Nb != Nb || L->tiles_H != H || L->tiles_W != W || L->tiles_cap != pplan.cap_rows) {
             L->tiles_rows = cut_row_tiles(L->host_mask, Nb, gp.P, gp.Wo, pplan.Hp, gp.kh, pplan.cap_rows, 128, &L->host_tiles);
@@ -706,7 +719,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             }
         }
         if (L->tiles_rows > 0 && L->tiles_rows == est_rows) {
-            plan_patch_cost(gp, L->num_sms, (long long)(L->host_tiles.size() / 4), &pplan);
+            plan_patch_cost(gp, L->num_sms, (long long)(L->host_tiles.size() / 4), in_compact, &pplan);
             use_patch = pplan.est_cost_us <= plan.est_cost_us || (flags & ASX_IMPL_WINDOW_PATCH);
         }
     }
@@ -737,7 +750,28 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         if (r != CUDA_SUCCESS) return ASX_ERR_CUDA;
         L->tmap_ptr = wsrc; L->tmap_BN = BNsel; L->tmap_Kw = Kw; L->tmap_es = ES;
     }
-    if (use_patch) {
+    // x as a matrix of [rows][channels of one box] for the row gathers: the row-gather form's, or a compact input's in either form
+    auto map_rows = [&]() -> asx_status {
+        const int64_t pixels = in_compact ? x_rows : (int64_t)Nb * g.H * g.W;
+        const int row_stride = x_row_stride ? x_row_stride : g.C_in * ES;
+        if (L->tmapx_ptr == xsrc && L->tmapx_pixels == pixels && L->tmapx_stride == row_stride && L->tmapx_es == ES) return ASX_OK;
+        EncodeTiledFn enc = encode_tiled_fn();
+        if (enc == nullptr) return ASX_ERR_CUDA;
+        const cuuint64_t dims[2] = {(cuuint64_t)g.C_in, (cuuint64_t)pixels};
+        const cuuint64_t strides[1] = {(cuuint64_t)row_stride};
+        const cuuint32_t box[2] = {box_k, 1u};
+        const cuuint32_t estr[2] = {1u, 1u};
+        const CUresult r = enc(&L->tmap_x, tm_type, 2, const_cast<void*>(xsrc), dims,
+                               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return ASX_ERR_CUDA;
+        L->tmapx_ptr = xsrc; L->tmapx_pixels = pixels; L->tmapx_stride = row_stride; L->tmapx_es = ES;
+        return ASX_OK;
+    };
+    if (use_patch && in_compact) {
+        s = map_rows();
+        if (s != ASX_OK) return s;
+    } else if (use_patch) {
         if (L->tmapx4_ptr != xsrc || L->tmapx4_Nb != Nb || L->tmapx4_H != g.H || L->tmapx4_W != g.W || L->tmapx4_Wp != pplan.Wp ||
             L->tmapx4_px32 != pplan.px32) {
             EncodeTiledFn enc = encode_tiled_fn();
@@ -756,27 +790,16 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             L->tmapx4_ptr = xsrc; L->tmapx4_Nb = Nb; L->tmapx4_H = g.H; L->tmapx4_W = g.W; L->tmapx4_Wp = pplan.Wp;
             L->tmapx4_px32 = pplan.px32;
         }
+    }
+    if (use_patch) {
         L->last_form = ASX_FORM_WINDOW_PATCH;
-        return from_cuda(launch_patch(gp, pplan, L->tmap, L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
+        return from_cuda(launch_patch(gp, pplan, L->tmap, in_compact ? L->tmap_x : L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
                                       fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
-                                      out_compact ? 1 : 0, L->wait_limit_kcycles, st));
+                                      out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->wait_limit_kcycles, st));
     }
     if (plan.vec == 2) {
-        const int64_t pixels = in_compact ? x_rows : (int64_t)Nb * g.H * g.W;
-        const int row_stride = x_row_stride ? x_row_stride : g.C_in * ES;
-        if (L->tmapx_ptr != xsrc || L->tmapx_pixels != pixels || L->tmapx_stride != row_stride || L->tmapx_es != ES) {
-            EncodeTiledFn enc = encode_tiled_fn();
-            if (enc == nullptr) return ASX_ERR_CUDA;
-            const cuuint64_t dims[2] = {(cuuint64_t)g.C_in, (cuuint64_t)pixels};
-            const cuuint64_t strides[1] = {(cuuint64_t)row_stride};
-            const cuuint32_t box[2] = {box_k, 1u};
-            const cuuint32_t estr[2] = {1u, 1u};
-            const CUresult r = enc(&L->tmap_x, tm_type, 2, const_cast<void*>(xsrc), dims,
-                                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return ASX_ERR_CUDA;
-            L->tmapx_ptr = xsrc; L->tmapx_pixels = pixels; L->tmapx_stride = row_stride; L->tmapx_es = ES;
-        }
+        s = map_rows();
+        if (s != ASX_OK) return s;
     }
     L->last_form = plan.vec == 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
     return from_cuda(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
@@ -894,7 +917,7 @@ asx_status asx_compact(const uint8_t* mask_dev, int64_t rows, int32_t* kept_dev,
     if (reinterpret_cast<uintptr_t>(scratch_dev) & 7) return ASX_ERR_ALIGN;
     if ((reinterpret_cast<uintptr_t>(kept_dev) & 3) || (reinterpret_cast<uintptr_t>(count_dev) & 3)) return ASX_ERR_ALIGN;
     return from_cuda(launch_compact(mask_dev, rows, kept_dev, count_dev, scratch_dev,
-                                    static_cast<cudaStream_t>(cuda_stream), false));
+                                    static_cast<cudaStream_t>(cuda_stream), false, nullptr));
 }
 
 asx_status asx_mask_from_activation(const void* x_dev, int64_t rows, int C, uint8_t* mask_dev, void* cuda_stream)

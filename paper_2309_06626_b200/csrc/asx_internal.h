@@ -62,8 +62,9 @@ constexpr int COMPACT_TILE = COMPACT_THREADS * COMPACT_PER_THREAD;
 int64_t compact_scratch_bytes(int64_t rows);
 // mask_written_by_copies_only: the mask buffer is never written by a kernel (a layer's own copy), so
 // the write pass may read it before its dependency wait; false for a caller's buffer.
+// copy: non-null, 16-byte aligned: the mask's bytes are also written there (which makes them written by a kernel).
 cudaError_t launch_compact(const uint8_t* mask, int64_t rows, int32_t* kept, int32_t* count,
-                           void* scratch, cudaStream_t st, bool mask_written_by_copies_only);
+                           void* scratch, cudaStream_t st, bool mask_written_by_copies_only, uint8_t* copy);
 
 // ---- debug reference kernels (naive.cu)
 cudaError_t launch_naive(const ConvGeom& g, const void* x, const void* w, const float* bias, void* y,
@@ -110,14 +111,14 @@ struct PatchPlan {
 // px32: g describes the 2x2-block form (64 channels = four 32-byte blocks, kw = 1, no padding, pixels 32 bytes apart)
 bool plan_patch(const ConvGeom& g, int fused_list_rows, int px32, PatchPlan* plan);
 // fills plan->est_cost_us for a mask that the host cut into n_mtiles row tiles
-void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, PatchPlan* plan);
+void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, bool in_compact, PatchPlan* plan);
 // tmap_x4: x as a 4-D tensor (C_in, W, H, Nb) with box (64, Wp, 1, 1), 128-byte swizzle, zero fill; for a px32 plan
-// W counts units of four blocks (64 values)
+// W counts units of four blocks (64 values).  With in_rank it is the compact input as a [rows][C_in] matrix, box (64, 1).
 cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x4,
                          const float* bias, void* y, const uint8_t* mask, const int32_t* kept, const int32_t* count,
                          int relu, int* dev_status, int num_sms, int fuse_compact, int write_list, long long host_kept,
                          const void* residual, const void* tiles, int n_mtiles, long long kept_rows, int out_compact,
-                         int wait_limit_kcycles, cudaStream_t st);
+                         const int32_t* in_rank, int in_kept, int wait_limit_kcycles, cudaStream_t st);
 // ---- the direct form (masked_conv_direct.cu): small filter matrices, dense input and output
 struct DirectPlan {
     int KQ;                // 16-byte chunks of a window in groups of four, or (words > 0) its words in groups of sixteen

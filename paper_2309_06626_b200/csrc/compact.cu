@@ -127,6 +127,39 @@ compact_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
     if (tid == 0) run_count[blockIdx.x] = (unsigned)total;
 }
 
+// Pass 1 of asx_set_mask with a device mask: the same counts, and the mask's bytes into the layer's own buffer on the way.
+// (A device-to-device copy in front of pass 1 cost 3.4 us and, as no kernel, kept both its neighbours from overlapping.)
+__global__ void __launch_bounds__(COMPACT_THREADS, COMPACT_RESIDENT)
+compact_copy_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles, uint8_t* __restrict__ copy, unsigned* __restrict__ run_count)
+{
+    __shared__ int s_warp[COMPACT_THREADS / 32];
+    __shared__ int s_total;
+    const int tid = threadIdx.x;
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();          // the mask may come from the kernel before; the layer's buffer may still be read
+    int t0, t1;
+    run_of_block(tiles, t0, t1);
+    const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;        // the copy is an allocation of its own
+    const long long end = (long long)t1 * COMPACT_BIG_TILE < rows ? (long long)t1 * COMPACT_BIG_TILE : rows;
+    int v = 0;
+#pragma unroll 4
+    for (long long first = (long long)t0 * COMPACT_BIG_TILE + tid * COMPACT_PER_THREAD; first < end; first += COMPACT_TILE) {
+        if (aligned && first + COMPACT_PER_THREAD <= rows) {
+            const uint4 m = __ldcg(reinterpret_cast<const uint4*>(mask + first));
+            *reinterpret_cast<uint4*>(copy + first) = m;
+            v += __popc(nonzero_flags16(m));
+        } else {
+            for (int j = 0; j < COMPACT_PER_THREAD && first + j < rows; ++j) {
+                const uint8_t m = __ldcg(mask + first + j);
+                copy[first + j] = m;
+                v += m != 0;
+            }
+        }
+    }
+    const int total = block_sum(v, s_warp, &s_total);
+    if (tid == 0) run_count[blockIdx.x] = (unsigned)total;
+}
+
 // Pass 2: the indices of a 4096-row sub-tile are put in order in shared memory and copied to the list
 // with full-width stores (direct stores of each 32-row ballot word's indices, without the staging,
 // write half-filled lines and were 12 % slower; 16-byte stores from the unaligned staging buffer 3 %; a
@@ -227,7 +260,7 @@ compact_write_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
 // the warps, and each thread writes its own indices.
 __global__ void __launch_bounds__(1024)
 compact_small_kernel(const uint8_t* __restrict__ mask, int rows, int32_t* __restrict__ kept,
-                     int32_t* __restrict__ count, ScratchHeader* hdr)
+                     int32_t* __restrict__ count, ScratchHeader* hdr, uint8_t* __restrict__ copy)
 {
     __shared__ int s_warp_total[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -238,11 +271,16 @@ compact_small_kernel(const uint8_t* __restrict__ mask, int rows, int32_t* __rest
     const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
     if (aligned && first + COMPACT_PER_THREAD <= rows) {
         const uint4 v = __ldcg(reinterpret_cast<const uint4*>(mask + first));      // past L1: a kernel may have written the mask
+        if (copy != nullptr) *reinterpret_cast<uint4*>(copy + first) = v;
         flags = nonzero_bytes4(v.x) | (nonzero_bytes4(v.y) << 4) | (nonzero_bytes4(v.z) << 8) |
                 (nonzero_bytes4(v.w) << 12);
     } else {
         for (int j = 0; j < COMPACT_PER_THREAD; ++j)
-            if (first + j < rows && __ldcg(mask + first + j) != 0) flags |= 1u << j;
+            if (first + j < rows) {
+                const uint8_t m = __ldcg(mask + first + j);
+                if (copy != nullptr) copy[first + j] = m;
+                if (m != 0) flags |= 1u << j;
+            }
     }
     const int mine = __popc(flags);
     int incl = mine;
@@ -302,17 +340,19 @@ int64_t compact_scratch_bytes(int64_t rows)
 }
 
 cudaError_t launch_compact(const uint8_t* mask, int64_t rows, int32_t* kept, int32_t* count,
-                           void* scratch, cudaStream_t st, bool mask_written_by_copies_only)
+                           void* scratch, cudaStream_t st, bool mask_written_by_copies_only, uint8_t* copy)
 {
     auto* hdr = static_cast<ScratchHeader*>(scratch);
     if (rows <= COMPACT_SMALL_MAX_ROWS)
-        return launch_pdl(compact_small_kernel, dim3(1), dim3(1024), 0, st, mask, (int)rows, kept, count, hdr);
+        return launch_pdl(compact_small_kernel, dim3(1), dim3(1024), 0, st, mask, (int)rows, kept, count, hdr, copy);
     const int tiles = (int)((rows + COMPACT_BIG_TILE - 1) / COMPACT_BIG_TILE);
     // one resident block per run of tiles: eight blocks per SM, never more blocks than tiles (the scratch has
     // 8 bytes per 4096 rows, i.e. room for eight 32-bit counts per tile)
     const int grid = tiles < COMPACT_RESIDENT * resident_sms() ? tiles : COMPACT_RESIDENT * resident_sms();
     unsigned* run_count = reinterpret_cast<unsigned*>(hdr + 1);
-    cudaError_t e = launch_pdl(compact_count_kernel, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, run_count);
+    cudaError_t e = copy != nullptr
+                        ? launch_pdl(compact_copy_count_kernel, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, copy, run_count)
+                        : launch_pdl(compact_count_kernel, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, run_count);
     if (e == cudaSuccess)
         e = mask_written_by_copies_only
                 ? launch_pdl(compact_write_kernel<true>, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, kept,
@@ -373,7 +413,7 @@ extern "C" asx_status asx_compact_static(const uint8_t* mask_dev, int64_t rows, 
     // launch_compact overwrites every word of the array it later reads (tile counts, header), in
     // stream order, so whatever the previous call left in the array does not matter.
     return asx::launch_compact(mask_dev, rows, kept_dev, count_dev, g_static_scratch_addr[dev],
-                               static_cast<cudaStream_t>(cuda_stream), false) == cudaSuccess
+                               static_cast<cudaStream_t>(cuda_stream), false, nullptr) == cudaSuccess
                ? ASX_OK
                : ASX_ERR_CUDA;
 }

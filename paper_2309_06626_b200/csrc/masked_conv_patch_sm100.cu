@@ -31,6 +31,7 @@
 // lanes of the tensor core idle; the host weighs that against the row-gather form).  The kernel
 // checks each tile again and reports a status word instead of running past a buffer.  All waits are
 // bounded.
+#include <algorithm>
 #include <cuda_bf16.h>
 #include "asx_internal.h"
 #include "ptx_sm100.cuh"
@@ -53,8 +54,12 @@ constexpr int FULL_RING = 24;           // 'stage full' barriers: a multiple of 
 constexpr int W_MMA = 0, W_INFO = 1, W_EPI0 = 2, NUM_EPI_WARPS = 4, W_ZERO_A = 6, W_FILL0 = 8, NUM_FILL_WARPS = 16,
               W_ZERO_B = 24, NUM_ZERO_WARPS = 4, W_FILTER = 26, W_PATCH = 27;
 constexpr int WORK_THREADS = 32 * W_FILTER;
-constexpr int NUM_THREADS = 32 * (W_PATCH + 1);
-static_assert(NUM_THREADS / 32 < 32, "the fused compaction keeps its running count in slot 31 of the warp totals");
+// A compact input is fetched pixel by pixel with row gathers (four pixels each): a warp issues one every 56 clocks, the
+// TMA unit takes one every 13, hence four patch warps.
+constexpr int COMPACT_PATCH_WARPS = 4;
+template <bool IN_COMPACT>
+constexpr int num_threads = 32 * (W_PATCH + (IN_COMPACT ? COMPACT_PATCH_WARPS : 1));
+static_assert(num_threads<true> / 32 < 32, "the fused compaction keeps its running count in slot 31 of the warp totals");
 static_assert((W_FILL0 & 3) == 0 && (NUM_FILL_WARPS & 3) == 0, "fill warps come in groups of four lane quarters");
 
 struct PatchArgs {
@@ -91,6 +96,9 @@ struct PatchArgs {
     const int4* tiles;  // per row tile: first kept lowered row, number of rows (1..128), first padded input row of
                         // its patch, patch rows; cut by the host from the mask
     int n_mtiles;       // row tiles
+    const int32_t* in_rank;   // compact input: row of each input position within its image's in_kept rows, -1 = dropped
+    int in_kept, in_oob;      // rows per image, a row index past all of them (reads zeros)
+    FastDiv fdQuads;          // division by the groups of four pixels of a padded row
     int Mk_host;        // kept lowered rows the tiles cover; must equal what the device counts
     int wait_limit_kcycles;
 };
@@ -164,11 +172,13 @@ __device__ __forceinline__ void decode_row(PShared* sh, int jj, int rr, int m_ti
     sh->rowpix[jj][rr] = rel;
 }
 
-template <bool RESIDUAL, bool SILU>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+// IN_COMPACT: the input holds the positions kept by its own mask only; tmap_x is then the [rows][C_in] matrix of them.
+template <bool RESIDUAL, bool SILU, bool IN_COMPACT>
+__global__ void __launch_bounds__(num_threads<IN_COMPACT>, 1)
 masked_conv_patch_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                                const ConvGeom g, const PatchArgs a)
 {
+    constexpr int NUM_THREADS = num_threads<IN_COMPACT>;
     extern __shared__ uint8_t smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -240,7 +250,50 @@ masked_conv_patch_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const
         // patch range, so the first filter slabs and the first patches are on their way while the other
         // warps still compact the mask and decode rows.  Each loader thread waits for the preceding
         // kernel by itself before its first load.
-        if (lane == 0) {
+        if (IN_COMPACT && warp >= W_PATCH) {
+            // ---------------------------------------------------------- input patches of a compact input
+            // The same buffers pixel by pixel: a padded pixel that is outside the image or was dropped reads the row past
+            // the end, which arrives as zeros.
+            ptx::grid_dependency_wait();
+            uint32_t use = 0;
+            bool ok = true;
+            const int quads = (int)a.fdQuads.d;
+            for (int t = blockIdx.x; t < host_tiles && ok; t += gridDim.x) {
+                const int4 tl = __ldg(a.tiles + pitem_of(t, a).m_tile);
+                int nrows = tl.w;
+                if (nrows > a.cap_rows || nrows < 1) {
+                    if (lane == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);
+                    nrows = nrows < 1 ? 1 : a.cap_rows;
+                }
+                const int n_lo = (int)fd_div((uint32_t)tl.z, a.fdHp), y_lo = tl.z - n_lo * a.Hp;
+                for (int sl = 0; sl < a.slices; ++sl, ++use) {
+                    const uint32_t b = use & (PB - 1u);
+                    ok = warp_wait_bar<40>(ptx::smem_u32(&sh->p_empty[b]), ((use >> a.p_bufs_log2) & 1u) ^ 1u, ctl, a.dev_status);
+                    if (!ok) break;
+                    const uint32_t full = ptx::smem_u32(&sh->p_full[b]), dst = smem_base + b * patch_bytes;
+                    if (warp == W_PATCH && lane == 0) ptx::mbar_arrive_expect_tx(full, (uint32_t)(nrows * quads) * 512u);
+                    for (int i = (warp - W_PATCH) * 32 + lane; i < nrows * quads; i += COMPACT_PATCH_WARPS * 32) {
+                        const int row = (int)fd_div((uint32_t)i, a.fdQuads), px = 4 * (i - row * quads);
+                        int yy = y_lo + row, n = n_lo;
+                        while (yy >= a.Hp) { yy -= a.Hp; ++n; }
+                        const int iy = yy - g.pad;
+                        int at[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int ix = px + j - g.pad_w;
+                            const bool in = (unsigned)iy < (unsigned)g.H && (unsigned)ix < (unsigned)g.W && n < g.Nb;
+                            const int rk = in ? __ldg(a.in_rank + iy * g.W + ix) : -1;      // written by stream-ordered copies
+                            at[j] = rk >= 0 ? n * a.in_kept + rk : a.in_oob;
+                        }
+                        ptx::tma_gather4_2d(dst + (uint32_t)row * row_bytes + (uint32_t)px * 128u, &tmap_x, full, sl * 64, at[0], at[1], at[2], at[3]);
+                    }
+                    __syncwarp();
+                }
+            }
+            if (!ok) {   // let loads already issued land before the block's shared memory goes away
+                for (int i = 0; i < 64; ++i) __nanosleep(1000);
+            }
+        } else if (lane == 0) {
             ptx::grid_dependency_wait();
             bool ok = true;
             if (warp == W_FILTER) {
@@ -665,7 +718,7 @@ bool plan_patch(const ConvGeom& g, int fused_list_rows, int px32, PatchPlan* pla
     return true;
 }
 
-void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, PatchPlan* plan)
+void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, bool in_compact, PatchPlan* plan)
 {
     // Estimated duration, in the terms of the row-gather planner and from the same kind of measurement:
     // a 64-wide k-block of a 128 x BN tile takes about 0.21 + 0.001 BN microseconds here (against
@@ -676,14 +729,16 @@ void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, PatchPl
     const long long waves = (items + num_sms - 1) / num_sms;
     const int KB = g.kh * g.kw * (g.C_in / 64);
     const double t_tile = KB * (0.21 + 0.001 * plan->BN);
-    plan->est_cost_us = (double)waves * (t_tile + 0.3) + 0.012 * plan->BN;
+    // a compact input's patches come as 128-byte rows, four to a request of 13 clocks
+    const double t_patch = in_compact ? (g.C_in / 64) * plan->cap_rows * plan->Wp / 4 * 13 / 1900.0 : 0.0;
+    plan->est_cost_us = (double)waves * (std::max(t_tile, t_patch) + 0.3) + 0.012 * plan->BN;
 }
 
 cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x4,
                          const float* bias, void* y, const uint8_t* mask, const int32_t* kept, const int32_t* count,
                          int relu, int* dev_status, int num_sms, int fuse_compact, int write_list, long long host_kept,
                          const void* residual, const void* tiles, int n_mtiles, long long kept_rows, int out_compact,
-                         int wait_limit_kcycles, cudaStream_t st)
+                         const int32_t* in_rank, int in_kept, int wait_limit_kcycles, cudaStream_t st)
 {
     PatchArgs a;
     a.fdcnt_host = make_fastdiv((uint32_t)(host_kept > 0 && host_kept < (1ll << 31) ? host_kept : 1));
@@ -700,6 +755,10 @@ cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtenso
     a.dev_status = dev_status;
     a.relu = relu == 1 ? 1 : 0;
     a.out_compact = out_compact;
+    a.in_rank = in_rank;
+    a.in_kept = in_kept;
+    a.in_oob = g.Nb * in_kept;
+    a.fdQuads = make_fastdiv((uint32_t)((plan.Wp + 3) / 4));
     a.st32 = (g.C_out % 16 == 0 && (reinterpret_cast<uintptr_t>(y) & 31) == 0) ? 1 : 0;
     a.BN = plan.BN;
     a.n_tiles = plan.n_tiles;
@@ -729,16 +788,20 @@ cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtenso
     if (grid < 1) grid = 1;
     const bool has_res = residual != nullptr, is_silu = relu == 2;
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const PatchArgs);
-    Kern kern = has_res ? (is_silu ? masked_conv_patch_sm100_kernel<true, true> : masked_conv_patch_sm100_kernel<true, false>)
-                        : (is_silu ? masked_conv_patch_sm100_kernel<false, true> : masked_conv_patch_sm100_kernel<false, false>);
-    static int smem_set[4] = {0, 0, 0, 0};      // largest dynamic shared memory size enabled so far, per instance
-    const int vi = (has_res ? 1 : 0) + (is_silu ? 2 : 0);
+    const bool compact = in_rank != nullptr;
+#define ASX_PICK(IC)                                                                                                              \
+    (has_res ? (is_silu ? masked_conv_patch_sm100_kernel<true, true, IC> : masked_conv_patch_sm100_kernel<true, false, IC>)          \
+             : (is_silu ? masked_conv_patch_sm100_kernel<false, true, IC> : masked_conv_patch_sm100_kernel<false, false, IC>))
+    Kern kern = compact ? ASX_PICK(true) : ASX_PICK(false);
+#undef ASX_PICK
+    static int smem_set[8] = {0, 0, 0, 0, 0, 0, 0, 0};      // largest dynamic shared memory size enabled so far, per instance
+    const int vi = (has_res ? 1 : 0) + (is_silu ? 2 : 0) + (compact ? 4 : 0);
     if (plan.smem_bytes > smem_set[vi]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
         if (e != cudaSuccess) return e;
         smem_set[vi] = plan.smem_bytes;
     }
-    return launch_pdl(kern, dim3(grid), dim3(NUM_THREADS), (size_t)plan.smem_bytes, st, tmap_w, tmap_x4, g, a);
+    return launch_pdl(kern, dim3(grid), dim3(compact ? num_threads<true> : num_threads<false>), (size_t)plan.smem_bytes, st, tmap_w, tmap_x4, g, a);
 }
 
 }  // namespace asx
