@@ -23,7 +23,8 @@ struct asx_layer {
     void* d_scratch = nullptr;
     int32_t* d_small = nullptr;        // [0] kept count, [1] status word
     bool has_mask = false;
-    bool mask_from_kernel = false;     // a kernel wrote d_mask, and nothing that reads it was launched in stream order since
+    int mask_from_kernel = 0;          // a kernel wrote d_mask, and no kernel was launched in stream order since: 2 at first, 1 once a
+                                       // launch has waited for it on its own SMs
     int64_t host_kept = -1;            // kept entries of the mask when it came from the host, else -1
     const void* residual = nullptr;    // caller-owned shortcut tensor added in the epilogue, or null
     int32_t* d_in_rank = nullptr;      // compact input: row of each input position within its image, -1 = dropped
@@ -131,7 +132,7 @@ asx_status ensure_mask_buffers(asx_layer* L, int64_t rows)
 
 asx_status run_compaction(asx_layer* L, cudaStream_t st)
 {
-    return from_cuda(launch_compact(L->d_mask, L->rows, L->d_kept, L->d_small, L->d_scratch, st, !L->mask_from_kernel, nullptr));
+    return from_cuda(launch_compact(L->d_mask, L->rows, L->d_kept, L->d_small, L->d_scratch, st, L->mask_from_kernel == 0, nullptr));
 }
 
 int64_t count_nonzero(const uint8_t* mask, int64_t rows)
@@ -276,13 +277,13 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
     if (on_device) {
         // one pass copies the mask and counts, or for a small one does everything; memory of another device is copied by
         // the runtime (it may not be mapped here)
-        L->mask_from_kernel = attr.device == L->device;
+        L->mask_from_kernel = attr.device == L->device ? 2 : 0;
         e = L->mask_from_kernel ? launch_compact(mask, rows, L->d_kept, L->d_small, L->d_scratch, st, false, L->d_mask)
                                 : cudaMemcpyAsync(L->d_mask, mask, (size_t)rows, cudaMemcpyDeviceToDevice, st);
         L->host_kept = -1;
         L->host_mask.clear();
     } else {
-        L->mask_from_kernel = false;
+        L->mask_from_kernel = 0;
         L->host_kept = count_nonzero(mask, rows);                 // only sizes the tiles (a launch heuristic)
         L->host_mask.clear();
         if (rows <= (1ll << 24)) {
@@ -474,13 +475,15 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     L->last_stream = st;
-    // The kernels below read the mask through L1, some before their dependency wait: right after a kernel wrote it they
-    // start in stream order.
+    // The kernels below read the mask through L1, some before their dependency wait: after a kernel wrote it they start in
+    // stream order.  The row gather with its list in global memory knows how to wait for a mask just written (this took
+    // 2.5 us off mask_from_activation, set_mask and run together); the run after that one then starts in stream order.
+    const int mask_from_kernel = L->mask_from_kernel;
     struct InOrder {
         explicit InOrder(bool on) { launch_in_stream_order = on; }
         ~InOrder() { launch_in_stream_order = false; }
-    } in_order(L->mask_from_kernel);
-    L->mask_from_kernel = false;
+    } in_order(mask_from_kernel != 0);
+    L->mask_from_kernel = 0;
     // Small masks are compacted inside the fused kernel itself (no launches of its own, and the list stays in
     // shared memory as 16-bit positions); the reference kernel and large masks take the stand-alone compaction
     // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
@@ -830,9 +833,15 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         if (s != ASX_OK) return s;
     }
     L->last_form = plan.vec == 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
+    const bool waits_for_mask = mask_from_kernel == 2 && !fuse_compact;
+    if (waits_for_mask) {
+        launch_in_stream_order = false;
+        L->mask_from_kernel = 1;
+    }
     return from_cuda(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
                                  L->num_sms, fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->d_wscnt,
-                                 out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles, st));
+                                 out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
+                                 waits_for_mask ? 1 : 0, st));
 }
 
 asx_status asx_get_kept(asx_layer* L, int64_t* count, const int32_t** dev_kept)

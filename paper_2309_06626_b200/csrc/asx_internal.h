@@ -54,7 +54,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 
 // ---- S1: mask compaction (compact.cu)
-constexpr int COMPACT_SMALL_MAX_ROWS = 1024 * 16;   // one block handles masks up to this size
+constexpr int COMPACT_SMALL_MAX_ROWS = 1024 * 16;   // masks of up to this size are compacted in one pass whatever their alignment
 constexpr int FUSED_COMPACT_MAX_ROWS = 1024 * 32;   // the fused kernels rebuild lists of up to this many rows themselves (positions fit 16 bits)
 constexpr int COMPACT_THREADS = 256;
 constexpr int COMPACT_PER_THREAD = 16;
@@ -92,7 +92,7 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
                         const int32_t* kept, const int32_t* count, int relu, int* dev_status,
                         int num_sms, int fuse_compact, int write_list, long long host_kept, int* split_hook,
                         int out_compact, const int32_t* in_rank, int in_kept, const void* residual, int f32, int wait_limit_kcycles,
-                        cudaStream_t st);
+                        int mask_from_kernel, cudaStream_t st);
 // ---- the window-patch form of the tensor-core path (masked_conv_patch_sm100.cu): stride-1 layers with
 // several filter taps and C_in % 64 == 0, bf16, dense input, dense or compact output
 struct PatchPlan {

@@ -5,8 +5,8 @@
 // exclusive prefix sum of the mask.  Here the prefix sum has two levels: inside a 16384-row
 // tile (4 x 16 mask bytes per thread, popcount, a shuffle scan inside each warp and across the
 // warp totals) and across runs of tiles (one run per resident block: a counting pass, then a
-// writing pass in which every block sums the counts in front of its run).  Masks of at most
-// 16384 rows take one block and one pass.
+// writing pass in which every block sums the counts in front of its run).  Small masks take one
+// pass in which every block counts all mask bytes in front of its own 4096.
 #include "asx_internal.h"
 #include "ptx_sm100.cuh"
 
@@ -18,12 +18,6 @@ struct ScratchHeader {       // first 8 bytes of the scratch; the tile counts fo
     unsigned int reserved;   // kept zero
     int error;               // device status word of the compaction (kept zero: nothing here can time out)
 };
-
-__device__ __forceinline__ unsigned nonzero_bytes4(unsigned w)
-{
-    unsigned t = ((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w;     // bit 7 of each byte: byte != 0
-    return ((t >> 7) & 1u) | ((t >> 14) & 2u) | ((t >> 21) & 4u) | ((t >> 28) & 8u);
-}
 
 // The sixteen flags of one 16-byte load, one bit per mask byte, in the order the arithmetic gives them
 // cheapest: byte b of word k (row 4 k + b of the sixteen) lands on bit 8 b + k.
@@ -43,33 +37,35 @@ __device__ __forceinline__ unsigned nonzero_flags16(const uint4& v)
 
 // A block takes COMPACT_SUB consecutive 4096-row sub-tiles and loads all their mask bytes before
 // anything else: four 16-byte loads in flight per thread instead of one.
+// Where that would leave SMs without a block (up to 4.8 million rows) a block takes one sub-tile.
 constexpr int COMPACT_SUB = 4;
-constexpr int COMPACT_BIG_TILE = COMPACT_SUB * COMPACT_TILE;
 constexpr int COMPACT_RESIDENT = 8;      // blocks per SM of the two passes over a large mask
+constexpr int64_t COMPACT_PREFIX_MAX_ROWS = 192 * 1024;
 
 // ---- Large masks: two passes over a grid of resident blocks, no block ever waits for another.  Block g
-// owns a run of consecutive 16384-row tiles.  Pass 1 counts the kept rows of every run; in pass 2 a block
+// owns a run of consecutive tiles of SUB sub-tiles.  Pass 1 counts the kept rows of every run; in pass 2 a block
 // adds up the counts of the runs in front of its own (a few loads per thread, all L2 hits), then writes
 // its tiles' indices one tile after another, carrying the offset along.  The mask is read twice, i.e.
 // `rows` more bytes than a single-pass chained scan (tiles that publish their totals and look back over
 // their predecessors' status words) would move; that form was built first and measured slower (0.150-0.152
 // ms on 2^27 rows), and it needs a ticket, cleared status words and bounded spin-waits, which this one
 // does not.
+template <int SUB>
 __device__ __forceinline__ void load_tile_flags(const uint8_t* __restrict__ mask, long long rows, long long tile_first,
-                                                int tid, unsigned (&flags)[COMPACT_SUB])
+                                                int tid, unsigned (&flags)[SUB])
 {
     const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
-    uint4 raw[COMPACT_SUB];
-    bool fast[COMPACT_SUB];
+    uint4 raw[SUB];
+    bool fast[SUB];
 #pragma unroll
-    for (int sub = 0; sub < COMPACT_SUB; ++sub) {
+    for (int sub = 0; sub < SUB; ++sub) {
         const long long first = tile_first + (long long)sub * COMPACT_TILE + (long long)tid * COMPACT_PER_THREAD;
         fast[sub] = aligned && first + COMPACT_PER_THREAD <= rows;
         raw[sub] = make_uint4(0, 0, 0, 0);
         if (fast[sub]) raw[sub] = __ldcg(reinterpret_cast<const uint4*>(mask + first));     // past L1: a kernel may have written the mask
     }
 #pragma unroll
-    for (int sub = 0; sub < COMPACT_SUB; ++sub) {
+    for (int sub = 0; sub < SUB; ++sub) {
         const long long first = tile_first + (long long)sub * COMPACT_TILE + (long long)tid * COMPACT_PER_THREAD;
         unsigned f = 0;
         if (fast[sub]) {
@@ -106,6 +102,7 @@ __device__ __forceinline__ int block_sum(int v, int* s_warp, int* s_total)
     return *s_total;
 }
 
+template <int SUB>
 __global__ void __launch_bounds__(COMPACT_THREADS, COMPACT_RESIDENT)
 compact_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles, unsigned* __restrict__ run_count)
 {
@@ -118,10 +115,10 @@ compact_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
     run_of_block(tiles, t0, t1);
     int v = 0;
     for (int t = t0; t < t1; ++t) {
-        unsigned flags[COMPACT_SUB];
-        load_tile_flags(mask, rows, (long long)t * COMPACT_BIG_TILE, tid, flags);
+        unsigned flags[SUB];
+        load_tile_flags(mask, rows, (long long)t * (SUB * COMPACT_TILE), tid, flags);
 #pragma unroll
-        for (int sub = 0; sub < COMPACT_SUB; ++sub) v += __popc(flags[sub]);
+        for (int sub = 0; sub < SUB; ++sub) v += __popc(flags[sub]);
     }
     const int total = block_sum(v, s_warp, &s_total);
     if (tid == 0) run_count[blockIdx.x] = (unsigned)total;
@@ -129,6 +126,7 @@ compact_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
 
 // Pass 1 of asx_set_mask with a device mask: the same counts, and the mask's bytes into the layer's own buffer on the way.
 // (A device-to-device copy in front of pass 1 cost 3.4 us and, as no kernel, kept both its neighbours from overlapping.)
+template <int SUB>
 __global__ void __launch_bounds__(COMPACT_THREADS, COMPACT_RESIDENT)
 compact_copy_count_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles, uint8_t* __restrict__ copy, unsigned* __restrict__ run_count)
 {
@@ -140,10 +138,10 @@ compact_copy_count_kernel(const uint8_t* __restrict__ mask, long long rows, int 
     int t0, t1;
     run_of_block(tiles, t0, t1);
     const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;        // the copy is an allocation of its own
-    const long long end = (long long)t1 * COMPACT_BIG_TILE < rows ? (long long)t1 * COMPACT_BIG_TILE : rows;
+    const long long end = (long long)t1 * (SUB * COMPACT_TILE) < rows ? (long long)t1 * (SUB * COMPACT_TILE) : rows;
     int v = 0;
 #pragma unroll 4
-    for (long long first = (long long)t0 * COMPACT_BIG_TILE + tid * COMPACT_PER_THREAD; first < end; first += COMPACT_TILE) {
+    for (long long first = (long long)t0 * (SUB * COMPACT_TILE) + tid * COMPACT_PER_THREAD; first < end; first += COMPACT_TILE) {
         if (aligned && first + COMPACT_PER_THREAD <= rows) {
             const uint4 m = __ldcg(reinterpret_cast<const uint4*>(mask + first));
             *reinterpret_cast<uint4*>(copy + first) = m;
@@ -169,21 +167,21 @@ compact_copy_count_kernel(const uint8_t* __restrict__ mask, long long rows, int 
 // still runs.  A caller's mask buffer may have been written by the kernel just before this call (a
 // data-dependent mask), which, launched as a programmatic predecessor, can still be storing it: then the
 // load waits like everything else.
-template <bool EARLY_MASK>
+template <int SUB, bool EARLY_MASK>
 __global__ void __launch_bounds__(COMPACT_THREADS, COMPACT_RESIDENT)
 compact_write_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles, int32_t* __restrict__ kept,
                      const unsigned* __restrict__ run_count, int32_t* __restrict__ count, ScratchHeader* hdr)
 {
     __shared__ int32_t s_idx[COMPACT_TILE];
-    __shared__ int s_warp_total[COMPACT_SUB][COMPACT_THREADS / 32];
+    __shared__ int s_warp_total[SUB][COMPACT_THREADS / 32];
     __shared__ int s_total;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     ptx::grid_launch_dependents();
     int t0, t1;
     run_of_block(tiles, t0, t1);
-    unsigned flags[COMPACT_SUB];
+    unsigned flags[SUB];
     if (!EARLY_MASK) ptx::grid_dependency_wait();
-    if (t0 < t1) load_tile_flags(mask, rows, (long long)t0 * COMPACT_BIG_TILE, tid, flags);
+    if (t0 < t1) load_tile_flags(mask, rows, (long long)t0 * (SUB * COMPACT_TILE), tid, flags);
     if (EARLY_MASK) ptx::grid_dependency_wait();          // the counts come from the pass before; the list may still be read
     // Offset of this block's run: the counts of all runs in front of it.  Read past L1: this block was
     // launched while the pass before was running, L1 is not invalidated in between, and the SM may hold
@@ -192,11 +190,11 @@ compact_write_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
     for (int i = tid; i < (int)blockIdx.x; i += COMPACT_THREADS) before += (int)__ldcg(run_count + i);
     int exclusive = block_sum(before, s_warp_total[0], &s_total);
     for (int t = t0; t < t1; ++t) {
-        const long long tile_first = (long long)t * COMPACT_BIG_TILE;
+        const long long tile_first = (long long)t * (SUB * COMPACT_TILE);
         if (t != t0) load_tile_flags(mask, rows, tile_first, tid, flags);
-        int mine[COMPACT_SUB], incl[COMPACT_SUB];
+        int mine[SUB], incl[SUB];
 #pragma unroll
-        for (int sub = 0; sub < COMPACT_SUB; ++sub) {
+        for (int sub = 0; sub < SUB; ++sub) {
             mine[sub] = __popc(flags[sub]);
             int v = mine[sub];
 #pragma unroll
@@ -209,7 +207,7 @@ compact_write_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
         }
         __syncthreads();
 #pragma unroll
-        for (int sub = 0; sub < COMPACT_SUB; ++sub) {
+        for (int sub = 0; sub < SUB; ++sub) {
             // lanes 0..7 hold the eight warp totals; a three-step scan gives every warp its prefix and the tile total
             const int wt = lane < COMPACT_THREADS / 32 ? s_warp_total[sub][lane] : 0;
             int winc = wt;
@@ -255,32 +253,40 @@ compact_write_kernel(const uint8_t* __restrict__ mask, long long rows, int tiles
     }
 }
 
-// Masks of up to 16 384 rows (every per-layer mask of a classification network) need no second
-// scan: one block of 1024 threads, 16 mask bytes per thread, a shuffle scan within and across
-// the warps, and each thread writes its own indices.
-__global__ void __launch_bounds__(1024)
-compact_small_kernel(const uint8_t* __restrict__ mask, int rows, int32_t* __restrict__ kept,
-                     int32_t* __restrict__ count, ScratchHeader* hdr, uint8_t* __restrict__ copy)
+// Small masks: one pass, one 4096-row sub-tile per block; the number of kept rows in front of it every block counts
+// itself, from the mask (up to 192 KB out of L2, loads in flight together, beside its own tile's scan), so no block needs
+// another one's result and there is one launch instead of two.
+__global__ void __launch_bounds__(COMPACT_THREADS)
+compact_prefix_kernel(const uint8_t* __restrict__ mask, int rows, int32_t* __restrict__ kept, int32_t* __restrict__ count,
+                      ScratchHeader* hdr, uint8_t* __restrict__ copy, int early_mask)
 {
-    __shared__ int s_warp_total[32];
+    __shared__ int32_t s_idx[COMPACT_TILE];
+    __shared__ int s_own[COMPACT_THREADS / 32], s_before[COMPACT_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
-    const int first = tid * COMPACT_PER_THREAD;
-    unsigned flags = 0;
+    if (!early_mask) ptx::grid_dependency_wait();         // see compact_write_kernel
     const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+    const int tile_first = blockIdx.x * COMPACT_TILE, first = tile_first + tid * COMPACT_PER_THREAD;
+    unsigned flags = 0;
     if (aligned && first + COMPACT_PER_THREAD <= rows) {
         const uint4 v = __ldcg(reinterpret_cast<const uint4*>(mask + first));      // past L1: a kernel may have written the mask
         if (copy != nullptr) *reinterpret_cast<uint4*>(copy + first) = v;
-        flags = nonzero_bytes4(v.x) | (nonzero_bytes4(v.y) << 4) | (nonzero_bytes4(v.z) << 8) |
-                (nonzero_bytes4(v.w) << 12);
+        flags = nonzero_flags16(v);
     } else {
-        for (int j = 0; j < COMPACT_PER_THREAD; ++j)
-            if (first + j < rows) {
-                const uint8_t m = __ldcg(mask + first + j);
-                if (copy != nullptr) copy[first + j] = m;
-                if (m != 0) flags |= 1u << j;
-            }
+        for (int j = 0; j < COMPACT_PER_THREAD && first + j < rows; ++j) {
+            const uint8_t m = __ldcg(mask + first + j);
+            if (copy != nullptr) copy[first + j] = m;
+            if (m != 0) flags |= 1u << flag_bit(j);
+        }
+    }
+    int before = 0;
+    if (aligned) {
+#pragma unroll 8
+        for (int i = tid * COMPACT_PER_THREAD; i < tile_first; i += COMPACT_TILE)
+            before += __popc(nonzero_flags16(__ldcg(reinterpret_cast<const uint4*>(mask + i))));
+    } else {
+#pragma unroll 8
+        for (int i = tid; i < tile_first; i += COMPACT_THREADS) before += __ldcg(mask + i) != 0;
     }
     const int mine = __popc(flags);
     int incl = mine;
@@ -289,26 +295,24 @@ compact_small_kernel(const uint8_t* __restrict__ mask, int rows, int32_t* __rest
         const int t = __shfl_up_sync(0xffffffffu, incl, d);
         if (lane >= d) incl += t;
     }
-    if (lane == 31) s_warp_total[warp] = incl;
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31) { s_own[warp] = incl; s_before[warp] = before; }
     __syncthreads();
-    // every warp scans the 32 warp totals itself: lane i holds the total of warp i
-    int wt = s_warp_total[lane], winc = wt;
+    int at = incl - mine, tot = 0, exclusive = 0;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, winc, d);
-        if (lane >= d) winc += t;
+    for (int i = 0; i < COMPACT_THREADS / 32; ++i) {
+        if (i < warp) at += s_own[i];
+        tot += s_own[i];
+        exclusive += s_before[i];
     }
-    const int warp_prefix = __shfl_sync(0xffffffffu, winc - wt, warp);
-    const int total = __shfl_sync(0xffffffffu, winc, 31);
-    int at = warp_prefix + incl - mine;
-    unsigned f = flags;
-    while (f) {
-        const int j = __ffs(f) - 1;
-        f &= f - 1;
-        kept[at++] = first + j;
-    }
-    if (tid == 0) {
-        *count = total;
+#pragma unroll
+    for (int j = 0; j < COMPACT_PER_THREAD; ++j)
+        if ((flags >> flag_bit(j)) & 1u) { s_idx[at] = first + j; ++at; }
+    __syncthreads();
+    if (early_mask) ptx::grid_dependency_wait();          // the list may still be read
+    for (int i = tid; i < tot; i += COMPACT_THREADS) kept[exclusive + i] = s_idx[i];
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+        *count = exclusive + tot;
         if (hdr != nullptr) { hdr->reserved = 0; hdr->error = 0; }     // a status query must find a clean word
     }
 }
@@ -328,7 +332,7 @@ static int resident_sms()               // SM count of the current device (looke
     return sms[dev];
 }
 
-static int tiles_for(int64_t rows)      // 4096-row units: sizes the scratch (8 bytes each; the passes use 4 bytes per resident block, at most one block per 16384 rows)
+static int tiles_for(int64_t rows)      // 4096-row units: sizes the scratch (8 bytes each; the passes use 4 bytes per resident block, at most one block per unit)
 {
     int64_t t = (rows + COMPACT_TILE - 1) / COMPACT_TILE;
     return (int)(t < 1 ? 1 : t);
@@ -339,27 +343,37 @@ int64_t compact_scratch_bytes(int64_t rows)
     return (int64_t)sizeof(ScratchHeader) + 8 * (int64_t)tiles_for(rows);
 }
 
+template <int SUB>
+static cudaError_t launch_two_passes(const uint8_t* mask, int64_t rows, int32_t* kept, int32_t* count, ScratchHeader* hdr, cudaStream_t st,
+                                     bool early_mask, uint8_t* copy)
+{
+    const int tiles = (int)((rows + SUB * COMPACT_TILE - 1) / (SUB * COMPACT_TILE));
+    // one resident block per run of tiles: eight blocks per SM, never more blocks than tiles (the scratch has
+    // 8 bytes per 4096 rows, i.e. room for two 32-bit counts per sub-tile)
+    const int grid = tiles < COMPACT_RESIDENT * resident_sms() ? tiles : COMPACT_RESIDENT * resident_sms();
+    unsigned* run_count = reinterpret_cast<unsigned*>(hdr + 1);
+    cudaError_t e = copy != nullptr
+                        ? launch_pdl(compact_copy_count_kernel<SUB>, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, copy, run_count)
+                        : launch_pdl(compact_count_kernel<SUB>, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, run_count);
+    if (e == cudaSuccess)
+        e = launch_pdl(early_mask ? compact_write_kernel<SUB, true> : compact_write_kernel<SUB, false>, dim3(grid), dim3(COMPACT_THREADS), 0, st,
+                       mask, (long long)rows, tiles, kept, static_cast<const unsigned*>(run_count), count, hdr);
+    return e;
+}
+
 cudaError_t launch_compact(const uint8_t* mask, int64_t rows, int32_t* kept, int32_t* count,
                            void* scratch, cudaStream_t st, bool mask_written_by_copies_only, uint8_t* copy)
 {
     auto* hdr = static_cast<ScratchHeader*>(scratch);
-    if (rows <= COMPACT_SMALL_MAX_ROWS)
-        return launch_pdl(compact_small_kernel, dim3(1), dim3(1024), 0, st, mask, (int)rows, kept, count, hdr, copy);
-    const int tiles = (int)((rows + COMPACT_BIG_TILE - 1) / COMPACT_BIG_TILE);
-    // one resident block per run of tiles: eight blocks per SM, never more blocks than tiles (the scratch has
-    // 8 bytes per 4096 rows, i.e. room for eight 32-bit counts per tile)
-    const int grid = tiles < COMPACT_RESIDENT * resident_sms() ? tiles : COMPACT_RESIDENT * resident_sms();
-    unsigned* run_count = reinterpret_cast<unsigned*>(hdr + 1);
-    cudaError_t e = copy != nullptr
-                        ? launch_pdl(compact_copy_count_kernel, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, copy, run_count)
-                        : launch_pdl(compact_count_kernel, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, run_count);
-    if (e == cudaSuccess)
-        e = mask_written_by_copies_only
-                ? launch_pdl(compact_write_kernel<true>, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, kept,
-                             static_cast<const unsigned*>(run_count), count, hdr)
-                : launch_pdl(compact_write_kernel<false>, dim3(grid), dim3(COMPACT_THREADS), 0, st, mask, (long long)rows, tiles, kept,
-                             static_cast<const unsigned*>(run_count), count, hdr);
-    return e;
+    // One pass while counting all bytes in front of the last block costs less than a second launch (about 2 us), and the
+    // bytes can be counted sixteen at a time; without that, while they are few.
+    const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+    if (rows <= (aligned ? COMPACT_PREFIX_MAX_ROWS : COMPACT_SMALL_MAX_ROWS))
+        return launch_pdl(compact_prefix_kernel, dim3((unsigned)tiles_for(rows)), dim3(COMPACT_THREADS), 0, st, mask,
+                          (int)rows, kept, count, hdr, copy, mask_written_by_copies_only ? 1 : 0);
+    return rows <= (int64_t)COMPACT_TILE * COMPACT_RESIDENT * resident_sms()
+               ? launch_two_passes<1>(mask, rows, kept, count, hdr, st, mask_written_by_copies_only, copy)
+               : launch_two_passes<COMPACT_SUB>(mask, rows, kept, count, hdr, st, mask_written_by_copies_only, copy);
 }
 
 }  // namespace asx

@@ -75,6 +75,7 @@ struct FastArgs {
     const int32_t* in_rank;   // non-null: x holds only the rows its own mask kept; in_rank[pos] = row of input position
                               // pos within its image's in_kept rows, or -1 for a dropped position (read as zeros)
     int in_kept;        // kept input positions per image
+    int mask_from_kernel;     // (without fuse_compact) the mask was written by a kernel that may still be running
     int ksplit;         // work items per output tile: each takes a contiguous share of the k-blocks
     int* split_hook;    // ksplit > 1: two ints per output tile, zero; a test makes a share wait for a partial sum that never comes
                         // by setting the first
@@ -175,8 +176,9 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Let the next kernel of the stream start its own prologue; everything up to the dependency
-    // wait below touches only this block's shared and tensor memory.
-    ptx::grid_launch_dependents();
+    // wait below touches only this block's shared and tensor memory.  (The next kernel may read the mask before its own
+    // wait, so while a kernel is still writing that, not yet.)
+    if (!a.mask_from_kernel) ptx::grid_launch_dependents();
     const int N = g.C_out;
 
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -250,6 +252,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     // for it here.  With it, the wait comes after the row decoding below, which needs only the list.
     if (!a.fuse_compact) {
         ptx::grid_dependency_wait();
+        if (a.mask_from_kernel) {
+            __threadfence();                 // the zero warps read the mask through L1, which may hold lines from before
+            ptx::grid_launch_dependents();
+        }
         cnt = __ldcg(a.count);
     }
     const int Mk = (g.rows == g.P) ? g.Nb * cnt : cnt;
@@ -1004,7 +1010,7 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
                         const int32_t* kept, const int32_t* count, int relu, int* dev_status,
                         int num_sms, int fuse_compact, int write_list, long long host_kept, int* split_hook,
                         int out_compact, const int32_t* in_rank, int in_kept, const void* residual, int f32, int wait_limit_kcycles,
-                        cudaStream_t st)
+                        int mask_from_kernel, cudaStream_t st)
 {
     if (f32 && (in_rank != nullptr || residual != nullptr)) return cudaErrorInvalidValue;
     FastArgs a;
@@ -1056,6 +1062,7 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
     long long tiles = split ? plan.items : ((long long)g.M + BM - 1) / BM * plan.n_tiles;
     int grid = (int)(split || tiles < num_sms ? tiles : num_sms);
     if (grid < 1) grid = 1;
+    a.mask_from_kernel = mask_from_kernel && !fuse_compact ? 1 : 0;
     const int variant = plan.vec + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
     const bool has_res = residual != nullptr, is_silu = relu == 2;
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const FastArgs);

@@ -187,3 +187,36 @@ def test_residual_add_before_the_activation(case, act):
     layer.close()
     plain = np.where(fm[:, None], f(lin), 0.0)
     _close(y.float().cpu().numpy().astype(np.float64), plain[rows] if compact else plain, spec.K, x, w)
+
+
+@pytest.mark.parametrize("case", [
+    # C_in, C_out, k, pad, H, W, Nb, kept input %, sparsity %, act
+    (64, 64, 3, 1, 17, 19, 3, 60, 30, 0), (128, 96, 3, 1, 28, 28, 2, 50, 50, 0), (64, 48, 5, 2, 9, 33, 2, 90, 0, 1),
+    (192, 256, 3, 0, 13, 14, 5, 3, 75, 0), (64, 64, 3, 1, 8, 61, 1, 50, 50, 1),
+], ids=lambda c: "x".join(str(v) for v in c))
+def test_window_patches_from_a_compact_input(case):
+    """The window-patch form fills its patches from the kept rows of the input: rows whose width is no multiple of
+    four, images that end inside a patch, nearly empty inputs."""
+    cin, cout, k, pad, H, W, Nb, keep, sp, act = case
+    spec = wl.LayerSpec("cpatch", cin, cout, k, k, 1, pad, H, W, Nb, sp, 1, "relu", wl.BASE_SEED + 310 + W)
+    x, w, b, m = wl.make_x(spec), wl.make_w(spec), wl.make_b(spec), wl.make_layer_mask(spec)
+    m_in = (np.random.default_rng(W).random(H * W) < keep / 100.0).astype(np.uint8)
+    m_in[H * W // 2] = 1
+    x_masked = x * np.tile(m_in, Nb).reshape(Nb, H, W, 1)
+    ref = oracle.masked_conv(x_masked, w, b, m, 1, pad, act == 1).reshape(spec.M, cout)
+    rows_in = (np.arange(Nb)[:, None] * H * W + np.flatnonzero(m_in)[None, :]).reshape(-1)
+    xc, wd, bd = to_dev_bf16(x.reshape(-1, cin)[rows_in]), to_dev_bf16(w), torch.from_numpy(b).cuda()
+    layer = asx.MaskedConvLayer(cin, cout, k, k, 1, pad)
+    layer.set_mask(m)
+    layer.set_input_mask(m_in)
+    flags = (asx.ACT_RELU if act else 0) | asx.IN_COMPACT | asx.IMPL_WINDOW_PATCH
+    rows_out = (np.arange(Nb)[:, None] * spec.P + np.flatnonzero(m)[None, :]).reshape(-1)
+    for more in (0, asx.RECOMPACT, asx.OUT_COMPACT):
+        n = rows_out.size if more == asx.OUT_COMPACT else spec.M
+        y = torch.full((n, cout), float("nan"), dtype=torch.bfloat16, device="cuda")
+        _run_raw(layer, xc, Nb, H, W, wd, bd, y, flags | more)
+        assert layer.last_run_form() == asx.FORM_WINDOW_PATCH
+        got = y.float().cpu().numpy().astype(np.float64)
+        assert not np.isnan(got).any()
+        _close(got, ref[rows_out] if more == asx.OUT_COMPACT else ref, spec.K, x, w)
+    layer.close()

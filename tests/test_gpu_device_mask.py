@@ -1,0 +1,65 @@
+"""Kept-row lists at the limits between the one-pass and the two-pass forms, from a caller's buffer and through
+set_mask with a mask that a kernel has just written."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2309_06626_b200 as asx
+import workloads as wl
+from gpu_util import to_dev_bf16
+
+pytestmark = pytest.mark.gpu
+
+ONE_PASS = 192 * 1024                    # largest mask of the one-pass form
+ONE_SUB_TILE = 4096 * 8 * 148            # largest mask whose blocks take one 4096-row sub-tile each (148 SMs)
+
+
+@pytest.mark.parametrize("rows", [1, 4095, 4096, 4097, 16384, 16385, ONE_PASS - 1, ONE_PASS, ONE_PASS + 1, ONE_SUB_TILE, ONE_SUB_TILE + 1])
+@pytest.mark.parametrize("offset", [0, 3], ids=["aligned", "unaligned"])
+def test_lists_at_the_limits(rows, offset):
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    mask = torch.randint(0, 3, (rows + offset,), generator=gen, device="cuda", dtype=torch.uint8)[offset:]
+    want = np.flatnonzero(mask.cpu().numpy()).astype(np.int32)
+    kept, count, _ = asx.compact_mask(mask)
+    assert int(count.item()) == want.size
+    assert np.array_equal(kept[:want.size].cpu().numpy(), want)
+    layer = asx.MaskedConvLayer(8, 8, 1, 1, 1, 0)
+    for m in (mask, torch.flip(mask, (0,)).contiguous()):       # the second one replaces the layer's copy of the first
+        layer.set_mask(m)
+        assert np.array_equal(layer.kept(), np.flatnonzero(m.cpu().numpy()).astype(np.int32))
+    layer.close()
+
+
+@pytest.mark.parametrize("cin,cout,k", [(64, 128, 3), (32, 48, 3), (128, 64, 1)])
+def test_masks_change_from_pass_to_pass(cin, cout, k):
+    """mask_from_activation, set_mask and three runs with no synchronisation in between, on rounds of other activations:
+    the first run waits for the mask on the device, the second starts in stream order, the third overlaps."""
+    spec = wl.LayerSpec("dyn", cin, cout, k, k, 1, k // 2, 24, 31, 5, 0, 1, "relu", wl.BASE_SEED + 900 + cin)
+    w, b = wl.make_w(spec), wl.make_b(spec)
+    wd, bd = to_dev_bf16(w), torch.from_numpy(b).cuda()
+    layer = asx.MaskedConvLayer(cin, cout, k, k, 1, k // 2)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    xs = []
+    for r in range(6):
+        x = torch.relu(torch.randn((spec.Nb, spec.H, spec.W, cin), generator=gen, device="cuda")).to(torch.bfloat16)
+        dead = torch.rand((spec.Nb, spec.H, spec.W, 1), generator=gen, device="cuda") < 0.15 * r
+        xs.append(x.masked_fill(dead, 0))
+    torch.cuda.synchronize()
+    got = []
+    for x in xs:
+        mask = asx.mask_from_activation(x)
+        layer.set_mask(mask)
+        got.append((mask, [layer.run(x, wd, bd).clone() for _ in range(2)] + [layer.run(x, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT).clone()]))
+    torch.cuda.synchronize()
+    assert layer.device_status() == 0
+    layer.close()
+    for x, (mask, ys) in zip(xs, got):
+        xf = x.float().cpu().numpy()
+        m = oracle.mask_from_activation(xf.reshape(spec.M, cin))
+        assert np.array_equal(mask.reshape(-1).cpu().numpy(), m)
+        ref = oracle.masked_conv(xf, w, b, m, 1, k // 2, True).reshape(spec.M, cout)
+        for y in ys:
+            g = y.float().cpu().numpy().astype(np.float64).reshape(spec.M, cout)
+            assert np.linalg.norm(g - ref) / np.linalg.norm(ref) < 5e-3
+            assert not g[m == 0].any()
