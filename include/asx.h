@@ -99,8 +99,8 @@ asx_status asx_create_layer(int C_in, int C_out, int kh, int kw, int stride, int
  *   rows : Ho*Wo (one mask shared by every image of a batch, the paper's constant per-layer
  *          mask) or Nb*Ho*Wo (one entry per lowered row); checked against the geometry at
  *          asx_run.  0 < rows < 2^31.
- * The copy and the compaction kernel are enqueued on `cuda_stream`; a host mask is copied
- * synchronously.  Device buffers owned by the layer are (re)allocated when `rows` grows.
+ * The copy and the compaction are enqueued on `cuda_stream`; a host mask has been read when the
+ * call returns (it waits for the copy of a page-locked one only).  Device buffers owned by the layer are (re)allocated when `rows` grows.
  */
 asx_status asx_set_mask(asx_layer* layer, const uint8_t* mask, int64_t rows, void* cuda_stream);
 
@@ -193,13 +193,13 @@ asx_status asx_recompact(asx_layer* layer, void* cuda_stream);
  *          mantissa bits are zero are multiplied exactly); sums, bias and activation are fp32 and y is
  *          written unrounded.  ASX_IMPL_NAIVE with ASX_F32 multiplies the full fp32 values.  Not
  *          together with ASX_OUT_COMPACT, ASX_IN_COMPACT or a residual (ASX_ERR_UNSUPPORTED).
- * Asynchronous on `cuda_stream`.  Allocates in two cases only, on first use and when the buffers
- * must grow: when C_in % 8 != 0 the layer keeps copies of x and w with the channels zero-padded to
- * a multiple of 8 (refreshed by a small kernel on every call); and when a layer has far fewer
- * 128-row tiles than the GPU has SMs and a long reduction (K of a few thousand), the k range of a
- * tile is shared between thread blocks that exchange fp32 partial tiles through a layer-owned
- * workspace (tiles x shares x 128 x tile width floats).  Partial sums are added in a fixed order,
- * so results do not depend on scheduling.  Errors: ASX_ERR_NO_MASK, ASX_ERR_SHAPE when
+ * Asynchronous on `cuda_stream`.  Allocates on first use and when a buffer must grow: copies of x and w
+ * with the channels zero-padded to a multiple of 8 (refreshed by a small kernel on every call) where
+ * C_in % 8 != 0 and the form that runs needs them, the row tiles of the window-patch form, and two
+ * words per tile for the test hook below.  When a layer has far fewer 128-row tiles than the GPU has SMs
+ * and a long reduction, the k range of a tile is shared between the thread blocks of a cluster, or the
+ * warps of a block, which exchange fp32 partial sums in shared memory.  Partial sums are added in a
+ * fixed order, so results do not depend on scheduling.  Errors: ASX_ERR_NO_MASK, ASX_ERR_SHAPE when
  * the mask length is neither Ho*Wo nor Nb*Ho*Wo, ASX_ERR_INVALID_ARG, ASX_ERR_ALIGN,
  * ASX_ERR_UNSUPPORTED when Nb*Ho*Wo or a tensor's element count reaches 2^31.
  */
@@ -254,13 +254,13 @@ asx_status asx_set_wait_limit(asx_layer* layer, int64_t cycles);
 
 /*
  * Test hook for the bounded waits (no counterpart in the paper).  Layers with few kept rows and a long
- * reduction share a tile's k-blocks between thread blocks, which meet at a per-tile arrival counter in
- * the layer's workspace.  This call overwrites the arrival counter of output tile `tile` with `value`
- * (in stream order); a value the arrivals can never lift to the number of shares makes the waiting
- * blocks run into their wait limit, which is how the time-out path is exercised from the host without
- * faulting or hanging the GPU.  ASX_ERR_UNSUPPORTED if the layer's last plan did not share k-blocks (no
- * counters exist), ASX_ERR_INVALID_ARG for a tile outside the workspace.  asx_last_device_status puts
- * the counters back to zero after a reported time-out.
+ * reduction share a tile's k-blocks between thread blocks, which wait for each other's partial sums.
+ * This call sets a word of output tile `tile` to `value` (in stream order); a value other than zero makes
+ * the tile's blocks wait for partial sums that nobody sends, until they run into their wait limit, which
+ * is how the time-out path is exercised from the host without faulting or hanging the GPU.
+ * ASX_ERR_UNSUPPORTED if no plan of the layer shared k-blocks so far (the words do not exist),
+ * ASX_ERR_INVALID_ARG for a tile outside the plan.  asx_last_device_status puts the words back to zero
+ * after a reported time-out.
  */
 asx_status asx_debug_set_split_counter(asx_layer* layer, int64_t tile, int32_t value, void* cuda_stream);
 
