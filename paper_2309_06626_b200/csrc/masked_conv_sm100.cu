@@ -34,6 +34,7 @@ namespace asx {
 namespace {
 
 constexpr int BM = 128;                 // kept rows per tile (UMMA M)
+constexpr int MIN_TILE_ROWS = 32;       // least kept rows per tile: every tile reads its filter slabs whole
 constexpr int BK = 64;                  // K elements per pipeline stage (one 128-byte swizzled row)
 constexpr int A_STAGE_BYTES = BM * BK * 2;
 static_assert(BK == 64, "the MMA loop issues four K=16 instructions per stage");
@@ -76,6 +77,7 @@ struct FastArgs {
                               // pos within its image's in_kept rows, or -1 for a dropped position (read as zeros)
     int in_kept;        // kept input positions per image
     int mask_from_kernel;     // (without fuse_compact) the mask was written by a kernel that may still be running
+    FastDiv fdGrid;     // division by the blocks of the launch
     int ksplit;         // work items per output tile: each takes a contiguous share of the k-blocks
     int* split_hook;    // ksplit > 1: two ints per output tile, zero; a test makes a share wait for a partial sum that never comes
                         // by setting the first
@@ -125,6 +127,21 @@ __device__ __forceinline__ Item item_of(int t, int KB, const FastArgs& a)
     it.m_tile = (int)fd_div((uint32_t)it.tile, a.fdNt);
     it.n_tile = it.tile - it.m_tile * a.n_tiles;
     return it;
+}
+
+// Kept rows per tile of the cp.async gather: as few as the waves that tiles of 128 need leave room for.  A tile's time is
+// mostly that of its row copies (missing rows cost a shared-memory write instead of a read from L2), so a few full tiles on
+// some of the SMs take longer than smaller ones on all of them: 12,240 rows of a 120 -> 255 channel 3x3 layer, 96 tiles of
+// 128 -> 148 of 84, 59.9 -> 45.8 us.  (The TMA gather, whose tiles cost their hand-overs, gained nothing on average: its
+// single-wave layers lost 5-30 %.)
+__device__ __forceinline__ int rows_per_tile(int Mk, const FastArgs& a)
+{
+    const int full = (Mk + BM - 1) / BM;                                                  // tiles of 128 rows
+    const uint32_t waves = fd_div((uint32_t)(full * a.n_tiles) + gridDim.x - 1, a.fdGrid);
+    const int tiles = (int)fd_div(waves * gridDim.x, a.fdNt);
+    if (tiles <= 0) return BM;
+    const int r = ((Mk + tiles - 1) / tiles + 3) & ~3;
+    return r < MIN_TILE_ROWS ? MIN_TILE_ROWS : r < BM ? r : BM;
 }
 
 // Rows of a tile that the TMA row gather fetches: the tile's kept rows in fours.  The rest of a last tile's stage keeps
@@ -261,7 +278,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     const int Mk = (g.rows == g.P) ? g.Nb * cnt : cnt;
     // With every position dropped there are no tiles; the zero warps then write the whole output
     // (Algorithm 2, mask == 0 branch).
-    const int m_tiles = (Mk + BM - 1) / BM;
+    const int rpt = MODE == GATHER_CPASYNC && !SPLIT ? rows_per_tile(Mk, a) : BM;
+    const int m_tiles = (Mk + rpt - 1) / rpt;
     int total_tiles = m_tiles * a.n_tiles * (SPLIT ? a.ksplit : 1);     // work items
     if (SPLIT && total_tiles > a.split_items) {       // cannot happen when the host sized the grid from this mask
         if (tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);
@@ -277,7 +295,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             const int jj = idx / BM, rr = idx - jj * BM;
             const long long t = blockIdx.x + (long long)jj * gridDim.x;
             if (t < total_tiles)
-                sh->rowinfo[jj][rr] = row_info_of(item_of<SPLIT>((int)t, KB, a).m_tile * BM + rr, Mk, fdcnt, g, a, kept_list);
+                sh->rowinfo[jj][rr] = row_info_of(rr < rpt ? item_of<SPLIT>((int)t, KB, a).m_tile * rpt + rr : Mk, Mk, fdcnt, g, a, kept_list);
         }
         __syncthreads();
         if (tid < INFO_RING && blockIdx.x + (long long)tid * gridDim.x < total_tiles) ptx::mbar_arrive(ptx::smem_u32(&sh->info_full[tid]));
@@ -334,8 +352,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             int rows4[4];
 #pragma unroll
             for (int q2 = 0; q2 < 4; ++q2) {
-                const int rk = m_tile * BM + lane * 4 + q2;
-                rows4[q2] = rk < Mk ? out_row_of(rk, fdcnt, g, kept_list) : -1;
+                const int rr = lane * 4 + q2, rk = m_tile * rpt + rr;
+                rows4[q2] = rr < rpt && rk < Mk ? out_row_of(rk, fdcnt, g, kept_list) : -1;
             }
 #pragma unroll
             for (int q2 = 0; q2 < 4; ++q2) sh->rowinfo[r][lane * 4 + q2] = row_info_from_row(rows4[q2], g, a);
@@ -403,8 +421,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             // kept rows from the accumulator
             const int buf = ti & 1;
             const uint32_t use = (uint32_t)(ti >> 1) & 1u;
-            const int rk = m_tile * BM + q * 32 + lane;
-            const bool valid = rk < Mk;
+            const int rk = m_tile * rpt + q * 32 + lane;
+            const bool valid = q * 32 + lane < rpt && rk < Mk;
             const long long yoff = valid ? (long long)(a.out_compact ? rk : out_row_of(rk, fdcnt, g, kept_list)) * N : 0;
             {
                 float* sb = sh->bias[buf];
@@ -961,13 +979,12 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     // three ran in two waves).
     int best_BN = 0, best_KS = 1;
     double best_cost = 0.0;
-    const double fill = std::min(1.0, (double)est_kept_rows / (double)(m_tiles * BM));       // rows gathered of a tile's 128
+    const bool level = g.C_in % bke != 0;                                                    // see rows_per_tile
     int halving = (N + 255) / 256;                // tile widths of whole tiles: 256 or less, then halves
     for (int n_tiles = halving; ; ++n_tiles) {
         const int per = (N + n_tiles - 1) / n_tiles;
         const int BN = ((per + 15) / 16) * 16;
         const int nt = (N + BN - 1) / BN;
-        const double t_kb = 0.12 + 0.18 * fill + 0.001 * BN;                  // microseconds
         const bool whole = n_tiles == halving;
         if (whole) halving *= 2;
         for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); KS += KS == 1 ? 1 : 2) {
@@ -979,6 +996,10 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
             if (KS > 1 && items > room) continue;
             const long long waves = (items + room - 1) / room;
             const int kbi = (KB + KS - 1) / KS;
+            // rows gathered of a tile's 128
+            const double tiles = KS == 1 && level ? std::max(1.0, (double)(waves * room / nt)) : (double)m_tiles;
+            const double fill = std::min(1.0, std::max(level ? (double)MIN_TILE_ROWS / BM : 0.0, (double)est_kept_rows / (tiles * BM)));
+            const double t_kb = 0.12 + 0.18 * fill + 0.001 * BN;                  // microseconds
             // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
             const double cost = (double)waves * (kbi * t_kb + 0.3) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
             if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_cost = cost; }
@@ -1059,9 +1080,11 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
 
     // Shared k-blocks: one item per block (the host knows the count).  Else as many resident blocks as there may be items.
     const bool split = plan.ksplit > 1;
-    long long tiles = split ? plan.items : ((long long)g.M + BM - 1) / BM * plan.n_tiles;
+    const long long least = !split && plan.vec == GATHER_CPASYNC ? MIN_TILE_ROWS : BM;      // rows per tile
+    const long long tiles = split ? plan.items : ((long long)g.M + least - 1) / least * plan.n_tiles;
     int grid = (int)(split || tiles < num_sms ? tiles : num_sms);
     if (grid < 1) grid = 1;
+    a.fdGrid = make_fastdiv((uint32_t)grid);
     a.mask_from_kernel = mask_from_kernel && !fuse_compact ? 1 : 0;
     const int variant = plan.vec + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
     const bool has_res = residual != nullptr, is_silu = relu == 2;
