@@ -823,7 +823,8 @@ def run_ours(args):
                        "ms_in_step": None if in_step_ms is None else in_step_ms[i],
                        "ms_serialised": per_layer_ms[i], "tflops": L.flops / (per_layer_ms[i] * 1e-3) / 1e12,
                        "gbs": L.bytes / (per_layer_ms[i] * 1e-3) / 1e9, "roof_ms": roofs[i],
-                       "form": {0: "none", 1: "naive", 2: "row gather (copies)", 3: "row gather (TMA)", 4: "window patch"}[forms[i]]}
+                       "form": {0: "none", 1: "naive", 2: "row gather (copies)", 3: "row gather (TMA)", 4: "window patch",
+                                5: "direct", 6: "direct, shared k range"}[forms[i]]}
                       for i, L in enumerate(layers)],
     }
     print(json.dumps(line), flush=True)
