@@ -439,7 +439,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 // ---- split K: this item holds a partial sum.  The shares of a tile are the blocks of a cluster; share k
                 // finishes 8-column groups gps k .. gps k + gps - 1 of the tile (gps = ceil(groups / ksplit)).  Every share
                 // sends each other one its partial sums of that one's columns straight from its registers to that block's
-                // shared memory ([share][group][half][R rows] 16 bytes, R the tile's rows rounded up to whole warps; a bulk copy
+                // shared memory ([other share][group][half][R rows] 16 bytes, R the tile's rows rounded up to whole warps; a bulk copy
                 // by the TMA unit from a staging area took 1.4 us to arrive, these stores 0.3), then adds what it received in
                 // share order (the result does not depend on which block finished first) and writes its columns of y.
                 const int KS = a.ksplit, gps = (int)a.fdGps.d, trow = q * 32 + lane;
@@ -454,7 +454,6 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                     ptx::mbar_arrive_expect_tx(recv_bar, (uint32_t)((KS - 1) * groups) * 2 * half + (uint32_t)never);
                 }
                 if (q * 32 < R) {
-                    const uint32_t mine = recv + (uint32_t)item.ks * slot + (uint32_t)trow * 16;
                     for (int c0 = 0; c0 < BN; c0 += 32) {
                         uint32_t r[32];
                         if (c0 + 32 <= BN) {
@@ -471,11 +470,9 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                             const int gq = (c0 >> 3) + h;
                             if (c0 + 8 * h >= BN) break;
                             const int dst = (int)fd_div((uint32_t)gq, a.fdGps);
-                            const uint32_t at = mine + (uint32_t)(gq - dst * gps) * 2 * half;
-                            if (dst == item.ks) {
-                                ptx::st_shared_v4(at, r[8 * h], r[8 * h + 1], r[8 * h + 2], r[8 * h + 3]);
-                                ptx::st_shared_v4(at + half, r[8 * h + 4], r[8 * h + 5], r[8 * h + 6], r[8 * h + 7]);
-                            } else {
+                            if (dst != item.ks) {            // this share's own columns stay in tensor memory
+                                const uint32_t at = recv + (uint32_t)(item.ks - (item.ks > dst ? 1 : 0)) * slot + (uint32_t)(gq - dst * gps) * 2 * half +
+                                                    (uint32_t)trow * 16;
                                 const uint32_t to = ptx::cluster_map(at, (uint32_t)dst), to_bar = ptx::cluster_map(recv_bar, (uint32_t)dst);
                                 ptx::st_cluster_v4(to, to_bar, r[8 * h], r[8 * h + 1], r[8 * h + 2], r[8 * h + 3]);
                                 ptx::st_cluster_v4(to + half, to_bar, r[8 * h + 4], r[8 * h + 5], r[8 * h + 6], r[8 * h + 7]);
@@ -483,22 +480,31 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                         }
                     }
                 }
-                ptx::tc_fence_before_sync();
                 if (!warp_wait_bar<20>(recv_bar, 0u, abort_flag, a.dev_status)) { ok = false; break; }
                 ptx::fence_cluster();
-                if (!valid) continue;
                 for (int gl = 0; gl < gps; ++gl) {
                     const int gq = item.ks * gps + gl;
                     if (gq * 8 >= BN || n0 + gq * 8 >= N) break;
+                    uint32_t own[8];
+                    __syncwarp();
+                    ptx::tmem_ld_8(tacc + (uint32_t)(gq * 8), own);
+                    ptx::tmem_ld_wait();
+                    if (!valid) continue;
                     float v[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[j] = 0.f;
                     uint32_t src = recv + (uint32_t)gl * 2 * half + (uint32_t)trow * 16;
 #pragma unroll 4
-                    for (int sp = 0; sp < KS; ++sp, src += slot) {                   // always in share order
+                    for (int sp = 0; sp < KS; ++sp) {                                // always in share order
                         uint32_t p[8];
-                        ptx::ld_shared_v4(src, p[0], p[1], p[2], p[3]);
-                        ptx::ld_shared_v4(src + half, p[4], p[5], p[6], p[7]);
+                        if (sp == item.ks) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) p[j] = own[j];
+                        } else {
+                            ptx::ld_shared_v4(src, p[0], p[1], p[2], p[3]);
+                            ptx::ld_shared_v4(src + half, p[4], p[5], p[6], p[7]);
+                            src += slot;
+                        }
 #pragma unroll
                         for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(p[j]);
                     }
@@ -522,6 +528,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
                     }
                 }
+                ptx::tc_fence_before_sync();
                 continue;                                         // one item per block: nobody waits for the accumulator
             }
             for (int c0 = 0; c0 < BN; c0 += 32) {
@@ -954,7 +961,7 @@ int cluster_room(int KS)
     return room;
 }
 // Shared memory for the partial sums that a share receives.
-int split_bytes(int BN, int KS) { return KS > 1 ? KS * ((BN / 8 + KS - 1) / KS) * 2 * BM * 16 : 0; }
+int split_bytes(int BN, int KS) { return (KS - 1) * ((BN / 8 + KS - 1) / KS) * 2 * BM * 16; }
 }  // namespace
 
 bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fused_list_rows, bool allow_split, int elem_bytes,
@@ -975,11 +982,11 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     // requests and bytes one SM can pull from L2: 16 KB of gathered rows in 32 requests of about
     // 13 clocks, plus the BN x 128-byte filter slab), the last tile's epilogue about 0.012 BN,
     // and the exchange SPLIT_US (cluster barriers, BN x 512 bytes through distributed shared memory in and out).
-    // A shared tile is its block's only one.  Clusters have an even size: SMs come in pairs (144 blocks in clusters of
-    // three ran in two waves).
+    // A shared tile is its block's only one, and clusters that do not all fit at once are not considered (a second wave costs
+    // more than sharing gains): the GPU tells how many do (148 blocks in twos, 132 in fours, 120 in eights).
     int best_BN = 0, best_KS = 1;
     double best_cost = 0.0;
-    const bool level = g.C_in % bke != 0;                                                    // see rows_per_tile
+    const double fill = std::min(1.0, (double)est_kept_rows / (double)(m_tiles * BM));       // rows gathered of a tile's 128
     int halving = (N + 255) / 256;                // tile widths of whole tiles: 256 or less, then halves
     for (int n_tiles = halving; ; ++n_tiles) {
         const int per = (N + n_tiles - 1) / n_tiles;
@@ -987,7 +994,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
         const int nt = (N + BN - 1) / BN;
         const bool whole = n_tiles == halving;
         if (whole) halving *= 2;
-        for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); KS += KS == 1 ? 1 : 2) {
+        for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); ++KS) {
             const int gps = (BN / 8 + KS - 1) / KS;
             if (KS > 1 && (KB / KS < 2 || (KS - 1) * gps >= BN / 8)) continue;       // every share finishes some columns
             if (227 * 1024 - fixed - split_bytes(BN, KS) < MIN_STAGES * (A_STAGE_BYTES + BN * BK * 2)) continue;
@@ -996,9 +1003,6 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
             if (KS > 1 && items > room) continue;
             const long long waves = (items + room - 1) / room;
             const int kbi = (KB + KS - 1) / KS;
-            // rows gathered of a tile's 128
-            const double tiles = KS == 1 && level ? std::max(1.0, (double)(waves * room / nt)) : (double)m_tiles;
-            const double fill = std::min(1.0, std::max(level ? (double)MIN_TILE_ROWS / BM : 0.0, (double)est_kept_rows / (tiles * BM)));
             const double t_kb = 0.12 + 0.18 * fill + 0.001 * BN;                  // microseconds
             // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
             const double cost = (double)waves * (kbi * t_kb + 0.3) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);

@@ -106,10 +106,6 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t bar, uint3
                  "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
 
 // ---------------------------------------------------------------- proxies, cp.async
 __device__ __forceinline__ void fence_proxy_async_smem()
@@ -270,6 +266,14 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
                  : "memory");
 }
 // 32 lanes x 16 consecutive 32-bit columns: thread i of the warp gets lane (base + i).
+__device__ __forceinline__ void tmem_ld_8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_ld_16(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(
