@@ -508,7 +508,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             FastPlan fp;
             PatchPlan pp;
             other = plan_fast(g, L->num_sms, known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp) ? fp.est_cost_us : 1e9;
-            if (!f32 && plan_patch(g, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
+            if (!f32 && plan_patch(g, recompact && L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
                 plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, false, &pp);
                 other = std::min(other, pp.est_cost_us);
             }
@@ -532,8 +532,10 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
                                        f32 ? 1 : 0, L->num_sms, st));
     }
     // Also without ASX_RECOMPACT: the list in global memory is behind the dependency wait (an earlier kernel may have
-    // written it), the mask is not.
-    bool fuse_compact = !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS;
+    // written it), the mask is not; that is worth 0.4 us a launch.  Right after a kernel wrote the mask it has to wait for
+    // that as well (3-4 us).  The window-patch form has its row tiles from the host and reads the list late: building it
+    // there costs 0.6 us for a mask of 3136 rows, 2 us for 15,000.
+    bool fuse_compact = !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS && (recompact || mask_from_kernel == 0);
     if (recompact && !fuse_compact) {
         s = run_compaction(L, st);
         if (s != ASX_OK) return s;
@@ -706,7 +708,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     ConvGeom gp = g;
     if (blocks2x2) gp.H = g.Ho + g.kh - 1;
     if (!f32 && !(flags & ASX_IMPL_ROW_GATHER) && !L->host_mask.empty() &&
-        (reinterpret_cast<uintptr_t>(y) & 15) == 0 && plan_patch(gp, fuse_compact ? (int)L->rows : 0, blocks2x2 ? 1 : 0, &pplan)) {
+        (reinterpret_cast<uintptr_t>(y) & 15) == 0 && plan_patch(gp, fuse_compact && recompact ? (int)L->rows : 0, blocks2x2 ? 1 : 0, &pplan)) {
         if (L->tiles_epoch != L->mask_epoch || L->tiles_Nb != Nb || L->tiles_H != H || L->tiles_W != W || L->tiles_cap != pplan.cap_rows) {
             std::vector<int32_t> kept;
             try {
@@ -825,7 +827,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     if (use_patch) {
         L->last_form = ASX_FORM_WINDOW_PATCH;
         return from_cuda(launch_patch(gp, pplan, L->tmap, in_compact ? L->tmap_x : L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
-                                      fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
+                                      fuse_compact && recompact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
                                       out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->wait_limit_kcycles, st));
     }
     if (plan.vec == 2) {
