@@ -43,7 +43,9 @@ constexpr int MIN_STAGES = 4;
 constexpr int WARP_TMA = 0, WARP_MMA = 1, WARP_EPI0 = 2, WARP_PROD0 = 6;
 constexpr int NUM_PROD_WARPS = 16, NUM_EPI_WARPS = 4;
 constexpr int GROUP_WARPS = 8;          // gather warps per group: 8 warps x 16 rows = one 128-row stage
-constexpr int INFO_RING = 8;            // tiles whose row coordinates are kept in shared memory (power of two)
+constexpr int PLAIN_INFO_RING = 8;      // tiles whose row coordinates are kept in shared memory (power of two); with shared
+                                        // k-blocks a block has one tile, and 7 KB more for stages (512 -> 512 channels at 7x7,
+                                        // batch 64: room for tiles 176 wide in three shares, 22.3 -> 19.9 us)
 constexpr int WARP_ZERO0 = WARP_PROD0 + NUM_PROD_WARPS, NUM_ZERO_WARPS = 4;
 constexpr int WARP_INFO = WARP_ZERO0 + NUM_ZERO_WARPS;
 constexpr int NUM_THREADS = 32 * (WARP_INFO + 1);
@@ -86,7 +88,8 @@ struct FastArgs {
     int wait_limit_kcycles;   // bound of every wait in the kernel, in units of 1024 clock cycles
 };
 
-struct alignas(16) Shared {           // lives after the operand stages
+template <int INFO_RING>
+struct alignas(16) SharedT {           // lives after the operand stages
     int2 rowinfo[INFO_RING][BM];   // per tile row: first input pixel index, (iy0 << 16) | (ix0 & 0xffff)
     float bias[2][256];   // bias of the tile's columns, double buffered
     unsigned long long info_full[INFO_RING];
@@ -189,6 +192,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                          const ConvGeom g, const FastArgs a)
 {
+    constexpr int INFO_RING = SPLIT ? 1 : PLAIN_INFO_RING;
+    using Shared = SharedT<INFO_RING>;
     extern __shared__ uint8_t smem_raw[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -973,7 +978,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const long long m_tiles = (est_kept_rows + BM - 1) / BM > 0 ? (est_kept_rows + BM - 1) / BM : 1;
     if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
     const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
-    const int fixed = 1024 + (int)sizeof(Shared) + list_bytes;
+    auto fixed_bytes = [&](int KS) { return 1024 + (int)(KS > 1 ? sizeof(SharedT<1>) : sizeof(SharedT<PLAIN_INFO_RING>)) + list_bytes; };
     // Tile width and k shares.  A wider tile does more work per gathered byte, a narrower one
     // gives more tiles when a layer has few kept rows, and sharing a tile's k-blocks between the blocks of a
     // cluster gives more work items still, at the price of exchanging fp32 partial tiles.  Pick
@@ -997,7 +1002,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
         for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); ++KS) {
             const int gps = (BN / 8 + KS - 1) / KS;
             if (KS > 1 && (KB / KS < 2 || (KS - 1) * gps >= BN / 8)) continue;       // every share finishes some columns
-            if (227 * 1024 - fixed - split_bytes(BN, KS) < MIN_STAGES * (A_STAGE_BYTES + BN * BK * 2)) continue;
+            if (227 * 1024 - fixed_bytes(KS) - split_bytes(BN, KS) < MIN_STAGES * (A_STAGE_BYTES + BN * BK * 2)) continue;
             const long long items = m_tiles * nt * KS;
             const int room = KS == 1 ? num_sms : cluster_room(KS);
             if (KS > 1 && items > room) continue;
@@ -1014,7 +1019,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const int BN = best_BN;
     const int n_tiles = (N + BN - 1) / BN;
     const int stage_bytes = A_STAGE_BYTES + BN * BK * 2;
-    int S = (227 * 1024 - fixed - split_bytes(BN, best_KS)) / stage_bytes;
+    int S = (227 * 1024 - fixed_bytes(best_KS) - split_bytes(BN, best_KS)) / stage_bytes;
     if (S > MAX_STAGES) S = MAX_STAGES;
     plan->BN = BN;
     plan->n_tiles = n_tiles;
@@ -1023,7 +1028,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     plan->items = (long long)m_tiles * n_tiles * best_KS;
     plan->stages = S;
     plan->list_bytes = list_bytes;
-    int smem = fixed + S * stage_bytes + split_bytes(BN, best_KS);
+    int smem = fixed_bytes(best_KS) + S * stage_bytes + split_bytes(BN, best_KS);
     if (smem < 120 * 1024) smem = 120 * 1024;      // one block per SM: tensor memory is not shared out
     plan->smem_bytes = smem;
     plan->vec = (g.C_in % bke == 0) ? GATHER_TMA : GATHER_CPASYNC;
