@@ -496,7 +496,10 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     const bool recompact = (flags & ASX_RECOMPACT) != 0, dense = !in_compact && !out_compact;
     DirectPlan dplan;
     DirectKPlan kplan;
+    // Its word form reads x in 4-byte words.  An x that lies between two words (allowed where the channels are no whole
+    // 16-byte chunks) takes the padded copy of the other forms.
     const bool direct = dense && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) &&
+                        (dplan.words == 0 || (reinterpret_cast<uintptr_t>(x) & 3) == 0) &&
                         (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, known_rows < 0 ? M : known_rows));
     bool direct_k = dense && (impl == 0 || impl == ASX_IMPL_DIRECT_K) && plan_direct_k(g, ES, known_rows, L->num_sms, &kplan);
     if (direct_k && impl == 0) {

@@ -1,0 +1,174 @@
+// A CUDA runtime of the host's own memory, and launches that only write a line to a log: with it the host side of the
+// C ABI (csrc/asx_api.cu, which holds no kernel) runs on a machine without a GPU, and a test can make a call of the runtime fail.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <string>
+#include "asx_internal.h"
+
+namespace {
+std::string log_text;
+int mallocs_left = -1;      // allocations that still succeed; -1: all
+int capturing = 0;
+int direct_words = 0;       // what plan_direct says: 0 the geometry does not take the direct form, else the words of a filter row
+int patch = 0;              // whether plan_patch accepts the geometry
+
+void say(const std::string& s) { log_text += s + "\n"; }
+std::string order() { return asx::launch_in_stream_order ? " in order" : ""; }
+
+CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill)
+{
+    return CUDA_SUCCESS;
+}
+}  // namespace
+
+extern "C" {
+
+void fake_set(const char* what, int value)
+{
+    const std::string w = what;
+    if (w == "mallocs_left") mallocs_left = value;
+    else if (w == "capturing") capturing = value;
+    else if (w == "direct_words") direct_words = value;
+    else if (w == "patch") patch = value;
+    else std::abort();
+}
+const char* fake_log() { return log_text.c_str(); }
+void fake_clear_log() { log_text.clear(); }
+
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int)
+{
+    *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : 148;
+    return cudaSuccess;
+}
+cudaError_t cudaMalloc(void** p, size_t n)
+{
+    if (mallocs_left == 0) return cudaErrorMemoryAllocation;
+    if (mallocs_left > 0) --mallocs_left;
+    *p = std::aligned_alloc(256, (n + 255) / 256 * 256);
+    std::memset(*p, 0x5a, n);                               // nothing is zero that was not set
+    return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { std::memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
+// in a capture work is recorded, not done, and a wait for it fails
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t)
+{
+    if (capturing) say("recorded a copy");
+    else std::memcpy(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t)
+{
+    if (!capturing) std::memset(p, v, n);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s)
+{
+    *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+// addresses with bit 62 set stand for device memory
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p)
+{
+    std::memset(a, 0, sizeof(*a));
+    a->type = ((uintptr_t)p >> 62) & 1 ? cudaMemoryTypeDevice : cudaMemoryTypeUnregistered;
+    return cudaSuccess;
+}
+cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetDriverEntryPoint(const char*, void** f, unsigned long long, cudaDriverEntryPointQueryResult* q)
+{
+    *f = reinterpret_cast<void*>(&encode);
+    *q = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
+
+}  // extern "C"
+
+namespace asx {
+
+int64_t compact_scratch_bytes(int64_t rows) { return 8 + 8 * ((rows + 4095) / 4096); }
+cudaError_t launch_compact(const uint8_t*, int64_t, int32_t*, int32_t*, void*, cudaStream_t, bool early, uint8_t* copy)
+{
+    say(std::string("compact") + (copy ? " copy" : "") + (early ? " early" : "") + order());
+    return cudaSuccess;
+}
+bool plan_direct(const ConvGeom&, int, DirectPlan* p)
+{
+    *p = DirectPlan{};
+    p->words = direct_words;
+    return direct_words != 0;
+}
+bool direct_pays(const DirectPlan&, int, int64_t) { return true; }
+double direct_est_us(const DirectPlan&, int, int64_t, int) { return 1.0; }
+bool plan_direct_k(const ConvGeom&, int, int64_t, int, DirectKPlan*) { return false; }
+bool plan_fast(const ConvGeom&, int, long long, int, bool, int, FastPlan* p)
+{
+    *p = FastPlan{64, 1, 4, 120 * 1024, 1, 1, 1, 0, 10.0};
+    return true;
+}
+bool plan_patch(const ConvGeom& g, int, int, PatchPlan* p)
+{
+    *p = PatchPlan{};
+    p->BN = 64;
+    p->n_tiles = 1;
+    p->cap_rows = 64;
+    p->Hp = g.H + 2 * g.pad;
+    p->Wp = g.W + 2 * g.pad_w;
+    return patch != 0;
+}
+void plan_patch_cost(const ConvGeom&, int, long long, bool, PatchPlan* p) { p->est_cost_us = 1.0; }
+cudaError_t launch_direct(const ConvGeom&, const DirectPlan&, const void*, const void*, const float*, void*, const uint8_t*, int32_t*, int32_t*, int, const void*, int,
+                          int, cudaStream_t)
+{
+    say("direct" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_direct_k(const ConvGeom&, const DirectKPlan&, const void*, const void*, const float*, void*, const uint8_t*, int32_t*, int32_t*, int64_t, int,
+                            const void*, int, int*, cudaStream_t)
+{
+    say("direct k" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_naive(const ConvGeom&, const void*, const void*, const float*, void*, const uint8_t*, const int32_t*, const int32_t*, int, int, cudaStream_t)
+{
+    say("naive" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_fast(const ConvGeom&, const FastPlan&, const CUtensorMap&, const CUtensorMap&, const void*, const float*, void*, const uint8_t*, const int32_t*,
+                        const int32_t*, int, int*, int, int, int, long long, int*, int, const int32_t*, int, const void*, int, int, int waits_for_mask, cudaStream_t)
+{
+    say(std::string("row gather") + (waits_for_mask ? " waits for the mask" : "") + order());
+    return cudaSuccess;
+}
+cudaError_t launch_patch(const ConvGeom&, const PatchPlan&, const CUtensorMap&, const CUtensorMap&, const float*, void*, const uint8_t*, const int32_t*,
+                         const int32_t*, int, int*, int, int, int, long long, const void*, const void* tiles, int n, long long, int, const int32_t*, int, int, cudaStream_t)
+{
+    const int32_t* t = static_cast<const int32_t*>(tiles);
+    char line[160];
+    std::snprintf(line, sizeof(line), "window patch, %d tiles, the first: row %d, %d rows", n, t ? t[0] : -1, t ? t[1] : -1);
+    say(line + order());
+    return cudaSuccess;
+}
+cudaError_t launch_pad_channels(const void*, void*, long long, int, int, cudaStream_t)
+{
+    say("pad channels" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_stage_blocks2x2(const void*, void*, int, int, int, int, int, int, int, const void*, void*, int, int, int, int, int, cudaStream_t)
+{
+    say("stage blocks" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_pack_pair_filters(const void*, void*, int, int, int, int, int, int, cudaStream_t)
+{
+    say("pack pairs" + order());
+    return cudaSuccess;
+}
+cudaError_t launch_mask_from_activation(const void*, long long, int, uint8_t*, int, cudaStream_t) { return cudaSuccess; }
+
+}  // namespace asx

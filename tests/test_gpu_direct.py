@@ -131,3 +131,31 @@ def test_residual(impl, form):
     ref = np.maximum(ref, 0) * np.tile(mask, spec.Nb)[:, None]
     got = y.float().cpu().numpy().reshape(spec.M, -1)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 5e-3
+
+
+@pytest.mark.parametrize("impl", [0, asx.IMPL_DIRECT], ids=["default", "direct"])
+@pytest.mark.parametrize("offset", [0, 1, 2])
+@pytest.mark.parametrize("case", [(3, 32, 3, 2, 1, 18, 20, 2, 40, 2), (3, 64, 7, 2, 3, 32, 30, 2, 50, 4), (6, 16, 3, 1, 1, 10, 9, 2, 20, 1)],
+                         ids=["3x3x3", "7x7x3", "3x3x6"])
+def test_input_between_two_words(case, offset, impl):
+    """Channels that are no whole 16-byte chunks: x at any 2-byte address, the word form at 4-byte ones."""
+    spec = _spec(case, 5)
+    x, w, b, mask = make_problem(spec)
+    room = torch.zeros(x.size + 8, dtype=torch.bfloat16, device="cuda")
+    xd = room[offset:offset + x.size].view(x.shape)
+    xd.copy_(torch.from_numpy(x))
+    assert xd.data_ptr() % 4 == 2 * (offset % 2)
+    layer = asx.MaskedConvLayer(spec.C_in, spec.C_out, spec.kh, spec.kw, spec.stride, spec.pad)
+    layer.set_mask(mask)
+    y = layer.run(xd, to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU | impl)
+    torch.cuda.synchronize()
+    assert layer.device_status() == 0
+    if offset % 2:
+        assert layer.last_run_form() != asx.FORM_DIRECT
+    elif impl:
+        assert layer.last_run_form() == asx.FORM_DIRECT
+    layer.close()
+    ref = oracle.masked_conv(x, w, b, mask, spec.stride, spec.pad, True)
+    got = y.float().cpu().numpy().astype(np.float64).reshape(ref.shape)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 5e-3
+    assert not got.reshape(spec.M, -1)[np.tile(mask, spec.Nb) == 0].any()

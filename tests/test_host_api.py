@@ -1,0 +1,79 @@
+"""The host side of the C ABI on a machine without a GPU: csrc/asx_api.cu against a runtime that uses host memory and
+launches that only write to a log (fake_cuda.cpp)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2309_06626_b200", "csrc")
+DEVICE = 1 << 62                                # an address that the fake runtime takes for device memory
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "libasx_fake.so")
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"),
+                           "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", so, "-x", "c++", os.path.join(CSRC, "asx_api.cu"),
+                           os.path.join(CSRC, "mask_from_scores.cpp"), os.path.join(ROOT, "tests", "fake_cuda.cpp")])
+    L = ctypes.CDLL(so)
+    vp, ci = ctypes.c_void_p, ctypes.c_int
+    L.asx_create_layer.argtypes = [ci] * 6 + [ctypes.POINTER(vp)]
+    L.asx_set_mask.argtypes = [vp, vp, ctypes.c_int64, vp]
+    L.asx_set_input_mask.argtypes = [vp, vp, ctypes.c_int64, vp]
+    L.asx_run.argtypes = [vp, vp, ci, ci, ci, vp, vp, vp, ci, vp]
+    L.asx_destroy.argtypes = [vp]
+    L.fake_log.restype = ctypes.c_char_p
+    L.fake_set.argtypes = [ctypes.c_char_p, ci]
+    return L
+
+
+class Layer:
+    def __init__(self, L, C_in, C_out, k, stride, pad):
+        self.L, self.h = L, ctypes.c_void_p()
+        for what, value in (("mallocs_left", -1), ("capturing", 0), ("direct_words", 0), ("patch", 0)):
+            self.set(what, value)
+        assert L.asx_create_layer(C_in, C_out, k, k, stride, pad, ctypes.byref(self.h)) == 0
+
+    def set(self, what, value):
+        self.L.fake_set(what.encode(), value)
+
+    def set_mask(self, mask):
+        return self.L.asx_set_mask(self.h, mask if isinstance(mask, int) else mask.ctypes.data, 64 if isinstance(mask, int) else mask.size, None)
+
+    def run(self, Nb, H, W, x=DEVICE, flags=0):
+        """Status and the launches of one asx_run."""
+        self.L.fake_clear_log()
+        rc = self.L.asx_run(self.h, x, Nb, H, W, DEVICE + (1 << 40), None, DEVICE + (2 << 40), flags, None)
+        return rc, self.L.fake_log().decode().split("\n")[:-1]
+
+
+@pytest.fixture
+def layer(fake):
+    made = []
+
+    def make(*geometry):
+        made.append(Layer(fake, *geometry))
+        return made[-1]
+    yield make
+    for m in made:
+        fake.asx_destroy(m.h)
+
+
+IMPL_DIRECT, F32 = 512, 64
+
+
+@pytest.mark.parametrize("flags", [0, IMPL_DIRECT])
+def test_word_form_takes_word_aligned_inputs_only(layer, flags):
+    """x of 3 channels may lie at any 2-byte address; the direct form reads it in 4-byte words."""
+    m = layer(3, 32, 3, 2, 1)
+    m.set("direct_words", 5)
+    assert m.set_mask(np.ones(64, np.uint8)) == 0
+    assert m.run(1, 16, 16, flags=flags) == (0, ["direct"])
+    rc, launches = m.run(1, 16, 16, x=DEVICE + 2, flags=flags)
+    assert rc == 0 and "direct" not in launches and launches[-1] == "row gather"
+    assert m.run(1, 16, 16, x=DEVICE + 4, flags=flags) == (0, ["direct"])
+    assert m.run(1, 16, 16, x=DEVICE + 4, flags=flags | F32) == (0, ["direct"])
