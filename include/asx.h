@@ -101,6 +101,9 @@ asx_status asx_create_layer(int C_in, int C_out, int kh, int kw, int stride, int
  *          asx_run.  0 < rows < 2^31.
  * The copy and the compaction are enqueued on `cuda_stream`; a host mask has been read when the
  * call returns (it waits for the copy of a page-locked one only).  Device buffers owned by the layer are (re)allocated when `rows` grows.
+ * While `cuda_stream` is being captured into a graph a host mask is refused (ASX_ERR_CUDA; the layer
+ * keeps its mask and the capture goes on), since every replay would read the caller's memory again; a
+ * device mask is read again by every replay.  The same holds for the two calls below that generate a mask.
  */
 asx_status asx_set_mask(asx_layer* layer, const uint8_t* mask, int64_t rows, void* cuda_stream);
 

@@ -264,8 +264,6 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
     asx_status s = bind_device(L);
     if (s != ASX_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    s = ensure_mask_buffers(L, rows);
-    if (s != ASX_OK) return s;
     cudaPointerAttributes attr;
     bool on_device = false, pinned = true;
     if (cudaPointerGetAttributes(&attr, mask) == cudaSuccess) {
@@ -273,6 +271,17 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
         pinned = attr.type != cudaMemoryTypeUnregistered;
     } else
         cudaGetLastError();
+    if (!on_device) {
+        // a capture would record the copy and read the caller's memory at every replay, long after this call
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+            cudaGetLastError();                                    // the legacy stream beside a capturing one
+            return ASX_ERR_CUDA;
+        }
+        if (capture != cudaStreamCaptureStatusNone) return ASX_ERR_CUDA;
+    }
+    s = ensure_mask_buffers(L, rows);
+    if (s != ASX_OK) return s;
     cudaError_t e;
     if (on_device) {
         // one pass copies the mask and counts, or for a small one does everything; memory of another device is copied by

@@ -63,3 +63,32 @@ def test_masks_change_from_pass_to_pass(cin, cout, k):
             g = y.float().cpu().numpy().astype(np.float64).reshape(spec.M, cout)
             assert np.linalg.norm(g - ref) / np.linalg.norm(ref) < 5e-3
             assert not g[m == 0].any()
+
+
+def test_host_mask_is_refused_under_capture():
+    """The call fails, the layer keeps its mask and the capture goes on."""
+    spec = wl.LayerSpec("capture", 64, 64, 3, 3, 1, 1, 20, 21, 2, 50, 1, "relu", wl.BASE_SEED + 950)
+    x, w, b, mask = wl.make_x(spec), wl.make_w(spec), wl.make_b(spec), wl.make_layer_mask(spec)
+    xd, wd, bd = to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda()
+    layer = asx.MaskedConvLayer(64, 64, 3, 3, 1, 1)
+    layer.set_mask(mask)
+    want = layer.run(xd, wd, bd).clone()
+    pinned = torch.from_numpy(1 - mask).pin_memory()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for refused in (lambda: layer.set_mask(1 - mask), lambda: layer.set_mask(pinned),
+                        lambda: layer.set_mask_random(spec.P, 0.5, 1, 3)):
+            with pytest.raises(asx.AsxError) as e:
+                refused()
+            assert e.value.code == 7                         # ASX_ERR_CUDA
+        y = layer.run(xd, wd, bd)
+    y.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    assert np.array_equal(layer.kept(), oracle.kept_list(mask))
+    layer.set_mask(1 - mask)                                 # outside it is taken
+    assert np.array_equal(layer.kept(), oracle.kept_list(1 - mask))
+    del graph
+    layer.close()

@@ -77,3 +77,17 @@ def test_word_form_takes_word_aligned_inputs_only(layer, flags):
     assert rc == 0 and "direct" not in launches and launches[-1] == "row gather"
     assert m.run(1, 16, 16, x=DEVICE + 4, flags=flags) == (0, ["direct"])
     assert m.run(1, 16, 16, x=DEVICE + 4, flags=flags | F32) == (0, ["direct"])
+
+
+def test_host_mask_is_refused_under_capture(layer):
+    """Recorded, the copy would read the caller's memory at every replay."""
+    m = layer(24, 32, 3, 1, 1)
+    assert m.set_mask(np.ones(64, np.uint8)) == 0
+    m.L.fake_clear_log()
+    m.set("capturing", 1)
+    assert m.set_mask(np.zeros(64, np.uint8)) == 7                      # ASX_ERR_CUDA
+    assert m.L.asx_set_mask_random(m.h, ctypes.c_int64(64), ctypes.c_double(0.5), 1, ctypes.c_uint64(1), None) == 7
+    assert m.L.fake_log() == b""
+    assert m.set_mask(DEVICE) == 0                                      # stays accepted
+    m.set("capturing", 0)
+    assert m.set_mask(np.zeros(64, np.uint8)) == 0
