@@ -492,7 +492,11 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         explicit InOrder(bool on) { launch_in_stream_order = on; }
         ~InOrder() { launch_in_stream_order = false; }
     } in_order(mask_from_kernel != 0);
-    L->mask_from_kernel = 0;
+    // Only a launch that was made changes what the next one may do: until here, and below, the call can still fail.
+    auto launched = [L](cudaError_t e, int mask_still_from_kernel = 0) {
+        if (e == cudaSuccess) L->mask_from_kernel = mask_still_from_kernel;
+        return from_cuda(e);
+    };
     // Small masks are compacted inside the fused kernel itself (no launches of its own, and the list stays in
     // shared memory as 16-bit positions); the reference kernel and large masks take the stand-alone compaction
     // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
@@ -530,8 +534,8 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     if (direct_k) {
         L->last_form = ASX_FORM_DIRECT_K;
-        return from_cuda(launch_direct_k(g, kplan, x, w, bias, y, L->d_mask, recompact ? L->d_kept : nullptr, L->d_small, L->host_kept, relu, L->residual,
-                                         f32 ? 1 : 0, reinterpret_cast<int*>(L->d_small + 1), st));
+        return launched(launch_direct_k(g, kplan, x, w, bias, y, L->d_mask, recompact ? L->d_kept : nullptr, L->d_small, L->host_kept, relu, L->residual,
+                                        f32 ? 1 : 0, reinterpret_cast<int*>(L->d_small + 1), st));
     }
     if (direct) {
         const bool list = recompact && L->rows <= DIRECT_LIST_MAX_ROWS;
@@ -540,8 +544,8 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             if (s != ASX_OK) return s;
         }
         L->last_form = ASX_FORM_DIRECT;
-        return from_cuda(launch_direct(g, dplan, x, w, bias, y, L->d_mask, list ? L->d_kept : nullptr, list ? L->d_small : nullptr, relu, L->residual,
-                                       f32 ? 1 : 0, L->num_sms, st));
+        return launched(launch_direct(g, dplan, x, w, bias, y, L->d_mask, list ? L->d_kept : nullptr, list ? L->d_small : nullptr, relu, L->residual,
+                                      f32 ? 1 : 0, L->num_sms, st));
     }
     // Also without ASX_RECOMPACT: the list in global memory is behind the dependency wait (an earlier kernel may have
     // written it), the mask is not; that is worth 0.4 us a launch.  Right after a kernel wrote the mask it has to wait for
@@ -557,7 +561,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 
     if (flags & ASX_IMPL_NAIVE) L->last_form = ASX_FORM_NAIVE;
     if (flags & ASX_IMPL_NAIVE)
-        return from_cuda(launch_naive(g, x, w, bias, y, L->d_mask, L->d_kept, d_count, relu, f32 ? 1 : 0, st));
+        return launched(launch_naive(g, x, w, bias, y, L->d_mask, L->d_kept, d_count, relu, f32 ? 1 : 0, st));
 
     // Channel counts that are not a multiple of 8 are padded with zero channels in staging
     // copies of x and w (a filter tap of a pixel is then a whole number of 16-byte chunks); the
@@ -838,9 +842,9 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     if (use_patch) {
         L->last_form = ASX_FORM_WINDOW_PATCH;
-        return from_cuda(launch_patch(gp, pplan, L->tmap, in_compact ? L->tmap_x : L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
-                                      fuse_compact && recompact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
-                                      out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->wait_limit_kcycles, st));
+        return launched(launch_patch(gp, pplan, L->tmap, in_compact ? L->tmap_x : L->tmap_x4, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status, L->num_sms,
+                                     fuse_compact && recompact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
+                                     out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->wait_limit_kcycles, st));
     }
     if (plan.vec == 2) {
         s = map_rows();
@@ -848,14 +852,11 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     L->last_form = plan.vec == 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
     const bool waits_for_mask = mask_from_kernel == 2 && !fuse_compact;
-    if (waits_for_mask) {
-        launch_in_stream_order = false;
-        L->mask_from_kernel = 1;
-    }
-    return from_cuda(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
-                                 L->num_sms, fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->d_wscnt,
-                                 out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
-                                 waits_for_mask ? 1 : 0, st));
+    if (waits_for_mask) launch_in_stream_order = false;
+    return launched(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
+                                L->num_sms, fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->d_wscnt,
+                                out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
+                                waits_for_mask ? 1 : 0, st), waits_for_mask ? 1 : 0);
 }
 
 asx_status asx_get_kept(asx_layer* L, int64_t* count, const int32_t** dev_kept)

@@ -63,7 +63,7 @@ def layer(fake):
         fake.asx_destroy(m.h)
 
 
-IMPL_DIRECT, F32 = 512, 64
+IMPL_DIRECT, F32, RECOMPACT = 512, 64, 2
 
 
 @pytest.mark.parametrize("flags", [0, IMPL_DIRECT])
@@ -91,3 +91,20 @@ def test_host_mask_is_refused_under_capture(layer):
     assert m.set_mask(DEVICE) == 0                                      # stays accepted
     m.set("capturing", 0)
     assert m.set_mask(np.zeros(64, np.uint8)) == 0
+
+
+@pytest.mark.parametrize("flags,first", [(0, "row gather waits for the mask"), (RECOMPACT, "row gather in order")])
+def test_failed_run_leaves_the_mask_as_unsettled_as_it_was(layer, flags, first):
+    """A kernel may still be writing a device mask: the next launch waits for it, also when a call failed in between."""
+    m = layer(24, 32, 3, 1, 1)
+    odd = layer(20, 32, 3, 1, 1)                                        # needs a padded copy, whose allocation fails
+    for n in (m, odd):
+        assert n.set_mask(DEVICE) == 0
+    assert m.run(1, 8, 8, flags=flags)[1][-1] == first
+    odd.set("mallocs_left", 0)
+    assert odd.run(1, 8, 8, flags=flags) == (6, [])                     # ASX_ERR_OOM
+    odd.set("mallocs_left", -1)
+    assert odd.run(1, 8, 8, flags=flags)[1][-1] == first
+    if not flags:                                                       # a launch that waited by itself: the next one is in order
+        assert odd.run(1, 8, 8)[1][-1] == "row gather in order"
+    assert odd.run(1, 8, 8, flags=flags)[1][-1] == "row gather"
