@@ -34,6 +34,9 @@ namespace {
 constexpr int THREADS = 256, WARPS = THREADS / 32;
 constexpr int CHUNK = 32;               // output rows a warp scans at a time
 constexpr int QUEUE = 48;               // row queue of a warp: up to 15 left over and 32 new ones
+// The filter row (upper half) of a chunk or word past the window: no corner -255 .. 32767 puts it into an image of up to
+// 32767 rows.
+constexpr int PAST_WINDOW = (int)0x80000000u;
 
 // How the zeros of dropped rows are written: the 16-byte units of a row's column range, and whether they are a power of
 // two up to 32 (1 << shift), so that every lane keeps its column.
@@ -150,7 +153,7 @@ __device__ __forceinline__ void fill_positions(const Tables& s, const ConvGeom& 
 {
     constexpr int EPC = F32 ? 4 : 8;
     for (int c = threadIdx.x; c < a.KQ * (WORDS ? 16 : 4); c += THREADS) {
-        int2 e = make_int2(WORDS ? -a.shift : 0, 0x7fff0000);  // past the window: no row has it inside the image (its filter entries are zero)
+        int2 e = make_int2(WORDS ? -a.shift : 0, PAST_WINDOW);  // no row has it inside the image (its filter entries are zero)
         if (WORDS) {
             const int ky = (int)fd_div((uint32_t)c, a.fdWords), i = c - ky * a.words;
             const int el = F32 ? i : 2 * i - a.shift;
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__(KTHREADS) masked_conv_direct_k_kernel(const Co
     unsigned short* const list = reinterpret_cast<unsigned short*>(pos + 4 * a.KQ);          // kept positions
     // Everything up to the dependency wait needs the mask and the geometry only.
     for (int c = tid; c < 4 * a.KQ; c += KTHREADS) {
-        int2 e = make_int2(0, 0x7fff0000);
+        int2 e = make_int2(0, PAST_WINDOW);
         if (c * EPC < g.K) {
             const int tap = (int)fd_div((uint32_t)(c * EPC), a.fdCin), ci = c * EPC - tap * g.C_in;
             const int ky = (int)fd_div((uint32_t)tap, a.fdkw), kx = tap - ky * g.kw;

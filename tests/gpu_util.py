@@ -21,8 +21,8 @@ def to_dev_bf16(a):
     return torch.from_numpy(np.ascontiguousarray(a)).to(torch.bfloat16).cuda().contiguous()
 
 
-def run_library(spec, x, w, b, mask, flags, prefill=None):
-    """Returns (y as float64 numpy [M][N], raw uint16 bits [M][N], kept list)."""
+def run_library(spec, x, w, b, mask, flags, prefill=None, form=None):
+    """`form`: the form of the kernel that the run has to take.  Returns (y as float64 numpy [M][N], raw uint16 bits [M][N], kept list)."""
     layer = asx.MaskedConvLayer(spec.C_in, spec.C_out, spec.kh, spec.kw, spec.stride, spec.pad)
     layer.set_mask(mask)
     xd, wd = to_dev_bf16(x), to_dev_bf16(w)
@@ -34,8 +34,10 @@ def run_library(spec, x, w, b, mask, flags, prefill=None):
     torch.cuda.synchronize()
     status = layer.device_status()
     kept = layer.kept()
+    ran = layer.last_run_form()
     layer.close()
     assert status == 0, f"device status {status}"
+    assert form is None or ran == form, f"form {ran} ran, not {form}"
     bits = out.view(torch.int16).cpu().numpy().view(np.uint16).reshape(spec.M, spec.C_out)
     y = out.float().cpu().numpy().astype(np.float64).reshape(spec.M, spec.C_out)
     return y, bits, kept
@@ -45,10 +47,10 @@ def full_row_mask(spec, mask):
     return mask if mask.size == spec.M else np.tile(mask, spec.Nb)
 
 
-def check_against_oracle(spec, x, w, b, mask, flags, rows_sel=None):
+def check_against_oracle(spec, x, w, b, mask, flags, rows_sel=None, form=None):
     """Full comparison (rows_sel None) or comparison on selected lowered rows."""
     relu = "silu" if flags & asx.ACT_SILU else bool(flags & asx.ACT_RELU)      # the oracle's activation argument
-    y, bits, kept = run_library(spec, x, w, b, mask, flags, prefill=0x7fc1)   # NaN canary
+    y, bits, kept = run_library(spec, x, w, b, mask, flags, prefill=0x7fc1, form=form)   # NaN canary
     # kept list: bit-exact
     assert np.array_equal(kept, oracle.kept_list(mask)), "kept-row list differs"
     fm = full_row_mask(spec, mask).astype(bool)

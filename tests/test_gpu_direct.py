@@ -41,8 +41,8 @@ def test_against_the_oracle(case, per_row):
     spec = _spec(case)
     x, w, b, mask = make_problem(spec, per_row=per_row)
     for flags in (asx.ACT_RELU, asx.ACT_SILU | asx.RECOMPACT):
-        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT)
-    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT)
+        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT, form=asx.FORM_DIRECT)
+    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT, form=asx.FORM_DIRECT)
 
 
 K_CASES = [
@@ -63,8 +63,8 @@ def test_shared_k_range(case, per_row):
     spec = _spec(case, 4)
     x, w, b, mask = make_problem(spec, per_row=per_row)
     for flags in (asx.ACT_RELU | asx.RECOMPACT, asx.ACT_SILU):
-        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT_K)
-    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT_K)
+        check_against_oracle(spec, x, w, b, mask, flags | asx.IMPL_DIRECT_K, form=asx.FORM_DIRECT_K)
+    check_against_oracle(spec, x, w, None, mask, asx.IMPL_DIRECT_K, form=asx.FORM_DIRECT_K)
 
 
 @pytest.mark.parametrize("impl", [asx.IMPL_DIRECT, asx.IMPL_DIRECT_K], ids=["direct", "direct_k"])
@@ -159,3 +159,14 @@ def test_input_between_two_words(case, offset, impl):
     got = y.float().cpu().numpy().astype(np.float64).reshape(ref.shape)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 5e-3
     assert not got.reshape(spec.M, -1)[np.tile(mask, spec.Nb) == 0].any()
+
+
+@pytest.mark.parametrize("C_in,W,impl", [(8, 1, asx.IMPL_DIRECT_K), (8, 1, asx.IMPL_DIRECT), (3, 2, asx.IMPL_DIRECT)], ids=["direct_k", "chunks", "words"])
+def test_images_of_the_largest_height(C_in, W, impl):
+    """What a group of chunks or words holds past the window stays outside an image of 32767 rows, whose windows' corners
+    are rows -1 .. 32765."""
+    spec = _spec((C_in, 16, 3, 2, 1, 32767, W, 1, 30, 1), 6)
+    assert spec.P == 16384
+    x, w, b, mask = make_problem(spec)
+    mask[:3] = mask[-3:] = 1
+    check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | impl, form=asx.FORM_DIRECT if impl == asx.IMPL_DIRECT else asx.FORM_DIRECT_K)
