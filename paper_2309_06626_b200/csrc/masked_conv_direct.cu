@@ -70,6 +70,7 @@ struct DirectArgs {
     int32_t* count_out;
     int relu;
     int KQ;                             // groups of four 16-byte chunks (word form: of sixteen words) of a window
+    int whole;                          // no chunk of the last group lies past the window
     int words;                          // word form: 4-byte words per filter row, else 0
     int shift;                          // word form: K-elements in front of a filter row's first (0 or 1)
     int block_rows;                     // output rows per block
@@ -144,6 +145,7 @@ struct Tables {
     uint4* b;          // [KQ][2][MTL][32]
     float* bias;       // [16 MTL]
     int2* pos;         // [KQ * 4] or [KQ * 16]: element offset from the window's corner, ky << 16 | kx (word form: the word's element)
+    uint32_t* own;     // word form, [KQ * 16]: the bits of a word that are the window's
     int4* queue;       // [WARPS][QUEUE]
 };
 
@@ -153,11 +155,12 @@ __device__ __forceinline__ void fill_positions(const Tables& s, const ConvGeom& 
 {
     constexpr int EPC = F32 ? 4 : 8;
     for (int c = threadIdx.x; c < a.KQ * (WORDS ? 16 : 4); c += THREADS) {
-        int2 e = make_int2(WORDS ? -a.shift : 0, PAST_WINDOW);  // no row has it inside the image (its filter entries are zero)
+        int2 e = make_int2(WORDS ? -a.shift : 0, PAST_WINDOW);  // no row has it inside the image
         if (WORDS) {
-            const int ky = (int)fd_div((uint32_t)c, a.fdWords), i = c - ky * a.words;
+            const int ky = (int)fd_div((uint32_t)c, a.fdWords), i = c - ky * a.words, run = g.kw * g.C_in;
             const int el = F32 ? i : 2 * i - a.shift;
             if (ky < g.kh) e = make_int2(ky * g.W * g.C_in + el, (ky << 16) | (el & 0xffff));
+            s.own[c] = ky >= g.kh ? 0u : F32 ? 0xffffffffu : (el >= 0 ? 0xffffu : 0u) | (el + 1 < run ? 0xffff0000u : 0u);
         } else if (c * EPC < g.K) {
             const int tap = (int)fd_div((uint32_t)(c * EPC), a.fdCin), ci = c * EPC - tap * g.C_in;
             const int ky = (int)fd_div((uint32_t)tap, a.fdkw), kx = tap - ky * g.kw;
@@ -222,7 +225,8 @@ __device__ __forceinline__ void load_filters(const Tables& s, const ConvGeom& g,
 }
 
 // A queued row: x its output row, y the element index of its window's corner, z the corner's coordinates (iy0 << 16 | ix0,
-// word form: ix0 * C_in), w 1 when every word or chunk the window's filter rows touch lies inside the image.
+// word form: ix0 * C_in), w 1 when every word or chunk that is loaded for the window lies inside the image (and every chunk in
+// the window: the check leaves the others out as well).
 using Row = int4;
 
 // One group of operand loads: chunk 4 q + t (or four words) of the two rows of this lane.  CHECK: some window of the tile
@@ -253,10 +257,23 @@ __device__ __forceinline__ void load_group(uint4 (&v)[2], int q, int t, const in
     }
 }
 
-// acc += the group whose two rows' values lie in v, against the filters at aq.
-template <bool F32, int MTL>
-__device__ __forceinline__ void multiply_group(float (&acc)[2][MTL][4], const uint4 (&v)[2], const uint4* aq)
+// acc += group q of KQ, whose two rows' values lie in v, against the filters at aq.
+// Word form: the half words beside a filter row and the words past the window (fp32: the latter, in the last group) hold values
+// of other windows.  They meet zeros of the filter, but infinity or NaN times zero is NaN, so `own` takes them out: 2 of 57 us
+// on a 7x7x3 stem of 64 images.  Dearer: these words in the first groups, the only ones with masks then (8 us: four lanes' words
+// no longer lie in one sector); the masks in registers beside the addresses (3 us: spills); a second pass over tiles
+// with a NaN among the sums (3 us there, 20 on a 3x3x3 stem at 640 x 640: spills).
+template <bool F32, bool WORDS, int MTL>
+__device__ __forceinline__ void multiply_group(float (&acc)[2][MTL][4], uint4 (&v)[2], const uint4* aq, int q, int KQ, const uint32_t* own, int t)
 {
+    if (WORDS && (!F32 || q == KQ - 1)) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t m = own[16 * q + 4 * k + t];
+            (&v[0].x)[k] &= m;
+            (&v[1].x)[k] &= m;
+        }
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -278,22 +295,22 @@ __device__ __forceinline__ void multiply(float (&acc)[2][MTL][4], const int2 (&r
     uint4 v[2], next[2];
     load_group<F32, WORDS, CHECK>(v, 0, t, row, s, g, xb);
     if (KQT == 1) {
-        multiply_group<F32, MTL>(acc, v, aq);
+        multiply_group<F32, WORDS, MTL>(acc, v, aq, 0, 1, s.own, t);
     } else if (KQT == 2) {
         load_group<F32, WORDS, CHECK>(next, 1, t, row, s, g, xb);
-        multiply_group<F32, MTL>(acc, v, aq);
-        multiply_group<F32, MTL>(acc, next, aq + STEP);
+        multiply_group<F32, WORDS, MTL>(acc, v, aq, 0, 2, s.own, t);
+        multiply_group<F32, WORDS, MTL>(acc, next, aq + STEP, 1, 2, s.own, t);
     } else {
         // two groups a turn, each loaded while the other is used (with an exit in the middle of the turn the compiler
         // copied every accumulator once per product)
 #pragma unroll 1
         for (int q = 1; q < KQ; q += 2, aq += 2 * STEP) {
             load_group<F32, WORDS, CHECK>(next, q, t, row, s, g, xb);
-            multiply_group<F32, MTL>(acc, v, aq);
+            multiply_group<F32, WORDS, MTL>(acc, v, aq, q - 1, KQ, s.own, t);
             if (q + 1 < KQ) load_group<F32, WORDS, CHECK>(v, q + 1, t, row, s, g, xb);
-            multiply_group<F32, MTL>(acc, next, aq + STEP);
+            multiply_group<F32, WORDS, MTL>(acc, next, aq + STEP, q, KQ, s.own, t);
         }
-        if (KQ & 1) multiply_group<F32, MTL>(acc, v, aq);
+        if (KQ & 1) multiply_group<F32, WORDS, MTL>(acc, v, aq, KQ - 1, KQ, s.own, t);
     }
 }
 
@@ -410,6 +427,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
     s.bias = reinterpret_cast<float*>(s.b + (size_t)a.KQ * 2 * MTL * 32);
     s.queue = reinterpret_cast<Row*>(s.bias + 16 * MTL);
     s.pos = reinterpret_cast<int2*>(s.queue + WARPS * QUEUE);
+    s.own = reinterpret_cast<uint32_t*>(s.pos + a.KQ * 16);
     fill_positions<F32, WORDS>(s, g, a);
 
     const int first = block * a.block_rows, end = g.M - first < a.block_rows ? g.M : first + a.block_rows;
@@ -444,7 +462,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
                 const int oy = (int)fd_div((uint32_t)p, a.fdWo), ox = p - oy * g.Wo;
                 const int iy0 = oy * g.stride - g.pad, ix0 = ox * g.stride - g.pad;
                 const int slack = WORDS ? 1 : 0;            // a filter row's first and last word may reach into the pixels beside it
-                const bool inner = iy0 >= 0 && iy0 + g.kh <= g.H && ix0 >= slack && ix0 + g.kw + slack <= g.W;
+                const bool inner = (WORDS || a.whole) && iy0 >= 0 && iy0 + g.kh <= g.H && ix0 >= slack && ix0 + g.kw + slack <= g.W;
                 queue[queued + __popc(kept & ((1u << lane) - 1u))] =
                     make_int4(rw, ((img * g.H + iy0) * g.W + ix0) * g.C_in, (iy0 << 16) | ((WORDS ? ix0 * g.C_in : ix0) & 0xffff), inner ? 1 : 0);
             }
@@ -680,7 +698,7 @@ bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan)
     }
     plan->NG = g.C_out <= 32 ? 1 : 2;
     plan->n_tiles = (g.C_out + 32 * plan->NG - 1) / (32 * plan->NG);
-    plan->smem_bytes = plan->KQ * plan->NG * 2048 + 128 * plan->NG + plan->KQ * (plan->words ? 16 : 4) * 8 + WARPS * QUEUE * 16;
+    plan->smem_bytes = plan->KQ * plan->NG * 2048 + 128 * plan->NG + plan->KQ * (plan->words ? 16 * 12 : 4 * 8) + WARPS * QUEUE * 16;
     return plan->smem_bytes <= 112 * 1024 && plan->n_tiles < 65536;
 }
 
@@ -725,6 +743,7 @@ cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void*
     a.count_out = count_out;
     a.relu = relu == 1 ? 1 : 0;
     a.KQ = plan.KQ;
+    a.whole = plan.words == 0 && 4 * plan.KQ * (16 / es) == g.K ? 1 : 0;
     a.words = plan.words;
     a.shift = plan.shift;
 

@@ -170,3 +170,48 @@ def test_images_of_the_largest_height(C_in, W, impl):
     x, w, b, mask = make_problem(spec)
     mask[:3] = mask[-3:] = 1
     check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | impl, form=asx.FORM_DIRECT if impl == asx.IMPL_DIRECT else asx.FORM_DIRECT_K)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+@pytest.mark.parametrize("case,f32,impl", [
+    ((3, 16, 3, 2, 1, 18, 20, 2, 20, 1), False, asx.IMPL_DIRECT), ((3, 64, 7, 2, 3, 32, 30, 2, 20, 1), False, asx.IMPL_DIRECT),
+    ((4, 24, 5, 2, 2, 14, 16, 2, 20, 1), False, asx.IMPL_DIRECT), ((5, 48, 3, 2, 1, 14, 16, 2, 20, 1), False, asx.IMPL_DIRECT),
+    ((3, 16, 3, 1, 1, 18, 21, 2, 20, 1), True, asx.IMPL_DIRECT), ((8, 16, 3, 1, 1, 12, 13, 2, 20, 1), False, asx.IMPL_DIRECT),
+    ((24, 56, 3, 1, 1, 13, 12, 2, 20, 1), False, asx.IMPL_DIRECT), ((4, 36, 3, 1, 1, 13, 12, 2, 20, 1), True, asx.IMPL_DIRECT),
+    ((8, 16, 1, 1, 0, 12, 13, 2, 20, 1), False, asx.IMPL_DIRECT), ((24, 56, 3, 1, 1, 13, 12, 2, 20, 1), False, asx.IMPL_DIRECT_K)],
+    ids=lambda v: "-".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_what_is_not_finite_stays_in_its_windows(case, f32, impl, value):
+    """Inf or NaN at single pixels: outputs whose window holds one become what the definition says, the others do not see it
+    (filters and the other pixels are positive, so that Inf stays Inf)."""
+    spec = _spec(case, 7)
+    x, w, b, mask = make_problem(spec)
+    x, w, b = np.abs(x) + 0.125, np.abs(w) + 0.125, np.abs(b)
+    rng = np.random.default_rng(spec.C_in)
+    for _ in range(3):                                      # whole pixels: every edge of every window is met
+        x[rng.integers(spec.Nb), rng.integers(spec.H), rng.integers(spec.W)] = value
+    x[0, spec.H // 2, spec.W // 2] = x[-1, 0, -1] = value
+    layer = asx.MaskedConvLayer(spec.C_in, spec.C_out, spec.kh, spec.kw, spec.stride, spec.pad)
+    layer.set_mask(mask)
+    if f32:
+        x, w = oracle.tf32_operand(x), oracle.tf32_operand(w)
+        y = layer.run(torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), torch.from_numpy(b).cuda(), flags=asx.F32 | impl)
+    else:
+        y = layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=impl)
+    torch.cuda.synchronize()
+    assert layer.last_run_form() == (asx.FORM_DIRECT if impl == asx.IMPL_DIRECT else asx.FORM_DIRECT_K)
+    layer.close()
+    got = y.double().cpu().reshape(spec.M, -1)
+    # the definition in which a padding pixel is left out and not multiplied: torch's unfolded windows of a padded image
+    xp = torch.nn.functional.pad(torch.from_numpy(x).double().permute(0, 3, 1, 2), (spec.pad,) * 4)
+    cols = torch.nn.functional.unfold(xp, (spec.kh, spec.kw), stride=spec.stride)                    # [Nb][C kh kw][P]
+    rows = cols.permute(0, 2, 1).reshape(spec.M, spec.C_in * spec.kh * spec.kw)
+    wr = torch.from_numpy(w).double().permute(0, 3, 1, 2).reshape(spec.C_out, -1)
+    bad = ~torch.isfinite(rows).all(1)
+    ref = torch.where(bad[:, None], torch.full((1, 1), value, dtype=torch.float64), rows.nan_to_num(0, 0, 0) @ wr.t() + torch.from_numpy(b).double())
+    ref = ref * torch.from_numpy(np.tile(mask, spec.Nb).astype(np.float64))[:, None].nan_to_num()
+    keep = torch.from_numpy(np.tile(mask, spec.Nb) != 0)
+    assert bad[keep].any() and (~bad)[keep].any()
+    assert torch.equal(torch.isnan(got[keep]), torch.isnan(ref[keep])) and torch.equal(torch.isinf(got[keep]), torch.isinf(ref[keep]))
+    fine = torch.isfinite(ref) & keep[:, None]
+    assert ((got - ref)[fine]).norm() < 5e-3 * ref[fine].norm()
+    assert not got[~keep].any()
