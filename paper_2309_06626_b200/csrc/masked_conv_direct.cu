@@ -691,7 +691,8 @@ bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan)
     } else {
         // 4-byte words of a filter row: in bf16 the windows' rows must all start at the same parity of elements
         if (elem_bytes == 2 && ((g.stride * g.C_in) % 2 != 0 || (g.W * g.C_in) % 2 != 0)) return false;
-        if (g.W * g.C_in > 32000 || g.kw * g.C_in > 1000) return false;
+        // a queued row keeps ix0 * C_in, from -pad * C_in up, in 16 bits
+        if ((long long)(g.W + g.pad) * g.C_in > 32000 || g.kw * g.C_in > 1000) return false;
         plan->shift = elem_bytes == 2 ? (g.pad * g.C_in) & 1 : 0;
         plan->words = elem_bytes == 2 ? (g.kw * g.C_in + plan->shift + 1) / 2 : g.kw * g.C_in;
         plan->KQ = (g.kh * plan->words + 15) / 16;

@@ -215,3 +215,11 @@ def test_what_is_not_finite_stays_in_its_windows(case, f32, impl, value):
     fine = torch.isfinite(ref) & keep[:, None]
     assert ((got - ref)[fine]).norm() < 5e-3 * ref[fine].norm()
     assert not got[~keep].any()
+
+
+@pytest.mark.parametrize("pad", [0, 66])
+def test_wide_words_and_padding(pad):
+    """Columns times channels that no longer fit 16 bits take another form."""
+    spec = wl.LayerSpec("wide", 998, 8, 1, 1, 1, pad, 1, 32, 1, 50, 1, "relu", wl.BASE_SEED + 8899)
+    x, w, b, mask = make_problem(spec)
+    check_against_oracle(spec, x, w, b, mask, asx.ACT_RELU | asx.IMPL_DIRECT, form=asx.FORM_ROW_GATHER_COPY if pad else asx.FORM_DIRECT)

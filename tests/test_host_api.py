@@ -108,3 +108,28 @@ def test_failed_run_leaves_the_mask_as_unsettled_as_it_was(layer, flags, first):
     if not flags:                                                       # a launch that waited by itself: the next one is in order
         assert odd.run(1, 8, 8)[1][-1] == "row gather in order"
     assert odd.run(1, 8, 8, flags=flags)[1][-1] == "row gather"
+
+
+def test_word_form_takes_geometries_whose_columns_fit_its_16_bits():
+    """A queued row keeps ix0 * C_in in 16 bits; one that wrapped could look as if it were inside the image."""
+    from paper_2309_06626_b200 import build, lib
+    build.build()
+    plan_direct = lib()["_ZN3asx11plan_directERKNS_8ConvGeomEiPNS_10DirectPlanE"]
+    plan_direct.restype = ctypes.c_bool
+    rng = np.random.default_rng(5)
+    words = 0
+    for i in range(4000):
+        W, C_in, k, stride = int(2 ** rng.uniform(0, 14.9)), int(2 ** rng.uniform(0, 10)), int(rng.integers(1, 8)), int(rng.integers(1, 4))
+        pad = int(rng.integers(0, 256)) if i % 2 else k // 2
+        if W + 2 * pad < k:
+            continue
+        Wo = (W + 2 * pad - k) // stride + 1
+        g = (ctypes.c_int * 17)(1, W, W, C_in, 16, k, k, stride, pad, Wo, Wo, stride, pad, k * k * C_in, Wo * Wo, Wo * Wo, Wo * Wo)
+        plan = (ctypes.c_int * 6)()
+        for elem in (2, 4):
+            if not plan_direct(g, elem, plan) or plan[1] == 0:
+                continue
+            words += 1
+            first, last = -pad * C_in, ((Wo - 1) * stride - pad) * C_in
+            assert -32768 <= first and last + k * C_in <= 32767, (W, C_in, k, stride, pad)
+    assert words > 200
