@@ -280,6 +280,7 @@ asx_status asx_set_mask(asx_layer* L, const uint8_t* mask, int64_t rows, void* c
         }
         if (capture != cudaStreamCaptureStatusNone) return ASX_ERR_CUDA;
     }
+    L->has_mask = false;                                           // until all of the new one is there
     s = ensure_mask_buffers(L, rows);
     if (s != ASX_OK) return s;
     cudaError_t e;

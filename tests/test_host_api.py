@@ -133,3 +133,16 @@ def test_word_form_takes_geometries_whose_columns_fit_its_16_bits():
             first, last = -pad * C_in, ((Wo - 1) * stride - pad) * C_in
             assert -32768 <= first and last + k * C_in <= 32767, (W, C_in, k, stride, pad)
     assert words > 200
+
+
+def test_failed_set_mask_leaves_no_mask(layer):
+    """A mask that outgrew the buffers took them along when their successors could not be allocated."""
+    m = layer(24, 32, 3, 1, 1)
+    assert m.set_mask(np.ones(64, np.uint8)) == 0
+    for mallocs in range(3):
+        m.set("mallocs_left", mallocs)
+        assert m.set_mask(np.ones(4096, np.uint8)) == 6                 # ASX_ERR_OOM
+        m.set("mallocs_left", -1)
+        assert m.run(1, 8, 8) == (3, [])                                # ASX_ERR_NO_MASK
+        assert m.set_mask(np.ones(64, np.uint8)) == 0
+        assert m.run(1, 8, 8) == (0, ["row gather"])
