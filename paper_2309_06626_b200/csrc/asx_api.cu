@@ -734,6 +734,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
                 return ASX_ERR_OOM;
             }
             const bool shared = L->rows == P;
+            L->tiles_epoch = ~0ull;                                       // until the new table is on the device
             L->tiles_rows = cut_row_tiles(kept, shared, Nb, gp.P, gp.Wo, pplan.Hp, gp.kh, pplan.cap_rows, 128, &L->host_tiles);
             // Level the waves: with T tiles of 128 rows on S blocks the last of ceil(T / S) waves is partly
             // empty; tiles of fewer rows that fill every wave cost less (a tile's patch reads and epilogue
@@ -753,7 +754,6 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
                         L->host_tiles.swap(level);
                 }
             }
-            L->tiles_epoch = L->mask_epoch; L->tiles_Nb = Nb; L->tiles_H = H; L->tiles_W = W; L->tiles_cap = pplan.cap_rows;
             const size_t need = L->host_tiles.size() * sizeof(int32_t);
             if (L->tiles_rows > 0 && need > 0) {
                 if (need > L->d_tiles_bytes) {
@@ -767,6 +767,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
                 if (cudaMemcpyAsync(L->d_tiles, L->host_tiles.data(), need, cudaMemcpyHostToDevice, st) != cudaSuccess) return ASX_ERR_CUDA;
                 if (cudaStreamSynchronize(st) != cudaSuccess) return ASX_ERR_CUDA;
             }
+            L->tiles_epoch = L->mask_epoch; L->tiles_Nb = Nb; L->tiles_H = H; L->tiles_W = W; L->tiles_cap = pplan.cap_rows;
         }
         if (L->tiles_rows > 0 && L->tiles_rows == est_rows) {
             plan_patch_cost(gp, L->num_sms, (long long)(L->host_tiles.size() / 4), in_compact, &pplan);

@@ -146,3 +146,23 @@ def test_failed_set_mask_leaves_no_mask(layer):
         assert m.run(1, 8, 8) == (3, [])                                # ASX_ERR_NO_MASK
         assert m.set_mask(np.ones(64, np.uint8)) == 0
         assert m.run(1, 8, 8) == (0, ["row gather"])
+
+
+def test_row_tiles_count_once_they_are_on_the_device(layer):
+    """A first run that fails on the way there (no memory, or a capture, whose copies do not happen) leaves nothing behind
+    that a later run takes for its tiles."""
+    m = layer(64, 32, 3, 1, 1)
+    m.set("patch", 1)
+    mask = np.ones(256, np.uint8)
+    mask[:7] = 0
+    assert m.set_mask(mask) == 0
+    m.set("mallocs_left", 0)
+    assert m.run(1, 16, 16) == (6, [])
+    m.set("mallocs_left", -1)
+    tiles = (0, ["window patch, 2 tiles, the first: row 0, 128 rows"])
+    assert m.run(1, 16, 16) == tiles
+    assert m.set_mask(1 - mask) == 0                                    # a shorter table: the buffer stays
+    m.set("capturing", 1)
+    assert m.run(1, 16, 16)[0] == 7
+    m.set("capturing", 0)
+    assert m.run(1, 16, 16) == (0, ["window patch, 1 tiles, the first: row 0, 7 rows"])
