@@ -398,6 +398,7 @@ asx_status asx_set_input_mask(asx_layer* L, const uint8_t* mask, int64_t rows, v
         cudaGetLastError();
         std::memcpy(host.data(), mask, (size_t)rows);
     }
+    L->in_rows = 0;                                               // until the new table is on the device
     int32_t kept = 0;
     for (int64_t p = 0; p < rows; ++p) rank[(size_t)p] = host[(size_t)p] != 0 ? kept++ : -1;
     if (rows > L->in_rank_cap) {
@@ -463,7 +464,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     const bool in_compact = (flags & ASX_IN_COMPACT) != 0, out_compact = (flags & ASX_OUT_COMPACT) != 0;
     if (out_compact && L->rows != P) return ASX_ERR_SHAPE;            // kept order n*P' + j needs one mask for the batch
     if (in_compact) {
-        if (L->d_in_rank == nullptr) return ASX_ERR_NO_MASK;
+        if (L->in_rows == 0) return ASX_ERR_NO_MASK;
         if (L->in_rows != (int64_t)H * W) return ASX_ERR_SHAPE;
         if (L->C_in % 8 != 0 || L->in_kept < 1) return ASX_ERR_UNSUPPORTED;
     }

@@ -63,7 +63,7 @@ def layer(fake):
         fake.asx_destroy(m.h)
 
 
-IMPL_DIRECT, F32, RECOMPACT = 512, 64, 2
+IMPL_DIRECT, F32, RECOMPACT, IN_COMPACT = 512, 64, 2, 16
 
 
 @pytest.mark.parametrize("flags", [0, IMPL_DIRECT])
@@ -166,3 +166,24 @@ def test_row_tiles_count_once_they_are_on_the_device(layer):
     assert m.run(1, 16, 16)[0] == 7
     m.set("capturing", 0)
     assert m.run(1, 16, 16) == (0, ["window patch, 1 tiles, the first: row 0, 7 rows"])
+
+
+def test_failed_set_input_mask_leaves_none(layer):
+    """The rank table of the input mask before went with its buffer."""
+    m = layer(24, 32, 3, 1, 1)
+    assert m.set_mask(np.ones(64, np.uint8)) == 0
+    assert m.run(1, 8, 8, flags=IN_COMPACT) == (3, [])                  # ASX_ERR_NO_MASK
+
+    def set_input_mask(rows):
+        mask = np.ones(rows, np.uint8)
+        return m.L.asx_set_input_mask(m.h, mask.ctypes.data, rows, None)
+    assert set_input_mask(64) == 0
+    assert m.run(1, 8, 8, flags=IN_COMPACT) == (0, ["row gather"])
+    for what, value, status in (("mallocs_left", 0, 6), ("capturing", 1, 7)):
+        before = -1 if what == "mallocs_left" else 0
+        m.set(what, value)
+        assert set_input_mask(4096) == status
+        m.set(what, before)
+        assert m.run(1, 8, 8, flags=IN_COMPACT) == (3, [])
+        assert set_input_mask(64) == 0
+        assert m.run(1, 8, 8, flags=IN_COMPACT) == (0, ["row gather"])
