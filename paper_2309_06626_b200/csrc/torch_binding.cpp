@@ -7,7 +7,8 @@
 //
 // Every function returns an int where it cannot do the call: the library's status code when the
 // C ABI returned one, or -1 when the arguments do not fit, upon which the Python wrapper goes through its own
-// checks and raises with a message.
+// checks and raises with a message.  So it does when torch throws here, as it does for tensors without a storage (under a
+// transform such as vmap, say): nothing C++ may leave a function that Python called.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <ATen/cuda/EmptyTensor.h>
@@ -43,7 +44,7 @@ at::Tensor empty_on(const at::Tensor& like, at::IntArrayRef sizes, at::ScalarTyp
 }
 
 // run(geometry, x, w, bias, out, flags, stream) with geometry = (handle, C_in, C_out, kh, kw, stride, pad)
-PyObject* run(PyObject*, PyObject* const* args, Py_ssize_t nargs)
+PyObject* run(PyObject* const* args, Py_ssize_t nargs)
 {
     if (nargs != 7 || !PyTuple_Check(args[0]) || PyTuple_GET_SIZE(args[0]) != 7) return refuse();
     PyObject* g = args[0];
@@ -73,6 +74,7 @@ PyObject* run(PyObject*, PyObject* const* args, Py_ssize_t nargs)
         if (b == nullptr || b->scalar_type() != at::kFloat || !b->is_cuda() || b->numel() != C_out) return refuse();
         bias = static_cast<const float*>(b->data_ptr());
     }
+    const void *xp = x->data_ptr(), *wp = w->data_ptr();
     void* st = nullptr;
     if (!stream_of(args[6], &st)) {
         PyErr_Clear();
@@ -95,7 +97,6 @@ PyObject* run(PyObject*, PyObject* const* args, Py_ssize_t nargs)
         y = t->data_ptr();
         Py_INCREF(out);
     }
-    const void *xp = x->data_ptr(), *wp = w->data_ptr();
     asx_status s;
     Py_BEGIN_ALLOW_THREADS
     s = asx_run(layer, xp, (int)Nb, (int)H, (int)W, wp, bias, y, (int)flags, st);
@@ -106,7 +107,7 @@ PyObject* run(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 }
 
 // set_mask(handle, mask, stream): a contiguous uint8 tensor on either side
-PyObject* set_mask(PyObject*, PyObject* const* args, Py_ssize_t nargs)
+PyObject* set_mask(PyObject* const* args, Py_ssize_t nargs)
 {
     if (nargs != 3) return refuse();
     asx_layer* layer = static_cast<asx_layer*>(PyLong_AsVoidPtr(args[0]));
@@ -126,7 +127,7 @@ PyObject* set_mask(PyObject*, PyObject* const* args, Py_ssize_t nargs)
 }
 
 // mask_from_activation(x, stream) -> uint8 mask, one entry per row
-PyObject* mask_from_activation(PyObject*, PyObject* const* args, Py_ssize_t nargs)
+PyObject* mask_from_activation(PyObject* const* args, Py_ssize_t nargs)
 {
     if (nargs != 2) return refuse();
     const at::Tensor* x = tensor_or_null(args[0]);
@@ -148,7 +149,7 @@ PyObject* mask_from_activation(PyObject*, PyObject* const* args, Py_ssize_t narg
 }
 
 // compact_mask(mask, stream) -> (kept, count, scratch)
-PyObject* compact_mask(PyObject*, PyObject* const* args, Py_ssize_t nargs)
+PyObject* compact_mask(PyObject* const* args, Py_ssize_t nargs)
 {
     if (nargs != 2) return refuse();
     const at::Tensor* m = tensor_or_null(args[0]);
@@ -177,11 +178,27 @@ PyObject* compact_mask(PyObject*, PyObject* const* args, Py_ssize_t nargs)
     return all;
 }
 
+template <PyObject* (*F)(PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject*, PyObject* const* args, Py_ssize_t nargs)
+{
+    try {
+        return F(args, nargs);
+    } catch (const std::exception&) {
+        PyErr_Clear();
+        return refuse();
+    }
+}
+template <PyObject* (*F)(PyObject* const*, Py_ssize_t)>
+PyCFunction entry()
+{
+    return reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<F>));
+}
+
 PyMethodDef methods[] = {
-    {"run", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(run)), METH_FASTCALL, nullptr},
-    {"set_mask", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(set_mask)), METH_FASTCALL, nullptr},
-    {"mask_from_activation", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(mask_from_activation)), METH_FASTCALL, nullptr},
-    {"compact_mask", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(compact_mask)), METH_FASTCALL, nullptr},
+    {"run", entry<run>(), METH_FASTCALL, nullptr},
+    {"set_mask", entry<set_mask>(), METH_FASTCALL, nullptr},
+    {"mask_from_activation", entry<mask_from_activation>(), METH_FASTCALL, nullptr},
+    {"compact_mask", entry<compact_mask>(), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_asx_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -1,0 +1,42 @@
+"""The native side of the binding (csrc/torch_binding.cpp)."""
+import subprocess
+import sys
+
+import pytest
+
+CALLS = {
+    "set_mask": "layer.set_mask(t.to(torch.uint8), stream=stream)",
+    "run": "layer.run(t.bfloat16().reshape(1, 2, 2, 8), torch.zeros(8, 1, 1, 8, dtype=torch.bfloat16, device=dev), stream=stream)",
+    "mask_from_activation": "asx.mask_from_activation(t.bfloat16().reshape(4, 8), stream=stream)",
+    "compact_mask": "asx.compact_mask(t.to(torch.uint8), stream=stream)",
+}
+PROGRAM = """
+import torch
+import paper_2309_06626_b200 as asx
+class stream: cuda_stream = 0
+dev = %r
+layer = asx.MaskedConvLayer(8, 8, 1, 1, 1, 0)
+def call(t):
+    try:
+        %s
+    except (RuntimeError, ValueError) as e:
+        print("refused", type(e).__name__)
+    return t
+torch.vmap(call)(torch.ones(2, 32, device=dev))
+"""
+
+
+def _refuses(call, dev):
+    p = subprocess.run([sys.executable, "-c", PROGRAM % (dev, CALLS[call])], capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0 and "refused" in p.stdout, p.stderr[-800:]
+
+
+def test_a_tensor_without_storage_raises_on_the_host():
+    """torch throws for it; the exception must not leave the extension as a C++ one, which ends the process."""
+    _refuses("set_mask", "cpu")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", CALLS)
+def test_a_tensor_without_storage_raises(call):
+    _refuses(call, "cuda")
