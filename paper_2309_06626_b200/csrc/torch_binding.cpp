@@ -144,7 +144,12 @@ PyObject* mask_from_activation(PyObject* const* args, Py_ssize_t nargs)
     } catch (const std::exception&) {
         return refuse();
     }
-    const asx_status s = asx_mask_from_activation(x->data_ptr(), rows, (int)C, static_cast<uint8_t*>(mask.data_ptr()), st);
+    const void* xp = x->data_ptr();
+    uint8_t* mp = static_cast<uint8_t*>(mask.data_ptr());
+    asx_status s;
+    Py_BEGIN_ALLOW_THREADS
+    s = asx_mask_from_activation(xp, rows, (int)C, mp, st);
+    Py_END_ALLOW_THREADS
     return s == ASX_OK ? THPVariable_Wrap(std::move(mask)) : PyLong_FromLong(s);
 }
 
@@ -167,8 +172,13 @@ PyObject* compact_mask(PyObject* const* args, Py_ssize_t nargs)
     } catch (const std::exception&) {
         return refuse();
     }
-    const asx_status s = asx_compact(static_cast<const uint8_t*>(m->data_ptr()), rows, static_cast<int32_t*>(kept.data_ptr()),
-                                     static_cast<int32_t*>(count.data_ptr()), scratch.data_ptr(), scratch.numel() * 8, st);
+    const uint8_t* mp = static_cast<const uint8_t*>(m->data_ptr());
+    int32_t *kp = static_cast<int32_t*>(kept.data_ptr()), *cp = static_cast<int32_t*>(count.data_ptr());
+    void* sp = scratch.data_ptr();
+    asx_status s;
+    Py_BEGIN_ALLOW_THREADS
+    s = asx_compact(mp, rows, kp, cp, sp, bytes, st);
+    Py_END_ALLOW_THREADS
     if (s != ASX_OK) return PyLong_FromLong(s);
     PyObject* all = PyTuple_New(3);
     if (all == nullptr) return nullptr;

@@ -40,3 +40,44 @@ def test_a_tensor_without_storage_raises_on_the_host():
 @pytest.mark.parametrize("call", CALLS)
 def test_a_tensor_without_storage_raises(call):
     _refuses(call, "cuda")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", ["run", "set_mask", "mask_from_activation", "compact_mask"])
+def test_other_threads_run_during_a_call(call):
+    """The interpreter's lock is given up around the call into the library: with switches on request only, another thread
+    gets it nowhere else in this loop."""
+    import threading
+    import time
+    import torch
+    import paper_2309_06626_b200 as asx
+    layer = asx.MaskedConvLayer(8, 8, 1, 1, 1, 0)
+    mask = torch.ones(64, dtype=torch.uint8, device="cuda")
+    layer.set_mask(mask)
+    x, w = torch.ones(1, 8, 8, 8, dtype=torch.bfloat16, device="cuda"), torch.ones(8, 1, 1, 8, dtype=torch.bfloat16, device="cuda")
+    y = layer.run(x, w)
+    todo = {"run": lambda: layer.run(x, w, None, y), "set_mask": lambda: layer.set_mask(mask), "mask_from_activation": lambda: asx.mask_from_activation(x),
+            "compact_mask": lambda: asx.compact_mask(mask)}[call]
+    todo()
+    turns, stop = [0], threading.Event()
+
+    def other():
+        while not stop.is_set():
+            turns[0] += 1
+            time.sleep(0)
+    before = sys.getswitchinterval()
+    thread = threading.Thread(target=other)
+    sys.setswitchinterval(1000)
+    try:
+        thread.start()
+        first = turns[0]
+        for _ in range(2000):
+            todo()
+        got = turns[0] - first
+    finally:
+        sys.setswitchinterval(before)
+        stop.set()
+        thread.join()
+    torch.cuda.synchronize()
+    layer.close()
+    assert got > 10, got
