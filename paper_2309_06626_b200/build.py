@@ -1,8 +1,9 @@
 """Builds the C-ABI shared library (libasx.so) in-tree with nvcc for sm_100a, and the torch side of the
-binding (_asx_torch.so, a CPython extension linked against it) with the host compiler."""
+binding (_asx_torch.so, a CPython extension linked against it) with the host compiler.  The library alone needs no torch."""
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
 import tempfile
@@ -59,7 +60,8 @@ def _build_ext() -> None:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source of the library into libasx.so (the CUDA runtime is linked
     statically and the driver is reached through the runtime, so the library loads on a
-    machine without a GPU driver), one nvcc process per source, and then the torch extension."""
+    machine without a GPU driver), one nvcc process per source, and then the torch extension where there is a
+    torch to build it for (a program that uses the C ABI needs none)."""
     stale = force or is_stale()
     if stale:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -78,7 +80,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             tmp = LIB + f".tmp{os.getpid()}"
             subprocess.check_call([nvcc] + arch + ["-shared", "-cudart", "static", "-o", tmp] + [obj for obj, _ in jobs])
         os.replace(tmp, LIB)
-    if force or _ext_is_stale():
+    if importlib.util.find_spec("torch") is not None and (force or _ext_is_stale()):
         _build_ext()
     return LIB
 
