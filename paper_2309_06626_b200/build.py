@@ -3,9 +3,11 @@ binding (_asx_torch.so, a CPython extension linked against it) with the host com
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import importlib.util
 import os
 import subprocess
+import sysconfig
 import tempfile
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -13,6 +15,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libasx.so")
 EXT = os.path.join(PKG, "_asx_torch.so")
+EXT_FOR = os.path.join(PKG, "_asx_torch.built_for")      # the torch and the interpreter whose headers the extension was compiled with
 EXT_SRC = os.path.join(CSRC, "torch_binding.cpp")
 
 
@@ -32,15 +35,21 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _deps())
 
 
+def _ext_target() -> str:
+    return f"torch {importlib.metadata.version('torch')}, {sysconfig.get_config_var('SOABI')}\n"
+
+
 def _ext_is_stale() -> bool:
-    if not os.path.exists(EXT):
+    if not os.path.exists(EXT) or not os.path.exists(EXT_FOR):
         return True
+    with open(EXT_FOR) as f:
+        if f.read() != _ext_target():
+            return True
     t = os.path.getmtime(EXT)
     return any(os.path.getmtime(f) > t for f in [EXT_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h")))
 
 
 def _build_ext() -> None:
-    import sysconfig
     import torch
     from torch.utils import cpp_extension
     tmp = EXT + f".tmp{os.getpid()}"
@@ -55,6 +64,8 @@ def _build_ext() -> None:
         cmd += ["-L", d]
     subprocess.check_call(cmd + ["-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
     os.replace(tmp, EXT)
+    with open(EXT_FOR, "w") as f:
+        f.write(_ext_target())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

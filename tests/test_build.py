@@ -1,4 +1,5 @@
 """What build.py builds, and when."""
+import importlib.metadata
 import importlib.util
 import os
 
@@ -13,6 +14,7 @@ def asked(monkeypatch, tmp_path):
     done = []
     monkeypatch.setattr(build, "is_stale", lambda: False)
     monkeypatch.setattr(build, "EXT", str(tmp_path / "_asx_torch.so"))
+    monkeypatch.setattr(build, "EXT_FOR", str(tmp_path / "_asx_torch.built_for"))
     monkeypatch.setattr(build, "_build_ext", lambda: done.append("extension"))
     return done
 
@@ -22,3 +24,27 @@ def test_the_library_is_built_without_torch(asked, monkeypatch):
     assert build.build() == build.LIB and asked == ["extension"]
     monkeypatch.setattr(importlib.util, "find_spec", lambda name, *a: None if name == "torch" else found(name, *a))
     assert build.build() == build.LIB and asked == ["extension"]
+
+
+def test_the_extension_is_built_anew_for_another_torch(asked, monkeypatch):
+    def put():
+        open(build.EXT, "w").close()
+        with open(build.EXT_FOR, "w") as f:
+            f.write(build._ext_target())
+    put()
+    build.build()
+    assert asked == []
+    version = importlib.metadata.version
+    with monkeypatch.context() as m:
+        m.setattr(importlib.metadata, "version", lambda name: "99.0" if name == "torch" else version(name))
+        build.build()
+        assert asked == ["extension"]
+        put()
+        build.build()
+        assert asked == ["extension"]
+    build.build()
+    assert asked == ["extension"] * 2
+    put()
+    os.remove(build.EXT_FOR)                     # one that does not say what it was built for
+    build.build()
+    assert asked == ["extension"] * 3
