@@ -1,5 +1,6 @@
 // Internal declarations shared by the library's translation units (not installed).
 #pragma once
+#include <atomic>
 #include <cuda_runtime.h>
 #include <cuda.h>
 #include <stdint.h>
@@ -51,6 +52,22 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
 {
     return launch_pdl_cluster(kernel, grid, block, 1, smem, st, args...);
+}
+
+// Lets a kernel have `bytes` of dynamic shared memory on the current device.  The limit is kept per device and function, so it is set
+// on each device that the function is launched on (`set_on`: a bit for each); and to the most that any plan takes, not to
+// what this launch takes: of two threads with different plans the one with the smaller could lower it under the other's launch.
+constexpr int MAX_DYN_SMEM = 227 * 1024;
+inline cudaError_t allow_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& set_on)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+    if (set_on.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) set_on.fetch_or(bit, std::memory_order_relaxed);
+    return e;
 }
 
 // ---- S1: mask compaction (compact.cu)

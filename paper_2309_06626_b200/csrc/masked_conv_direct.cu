@@ -32,6 +32,7 @@ namespace asx {
 namespace {
 
 constexpr int THREADS = 256, WARPS = THREADS / 32;
+constexpr int DIRECT_MAX_SMEM = 112 * 1024;
 constexpr int CHUNK = 32;               // output rows a warp scans at a time
 constexpr int QUEUE = 48;               // row queue of a warp: up to 15 left over and 32 new ones
 // The filter row (upper half) of a chunk or word past the window: no corner -255 .. 32767 puts it into an image of up to
@@ -500,6 +501,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
 // eight warps, and both operands come straight from global memory: a filter value is used by one block once, so there
 // is nothing to stage.
 constexpr int KWARPS = 8, KZERO = 2, KTHREADS = 32 * (KWARPS + KZERO);
+constexpr int DIRECT_K_MAX_SMEM = 100 * 1024;
 
 struct DirectKArgs {
     FastDiv fdP, fdWo, fdCin, fdkw, fdcnt;
@@ -700,7 +702,7 @@ bool plan_direct(const ConvGeom& g, int elem_bytes, DirectPlan* plan)
     plan->NG = g.C_out <= 32 ? 1 : 2;
     plan->n_tiles = (g.C_out + 32 * plan->NG - 1) / (32 * plan->NG);
     plan->smem_bytes = plan->KQ * plan->NG * 2048 + 128 * plan->NG + plan->KQ * (plan->words ? 16 * 12 : 4 * 8) + WARPS * QUEUE * 16;
-    return plan->smem_bytes <= 112 * 1024 && plan->n_tiles < 65536;
+    return plan->smem_bytes <= DIRECT_MAX_SMEM && plan->n_tiles < 65536;
 }
 
 // Measured against the tensor-memory forms on 147 layers (networks' layers and random ones, bf16 and fp32).  The k loop
@@ -777,13 +779,10 @@ cudaError_t launch_direct(const ConvGeom& g, const DirectPlan& plan, const void*
     const long long per = (chunks + slots - 1) / slots;
     a.block_rows = (int)per * CHUNK;
     const int grid = (int)((chunks + per - 1) / per) + a.list_blocks;
-    static std::atomic<int> smem_set[96];                // largest dynamic shared memory size enabled so far, per instance
+    static std::atomic<unsigned long long> smem_set[96];     // per instance
     const int vi = ((plan.KQ <= 2 ? plan.KQ : 0) * 2 + (plan.NG - 1)) * 16 + (f32 ? 8 : 0) + (wd ? 4 : 0) + (res ? 2 : 0) + (is_silu ? 1 : 0);
-    if (plan.smem_bytes > smem_set[vi].load(std::memory_order_relaxed)) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
-        if (e != cudaSuccess) return e;
-        smem_set[vi].store(plan.smem_bytes, std::memory_order_relaxed);
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), DIRECT_MAX_SMEM, smem_set[vi]);
+    if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(grid, plan.n_tiles), dim3(THREADS), (size_t)plan.smem_bytes, st, g, a);
 }
 
@@ -809,7 +808,7 @@ bool plan_direct_k(const ConvGeom& g, int elem_bytes, int64_t kept_rows, int num
         plan->grid_y = gy;
     }
     plan->smem_bytes = KWARPS * 4 * plan->NT * plan->MTL * 128 + plan->KQ * 32 + (g.rows * 2 + 15) / 16 * 16;
-    return plan->smem_bytes <= 100 * 1024 && plan->grid_y < 65536;
+    return plan->smem_bytes <= DIRECT_K_MAX_SMEM && plan->grid_y < 65536;
 }
 
 cudaError_t launch_direct_k(const ConvGeom& g, const DirectKPlan& plan, const void* x, const void* w, const float* bias, void* y, const uint8_t* mask,
@@ -847,13 +846,10 @@ cudaError_t launch_direct_k(const ConvGeom& g, const DirectKPlan& plan, const vo
     else { ASX_PICK(4, 2); }
 #undef ASX_PICK
 #undef ASX_PICK2
-    static std::atomic<int> smem_set[24];                // largest dynamic shared memory size enabled so far, per instance
+    static std::atomic<unsigned long long> smem_set[24];     // per instance
     const int vi = (plan.NT == 2 ? 0 : plan.MTL) * 8 + (f32 ? 4 : 0) + (res ? 2 : 0) + (is_silu ? 1 : 0);
-    if (plan.smem_bytes > smem_set[vi].load(std::memory_order_relaxed)) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
-        if (e != cudaSuccess) return e;
-        smem_set[vi].store(plan.smem_bytes, std::memory_order_relaxed);
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), DIRECT_K_MAX_SMEM, smem_set[vi]);
+    if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(plan.grid_x, plan.grid_y), dim3(KTHREADS), (size_t)plan.smem_bytes, st, g, a);
 }
 

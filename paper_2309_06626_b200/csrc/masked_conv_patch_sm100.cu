@@ -794,13 +794,10 @@ cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtenso
              : (is_silu ? masked_conv_patch_sm100_kernel<false, true, IC> : masked_conv_patch_sm100_kernel<false, false, IC>))
     Kern kern = compact ? ASX_PICK(true) : ASX_PICK(false);
 #undef ASX_PICK
-    static int smem_set[8] = {0, 0, 0, 0, 0, 0, 0, 0};      // largest dynamic shared memory size enabled so far, per instance
+    static std::atomic<unsigned long long> smem_set[8];      // per instance
     const int vi = (has_res ? 1 : 0) + (is_silu ? 2 : 0) + (compact ? 4 : 0);
-    if (plan.smem_bytes > smem_set[vi]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
-        if (e != cudaSuccess) return e;
-        smem_set[vi] = plan.smem_bytes;
-    }
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), MAX_DYN_SMEM, smem_set[vi]);
+    if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(grid), dim3(compact ? num_threads<true> : num_threads<false>), (size_t)plan.smem_bytes, st, tmap_w, tmap_x4, g, a);
 }
 

@@ -955,7 +955,7 @@ int cluster_room(int KS)
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int clusters = 0;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
         if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
             cudaGetLastError();
             clusters = 148 / KS * 3 / 4;
@@ -1116,13 +1116,10 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
 #undef ASX_PICK2
 #undef ASX_PICK_F32
 #undef ASX_PICK
-    static int smem_set_all[80] = {0};          // largest dynamic shared memory size enabled so far, per instance
-    int* smem_set = smem_set_all + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0) + (split ? 40 : 0);
-    if (plan.smem_bytes > smem_set[variant]) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
-        if (e != cudaSuccess) return e;
-        smem_set[variant] = plan.smem_bytes;
-    }
+    static std::atomic<unsigned long long> smem_set[80];     // per instance
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), MAX_DYN_SMEM,
+                                     smem_set[variant + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0) + (split ? 40 : 0)]);
+    if (e != cudaSuccess) return e;
     return launch_pdl_cluster(kern, dim3(grid), dim3(NUM_THREADS), plan.ksplit, (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
 }
 

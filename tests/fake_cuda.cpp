@@ -12,6 +12,8 @@ int mallocs_left = -1;      // allocations that still succeed; -1: all
 int capturing = 0;
 int direct_words = 0;       // what plan_direct says: 0 the geometry does not take the direct form, else the words of a filter row
 int patch = 0;              // whether plan_patch accepts the geometry
+int device = 0;             // the current one
+int attribute_fails = 0;    // whether cudaFuncSetAttribute does
 
 void say(const std::string& s) { log_text += s + "\n"; }
 std::string order() { return asx::launch_in_stream_order ? " in order" : ""; }
@@ -32,12 +34,26 @@ void fake_set(const char* what, int value)
     else if (w == "capturing") capturing = value;
     else if (w == "direct_words") direct_words = value;
     else if (w == "patch") patch = value;
+    else if (w == "device") device = value;
+    else if (w == "attribute_fails") attribute_fails = value;
     else std::abort();
 }
 const char* fake_log() { return log_text.c_str(); }
 void fake_clear_log() { log_text.clear(); }
 
-cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+// a launch of the one kernel there is
+int fake_allow_smem(int bytes)
+{
+    static std::atomic<unsigned long long> set_on;
+    return (int)asx::allow_smem(reinterpret_cast<const void*>(&fake_log), bytes, set_on);
+}
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int bytes)
+{
+    if (attribute_fails) return cudaErrorInvalidValue;
+    say(std::to_string(bytes) + " bytes on device " + std::to_string(device));
+    return cudaSuccess;
+}
+cudaError_t cudaGetDevice(int* d) { *d = device; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int)
 {
     *v = a == cudaDevAttrComputeCapabilityMajor ? 10 : 148;

@@ -187,3 +187,22 @@ def test_failed_set_input_mask_leaves_none(layer):
         assert m.run(1, 8, 8, flags=IN_COMPACT) == (3, [])
         assert set_input_mask(64) == 0
         assert m.run(1, 8, 8, flags=IN_COMPACT) == (0, ["row gather"])
+
+
+def test_shared_memory_is_allowed_on_every_device(fake):
+    """A kernel's limit is kept per device: each one it is launched on gets it, once, and the most any plan takes."""
+    def launch(device):
+        fake.fake_clear_log()
+        fake.fake_set(b"device", device)
+        rc = fake.fake_allow_smem(227 * 1024)
+        fake.fake_set(b"device", 0)
+        return rc, fake.fake_log().decode()
+    fake.fake_set(b"attribute_fails", 1)
+    assert launch(1) == (1, "")
+    fake.fake_set(b"attribute_fails", 0)
+    for device in (0, 1, 63):
+        assert launch(device) == (0, f"232448 bytes on device {device}\n")
+        assert launch(device) == (0, "")
+    for _ in range(2):                                                  # past the devices that are remembered
+        assert launch(64) == (0, "232448 bytes on device 64\n")
+
