@@ -936,12 +936,16 @@ namespace {
 // Sharing k-blocks: fewest k-blocks of a tile, and what the exchange costs beside the bytes.
 constexpr int SPLIT_MIN_KB = 12;
 constexpr double SPLIT_US = 2.5;
-// Blocks in clusters of KS (one block per SM) that find a place on the device at a time; asked once per size.
+// Blocks in clusters of KS (one block per SM) that find a place on the current device at a time; asked once per device and
+// size.  0 where the device does not say: such a plan is not considered.
 int cluster_room(int KS)
 {
-    static std::atomic<int> known[9];
-    int room = known[KS].load(std::memory_order_relaxed);
-    if (room == 0) {
+    constexpr int DEVICES = 64;
+    static std::atomic<int> known[DEVICES][9];      // the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) return 0;
+    int room = known[dev][KS].load(std::memory_order_relaxed) - 1;
+    if (room < 0) {
         constexpr int bytes = 200 * 1024;
         auto kern = masked_conv_sm100_kernel<GATHER_TMA, false, false, false, false, true>;
         cudaLaunchConfig_t cfg = {};
@@ -956,12 +960,12 @@ int cluster_room(int KS)
         cfg.numAttrs = 1;
         int clusters = 0;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
-        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 0) {
             cudaGetLastError();
-            clusters = 148 / KS * 3 / 4;
+            return 0;
         }
         room = clusters * KS;
-        known[KS].store(room, std::memory_order_relaxed);
+        known[dev][KS].store(room + 1, std::memory_order_relaxed);
     }
     return room;
 }

@@ -206,3 +206,18 @@ def test_shared_memory_is_allowed_on_every_device(fake):
     for _ in range(2):                                                  # past the devices that are remembered
         assert launch(64) == (0, "232448 bytes on device 64\n")
 
+
+
+def test_k_blocks_are_shared_only_where_the_device_tells_its_room():
+    """No device here, so no clusters are known to fit; a guess could be more than a device takes at a time."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("there is a device")
+    from paper_2309_06626_b200 import build, lib
+    build.build()
+    plan_fast = lib()["_ZN3asx9plan_fastERKNS_8ConvGeomEixibiPNS_8FastPlanE"]
+    plan_fast.restype = ctypes.c_bool
+    plan_fast.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_bool, ctypes.c_int, ctypes.c_void_p]
+    g = (ctypes.c_int * 17)(1, 7, 7, 512, 512, 3, 3, 1, 1, 7, 7, 1, 1, 9 * 512, 49, 49, 49)      # one row tile, 72 k-blocks
+    plan = (ctypes.c_int * 12)()
+    assert plan_fast(g, 148, 49, 0, True, 2, plan) and plan[5] == 1
