@@ -43,6 +43,12 @@ def run_library(spec, x, w, b, mask, flags, prefill=None, form=None):
     return y, bits, kept
 
 
+def shares_k_blocks(layer):
+    """Whether a run of this layer shared k-blocks between thread blocks: the words of the time-out test exist then (the call
+    writes a zero, which they hold)."""
+    return asx.lib().asx_debug_set_split_counter(layer._h, 0, 0, int(torch.cuda.current_stream().cuda_stream)) == 0
+
+
 def full_row_mask(spec, mask):
     return mask if mask.size == spec.M else np.tile(mask, spec.Nb)
 

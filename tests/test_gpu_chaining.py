@@ -10,7 +10,7 @@ import torch
 import oracle
 import paper_2309_06626_b200 as asx
 import workloads as wl
-from gpu_util import to_dev_bf16
+from gpu_util import shares_k_blocks, to_dev_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -73,6 +73,7 @@ def test_two_layers_chained_compact(case):
     y2c = torch.full((Nb * kept2, cout), float("nan"), dtype=torch.bfloat16, device="cuda")
     _run_raw(A, xd, Nb, H, W, w1d, b1d, y1c, asx.ACT_RELU | asx.RECOMPACT | asx.OUT_COMPACT)
     _run_raw(B, y1c, Nb, l1.Ho, l1.Wo, w2d, b2d, y2c, asx.ACT_RELU | asx.RECOMPACT | asx.IN_COMPACT | asx.OUT_COMPACT)
+    assert cmid != 512 or shares_k_blocks(B)
     A.close(); B.close()
 
     rows1 = (np.arange(Nb)[:, None] * l1.P + np.flatnonzero(m1)[None, :]).reshape(-1)
@@ -143,13 +144,15 @@ RES_CASES = [
 ]
 
 
+@pytest.mark.parametrize("impl", [0, asx.IMPL_ROW_GATHER], ids=["default", "row_gather"])
 @pytest.mark.parametrize("act", ["relu", "silu"])
 @pytest.mark.parametrize("case", RES_CASES, ids=[f"r{i}" for i in range(len(RES_CASES))])
-def test_residual_add_before_the_activation(case, act):
+def test_residual_add_before_the_activation(case, act, impl):
     """y = mask ? act(conv + bias + residual) : 0, the shortcut of a residual block fused into the
-    epilogue.  The oracle gives conv + bias without activation; the rest is written out here."""
+    epilogue.  The oracle gives conv + bias without activation; the rest is written out here.  The cases' comments
+    say what the row gather does with them; by default the small dense ones take a direct form."""
     cin, cout, k, s, p, H, W, Nb, sp, blk, compact = case
-    act_flag = asx.ACT_RELU if act == "relu" else asx.ACT_SILU
+    act_flag = (asx.ACT_RELU if act == "relu" else asx.ACT_SILU) | impl
     f = (lambda z: np.maximum(z, 0.0)) if act == "relu" else (lambda z: z / (1.0 + np.exp(-z)))
     spec = wl.LayerSpec("res", cin, cout, k, k, s, p, H, W, Nb, sp, blk, "relu", wl.BASE_SEED + 310)
     x, w, b, m = wl.make_x(spec), wl.make_w(spec), wl.make_b(spec), wl.make_layer_mask(spec)
@@ -172,7 +175,7 @@ def test_residual_add_before_the_activation(case, act):
         flags = act_flag | asx.RECOMPACT
     layer.set_residual(rd)
     st = int(torch.cuda.current_stream().cuda_stream)
-    assert layer.run_raw(xd.data_ptr(), Nb, H, W, wd.data_ptr(), bd.data_ptr(), y.data_ptr(), flags | asx.IMPL_NAIVE, st) == 1
+    assert layer.run_raw(xd.data_ptr(), Nb, H, W, wd.data_ptr(), bd.data_ptr(), y.data_ptr(), (flags & ~impl) | asx.IMPL_NAIVE, st) == 1
     _run_raw(layer, xd, Nb, H, W, wd, bd, y, flags)
     got = y.float().cpu().numpy().astype(np.float64)
     assert not np.isnan(got).any()
@@ -181,6 +184,9 @@ def test_residual_add_before_the_activation(case, act):
     _close(got, want, spec.K, x, w, extra_abs=2.0 ** -8 * float(np.abs(want).max()))
     if not compact:
         assert not got[~fm].any()
+    if impl:
+        assert layer.last_run_form() in (asx.FORM_ROW_GATHER_TMA, asx.FORM_ROW_GATHER_COPY)
+        assert shares_k_blocks(layer) == (cin == 512)
     # switching the residual off gives the plain layer again
     layer.set_residual(None)
     _run_raw(layer, xd, Nb, H, W, wd, bd, y, flags)

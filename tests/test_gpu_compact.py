@@ -132,6 +132,7 @@ def test_mask_written_by_the_kernel_just_before(rows):
         assert np.array_equal(k2[:want.size].cpu().numpy(), want), r
 
 
+@pytest.mark.parametrize("impl", [0, asx.IMPL_ROW_GATHER], ids=["default", "row_gather"])
 @pytest.mark.parametrize("case", [
     # name, C_in, C_out, k, pad, H, W, Nb, pct, block, fused list expected to fit beside the pipeline stages
     ("pw_160", 32, 32, 1, 0, 160, 160, 1, 40, 4),              # 25600-row mask: compacted inside the fused kernel
@@ -139,18 +140,18 @@ def test_mask_written_by_the_kernel_just_before(rows):
     ("pw_182x182", 64, 64, 1, 0, 182, 182, 1, 50, 1),          # 33124 rows: the stand-alone passes
     ("c3_150_wide", 64, 256, 3, 1, 150, 150, 1, 70, 2),        # 22500 rows, 256-wide tiles: no room for the list, falls back
 ], ids=lambda c: c[0])
-def test_masks_between_the_one_block_limit_and_the_fused_limit(case):
+def test_masks_between_the_one_block_limit_and_the_fused_limit(case, impl):
     """Masks of 16385..32768 rows are compacted inside the fused kernel when their 2-byte list fits beside the
     pipeline stages, by the stand-alone passes otherwise; either way ASX_RECOMPACT must give the stored list's result
-    and the oracle's."""
+    and the oracle's.  (By default the 1x1 layers take the direct form, which rebuilds the list beside the convolution.)"""
     name, cin, cout, k, pad, H, W, Nb, pct, blk = case
     spec = wl.LayerSpec(name, cin, cout, k, k, 1, pad, H, W, Nb, pct, blk, "relu", wl.BASE_SEED + 8800 + H)
     x, w, b, mask = make_problem(spec, per_row=False)
     layer = asx.MaskedConvLayer(cin, cout, k, k, 1, pad)
     layer.set_mask(mask)
     xd, wd, bd = to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda()
-    y_stored = layer.run(xd, wd, bd, flags=asx.ACT_RELU).clone()
-    y_re = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT).clone()
+    y_stored = layer.run(xd, wd, bd, flags=asx.ACT_RELU | impl).clone()
+    y_re = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT | impl).clone()
     torch.cuda.synchronize()
     assert layer.device_status() == 0
     assert np.array_equal(layer.kept(), oracle.kept_list(mask))
@@ -158,8 +159,9 @@ def test_masks_between_the_one_block_limit_and_the_fused_limit(case):
     # a new mask through the device copy only (no host-side list): the next RECOMPACT run must follow it
     mask2 = np.roll(mask, 7)
     layer.set_mask(mask2)
-    y2 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT)
+    y2 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT | impl)
     torch.cuda.synchronize()
+    assert impl == 0 or layer.last_run_form() == (asx.FORM_ROW_GATHER_TMA if cin == 64 else asx.FORM_ROW_GATHER_COPY)
     assert np.array_equal(layer.kept(), oracle.kept_list(mask2))
     ref = oracle.masked_conv(x, w, b, mask2, 1, pad, True).reshape(spec.M, cout)
     got = y2.float().cpu().numpy().astype(np.float64).reshape(spec.M, cout)

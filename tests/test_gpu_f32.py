@@ -21,7 +21,7 @@ from gpu_util import full_row_mask, make_problem
 pytestmark = pytest.mark.gpu
 
 SMALL = list(wl.iter_small_cases())
-IMPLS = [("naive", asx.IMPL_NAIVE), ("tcgen05", 0)]
+IMPLS = [("naive", asx.IMPL_NAIVE), ("default", 0), ("row_gather", asx.IMPL_ROW_GATHER)]
 REL_TOL_F32 = 2e-4
 
 
@@ -79,12 +79,13 @@ def test_small_cases_full_compare(spec, impl):
     check_f32(spec, x, w, b, mask, asx.ACT_RELU | impl[1])
 
 
+@pytest.mark.parametrize("impl", IMPLS[1:], ids=[i[0] for i in IMPLS[1:]])
 @pytest.mark.parametrize("spec", SMALL[:6], ids=[s.name for s in SMALL[:6]])
-def test_silu_per_row_mask_and_recompact(spec):
+def test_silu_per_row_mask_and_recompact(spec, impl):
     x, w, b, mask = tf32_problem(spec, per_row=True)
-    check_f32(spec, x, w, None, mask, asx.ACT_SILU)
+    check_f32(spec, x, w, None, mask, asx.ACT_SILU | impl[1])
     x, w, b, mask = tf32_problem(spec)
-    check_f32(spec, x, w, b, mask, asx.RECOMPACT)
+    check_f32(spec, x, w, b, mask, asx.RECOMPACT | impl[1])
 
 
 @pytest.mark.parametrize("impl", IMPLS, ids=[i[0] for i in IMPLS])
@@ -113,7 +114,8 @@ def test_tiny_integer_cases_bit_exact(k, p, impl):
             assert np.array_equal(y, ref), (C_in, C_out, relu)
 
 
-def test_lower_mantissa_bits_of_the_operands_are_ignored():
+@pytest.mark.parametrize("impl", IMPLS[1:], ids=[i[0] for i in IMPLS[1:]])
+def test_lower_mantissa_bits_of_the_operands_are_ignored(impl):
     """The contraction reads only the TF32 part of an fp32 operand: full-precision inputs give the
     same bits as the inputs with their lower 13 mantissa bits cleared.  Note what this does and does
     not show: it compares the GPU with ITSELF (two runs of the same kernel), which is how the reading
@@ -122,8 +124,8 @@ def test_lower_mantissa_bits_of_the_operands_are_ignored():
     file) runs on inputs that are already TF32 values, where no reading of the conversion enters."""
     for spec in (SMALL[0], SMALL[2], SMALL[6]):
         x, w, b, mask = make_problem(spec)
-        y_full, bits_full, _ = run_f32(spec, x, w, b, mask, asx.ACT_RELU)
-        y_t, bits_t, _ = run_f32(spec, oracle.tf32_operand(x), oracle.tf32_operand(w), b, mask, asx.ACT_RELU)
+        y_full, bits_full, _ = run_f32(spec, x, w, b, mask, asx.ACT_RELU | impl[1])
+        y_t, bits_t, _ = run_f32(spec, oracle.tf32_operand(x), oracle.tf32_operand(w), b, mask, asx.ACT_RELU | impl[1])
         assert np.array_equal(bits_full, bits_t), spec.name
 
 

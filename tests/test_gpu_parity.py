@@ -11,13 +11,13 @@ import torch
 import oracle
 import paper_2309_06626_b200 as asx
 import workloads as wl
-from gpu_util import check_against_oracle, make_problem, run_library, to_dev_bf16
+from gpu_util import check_against_oracle, make_problem, run_library, shares_k_blocks, to_dev_bf16
 from philox_ref import random_block_mask
 
 pytestmark = pytest.mark.gpu
 
 SMALL = list(wl.iter_small_cases())
-IMPLS = [("naive", asx.IMPL_NAIVE), ("tcgen05", 0), ("row_gather", asx.IMPL_ROW_GATHER)]
+IMPLS = [("naive", asx.IMPL_NAIVE), ("default", 0), ("row_gather", asx.IMPL_ROW_GATHER)]
 
 
 @pytest.mark.parametrize("impl", IMPLS, ids=[i[0] for i in IMPLS])
@@ -121,19 +121,20 @@ def test_generated_mask_matches_documented_rule():
     layer.close()
 
 
-def test_recompact_flag_and_mask_change():
+@pytest.mark.parametrize("impl", [0, asx.IMPL_ROW_GATHER], ids=["default", "row_gather"])
+def test_recompact_flag_and_mask_change(impl):
     spec = SMALL[0]
     x, w, b, mask = make_problem(spec)
     layer = asx.MaskedConvLayer(spec.C_in, spec.C_out, 3, 3, spec.stride, spec.pad)
     from gpu_util import to_dev_bf16
     xd, wd, bd = to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda()
     layer.set_mask(mask)
-    y1 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT)
-    y2 = layer.run(xd, wd, bd, flags=asx.ACT_RELU)
+    y1 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | asx.RECOMPACT | impl)
+    y2 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | impl)
     assert torch.equal(y1.view(torch.int16), y2.view(torch.int16))
     mask2 = 1 - mask
     layer.set_mask(torch.from_numpy(mask2).cuda())           # device-side mask
-    y3 = layer.run(xd, wd, bd, flags=asx.ACT_RELU)
+    y3 = layer.run(xd, wd, bd, flags=asx.ACT_RELU | impl)
     torch.cuda.synchronize()
     ref = oracle.masked_conv(x, w, b, mask2, spec.stride, spec.pad, True)
     assert np.array_equal(layer.kept(), oracle.kept_list(mask2))
@@ -176,10 +177,10 @@ def test_shared_k_blocks_give_the_same_bits_every_run():
     xd, wd, bd = to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda()
     runs = []
     for flags in (asx.ACT_RELU, asx.ACT_RELU | asx.RECOMPACT, asx.ACT_RELU):
-        y = layer.run(xd, wd, bd, flags=flags)
+        y = layer.run(xd, wd, bd, flags=flags | asx.IMPL_ROW_GATHER)
         torch.cuda.synchronize()
         runs.append(y.view(torch.int16).cpu().numpy().copy())
-    assert layer.device_status() == 0
+    assert layer.device_status() == 0 and shares_k_blocks(layer)
     layer.close()
     assert np.array_equal(runs[0], runs[1]) and np.array_equal(runs[0], runs[2])
     ref = oracle.masked_conv(x, w, b, mask, spec.stride, spec.pad, True)

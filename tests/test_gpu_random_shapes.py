@@ -39,7 +39,9 @@ def test_random_geometry(i):
     per_row = bool(rng.random() < 0.3)
     x, w, b, mask = make_problem(spec, per_row=per_row)
     flags = (asx.ACT_RELU if rng.random() < 0.7 else 0) | (asx.RECOMPACT if rng.random() < 0.5 else 0)
-    check_against_oracle(spec, x, w, b if rng.random() < 0.8 else None, mask, flags)
+    b = b if rng.random() < 0.8 else None
+    for impl in (0, asx.IMPL_ROW_GATHER):              # most of these are small enough for a direct form
+        check_against_oracle(spec, x, w, b, mask, flags | impl)
 
 
 def _random_patch_spec(i):

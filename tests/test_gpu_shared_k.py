@@ -4,6 +4,7 @@ import pytest
 import torch
 
 import paper_2309_06626_b200 as asx
+from gpu_util import shares_k_blocks
 
 pytestmark = pytest.mark.gpu
 
@@ -32,7 +33,7 @@ def test_shares_of_every_size(case, f32):
     for flags in (asx.IMPL_ROW_GATHER, asx.IMPL_ROW_GATHER | asx.RECOMPACT):
         got = layer.run(x, w, b, flags=base | asx.ACT_RELU | flags).float()
         torch.cuda.synchronize()
-        assert layer.device_status() == 0
+        assert layer.device_status() == 0 and shares_k_blocks(layer)
         assert (got - want).norm() <= (2e-5 if f32 else 5e-3) * want.norm()
         assert not got.reshape(Nb, H * W, cout)[:, (mask == 0).cuda()].any()
     layer.close()

@@ -1,9 +1,8 @@
 """The bounded waits of the fused kernel, exercised from the host in the safe form.
 
-A layer with few kept rows and a long reduction shares each tile's k-blocks between thread blocks;
-the blocks of a tile meet at an arrival counter.  The test overwrites one tile's counter with a value
-the arrivals can never lift to the number of shares and shortens the wait limit to about a
-millisecond: the waiting blocks must give up, every role of the kernel must leave, the kernel must
+A layer with few kept rows and a long reduction shares each tile's k-blocks between thread blocks,
+which wait for each other's partial sums.  The test sets a word of one tile that makes its blocks expect
+more bytes than are sent and shortens the wait limit to about a millisecond: the waiting blocks must give up, every role of the kernel must leave, the kernel must
 return, the status word must say so, and the next run on the same handle must be correct again.
 Nothing here faults, traps or hangs the GPU: the wait simply runs out."""
 import numpy as np
@@ -40,7 +39,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_layer_recovers():
         assert np.abs(got - ref).max() <= tol
 
     run_and_compare()
-    # the plan of this layer shares k-blocks: the counters exist (else this case tests nothing)
+    # the plan of this layer shares k-blocks: the words exist (else this case tests nothing)
     rc = asx.lib().asx_debug_set_split_counter(layer._h, 0, -100000, st)
     assert rc == 0, f"the layer was expected to share k-blocks between blocks (status {rc})"
     assert asx.lib().asx_debug_set_split_counter(layer._h, 1 << 40, 0, st) == 1       # outside the workspace
@@ -64,8 +63,9 @@ def test_hook_refuses_layers_without_shared_k_blocks():
     x, w, b, mask = make_problem(spec)
     layer = asx.MaskedConvLayer(64, 64, 3, 3, 1, 1)
     layer.set_mask(mask)
-    layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU)
+    layer.run(to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda(), flags=asx.ACT_RELU | asx.IMPL_ROW_GATHER)
     torch.cuda.synchronize()
+    assert layer.last_run_form() == asx.FORM_ROW_GATHER_TMA
     st = int(torch.cuda.current_stream().cuda_stream)
     assert asx.lib().asx_debug_set_split_counter(layer._h, 0, 5, st) == 2       # ASX_ERR_UNSUPPORTED
     layer.close()
