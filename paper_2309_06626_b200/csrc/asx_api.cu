@@ -50,7 +50,6 @@ struct asx_layer {
     // what the host knows about the current mask (masks that came from host memory, up to 2^24 rows)
     std::vector<uint8_t> host_mask;
     uint64_t mask_epoch = 0;           // bumped by every asx_set_mask*
-    // window-patch form: rows of padded input the windows of one 128-row tile span at most, cached per geometry
     // window-patch form: the row tiles cut from the host's mask, cached per geometry and buffer size
     uint64_t tiles_epoch = ~0ull;
     int tiles_Nb = 0, tiles_H = 0, tiles_W = 0, tiles_cap = 0;
@@ -62,8 +61,8 @@ struct asx_layer {
     const void* tmapx4_ptr = nullptr;
     int tmapx4_Nb = 0, tmapx4_H = 0, tmapx4_W = 0, tmapx4_Wp = 0;
     int tmapx4_px32 = 0;
-    int wait_limit_kcycles = 0;
-    int last_form = ASX_FORM_NONE;     // producer form of the last asx_run        // bound of the in-kernel waits in units of 1024 cycles (0: the default, about 2 s)
+    int wait_limit_kcycles = 0;        // bound of the in-kernel waits in units of 1024 cycles (0: the default, about 2 s)
+    int last_form = ASX_FORM_NONE;     // producer form of the last asx_run
 };
 
 namespace {
@@ -501,7 +500,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     };
     // Small masks are compacted inside the fused kernel itself (no launches of its own, and the list stays in
     // shared memory as 16-bit positions); the reference kernel and large masks take the stand-alone compaction
-    // kernels.  Up to 16384 rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
+    // kernels.  Up to COMPACT_SMALL_MAX_ROWS rows always; up to FUSED_COMPACT_MAX_ROWS when the list (2 bytes per row) still
     // leaves the plan its pipeline stages (decided below, once the geometry the kernel sees is known).
     const int relu = (flags & ASX_ACT_SILU) ? 2 : (flags & ASX_ACT_RELU) ? 1 : 0;      // activation code: 0 identity, 1 ReLU, 2 SiLU
     // Small filter matrices take the direct form, which needs no list and rebuilds it beside the convolution when asked to;
@@ -701,7 +700,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     FastPlan plan;
     long long est_rows = M;                                       // unknown on the host: assume every row kept
     if (L->host_kept >= 0) est_rows = (L->rows == P) ? L->host_kept * Nb : L->host_kept;
-    // Sharing a tile's k-blocks between blocks needs the exact tile count (to size the workspace)
+    // Sharing a tile's k-blocks between blocks needs the exact tile count (one item per block, all clusters at once)
     // and 16-byte output stores.
     const bool allow_split = L->host_kept >= 0 && L->C_out % 8 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
     if (!plan_fast(g, L->num_sms, est_rows, fuse_compact ? (int)L->rows : 0, allow_split, ES, &plan)) {
@@ -909,7 +908,7 @@ asx_status asx_last_device_status(asx_layer* L)
         cudaMemcpy(&scan_err, static_cast<int32_t*>(L->d_scratch) + 1, sizeof(scan_err), cudaMemcpyDeviceToHost) != cudaSuccess)
         return ASX_ERR_CUDA;
     if (word != 0 && cudaMemset(L->d_small + 1, 0, sizeof(word)) != cudaSuccess) return ASX_ERR_CUDA;
-    // a launch that gave up may have left tile counters of the split-K exchange half way
+    // the words with which a test keeps the shares of a tile waiting
     if (word != 0 && L->d_wscnt != nullptr && cudaMemset(L->d_wscnt, 0, L->wscnt_ints * sizeof(int)) != cudaSuccess) return ASX_ERR_CUDA;
     return (word != 0 || scan_err != 0) ? ASX_ERR_TIMEOUT : ASX_OK;
 }

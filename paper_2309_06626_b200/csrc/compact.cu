@@ -161,9 +161,10 @@ compact_copy_count_kernel(const uint8_t* __restrict__ mask, long long rows, int 
 // Pass 2: the indices of a 4096-row sub-tile are put in order in shared memory and copied to the list
 // with full-width stores (direct stores of each 32-row ballot word's indices, without the staging,
 // write half-filled lines and were 12 % slower; 16-byte stores from the unaligned staging buffer 3 %; a
-// staging index swizzled against bank conflicts 18 %: the pass is bound by the instructions it issues).
-// EARLY_MASK: the mask is only ever written by stream-ordered copies (a layer's own copy of its mask), so
-// the first tile's mask bytes may be loaded and scanned before the dependency wait, while the pass before
+// staging index swizzled against bank conflicts 18 %).  On 2^27 rows, half of them kept, the shared-memory pipe is busy 75 % of
+// the time (two thirds of it the staging stores, more than half of those bank conflicts), the issue slots 67 %, DRAM 46 %.
+// EARLY_MASK: no kernel that may still be running wrote the mask (a layer's own copy of its mask, unless it has just been taken
+// from the device), so the first tile's mask bytes may be loaded and scanned before the dependency wait, while the pass before
 // still runs.  A caller's mask buffer may have been written by the kernel just before this call (a
 // data-dependent mask), which, launched as a programmatic predecessor, can still be storing it: then the
 // load waits like everything else.
@@ -362,7 +363,7 @@ static cudaError_t launch_two_passes(const uint8_t* mask, int64_t rows, int32_t*
 }
 
 cudaError_t launch_compact(const uint8_t* mask, int64_t rows, int32_t* kept, int32_t* count,
-                           void* scratch, cudaStream_t st, bool mask_written_by_copies_only, uint8_t* copy)
+                           void* scratch, cudaStream_t st, bool mask_settled, uint8_t* copy)
 {
     auto* hdr = static_cast<ScratchHeader*>(scratch);
     // One pass while counting all bytes in front of the last block costs less than a second launch (about 2 us), and the
@@ -370,10 +371,10 @@ cudaError_t launch_compact(const uint8_t* mask, int64_t rows, int32_t* kept, int
     const bool aligned = (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
     if (rows <= (aligned ? COMPACT_PREFIX_MAX_ROWS : COMPACT_SMALL_MAX_ROWS))
         return launch_pdl(compact_prefix_kernel, dim3((unsigned)tiles_for(rows)), dim3(COMPACT_THREADS), 0, st, mask,
-                          (int)rows, kept, count, hdr, copy, mask_written_by_copies_only ? 1 : 0);
+                          (int)rows, kept, count, hdr, copy, mask_settled ? 1 : 0);
     return rows <= (int64_t)COMPACT_TILE * COMPACT_RESIDENT * resident_sms()
-               ? launch_two_passes<1>(mask, rows, kept, count, hdr, st, mask_written_by_copies_only, copy)
-               : launch_two_passes<COMPACT_SUB>(mask, rows, kept, count, hdr, st, mask_written_by_copies_only, copy);
+               ? launch_two_passes<1>(mask, rows, kept, count, hdr, st, mask_settled, copy)
+               : launch_two_passes<COMPACT_SUB>(mask, rows, kept, count, hdr, st, mask_settled, copy);
 }
 
 }  // namespace asx

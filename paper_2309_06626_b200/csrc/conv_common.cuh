@@ -72,7 +72,7 @@ __device__ __forceinline__ bool warp_wait_bar(uint32_t bar, uint32_t parity, vol
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// S1 inside the fused kernel, for masks of at most 16384 rows: the whole block scans the mask
+// S1 inside the fused kernel, for masks of at most 32768 rows: the whole block scans the mask
 // (16 bytes per thread, popcount, shuffle scan within the warps, warp totals through shared
 // memory) and writes the ascending kept positions as 16-bit values into its own shared memory
 // (every block writing the list to the same global addresses serialises in L2 and cost 10-20 us;

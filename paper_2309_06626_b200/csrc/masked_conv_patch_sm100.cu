@@ -183,8 +183,8 @@ masked_conv_patch_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // Let the next kernel of the stream start its own prologue; everything up to the dependency
-    // wait below touches only this block's shared and tensor memory (and the layer's mask, which
-    // is only ever written by stream-ordered copies).
+    // wait below touches only this block's shared and tensor memory (and the layer's mask: behind a kernel
+    // that wrote it this one is launched in stream order).
     ptx::grid_launch_dependents();
     const int N = g.C_out, BN = a.BN, BS = a.b_stages, AS = a.a_stages;
     const int taps = g.kh * g.kw, G = a.G;

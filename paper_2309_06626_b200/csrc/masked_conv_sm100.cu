@@ -17,8 +17,8 @@
 //   zero warps      write zeros to the dropped rows of this block's share of the output,
 //                   straight from the mask.  Every output element is written exactly once.
 //
-// The kept-row list comes from device memory or, for masks of at most 16384 rows, is built by
-// every block in its own shared memory at the start of this kernel (stage i of Section 3.2 fused
+// The kept-row list comes from device memory or, for masks of at most 32768 rows whose list fits beside the
+// stages, is built by every block in its own shared memory at the start of this kernel (stage i of Section 3.2 fused
 // in); either way the host never has to know the count.  Layers with few kept rows and a long
 // reduction may share a tile's k-blocks between blocks (split K with a fixed-order exchange).
 // All waits are bounded: a wait that runs out sets the status word and every role leaves.
@@ -214,9 +214,9 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     constexpr int EPC = 16 / ES;            // elements per 16-byte chunk
     const int KB = (g.K + BKE - 1) / BKE;
 
-    // The layer's mask is only ever written by stream-ordered copies, never by a kernel, so the
-    // fused compaction may read it while the preceding kernel is still running; the read is
-    // issued first so that its latency overlaps the set-up below.
+    // The preceding kernel, which may still be running, did not write the mask (behind one that did, a launch with the fused
+    // compaction is in stream order), so it may be read here; the read is issued first so that its latency overlaps
+    // the set-up below.
     uint4 early_mask = make_uint4(0, 0, 0, 0);
     const bool early_ok = a.fuse_compact && tid * 16 + 16 <= g.rows && (reinterpret_cast<uintptr_t>(a.mask) & 15) == 0;
     if (early_ok) early_mask = ptx::ld_global_v4_keep_in_l2(a.mask + tid * 16);
@@ -987,9 +987,9 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     // gives more tiles when a layer has few kept rows, and sharing a tile's k-blocks between the blocks of a
     // cluster gives more work items still, at the price of exchanging fp32 partial tiles.  Pick
     // the pair with the lowest estimated time, from figures measured on B200: a 64-wide k-block
-    // of a 128 x BN tile takes about 0.30 + 0.001 BN microseconds (the loop is bound by the TMA
-    // requests and bytes one SM can pull from L2: 16 KB of gathered rows in 32 requests of about
-    // 13 clocks, plus the BN x 128-byte filter slab), the last tile's epilogue about 0.012 BN,
+    // of a 128 x BN tile takes about 0.12 + 0.18 fill + 0.001 BN microseconds, fill being the share of its
+    // 128 rows that is gathered (the loop is bound by the TMA requests and bytes one SM can pull from L2: a full tile's
+    // 16 KB of gathered rows in 32 requests of about 13 clocks, plus the BN x 128-byte filter slab), the last tile's epilogue about 0.012 BN,
     // and the exchange SPLIT_US (cluster barriers, BN x 512 bytes through distributed shared memory in and out).
     // A shared tile is its block's only one, and clusters that do not all fit at once are not considered (a second wave costs
     // more than sharing gains): the GPU tells how many do (148 blocks in twos, 132 in fours, 120 in eights).
