@@ -46,7 +46,7 @@ typedef enum {
     ASX_ERR_ALIGN = 5,         /* a pointer is not aligned as documented */
     ASX_ERR_OOM = 6,           /* device or host allocation failed */
     ASX_ERR_CUDA = 7,          /* a CUDA runtime or driver call failed */
-    ASX_ERR_TIMEOUT = 8        /* a bounded wait inside a kernel gave up */
+    ASX_ERR_TIMEOUT = 8        /* a bounded wait inside a kernel gave up, or a kernel found another mask than it was launched for */
 } asx_status;
 
 /* flags of asx_run */
@@ -71,7 +71,8 @@ enum {
                               (ASX_ERR_INVALID_ARG) */
     ASX_IMPL_DIRECT = 512, /* take the direct form (operands gathered into registers, no kept-row list; meant for small
                               filter matrices) wherever it can run: dense input and output, a filter matrix that fits
-                              in shared memory */
+                              in shared memory; where the channels are no whole number of 16-byte chunks, x at a 4-byte
+                              address and rows of at most 32000 values, the padding included */
     ASX_IMPL_DIRECT_K = 1024  /* take the direct form whose warps share a small tile's k range (meant for few kept rows)
                               wherever it can run: dense input and output, C_in a whole number of 16-byte chunks, a mask of
                               at most 16384 rows from host memory.  At most one of the four form switches
@@ -196,6 +197,10 @@ asx_status asx_recompact(asx_layer* layer, void* cuda_stream);
  *          mantissa bits are zero are multiplied exactly); sums, bias and activation are fp32 and y is
  *          written unrounded.  ASX_IMPL_NAIVE with ASX_F32 multiplies the full fp32 values.  Not
  *          together with ASX_OUT_COMPACT, ASX_IN_COMPACT or a residual (ASX_ERR_UNSUPPORTED).
+ * In a CUDA graph the call is the launch for the mask that the layer had during the capture, on the buffers that
+ * it had then: capture it again after asx_set_mask* outside the graph, asx_set_input_mask, or a run with larger
+ * tensors.  A replay under another mask of the same length computes what its launch allows or nothing, and
+ * asx_last_device_status says so (ASX_ERR_TIMEOUT).  Make a layer's first run before the capture: it allocates.
  * Asynchronous on `cuda_stream`.  Allocates on first use and when a buffer must grow: copies of x and w
  * with the channels zero-padded to a multiple of 8 (refreshed by a small kernel on every call) where
  * C_in % 8 != 0 and the form that runs needs them, the row tiles of the window-patch form, and two
@@ -229,7 +234,8 @@ asx_status asx_get_mask(asx_layer* layer, uint8_t* host_mask_out, int64_t rows);
 
 /*
  * Waits for the stream last used with this layer and reports the kernels' status word:
- * ASX_OK, or ASX_ERR_TIMEOUT if a bounded wait inside a kernel ran out (the output of that
+ * ASX_OK, or ASX_ERR_TIMEOUT if a bounded wait inside a kernel ran out or the mask on the device was
+ * not the one the launch was made for (the output of that
  * call is then undefined; the CUDA context stays usable).  The word is cleared by the call.
  */
 asx_status asx_last_device_status(asx_layer* layer);

@@ -545,8 +545,11 @@ __global__ void __launch_bounds__(KTHREADS) masked_conv_direct_k_kernel(const Co
         pos[c] = e;
     }
     const int cnt = block_compact(a.mask, g.rows, make_uint4(0, 0, 0, 0), false, list, scan_total, KTHREADS);
-    const int Mk = (g.rows == g.P) ? g.Nb * cnt : cnt;
-    if (Mk != a.Mk && tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);                      // the grid was sized for another mask
+    int Mk = (g.rows == g.P) ? g.Nb * cnt : cnt;
+    if (Mk != a.Mk) {                   // grid and divisor are those of another mask (a graph replayed under a new one): nothing can be computed
+        if (tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);
+        Mk = 0;
+    }
     const int r_first = blockIdx.x * ROWS, n0 = blockIdx.y * CH;
     if (tid < ROWS) {
         const int rk = r_first + tid;

@@ -92,3 +92,42 @@ def test_host_mask_is_refused_under_capture():
     assert np.array_equal(layer.kept(), oracle.kept_list(1 - mask))
     del graph
     layer.close()
+
+
+@pytest.mark.parametrize("per_row", [False, True], ids=["shared", "per_row"])
+def test_a_graph_replayed_under_another_mask(per_row):
+    """The direct form whose warps share the k range is launched for a number of kept rows: under a mask with as many it
+    computes that one, under another it stores nothing but zeros, says so, and stays inside its tensors."""
+    spec = wl.LayerSpec("replay", 64, 64, 3, 3, 1, 1, 13, 11, 3, 50, 1, "relu", wl.BASE_SEED + 951)
+    x, w, b, mask = wl.make_x(spec), wl.make_w(spec), wl.make_b(spec), wl.make_layer_mask(spec, per_row)
+    xd, wd, bd = to_dev_bf16(x), to_dev_bf16(w), torch.from_numpy(b).cuda()
+    room = torch.full((spec.M + 256, 64), 7.0, dtype=torch.bfloat16, device="cuda")
+    y = room[128:128 + spec.M].view(spec.Nb, spec.Ho, spec.Wo, 64)
+    layer = asx.MaskedConvLayer(64, 64, 3, 3, 1, 1)
+    layer.set_mask(mask)
+    layer.run(xd, wd, bd, y, flags=asx.ACT_RELU | asx.IMPL_DIRECT_K)
+    torch.cuda.synchronize()
+    assert layer.last_run_form() == asx.FORM_DIRECT_K
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layer.run(xd, wd, bd, y, flags=asx.ACT_RELU | asx.IMPL_DIRECT_K)
+    more, fewer = mask.copy(), mask.copy()
+    more[np.flatnonzero(mask == 0)[:5]] = 1
+    fewer[np.flatnonzero(mask)[:7]] = 0
+    for m in (mask, np.roll(mask, 3), more, fewer, np.zeros_like(mask), np.ones_like(mask), mask):
+        layer.set_mask(m)
+        y.fill_(7.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        same = int(m.sum()) == int(mask.sum())
+        assert layer.device_status() == (0 if same else 8)
+        got, full = y.float().cpu().numpy().reshape(spec.M, 64), m if per_row else np.tile(m, spec.Nb)
+        assert not got[full == 0].any()
+        if same:
+            ref = oracle.masked_conv(x, w, b, m, 1, 1, True).reshape(spec.M, 64)
+            assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < 5e-3
+        else:
+            assert (got[full != 0] == 7.0).all()
+        assert bool((room[:128] == 7.0).all()) and bool((room[128 + spec.M:] == 7.0).all())
+    del graph
+    layer.close()
