@@ -37,18 +37,18 @@ L2_BYTES = 126 * 1024 * 1024
 
 # DRAM traffic of the fused kernels from one ncu capture of the default workload (ResNet-18 stack, batch 64):
 # dram__bytes_read.sum + dram__bytes_write.sum averaged over the 20 fused-kernel launches of a step
-# (12.79 MB read + 2.35 MB written; ncu flushes the caches before every captured launch, so reads are
+# (12.47 MB read + 2.15 MB written; ncu flushes the caches before every captured launch, so reads are
 # cold-cache and most of a launch's output is still in L2 when its counters stop).  The figure belongs to
 # the kernel sources whose digest is recorded with it; with any other sources the bench reports null.
-NCU_TRAFFIC = {"workload_config": 3, "bytes_per_launch": 15.15e6,
-               "csrc_sha256": "31c31102a1af22b7012d9a7e070229ec88cbaf102c67d75daddabe819296c3ee"}
+NCU_TRAFFIC = {"workload_config": 3, "bytes_per_launch": 14.63e6,
+               "csrc_sha256": "4b56283805d82252b6fe25cbc4ddcde5d37788c3507ea9df6a5681acd832a437"}
 
 
 def csrc_digest() -> str:
-    """Digest of the sources the fused kernel is compiled from."""
+    """Digest of the sources the fused kernels are compiled from."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("asx_internal.h", "conv_common.cuh", "masked_conv_sm100.cu", "masked_conv_patch_sm100.cu", "ptx_sm100.cuh"):
+    for name in ("asx_internal.h", "conv_common.cuh", "masked_conv_direct.cu", "masked_conv_sm100.cu", "masked_conv_patch_sm100.cu", "ptx_sm100.cuh"):
         h.update(name.encode())
         with open(os.path.join(ROOT, "paper_2309_06626_b200", "csrc", name), "rb") as fh:
             h.update(fh.read())
@@ -771,7 +771,7 @@ def run_ours(args):
                 "ms_per_step": e2e_ms},
         "gpu_launches": K * sum(L.launches for L in layers),
         "roofline": {
-            "bound": "tensor", "kernel": "masked_conv_sm100_kernel / masked_conv_patch_sm100_kernel (one launch per layer)",
+            "bound": "tensor", "kernel": "masked_conv_sm100_kernel / masked_conv_patch_sm100_kernel / masked_conv_direct_kernel (one launch per layer)",
             "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
             # frac is the spec quantity: per layer the slower of its kept-row FLOPs at the tensor peak and
             # its algorithmic bytes at the HBM peak, summed over the layers, over the measured step time
@@ -782,7 +782,7 @@ def run_ours(args):
             "frac_tensor_only_vs_other_peak": achieved / (peaks["bf16_tflops_sustained"] if burst else peaks["bf16_tflops"]),
             "layer_roofs_ms_per_step": roof_ms,
             "kernel_ms_per_step": ms_step,
-            "kernel_ms_note": "the graph-replayed step: the fused kernel's launches (plus the stem's staging kernel), "
+            "kernel_ms_note": "the graph-replayed step: the fused kernels' launches, "
                               "overlapping by programmatic dependent launch as in the timed region",
             "in_step_ms_sum": None if in_step_ms is None else sum(in_step_ms),
             "in_step_note": "per_layer.ms_in_step: replay time of the captured prefix of layers [0..i] minus that of [0..i-1]; "
@@ -815,7 +815,7 @@ def run_ours(args):
                 "chain": chain,
                 "sweep": None if sweep is None else [{k: e[k] for k in ("sparsity_pct", "block", "tflops", "speedup_vs_sparsity0")}
                                                      for e in sweep],
-                "window_patch_layers": sum(1 for f in forms if f == 4), "row_gather_layers": sum(1 for f in forms if f in (2, 3))}},
+                "window_patch_layers": sum(1 for f in forms if f == 4), "row_gather_layers": sum(1 for f in forms if f in (2, 3)), "direct_layers": sum(1 for f in forms if f in (5, 6))}},
         "cpu_baseline": cpu,
         "cpu_alg2_fp32": cpu_alg2,
         "s1_compaction": s1,
