@@ -16,7 +16,7 @@
 // The legacy tensor path runs at a quarter of the tcgen05 rate (1017 of 4096 multiply-adds per clock and SM,
 // measured), which is why only small filter matrices come here; the warps are independent, so 16 to 24 of them
 // per SM hide each other's latencies.  What bounds it is the L1 and shared-memory pipe, and latency beside it: on a
-// 7x7x3 stem of 64 images (65 us cold) it is busy 61 % of the time, four fifths of that with filter fragments, which every
+// 7x7x3 stem of 64 images (65 us cold) it is busy 61 % of the time, three quarters of that with filter fragments, which every
 // 16-row tile reads anew; the issue slots 47 %, the mma pipe 28 %.
 //
 // There is no kept-row list: a warp walks over 32 output rows at a time, reads their mask bytes, writes the zeros of
