@@ -784,7 +784,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             if (cudaMemsetAsync(L->d_wscnt, 0, ints * sizeof(int), st) != cudaSuccess) return ASX_ERR_CUDA;
         }
     }
-    const int BNsel = use_patch ? pplan.BN : plan.BN;
+    const int BNsel = use_patch ? pplan.BN : plan.pair ? plan.BN / 2 : plan.BN;      // filters of one slab load
     const int Kw = g.K;
     const CUtensorMapDataType tm_type = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const cuuint32_t box_k = (cuuint32_t)(128 / ES);           // one 128-byte swizzled row of K elements

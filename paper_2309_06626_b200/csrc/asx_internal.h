@@ -96,7 +96,8 @@ struct FastPlan {
     int smem_bytes;
     int vec;          // gather mode: 1 cp.async 16 B (a pixel's channels are whole 16-byte chunks), 2 TMA row
                       // gather (they are whole 128-byte runs)
-    int ksplit;       // work items per output tile (shares of the k-blocks), the blocks of a cluster
+    int pair;         // a work item is a pair of blocks on 256 rows, each with its own 128 rows and half of every filter slab
+    int ksplit;       // work items per output tile (shares of the k-blocks), which form a cluster
     long long items;  // m_tiles * n_tiles * ksplit for the estimated kept rows
     int list_bytes;   // shared memory set aside for the fused compaction's list
     double est_cost_us;   // the planner's estimate of the launch's duration

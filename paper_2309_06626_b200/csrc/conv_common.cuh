@@ -46,12 +46,14 @@ struct WaitCtl {
 // (and woken when the phase completes), so waiting warps do not take issue slots from the warps
 // that share their scheduler.  SLEEP_NS is kept as a per-call-site label of how relaxed the
 // waiter may be; it scales the suspend-time hint.
-template <int SLEEP_NS>
+// CLUSTER: threads of another block of the cluster arrive on it too, and what they did before is to be seen.
+template <int SLEEP_NS, bool CLUSTER = false>
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile WaitCtl* ctl, int* dev_status)
 {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity, 20u) : ptx::mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
-    while (!ptx::mbar_try_wait_suspend(bar, parity, 2000u + 10u * SLEEP_NS)) {
+    while (!(CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity, 2000u + 10u * SLEEP_NS)
+                     : ptx::mbar_try_wait_suspend(bar, parity, 2000u + 10u * SLEEP_NS))) {
         if (ctl->abort) return false;
         if (clock64() - t0 > ((long long)ctl->limit_kcycles << 10)) {
             ctl->abort = 1;
@@ -64,11 +66,11 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
 
 // The same wait for a whole converged warp: lane 0 polls, the result is broadcast.  Polling from
 // every lane multiplies the barrier traffic in shared memory by 32 and slows every waiter down.
-template <int SLEEP_NS>
+template <int SLEEP_NS, bool CLUSTER = false>
 __device__ __forceinline__ bool warp_wait_bar(uint32_t bar, uint32_t parity, volatile WaitCtl* ctl, int* dev_status)
 {
     int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = wait_bar<SLEEP_NS>(bar, parity, ctl, dev_status) ? 1 : 0;
+    if ((threadIdx.x & 31) == 0) ok = wait_bar<SLEEP_NS, CLUSTER>(bar, parity, ctl, dev_status) ? 1 : 0;
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 

@@ -112,7 +112,8 @@ enum : int { GATHER_CPASYNC = 1, GATHER_TMA = 2 };
 struct Item {
     int tile, ks, m_tile, n_tile, kb_lo, kb_hi;
 };
-template <bool SPLIT>
+// PAIR: the item belongs to two blocks, tile rows 2 m_tile and 2 m_tile + 1 in units of 128; m_tile is this block's own.
+template <bool SPLIT, bool PAIR>
 __device__ __forceinline__ Item item_of(int t, int KB, const FastArgs& a)
 {
     Item it;
@@ -129,6 +130,7 @@ __device__ __forceinline__ Item item_of(int t, int KB, const FastArgs& a)
     }
     it.m_tile = (int)fd_div((uint32_t)it.tile, a.fdNt);
     it.n_tile = it.tile - it.m_tile * a.n_tiles;
+    if (PAIR) it.m_tile = 2 * it.m_tile + (int)(blockIdx.x & 1);
     return it;
 }
 
@@ -151,8 +153,8 @@ __device__ __forceinline__ int rows_per_tile(int Mk, const FastArgs& a)
 // what was there; a row of the product depends on its own row of the stage alone, and those are not stored.
 __device__ __forceinline__ int gathered_rows(int Mk, int m_tile)
 {
-    const int left = Mk - m_tile * BM;
-    return left < BM ? (left + 3) & ~3 : BM;
+    const int left = Mk - m_tile * BM;                  // the second block of a pair may have none of its last tile
+    return left < BM ? (left > 0 ? (left + 3) & ~3 : 0) : BM;
 }
 
 // What the gather warps need to know about the rk-th kept lowered row: the pixel index of its
@@ -187,7 +189,12 @@ __device__ __forceinline__ int2 row_info_of(int rk, int Mk, const FastDiv& fdcnt
 // F32: x, w and y are fp32 (the storage type of Appendix A); a pipeline stage is still 128 rows of
 // 128 bytes, i.e. 32 K-elements, and the tensor core reads the operands as TF32.
 // SPLIT: a.ksplit > 1 (an instance of its own as well: with the exchange in the plain one every launch took 0.8 us longer).
-template <int MODE, bool IN_COMPACT, bool RESIDUAL, bool SILU, bool F32, bool SPLIT>
+// PAIR: two blocks on two SMs (a cluster) take 256 rows together: each gathers its own 128 and loads half of the filter slab,
+// the first issues the products of both (cta_group::2), and each has its rows' results in its own tensor memory.  A 64-wide k-block of a
+// 128 x 256 tile alone is 16 KB of rows and 32 KB of filters through the SM's TMA unit, one after the other; in a pair it is
+// 16 + 16 KB: 0.51 -> 0.42 us per k-block.  100,352 kept rows at 50 %, 256 -> 256 channels, 3x3: 61.9 -> 52.1 us a launch; at 10 %
+// 89.8 -> 82.9; 512 -> 512 channels at 14x14 (12,544 rows) 70.5 -> 62.4.
+template <int MODE, bool IN_COMPACT, bool RESIDUAL, bool SILU, bool F32, bool SPLIT, bool PAIR>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                          const ConvGeom g, const FastArgs a)
@@ -205,7 +212,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
 
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const int BN = a.BN, S = a.stages;
-    const int stage_bytes = A_STAGE_BYTES + BN * (BK * 2);
+    const int BNB = PAIR ? BN >> 1 : BN;                       // filters of a slab that this block loads
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;         // 0: this block issues the pair's products
+    const int t_first = PAIR ? blockIdx.x >> 1 : blockIdx.x, t_step = PAIR ? gridDim.x >> 1 : gridDim.x;
+    const int stage_bytes = A_STAGE_BYTES + BNB * (BK * 2);
     Shared* sh = reinterpret_cast<Shared*>(smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + S * stage_bytes);
     volatile WaitCtl* abort_flag = &sh->ctl;
 
@@ -230,13 +240,13 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             unsigned long long* bar;
             uint32_t count;
             // full: the filter thread's expect_tx arrival (which in TMA mode also announces the gathered
-            // bytes) + in the copy modes every gather lane's arrival
+            // bytes, of both blocks of a pair on the first one's barrier) + in the copy modes every gather lane's arrival
             if (i < MAX_STAGES) { bar = &sh->full[i]; count = 1 + (MODE == GATHER_TMA ? 0 : GROUP_WARPS * 32); }
             else if ((i -= MAX_STAGES) < MAX_STAGES) { bar = &sh->empty[i]; count = 1; }
             else if ((i -= MAX_STAGES) < INFO_RING) { bar = &sh->info_full[i]; count = 1; }
             else if ((i -= INFO_RING) < INFO_RING) { bar = &sh->info_empty[i]; count = NUM_PROD_WARPS; }    // one arrival per gather warp
             else if ((i -= INFO_RING) < 2) { bar = &sh->acc_full[i]; count = 1; }
-            else { i -= 2; bar = &sh->acc_empty[i]; count = NUM_EPI_WARPS; }
+            else { i -= 2; bar = &sh->acc_empty[i]; count = PAIR ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS; }
             ptx::mbar_init(ptx::smem_u32(bar), count);
             ptx::fence_mbar_init();
         }
@@ -250,8 +260,13 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         }
     }
     if (warp == WARP_MMA) {
-        ptx::tmem_alloc(ptx::smem_u32(&sh->tmem_base), (uint32_t)a.tmem_cols);
-        ptx::tmem_relinquish();
+        if (PAIR) {
+            ptx::tmem_alloc_pair(ptx::smem_u32(&sh->tmem_base), (uint32_t)a.tmem_cols);
+            ptx::tmem_relinquish_pair();
+        } else {
+            ptx::tmem_alloc(ptx::smem_u32(&sh->tmem_base), (uint32_t)a.tmem_cols);
+            ptx::tmem_relinquish();
+        }
     }
     if (warp == WARP_TMA && lane == 0) {
         ptx::prefetch_tensormap(&tmap_w);
@@ -261,7 +276,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = sh->tmem_base;
-    if (SPLIT) ptx::cluster_arrive();        // this block's barrier can take the others' partial sums
+    if (SPLIT || PAIR) ptx::cluster_arrive();        // this block's barriers can take the others' arrivals and partial sums
+
+    // Both blocks of a pair report the bytes of a stage to the first one, which issues the products.
+    const uint32_t pair_full = PAIR ? ptx::cluster_map(ptx::smem_u32(&sh->full[0]), 0u) : 0u;
 
     int cnt = 0;
     KeptList kept_list{a.kept, nullptr};
@@ -284,7 +302,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     // With every position dropped there are no tiles; the zero warps then write the whole output
     // (Algorithm 2, mask == 0 branch).
     const int rpt = MODE == GATHER_CPASYNC && !SPLIT ? rows_per_tile(Mk, a) : BM;
-    const int m_tiles = (Mk + rpt - 1) / rpt;
+    const int m_tiles = PAIR ? (Mk + 2 * BM - 1) / (2 * BM) : (Mk + rpt - 1) / rpt;
     int total_tiles = m_tiles * a.n_tiles * (SPLIT ? a.ksplit : 1);     // work items
     if (SPLIT && total_tiles > a.split_items) {       // cannot happen when the host sized the grid from this mask
         if (tid == 0) atomicOr(a.dev_status, DEV_BAD_INDEX);
@@ -298,14 +316,14 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     {
         for (int idx = tid; idx < INFO_RING * BM; idx += NUM_THREADS) {
             const int jj = idx / BM, rr = idx - jj * BM;
-            const long long t = blockIdx.x + (long long)jj * gridDim.x;
+            const long long t = t_first + (long long)jj * t_step;
             if (t < total_tiles)
-                sh->rowinfo[jj][rr] = row_info_of(rr < rpt ? item_of<SPLIT>((int)t, KB, a).m_tile * rpt + rr : Mk, Mk, fdcnt, g, a, kept_list);
+                sh->rowinfo[jj][rr] = row_info_of(rr < rpt ? item_of<SPLIT, PAIR>((int)t, KB, a).m_tile * rpt + rr : Mk, Mk, fdcnt, g, a, kept_list);
         }
         __syncthreads();
-        if (tid < INFO_RING && blockIdx.x + (long long)tid * gridDim.x < total_tiles) ptx::mbar_arrive(ptx::smem_u32(&sh->info_full[tid]));
+        if (tid < INFO_RING && t_first + (long long)tid * t_step < total_tiles) ptx::mbar_arrive(ptx::smem_u32(&sh->info_full[tid]));
     }
-    if (SPLIT) ptx::cluster_wait();
+    if (SPLIT || PAIR) ptx::cluster_wait();
     // From here on the kernel reads what earlier kernels wrote (the input, the filters) and writes
     // the output and the list, so it waits for them to have finished.
     if (a.fuse_compact) {
@@ -322,15 +340,20 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-                const Item item = item_of<SPLIT>(t, KB, a);
+            for (int t = t_first; t < total_tiles && ok; t += t_step) {
+                const Item item = item_of<SPLIT, PAIR>(t, KB, a);
                 const int n_tile = item.n_tile;
-                const int row_bytes = gathered_rows(Mk, item.m_tile) * BK * 2;
+                const int row_bytes = (gathered_rows(Mk, item.m_tile) + (PAIR ? gathered_rows(Mk, item.m_tile + 1) : 0)) * BK * 2;
                 for (int kb = item.kb_lo; kb < item.kb_hi; ++kb) {
                     if (!wait_bar<40>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
                     const uint32_t full = ptx::smem_u32(&sh->full[s]);
-                    ptx::mbar_arrive_expect_tx(full, (uint32_t)(BN * BK * 2 + (MODE == GATHER_TMA ? row_bytes : 0)));
-                    ptx::tma_load_2d(smem_base + s * stage_bytes + A_STAGE_BYTES, &tmap_w, full, kb * BKE, n_tile * BN);
+                    if (PAIR) {
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full, (uint32_t)(BN * BK * 2 + row_bytes));
+                        ptx::tma_load_2d_pair(smem_base + s * stage_bytes + A_STAGE_BYTES, &tmap_w, pair_full + 8u * s, kb * BKE, n_tile * BN + rank * BNB);
+                    } else {
+                        ptx::mbar_arrive_expect_tx(full, (uint32_t)(BN * BK * 2 + (MODE == GATHER_TMA ? row_bytes : 0)));
+                        ptx::tma_load_2d(smem_base + s * stage_bytes + A_STAGE_BYTES, &tmap_w, full, kb * BKE, n_tile * BN);
+                    }
                     if (++s == S) { s = 0; ph ^= 1u; }
                 }
             }
@@ -343,14 +366,14 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         // Decodes the kept rows of upcoming tiles into the shared-memory ring, four rows per lane,
         // running ahead of the gather warps by up to INFO_RING tiles.
         int j = INFO_RING;                        // the first INFO_RING tiles were decoded by the whole block
-        for (long long t = blockIdx.x + (long long)INFO_RING * gridDim.x; t < total_tiles; t += gridDim.x, ++j) {
+        for (long long t = t_first + (long long)INFO_RING * t_step; t < total_tiles; t += t_step, ++j) {
             const int r = j % INFO_RING;
             int good = 1;
             if (lane == 0)
                 good = wait_bar<200>(ptx::smem_u32(&sh->info_empty[r]), ((uint32_t)(j / INFO_RING) & 1u) ^ 1u, abort_flag, a.dev_status) ? 1 : 0;
             good = __shfl_sync(0xffffffffu, good, 0);
             if (!good) break;
-            const int m_tile = item_of<SPLIT>((int)t, KB, a).m_tile;
+            const int m_tile = item_of<SPLIT, PAIR>((int)t, KB, a).m_tile;
             // the four list entries first (with the list in global memory each is a trip to L2: one after the other
             // they were 2.7 us per tile, which paced every layer with one k-block per tile and a mask too large for
             // the fused compaction), then the arithmetic
@@ -365,24 +388,26 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->info_full[r]));
         }
+    } else if (warp == WARP_MMA && rank != 0) {
+        // the first block of a pair issues the products of both
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issue
         // The whole warp runs the loop so that descriptors and counters stay in uniform registers;
         // one elected lane issues the tcgen05 instructions (issuing from inside a divergent
         // single-lane branch costs about 100 cycles per instruction).
-        const uint32_t idesc = F32 ? ptx::umma_idesc_tf32(BM, BN) : ptx::umma_idesc_bf16(BM, BN);
+        const uint32_t idesc = F32 ? ptx::umma_idesc_tf32(PAIR ? 2 * BM : BM, BN) : ptx::umma_idesc_bf16(PAIR ? 2 * BM : BM, BN);
         const uint64_t adesc0 = ptx::umma_desc_k_major_sw128(smem_base);
         int s = 0, ti = 0;
         uint32_t ph = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++ti) {
+        for (int t = t_first; t < total_tiles && ok; t += t_step, ++ti) {
             const int buf = ti & 1;
             const uint32_t use = (uint32_t)(ti >> 1) & 1u;
-            ok = warp_wait_bar<0>(ptx::smem_u32(&sh->acc_empty[buf]), use ^ 1u, abort_flag, a.dev_status);
+            ok = warp_wait_bar<0, PAIR>(ptx::smem_u32(&sh->acc_empty[buf]), use ^ 1u, abort_flag, a.dev_status);
             if (!ok) break;
             ptx::tc_fence_after_sync();
             const uint32_t d = tmem_base + (uint32_t)(buf * BN);
-            const Item item = item_of<SPLIT>(t, KB, a);
+            const Item item = item_of<SPLIT, PAIR>(t, KB, a);
             for (int kb = item.kb_lo; kb < item.kb_hi; ++kb) {
                 ok = warp_wait_bar<0>(ptx::smem_u32(&sh->full[s]), ph, abort_flag, a.dev_status);
                 if (!ok) break;
@@ -394,23 +419,27 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 const uint64_t adesc = adesc0 + (uint64_t)(s * (stage_bytes >> 4));   // start-address field
                 const uint64_t bdesc = adesc + (A_STAGE_BYTES >> 4);
                 if (ptx::elect_one()) {
-                    if (F32) {                                                          // 8 K-elements = 32 bytes
-                        ptx::umma_tf32(d, adesc, bdesc, idesc, kb != item.kb_lo ? 1u : 0u);
-                        ptx::umma_tf32(d, adesc + 2, bdesc + 2, idesc, 1u);
-                        ptx::umma_tf32(d, adesc + 4, bdesc + 4, idesc, 1u);
-                        ptx::umma_tf32(d, adesc + 6, bdesc + 6, idesc, 1u);
-                    } else {
-                        ptx::umma_bf16(d, adesc, bdesc, idesc, kb != item.kb_lo ? 1u : 0u);       // 16 K-elements = 32 bytes
-                        ptx::umma_bf16(d, adesc + 2, bdesc + 2, idesc, 1u);             //   = 2 descriptor units
-                        ptx::umma_bf16(d, adesc + 4, bdesc + 4, idesc, 1u);
-                        ptx::umma_bf16(d, adesc + 6, bdesc + 6, idesc, 1u);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {          // 32 bytes = 2 descriptor units each: 16 bf16 or 8 fp32 K-elements
+                        const uint32_t acc = i > 0 || kb != item.kb_lo ? 1u : 0u;
+                        if (PAIR) {
+                            if (F32) ptx::umma_tf32_pair(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
+                            else ptx::umma_bf16_pair(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
+                        } else {
+                            if (F32) ptx::umma_tf32(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
+                            else ptx::umma_bf16(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
+                        }
                     }
-                    ptx::umma_commit(ptx::smem_u32(&sh->empty[s]));
+                    if (PAIR) ptx::umma_commit_pair(ptx::smem_u32(&sh->empty[s]), 3);
+                    else ptx::umma_commit(ptx::smem_u32(&sh->empty[s]));
                 }
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (ok && ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&sh->acc_full[buf]));
+            if (ok && ptx::elect_one()) {
+                if (PAIR) ptx::umma_commit_pair(ptx::smem_u32(&sh->acc_full[buf]), 3);
+                else ptx::umma_commit(ptx::smem_u32(&sh->acc_full[buf]));
+            }
             __syncwarp();
         }
     } else if (warp < WARP_PROD0) {
@@ -419,8 +448,8 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         unsigned short* y2 = reinterpret_cast<unsigned short*>(a.y);
         int ti = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++ti) {
-            const Item item = item_of<SPLIT>(t, KB, a);
+        for (int t = t_first; t < total_tiles && ok; t += t_step, ++ti) {
+            const Item item = item_of<SPLIT, PAIR>(t, KB, a);
             const int m_tile = item.m_tile, n_tile = item.n_tile;
             const int n0 = n_tile * BN;
             // kept rows from the accumulator
@@ -604,7 +633,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->acc_empty[buf]));
+            if (lane == 0) {
+                if (PAIR) ptx::mbar_arrive_cluster(ptx::cluster_map(ptx::smem_u32(&sh->acc_empty[buf]), 0u));
+                else ptx::mbar_arrive(ptx::smem_u32(&sh->acc_empty[buf]));
+            }
         }
     } else if (warp >= WARP_ZERO0 && a.out_compact) {
         // a compact output has no dropped rows
@@ -633,7 +665,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 int s = 0, j = 0, it = 0;
                 uint32_t ph = 0;
                 bool ok = true;
-                for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++j) {
+                for (int t = t_first; t < total_tiles && ok; t += t_step, ++j) {
                     const int r = j & (INFO_RING - 1);
                     if (!wait_bar<100>(ptx::smem_u32(&sh->info_full[r]), (uint32_t)(j / INFO_RING) & 1u, abort_flag, a.dev_status)) break;
                     const int2* info = sh->rowinfo[r] + 16 * pwg + 4 * lane;
@@ -642,7 +674,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                     const int pix[4] = {ra.x, ra.z, rb.x, rb.z}, yx[4] = {ra.y, ra.w, rb.y, rb.w};
                     __syncwarp(0xfu);
                     if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->info_empty[r]));    // the ring slot is in registers now
-                    const Item item = item_of<SPLIT>(t, KB, a);
+                    const Item item = item_of<SPLIT, PAIR>(t, KB, a);
                     const bool fetch = 16 * pwg + 4 * lane < gathered_rows(Mk, item.m_tile);
                     int ky = 0, kx = 0, ci = 0;
                     if (item.kb_lo != 0) {                 // a later k share starts inside the window
@@ -686,8 +718,11 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                                 }
                             }
                             if (!wait_bar<20>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
-                            if (fetch) ptx::tma_gather4_2d(smem_base + s * stage_bytes + (uint32_t)(16 * pwg + 4 * lane) * 128u, &tmap_x,
-                                                ptx::smem_u32(&sh->full[s]), ci, idx[0], idx[1], idx[2], idx[3]);
+                            if (fetch) {
+                                const uint32_t dst = smem_base + s * stage_bytes + (uint32_t)(16 * pwg + 4 * lane) * 128u;
+                                if (PAIR) ptx::tma_gather4_2d_pair(dst, &tmap_x, pair_full + 8u * s, ci, idx[0], idx[1], idx[2], idx[3]);
+                                else ptx::tma_gather4_2d(dst, &tmap_x, ptx::smem_u32(&sh->full[s]), ci, idx[0], idx[1], idx[2], idx[3]);
+                            }
                             if (IN_COMPACT && kb + 2 < item.kb_hi) request_ranks(kb + 2);
                         }
                         ci += BKE;                         // next 128 bytes of channels, or the next tap
@@ -713,7 +748,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
             int j = 0;
             uint32_t it0 = 0;                              // k-blocks of the launch before this tile
             bool ok = true;
-            for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++j) {
+            for (int t = t_first; t < total_tiles && ok; t += t_step, ++j) {
                 const int r = j & (INFO_RING - 1);
                 if (!warp_wait_bar<100>(ptx::smem_u32(&sh->info_full[r]), (uint32_t)(j / INFO_RING) & 1u, abort_flag, a.dev_status)) break;
                 const int2* info = sh->rowinfo[r] + 16 * pwg;
@@ -727,7 +762,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->info_empty[r]));    // the ring slot is in registers now
 
-                const Item item = item_of<SPLIT>(t, KB, a);
+                const Item item = item_of<SPLIT, PAIR>(t, KB, a);
                 const int kb0 = item.kb_lo + (int)((it0 ^ (uint32_t)grp) & 1u);          // this group's first k-block of the tile
                 // window position (filter tap, channel) of this lane's chunk in k-block kb0
                 int tap, ci;
@@ -770,15 +805,21 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
     }
 
     ptx::tc_fence_before_sync();
-    __syncthreads();
+    if (PAIR) {                              // neither block gives up memory that the other still works in
+        ptx::cluster_arrive();
+        ptx::cluster_wait();
+    } else {
+        __syncthreads();
+    }
     if (warp == WARP_MMA) {
         __syncwarp();
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
+        if (PAIR) ptx::tmem_dealloc_pair(tmem_base, (uint32_t)a.tmem_cols);
+        else ptx::tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
     }
     // Another share may still send to this block's shared memory when this one has given up a wait.  Every block gets
     // here, because every wait is bounded.
-    if (SPLIT) {
+    if (SPLIT || PAIR) {
         ptx::cluster_arrive_relaxed();
         ptx::cluster_wait();
     }
@@ -944,10 +985,11 @@ int cluster_room(int KS)
     static std::atomic<int> known[DEVICES][9];      // the answer + 1
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= DEVICES) return 0;
-    int room = known[dev][KS].load(std::memory_order_relaxed) - 1;
+    std::atomic<int>& slot = known[dev][KS];
+    int room = slot.load(std::memory_order_relaxed) - 1;
     if (room < 0) {
         constexpr int bytes = 200 * 1024;
-        auto kern = masked_conv_sm100_kernel<GATHER_TMA, false, false, false, false, true>;
+        auto kern = masked_conv_sm100_kernel<GATHER_TMA, false, false, false, false, true, false>;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(KS * 64));
         cfg.blockDim = dim3(NUM_THREADS);
@@ -965,7 +1007,7 @@ int cluster_room(int KS)
             return 0;
         }
         room = clusters * KS;
-        known[dev][KS].store(room + 1, std::memory_order_relaxed);
+        slot.store(room + 1, std::memory_order_relaxed);
     }
     return room;
 }
@@ -979,9 +1021,9 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const int N = g.C_out;
     const int bke = 128 / elem_bytes;             // K elements per stage: 64 bf16 or 32 fp32
     const int KB = (g.K + bke - 1) / bke;
-    const long long m_tiles = (est_kept_rows + BM - 1) / BM > 0 ? (est_kept_rows + BM - 1) / BM : 1;
     if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
     const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
+    auto stage_bytes_of = [](int BN, int pair) { return A_STAGE_BYTES + (pair ? BN / 2 : BN) * BK * 2; };
     auto fixed_bytes = [&](int KS) { return 1024 + (int)(KS > 1 ? sizeof(SharedT<1>) : sizeof(SharedT<PLAIN_INFO_RING>)) + list_bytes; };
     // Tile width and k shares.  A wider tile does more work per gathered byte, a narrower one
     // gives more tiles when a layer has few kept rows, and sharing a tile's k-blocks between the blocks of a
@@ -993,41 +1035,52 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     // and the exchange SPLIT_US (cluster barriers, BN x 512 bytes through distributed shared memory in and out).
     // A shared tile is its block's only one, and clusters that do not all fit at once are not considered (a second wave costs
     // more than sharing gains): the GPU tells how many do (148 blocks in twos, 132 in fours, 120 in eights).
-    int best_BN = 0, best_KS = 1;
+    // Pairs of blocks share tiles of 256 rows where the tiles are 256 wide and there is a wave of them: with narrower ones the row
+    // requests, which a pair does not save, are all that counts (128 and 192 wide: 0-8 % slower than alone), and an item's hand-overs between the
+    // two blocks take longer (1.2 us an item: a 256 -> 256 channel 1x1 layer, four k-blocks an item, 21.4 us alone, 25.0 in pairs).
+    int best_BN = 0, best_KS = 1, best_pair = 0;
     double best_cost = 0.0;
-    const double fill = std::min(1.0, (double)est_kept_rows / (double)(m_tiles * BM));       // rows gathered of a tile's 128
-    int halving = (N + 255) / 256;                // tile widths of whole tiles: 256 or less, then halves
-    for (int n_tiles = halving; ; ++n_tiles) {
-        const int per = (N + n_tiles - 1) / n_tiles;
-        const int BN = ((per + 15) / 16) * 16;
-        const int nt = (N + BN - 1) / BN;
-        const bool whole = n_tiles == halving;
-        if (whole) halving *= 2;
-        for (int KS = whole ? 1 : 2; KS <= (allow_split && KB >= SPLIT_MIN_KB ? 8 : 1); ++KS) {
-            const int gps = (BN / 8 + KS - 1) / KS;
-            if (KS > 1 && (KB / KS < 2 || (KS - 1) * gps >= BN / 8)) continue;       // every share finishes some columns
-            if (227 * 1024 - fixed_bytes(KS) - split_bytes(BN, KS) < MIN_STAGES * (A_STAGE_BYTES + BN * BK * 2)) continue;
-            const long long items = m_tiles * nt * KS;
-            const int room = KS == 1 ? num_sms : cluster_room(KS);
-            if (KS > 1 && items > room) continue;
-            const long long waves = (items + room - 1) / room;
-            const int kbi = (KB + KS - 1) / KS;
-            const double t_kb = 0.12 + 0.18 * fill + 0.001 * BN;                  // microseconds
-            // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
-            const double cost = (double)waves * (kbi * t_kb + 0.3) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
-            if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_cost = cost; }
+    const bool tma = g.C_in % bke == 0;
+    for (int pair = 0; pair <= (tma && num_sms > 1 ? 1 : 0); ++pair) {
+        const long long tile_rows = pair ? 2 * BM : BM;
+        const long long m_tiles = std::max<long long>(1, (est_kept_rows + tile_rows - 1) / tile_rows);
+        const double fill = std::min(1.0, (double)est_kept_rows / (double)(m_tiles * tile_rows));       // rows gathered of a tile's
+        int halving = (N + 255) / 256;                // tile widths of whole tiles: 256 or less, then halves
+        for (int n_tiles = halving; ; ++n_tiles) {
+            const int per = (N + n_tiles - 1) / n_tiles;
+            const int BN = ((per + 15) / 16) * 16;
+            const int nt = (N + BN - 1) / BN;
+            const bool whole = n_tiles == halving;
+            if (whole) halving *= 2;
+            if (pair && BN != 256) break;
+            for (int KS = whole ? 1 : 2; KS <= (allow_split && !pair && KB >= SPLIT_MIN_KB ? 8 : 1); ++KS) {
+                const int gps = (BN / 8 + KS - 1) / KS;
+                if (KS > 1 && (KB / KS < 2 || (KS - 1) * gps >= BN / 8)) continue;       // every share finishes some columns
+                if (227 * 1024 - fixed_bytes(KS) - split_bytes(BN, KS) < MIN_STAGES * stage_bytes_of(BN, pair)) continue;
+                const long long items = m_tiles * nt * KS;
+                const int room = KS == 1 ? (pair ? num_sms / 2 : num_sms) : cluster_room(KS);
+                if (KS > 1 && items > room) continue;
+                const long long waves = (items + room - 1) / room;
+                const int kbi = (KB + KS - 1) / KS;
+                const double t_kb = 0.12 + 0.18 * fill + (pair ? 0.0005 : 0.001) * BN;                  // microseconds
+                // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
+                const double cost = (double)waves * (kbi * t_kb + (pair ? 1.5 : 0.3)) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
+                if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_pair = pair; best_cost = cost; }
+            }
+            if (BN <= 64 && whole) break;
         }
-        if (BN <= 64 && whole) break;
     }
     if (best_BN == 0) return false;
     const int BN = best_BN;
     const int n_tiles = (N + BN - 1) / BN;
-    const int stage_bytes = A_STAGE_BYTES + BN * BK * 2;
+    const int stage_bytes = stage_bytes_of(BN, best_pair);
+    const long long tile_rows = best_pair ? 2 * BM : BM, m_tiles = std::max<long long>(1, (est_kept_rows + tile_rows - 1) / tile_rows);
     int S = (227 * 1024 - fixed_bytes(best_KS) - split_bytes(BN, best_KS)) / stage_bytes;
     if (S > MAX_STAGES) S = MAX_STAGES;
     plan->BN = BN;
     plan->n_tiles = n_tiles;
     plan->ksplit = best_KS;
+    plan->pair = best_pair;
     plan->est_cost_us = best_cost;
     plan->items = (long long)m_tiles * n_tiles * best_KS;
     plan->stages = S;
@@ -1094,37 +1147,42 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
     // Shared k-blocks: one item per block (the host knows the count).  Else as many resident blocks as there may be items.
     const bool split = plan.ksplit > 1;
     const long long least = !split && plan.vec == GATHER_CPASYNC ? MIN_TILE_ROWS : BM;      // rows per tile
-    const long long tiles = split ? plan.items : ((long long)g.M + least - 1) / least * plan.n_tiles;
-    int grid = (int)(split || tiles < num_sms ? tiles : num_sms);
-    if (grid < 1) grid = 1;
+    const bool pair = plan.pair != 0;
+    const int blocks = pair ? 2 : 1;              // of a work item
+    const long long tiles = split ? plan.items : ((long long)g.M + blocks * least - 1) / (blocks * least) * plan.n_tiles;
+    int grid = (split || tiles < num_sms / blocks ? (int)tiles : num_sms / blocks) * blocks;
+    if (grid < blocks) grid = blocks;
     a.fdGrid = make_fastdiv((uint32_t)grid);
     a.mask_from_kernel = mask_from_kernel && !fuse_compact ? 1 : 0;
     const int variant = plan.vec + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
     const bool has_res = residual != nullptr, is_silu = relu == 2;
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const FastArgs);
     Kern kern = nullptr;
-#define ASX_PICK2(MODE, IC, SPLIT)                                                                                              \
-    (has_res ? (is_silu ? masked_conv_sm100_kernel<MODE, IC, true, true, false, SPLIT> : masked_conv_sm100_kernel<MODE, IC, true, false, false, SPLIT>) \
-             : (is_silu ? masked_conv_sm100_kernel<MODE, IC, false, true, false, SPLIT> : masked_conv_sm100_kernel<MODE, IC, false, false, false, SPLIT>))
-#define ASX_PICK_F32(MODE, SPLIT) \
-    (is_silu ? masked_conv_sm100_kernel<MODE, false, false, true, true, SPLIT> : masked_conv_sm100_kernel<MODE, false, false, false, true, SPLIT>)
-#define ASX_PICK(WHICH, ...) kern = split ? WHICH(__VA_ARGS__, true) : WHICH(__VA_ARGS__, false)
+#define ASX_PICK2(MODE, IC, SPLIT, PAIR)                                                                                              \
+    (has_res ? (is_silu ? masked_conv_sm100_kernel<MODE, IC, true, true, false, SPLIT, PAIR> : masked_conv_sm100_kernel<MODE, IC, true, false, false, SPLIT, PAIR>) \
+             : (is_silu ? masked_conv_sm100_kernel<MODE, IC, false, true, false, SPLIT, PAIR> : masked_conv_sm100_kernel<MODE, IC, false, false, false, SPLIT, PAIR>))
+#define ASX_PICK_F32(MODE, SPLIT, PAIR) \
+    (is_silu ? masked_conv_sm100_kernel<MODE, false, false, true, true, SPLIT, PAIR> : masked_conv_sm100_kernel<MODE, false, false, false, true, SPLIT, PAIR>)
+#define ASX_PICK(WHICH, ...) kern = split ? WHICH(__VA_ARGS__, true, false) : WHICH(__VA_ARGS__, false, false)
+#define ASX_PICK_PAIR(WHICH, ...) \
+    if (pair) kern = WHICH(__VA_ARGS__, false, true); else ASX_PICK(WHICH, __VA_ARGS__)
     if (f32) {      // fp32 storage: dense input, no residual
-        if (variant == 2) { ASX_PICK(ASX_PICK_F32, GATHER_TMA); }
+        if (variant == 2) { ASX_PICK_PAIR(ASX_PICK_F32, GATHER_TMA); }
         else { ASX_PICK(ASX_PICK_F32, GATHER_CPASYNC); }
     }
-    else if (variant == 2) { ASX_PICK(ASX_PICK2, GATHER_TMA, false); }
+    else if (variant == 2) { ASX_PICK_PAIR(ASX_PICK2, GATHER_TMA, false); }
     else if (variant == 1) { ASX_PICK(ASX_PICK2, GATHER_CPASYNC, false); }
-    else if (variant == 4) { ASX_PICK(ASX_PICK2, GATHER_TMA, true); }
+    else if (variant == 4) { ASX_PICK_PAIR(ASX_PICK2, GATHER_TMA, true); }
     else { ASX_PICK(ASX_PICK2, GATHER_CPASYNC, true); }
 #undef ASX_PICK2
 #undef ASX_PICK_F32
 #undef ASX_PICK
-    static std::atomic<unsigned long long> smem_set[80];     // per instance
+#undef ASX_PICK_PAIR
+    static std::atomic<unsigned long long> smem_set[160];     // per instance
     const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), MAX_DYN_SMEM,
-                                     smem_set[variant + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0) + (split ? 40 : 0)]);
+                                     smem_set[variant + (has_res ? 5 : 0) + (is_silu ? 10 : 0) + (f32 ? 20 : 0) + (split ? 40 : 0) + (pair ? 80 : 0)]);
     if (e != cudaSuccess) return e;
-    return launch_pdl_cluster(kern, dim3(grid), dim3(NUM_THREADS), plan.ksplit, (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
+    return launch_pdl_cluster(kern, dim3(grid), dim3(NUM_THREADS), pair ? 2 : plan.ksplit, (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
 }
 
 cudaError_t launch_pad_channels(const void* src, void* dst, long long rows, int C, int Cp, cudaStream_t st)

@@ -1,0 +1,77 @@
+"""Tiles that two blocks share in the row gather (256 wide, a wave of them or more): last tiles that the second block has no rows of, or one,
+column counts under 256, more tiles than one wave, and every variant of the kernel; against the library's plain kernel."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2309_06626_b200 as asx
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(cout, kept, f32, per_row, Nb=128, H=14, cin=128):
+    gen = torch.Generator(device="cuda").manual_seed(cout + kept)
+    dt = torch.float32 if f32 else torch.bfloat16
+
+    def values(shape, scale=1.0):
+        t = torch.randn(shape, generator=gen, device="cuda") * scale
+        return (t.view(torch.int32) & ~0x1fff).view(torch.float32) if f32 else t.to(dt)      # fp32: values that TF32 holds exactly
+    rows = Nb * H * H if per_row else H * H
+    mask = np.zeros(rows, np.uint8)
+    mask[np.random.default_rng(kept).permutation(rows)[:kept]] = 1
+    return values((Nb, H, H, cin)), values((cout, 3, 3, cin), (9 * cin) ** -0.5), torch.randn((cout,), generator=gen, device="cuda"), mask
+
+
+# kept lowered rows: one more than whole tiles of 256 (the last has a row for the first block only), a row for the second, whole
+# tiles, a second wave of 74 tiles
+@pytest.mark.parametrize("f32", [False, True], ids=["bf16", "f32"])
+@pytest.mark.parametrize("cout,kept", [(256, 10241), (250, 10240 + 129), (256, 10240), (512, 9600), (241, 18950), (256, 25088)])
+def test_pairs_of_blocks(cout, kept, f32):
+    x, w, b, mask = _problem(cout, kept, f32, per_row=True)
+    layer = asx.MaskedConvLayer(128, cout, 3, 3, 1, 1)
+    layer.set_mask(mask)
+    base = asx.F32 if f32 else 0
+    for act in (asx.ACT_RELU, asx.ACT_SILU):
+        want = layer.run(x, w, b, flags=base | act | asx.IMPL_NAIVE).float().clone()
+        got = layer.run(x, w, b, flags=base | act | asx.IMPL_ROW_GATHER).float()
+        torch.cuda.synchronize()
+        assert layer.device_status() == 0 and layer.last_run_form() == asx.FORM_ROW_GATHER_TMA
+        # bf16: one rounding of the result; fp32: sums of 1152 products in another order
+        assert (got - want).norm() <= (2e-5 if f32 else 5e-3) * want.norm()
+        assert not got.reshape(-1, cout)[torch.from_numpy(mask == 0).cuda()].any()
+    layer.close()
+
+
+@pytest.mark.parametrize("residual", [False, True])
+@pytest.mark.parametrize("act", [asx.ACT_RELU, asx.ACT_SILU])
+def test_pairs_with_compact_tensors(act, residual):
+    """The compact input is the dense one's kept rows, the compact output the dense one's."""
+    Nb, H, cin, cout = 128, 14, 128, 256
+    x, w, b, mask = _problem(cout, 101, False, per_row=False)
+    in_mask = np.zeros(H * H, np.uint8)
+    in_mask[np.random.default_rng(3).permutation(H * H)[:150]] = 1
+    on = torch.from_numpy(in_mask != 0).cuda()
+    xd = (x.reshape(Nb, H * H, cin) * on[None, :, None]).reshape(x.shape).contiguous()
+    xc = xd.reshape(Nb, H * H, cin)[:, on].contiguous()
+    keep = torch.from_numpy(mask != 0).cuda()
+    res = torch.randn((Nb, H, H, cout), device="cuda").to(torch.bfloat16)
+    resc = res.reshape(Nb, H * H, cout)[:, keep].contiguous()
+    layer = asx.MaskedConvLayer(cin, cout, 3, 3, 1, 1)
+    layer.set_mask(mask)
+    layer.set_input_mask(in_mask)
+    st = int(torch.cuda.current_stream().cuda_stream)
+
+    def run(src, dst, shortcut, flags):
+        layer.set_residual(shortcut if residual else None)
+        assert layer.run_raw(src.data_ptr(), Nb, H, H, w.data_ptr(), b.data_ptr(), dst.data_ptr(), act | asx.IMPL_ROW_GATHER | flags, st) == 0
+        torch.cuda.synchronize()
+        assert layer.device_status() == 0 and layer.last_run_form() == asx.FORM_ROW_GATHER_TMA
+        return dst
+    dense = run(xd, torch.empty_like(res), res, 0)
+    z = torch.nn.functional.conv2d(xd.permute(0, 3, 1, 2).double(), w.permute(0, 3, 1, 2).double(), b.double(), padding=1)
+    z = z.permute(0, 2, 3, 1) + (res.double() if residual else 0)
+    want = (z.clamp(min=0) if act == asx.ACT_RELU else z * torch.sigmoid(z)) * keep.reshape(1, H, H, 1)
+    assert (dense.double() - want).norm() <= 5e-3 * want.norm()                      # one rounding to bf16
+    compact = run(xc, torch.empty_like(resc), resc, asx.IN_COMPACT | asx.OUT_COMPACT)
+    assert torch.equal(compact, dense.reshape(Nb, H * H, cout)[:, keep])
+    layer.close()
