@@ -96,11 +96,11 @@ struct FastPlan {
     int smem_bytes;
     int vec;          // gather mode: 1 cp.async 16 B (a pixel's channels are whole 16-byte chunks), 2 TMA row
                       // gather (they are whole 128-byte runs)
-    int pair;         // a work item is a pair of blocks on 256 rows, each with its own 128 rows and half of every filter slab
     int ksplit;       // work items per output tile (shares of the k-blocks), which form a cluster
     long long items;  // m_tiles * n_tiles * ksplit for the estimated kept rows
     int list_bytes;   // shared memory set aside for the fused compaction's list
     double est_cost_us;   // the planner's estimate of the launch's duration
+    int pair = 0;         // a work item is a pair of blocks on 256 rows, each with its own 128 rows and half of every filter slab
 };
 // elem_bytes: 2 (bf16 storage) or 4 (fp32 storage, TF32 contraction)
 bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fused_list_rows, bool allow_split, int elem_bytes,
