@@ -74,6 +74,9 @@ __device__ __forceinline__ bool warp_wait_bar(uint32_t bar, uint32_t parity, vol
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// A value that is the same in every lane of a converged warp, in a form from which the compiler sees that it is.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+
 // S1 inside the fused kernel, for masks of at most 32768 rows: the whole block scans the mask
 // (16 bytes per thread, popcount, shuffle scan within the warps, warp totals through shared
 // memory) and writes the ascending kept positions as 16-bit values into its own shared memory

@@ -392,54 +392,43 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
         // the first block of a pair issues the products of both
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------------------------ MMA issue
-        // The whole warp runs the loop so that descriptors and counters stay in uniform registers;
-        // one elected lane issues the tcgen05 instructions (issuing from inside a divergent
-        // single-lane branch costs about 100 cycles per instruction).
+        // The whole warp runs the loop, and its control flow is the same for all lanes in a way that the compiler sees (counts made uniform,
+        // waits decided by a vote), so that descriptors and counters stay in uniform registers and the products need no branch around
+        // them (ptx::umma says what that is worth).  No lane may run ahead of a wait: a lane that lags behind the issuing one by a
+        // refilled stage finds the barrier two phases on, which a parity cannot tell from none.
         const uint32_t idesc = F32 ? ptx::umma_idesc_tf32(PAIR ? 2 * BM : BM, BN) : ptx::umma_idesc_bf16(PAIR ? 2 * BM : BM, BN);
-        const uint64_t adesc0 = ptx::umma_desc_k_major_sw128(smem_base);
+        const uint32_t a0 = ptx::umma_desc_lo(smem_base), d0 = uniform(tmem_base);
+        const int tiles = (int)uniform((uint32_t)total_tiles);
+        const uint32_t lead = ptx::elect_one() ? 1u : 0u;
+        bool ok = true;
         int s = 0, ti = 0;
         uint32_t ph = 0;
-        bool ok = true;
-        for (int t = t_first; t < total_tiles && ok; t += t_step, ++ti) {
+        for (int t = t_first; t < tiles && ok; t += t_step, ++ti) {
             const int buf = ti & 1;
             const uint32_t use = (uint32_t)(ti >> 1) & 1u;
-            ok = warp_wait_bar<0, PAIR>(ptx::smem_u32(&sh->acc_empty[buf]), use ^ 1u, abort_flag, a.dev_status);
+            ok = __all_sync(0xffffffffu, wait_bar<0, PAIR>(ptx::smem_u32(&sh->acc_empty[buf]), use ^ 1u, abort_flag, a.dev_status));
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            const uint32_t d = tmem_base + (uint32_t)(buf * BN);
+            const uint32_t d = d0 + (uint32_t)(buf * BN);
             const Item item = item_of<SPLIT, PAIR>(t, KB, a);
-            for (int kb = item.kb_lo; kb < item.kb_hi; ++kb) {
-                ok = warp_wait_bar<0>(ptx::smem_u32(&sh->full[s]), ph, abort_flag, a.dev_status);
+            const int kbs = SPLIT ? (int)uniform((uint32_t)(item.kb_hi - item.kb_lo)) : KB;
+            for (int kb = 0; kb < kbs; ++kb) {
+                ok = __all_sync(0xffffffffu, wait_bar<0>(ptx::smem_u32(&sh->full[s]), ph, abort_flag, a.dev_status));
                 if (!ok) break;
                 // Only the cp.async gather writes the stage through the generic proxy without a fence
                 // of its own (TMA writes through the async proxy, the element gather fences after
                 // its stores).
                 if (MODE == GATHER_CPASYNC) ptx::fence_proxy_async_smem();
                 ptx::tc_fence_after_sync();
-                const uint64_t adesc = adesc0 + (uint64_t)(s * (stage_bytes >> 4));   // start-address field
-                const uint64_t bdesc = adesc + (A_STAGE_BYTES >> 4);
-                if (ptx::elect_one()) {
+                const uint32_t al = a0 + (uint32_t)(s * (stage_bytes >> 4)), bl = al + (A_STAGE_BYTES >> 4);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {          // 32 bytes = 2 descriptor units each: 16 bf16 or 8 fp32 K-elements
-                        const uint32_t acc = i > 0 || kb != item.kb_lo ? 1u : 0u;
-                        if (PAIR) {
-                            if (F32) ptx::umma_tf32_pair(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
-                            else ptx::umma_bf16_pair(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
-                        } else {
-                            if (F32) ptx::umma_tf32(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
-                            else ptx::umma_bf16(d, adesc + 2 * i, bdesc + 2 * i, idesc, acc);
-                        }
-                    }
-                    if (PAIR) ptx::umma_commit_pair(ptx::smem_u32(&sh->empty[s]), 3);
-                    else ptx::umma_commit(ptx::smem_u32(&sh->empty[s]));
-                }
+                for (int i = 0; i < 4; ++i)                // 32 bytes of K a step: 16 bf16 or 8 fp32 elements, 2 descriptor units
+                    ptx::umma<F32, PAIR>(lead, d, al + 2 * i, bl + 2 * i, idesc, i > 0 || kb > 0 ? 1u : 0u);
+                ptx::umma_commit<PAIR>(lead, ptx::smem_u32(&sh->empty[s]));
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (ok && ptx::elect_one()) {
-                if (PAIR) ptx::umma_commit_pair(ptx::smem_u32(&sh->acc_full[buf]), 3);
-                else ptx::umma_commit(ptx::smem_u32(&sh->acc_full[buf]));
-            }
+            ptx::umma_commit<PAIR>(ok ? lead : 0u, ptx::smem_u32(&sh->acc_full[buf]));
             __syncwarp();
         }
     } else if (warp < WARP_PROD0) {

@@ -276,50 +276,63 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// The product of a pair, issued by one thread of its first block: 256 rows, of which each block holds 128 in its shared memory
-// and gets those rows' results in its tensor memory, by N filters, of which each block holds half.
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// ---- products, issued by the lanes with lead != 0 (one of the warp)
+// The predicate stands on the instruction itself: in the warp's ordinary control flow, without a branch, every operand stays in uniform
+// registers.  In a branch of one lane, behind a wait that only one lane decides, they did not, and four products with their wait and
+// commit took 590 clocks whatever their width; as they are here, behind a wait decided by a vote, 340 (280 without the wait; 148 SMs,
+// 128 x 64 and 128 x 128 x 64, operands at rest).  An operand's descriptor is its lower word, the upper one is the same for all (UMMA_DESC_HI).
+constexpr uint32_t UMMA_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // of umma_desc_k_major_sw128
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t smem_addr) { return ((smem_addr & 0x3ffffu) >> 4) | (1u << 16); }
+// D[tmem] (+)= A[smem] * B[smem], fp32 accumulate; TF32: fp32 operands read as TF32 (sign, exponent and the upper 10 mantissa bits of
+// each value), 8 K-elements an instruction, else bf16, 16.  PAIR: 256 rows, of which each block of the pair holds 128 in its shared memory and gets those rows' results in
+// its tensor memory, by N filters, of which each block holds half; issued by the first block.
+template <bool TF32, bool PAIR>
+__device__ __forceinline__ void umma(uint32_t lead, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+#define ASX_UMMA(GROUP, KIND)                                                                                               \
+    asm volatile(                                                                                                           \
+        "{\n"                                                                                                              \
+        ".reg .pred p, q;\n"                                                                                               \
+        ".reg .b64 da, db;\n"                                                                                              \
+        "setp.ne.b32 q, %6, 0;\n"                                                                                          \
+        "setp.ne.b32 p, %5, 0;\n"                                                                                          \
+        "mov.b64 da, {%1, %3};\n"                                                                                          \
+        "mov.b64 db, {%2, %3};\n"                                                                                          \
+        "@q tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], da, db, %4, p;\n"                                        \
+        "}\n" ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate), "r"(lead)               \
+        : "memory")
+    if (TF32) {
+        if (PAIR) ASX_UMMA("2", "tf32");
+        else ASX_UMMA("1", "tf32");
+    } else {
+        if (PAIR) ASX_UMMA("2", "f16");
+        else ASX_UMMA("1", "f16");
+    }
+#undef ASX_UMMA
 }
-__device__ __forceinline__ void umma_tf32_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// mbarrier arrive, PAIR: in both blocks of the pair, once every product issued so far by this thread has completed.
+template <bool PAIR>
+__device__ __forceinline__ void umma_commit(uint32_t lead, uint32_t bar)
 {
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if (PAIR)
+        asm volatile(
+            "{\n"
+            ".reg .pred q;\n"
+            "setp.ne.b32 q, %1, 0;\n"
+            "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %2;\n"
+            "}\n" ::"r"(bar), "r"(lead), "h"((uint16_t)3)
+            : "memory");
+    else
+        asm volatile(
+            "{\n"
+            ".reg .pred q;\n"
+            "setp.ne.b32 q, %1, 0;\n"
+            "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+            "}\n" ::"r"(bar), "r"(lead)
+            : "memory");
 }
-// mbarrier arrive, in every block of `blocks` (a bit for each rank of the cluster), once every pair product issued so far has completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t blocks)
-{
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-                 "h"(blocks)
-                 : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate, issued by one thread.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
+// ---- products of the window-patch form, issued from a branch of one lane: with the predicate on the instruction instead its layers took 10 % longer
+// (64 -> 64 channels at 56x56, batch 64: 23.0 against 20.6 us), there the loop waits once per three taps
 // D[tmem] (+)= A[tmem] * B[smem]: the A operand comes from tensor memory (lane = row of the
 // 128-row tile, two bf16 per 32-bit column: 8 columns per K = 16 instruction), B from shared memory.
 __device__ __forceinline__ void umma_bf16_a_tmem(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
@@ -332,20 +345,6 @@ __device__ __forceinline__ void umma_bf16_a_tmem(uint32_t tmem_d, uint32_t tmem_
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
         "}\n" ::"r"(tmem_d),
         "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The same with fp32 operands in shared memory read as TF32 (the tensor core uses the sign, the
-// exponent and the upper 10 mantissa bits of each value); one instruction covers 8 K-elements.
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // mbarrier arrive once every MMA issued so far by this thread has completed.
