@@ -706,8 +706,10 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                                     idx[i] = rn[i] >= 0 ? pix[i] + rn[i] : oob;
                                 }
                             }
-                            if (!wait_bar<20>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
+                            // A lane without rows waits for nothing: the stages do not wait for it either, and once two uses behind it would
+                            // find its phase neither over nor to come.  (A block's later tiles have no more rows for it than this one.)
                             if (fetch) {
+                                if (!wait_bar<20>(ptx::smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, a.dev_status)) { ok = false; break; }
                                 const uint32_t dst = smem_base + s * stage_bytes + (uint32_t)(16 * pwg + 4 * lane) * 128u;
                                 if (PAIR) ptx::tma_gather4_2d_pair(dst, &tmap_x, pair_full + 8u * s, ci, idx[0], idx[1], idx[2], idx[3]);
                                 else ptx::tma_gather4_2d(dst, &tmap_x, ptx::smem_u32(&sh->full[s]), ci, idx[0], idx[1], idx[2], idx[3]);
