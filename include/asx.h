@@ -73,9 +73,12 @@ enum {
                               filter matrices) wherever it can run: dense input and output, a filter matrix that fits
                               in shared memory; where the channels are no whole number of 16-byte chunks, x at a 4-byte
                               address and rows of at most 32000 values, the padding included */
+    ASX_IMPL_ALL_ROWS = 2048, /* take the form that computes the dropped rows too and writes zeros in their place (meant for masks
+                              that drop little, and for channel counts that the other forms handle badly) wherever it can run: dense input
+                              and output, stride up to 8, filters and padding up to 120 */
     ASX_IMPL_DIRECT_K = 1024  /* take the direct form whose warps share a small tile's k range (meant for few kept rows)
                               wherever it can run: dense input and output, C_in a whole number of 16-byte chunks, a mask of
-                              at most 16384 rows from host memory.  At most one of the four form switches
+                              at most 16384 rows from host memory.  At most one of the five form switches
                               (ASX_ERR_INVALID_ARG) */
 };
 
@@ -186,7 +189,7 @@ asx_status asx_recompact(asx_layer* layer, void* cuda_stream);
  *   y    : device, bf16 [Nb][Ho][Wo][C_out], Ho = (H + 2*pad - kh)/stride + 1 (Wo alike);
  *          16-byte aligned when C_out % 8 == 0, else 2-byte; must not overlap x.
  *   flags: OR of ASX_ACT_RELU or ASX_ACT_SILU, ASX_RECOMPACT, ASX_IMPL_NAIVE, ASX_OUT_COMPACT, ASX_IN_COMPACT, ASX_F32,
- *          ASX_IMPL_ROW_GATHER, ASX_IMPL_WINDOW_PATCH, ASX_IMPL_DIRECT or ASX_IMPL_DIRECT_K.
+ *          ASX_IMPL_ROW_GATHER, ASX_IMPL_WINDOW_PATCH, ASX_IMPL_DIRECT, ASX_IMPL_DIRECT_K or ASX_IMPL_ALL_ROWS.
  *          Dropped positions are 0 under every activation (each maps 0 to 0; no bias is added there).  With
  *          ASX_OUT_COMPACT y is bf16 [Nb*P'][C_out] (P' = kept entries of the mask, which must then be
  *          shared by the batch); with ASX_IN_COMPACT x is bf16 [Nb*P'_in][C_in] (see asx_set_input_mask).
@@ -246,10 +249,11 @@ asx_status asx_last_device_status(asx_layer* layer);
  *   filter tap and kept row), ASX_FORM_ROW_GATHER_TMA (TMA row gather per filter tap and kept row),
  *   ASX_FORM_WINDOW_PATCH (a tile's window range loaded once, filter taps cut out of it into tensor memory),
  *   ASX_FORM_DIRECT (operands gathered into registers; small filter matrices),
- *   ASX_FORM_DIRECT_K (the same with a tile's k range shared by the warps of a block; few kept rows).
+ *   ASX_FORM_DIRECT_K (the same with a tile's k range shared by the warps of a block; few kept rows),
+ *   ASX_FORM_ALL_ROWS (every position's window, dropped ones included, by im2col loads).
  * All forms compute the same result up to summation order; this only reports the choice (tests, tuning).
  */
-enum { ASX_FORM_NONE = 0, ASX_FORM_NAIVE = 1, ASX_FORM_ROW_GATHER_COPY = 2, ASX_FORM_ROW_GATHER_TMA = 3, ASX_FORM_WINDOW_PATCH = 4, ASX_FORM_DIRECT = 5, ASX_FORM_DIRECT_K = 6 };
+enum { ASX_FORM_NONE = 0, ASX_FORM_NAIVE = 1, ASX_FORM_ROW_GATHER_COPY = 2, ASX_FORM_ROW_GATHER_TMA = 3, ASX_FORM_WINDOW_PATCH = 4, ASX_FORM_DIRECT = 5, ASX_FORM_DIRECT_K = 6, ASX_FORM_ALL_ROWS = 7 };
 asx_status asx_last_run_form(const asx_layer* layer, int* form);
 
 /*

@@ -11,7 +11,7 @@ _EXT_PATH = os.path.join(_PKG, "_asx_torch.so")
 _lib = None
 _fast = None
 
-ACT_RELU, RECOMPACT, IMPL_NAIVE, OUT_COMPACT, IN_COMPACT, ACT_SILU, F32, IMPL_ROW_GATHER, IMPL_WINDOW_PATCH, IMPL_DIRECT, IMPL_DIRECT_K = 1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024
+ACT_RELU, RECOMPACT, IMPL_NAIVE, OUT_COMPACT, IN_COMPACT, ACT_SILU, F32, IMPL_ROW_GATHER, IMPL_WINDOW_PATCH, IMPL_DIRECT, IMPL_DIRECT_K, IMPL_ALL_ROWS = 1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048
 
 # every symbol include/asx.h declares
 EXPORTS = (
@@ -22,7 +22,7 @@ EXPORTS = (
     "asx_last_run_form", "asx_set_wait_limit", "asx_debug_set_split_counter",
 )
 COMPACT_STATIC_MAX_ROWS = 1 << 24
-FORM_NONE, FORM_NAIVE, FORM_ROW_GATHER_COPY, FORM_ROW_GATHER_TMA, FORM_WINDOW_PATCH, FORM_DIRECT, FORM_DIRECT_K = 0, 1, 2, 3, 4, 5, 6
+FORM_NONE, FORM_NAIVE, FORM_ROW_GATHER_COPY, FORM_ROW_GATHER_TMA, FORM_WINDOW_PATCH, FORM_DIRECT, FORM_DIRECT_K, FORM_ALL_ROWS = 0, 1, 2, 3, 4, 5, 6, 7
 
 
 class AsxError(RuntimeError):

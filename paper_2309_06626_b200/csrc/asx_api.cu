@@ -61,6 +61,19 @@ struct asx_layer {
     const void* tmapx4_ptr = nullptr;
     int tmapx4_Nb = 0, tmapx4_H = 0, tmapx4_W = 0, tmapx4_Wp = 0;
     int tmapx4_px32 = 0;
+    struct Choice {                    // of the form of a call, for the values that it depends on
+        int64_t key[8] = {-1};
+        bool direct = false, direct_k = false, all_rows = false;
+        DirectPlan dplan;
+        DirectKPlan kplan;
+    } choice;
+    struct Im2colKey {                 // what the maps of the all-rows form were made for
+        const void *x = nullptr, *w = nullptr;
+        int geom[18] = {0};
+        bool operator==(const Im2colKey& o) const { return x == o.x && w == o.w && std::memcmp(geom, o.geom, sizeof(geom)) == 0; }
+    };
+    Im2colKey tmap_all_key;
+    CUtensorMap tmap_all_x, tmap_all_w;
     int wait_limit_kcycles = 0;        // bound of the in-kernel waits in units of 1024 cycles (0: the default, about 2 s)
     int last_form = ASX_FORM_NONE;     // producer form of the last asx_run
 };
@@ -83,6 +96,75 @@ EncodeTiledFn encode_tiled_fn()
             fn = reinterpret_cast<EncodeTiledFn>(p);
     }
     return fn;
+}
+
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                   const int*, const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave,
+                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeIm2colFn encode_im2col_fn()
+{
+    static EncodeIm2colFn fn = nullptr;
+    if (fn == nullptr) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &p, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeIm2colFn>(p);
+    }
+    return fn;
+}
+
+// The maps of the all-rows form: x (g.H x g.W pixels of g.C_in channels, `pixel_bytes` apart, `row_bytes` and `image_bytes` per row and
+// image) for loads of 128 window positions, w as [C_out][taps][C_in] with `slab` filters a load.  Channels past g.C_in read zeros
+// in both.
+asx_status map_all_rows(asx_layer* L, const ConvGeom& g, const void* x, const void* w, int ES, const AllRowsPlan& plan, int64_t pixel_bytes,
+                        int64_t row_bytes, int64_t image_bytes)
+{
+    const int slab = plan.pair ? plan.BN / 2 : plan.BN, patch = plan.patch ? plan.pitch : 0;
+    asx_layer::Im2colKey key;
+    key.x = x;
+    key.w = w;
+    const int geom[18] = {g.Nb, g.H, g.W, g.C_in, g.kh, g.kw, g.stride, g.stride_w, g.pad, g.pad_w, g.Ho, g.Wo, g.C_out, ES, slab, (int)pixel_bytes, (int)row_bytes, patch};
+    std::memcpy(key.geom, geom, sizeof(geom));
+    if (key == L->tmap_all_key) return ASX_OK;
+    EncodeTiledFn tiled = encode_tiled_fn();
+    EncodeIm2colFn im2col = patch ? nullptr : encode_im2col_fn();
+    if (tiled == nullptr || (!patch && im2col == nullptr)) return ASX_ERR_CUDA;
+    const CUtensorMapDataType type = ES == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const cuuint32_t channels = (cuuint32_t)(plan.rb / ES), ones[4] = {1u, 1u, 1u, 1u};
+    L->tmap_all_key = asx_layer::Im2colKey();
+    const CUtensorMapSwizzle swizzle = plan.rb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : plan.rb == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+    if (patch) {
+        const cuuint64_t pixels = (cuuint64_t)g.Nb * g.H * g.W;
+        const cuuint64_t dims[4] = {(cuuint64_t)g.C_in, plan.flat ? pixels : (cuuint64_t)g.W, plan.flat ? 1u : (cuuint64_t)g.H, plan.flat ? 1u : (cuuint64_t)g.Nb};
+        const cuuint64_t strides[3] = {(cuuint64_t)pixel_bytes, plan.flat ? pixels * pixel_bytes : (cuuint64_t)row_bytes,
+                                       plan.flat ? pixels * pixel_bytes : (cuuint64_t)image_bytes};
+        const cuuint32_t box[4] = {channels, (cuuint32_t)patch, 1u, 1u};
+        if (tiled(&L->tmap_all_x, type, 4, const_cast<void*>(x), dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return ASX_ERR_CUDA;
+    } else {
+        const cuuint64_t dims[4] = {(cuuint64_t)g.C_in, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.Nb};
+        const cuuint64_t strides[3] = {(cuuint64_t)pixel_bytes, (cuuint64_t)row_bytes, (cuuint64_t)image_bytes};
+        // the window corners of a row lie at lower, lower + stride .. extent - 1 + upper
+        const int lower[2] = {-g.pad_w, -g.pad};
+        const int upper[2] = {(g.Wo - 1) * g.stride_w - g.pad_w - (g.W - 1), (g.Ho - 1) * g.stride - g.pad - (g.H - 1)};
+        const cuuint32_t step[4] = {1u, (cuuint32_t)g.stride_w, (cuuint32_t)g.stride, 1u};
+        if (im2col(&L->tmap_all_x, type, 4, const_cast<void*>(x), dims, strides, lower, upper, channels, 128u, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return ASX_ERR_CUDA;
+    }
+    {
+        const cuuint64_t dims[3] = {(cuuint64_t)g.C_in, (cuuint64_t)(g.kh * g.kw), (cuuint64_t)g.C_out};
+        const cuuint64_t strides[2] = {(cuuint64_t)g.C_in * ES, (cuuint64_t)g.K * ES};
+        const cuuint32_t box[3] = {channels, 1u, (cuuint32_t)slab};
+        if (tiled(&L->tmap_all_w, type, 3, const_cast<void*>(w), dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return ASX_ERR_CUDA;
+    }
+    L->tmap_all_key = key;
+    return ASX_OK;
 }
 
 asx_status from_cuda(cudaError_t e)
@@ -432,8 +514,8 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
 {
     if (L == nullptr || x == nullptr || w == nullptr || y == nullptr) return ASX_ERR_INVALID_ARG;
     if (Nb < 1 || H < 1 || W < 1) return ASX_ERR_INVALID_ARG;
-    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K)) return ASX_ERR_INVALID_ARG;
-    if (((flags & ASX_IMPL_ROW_GATHER) != 0) + ((flags & ASX_IMPL_WINDOW_PATCH) != 0) + ((flags & ASX_IMPL_DIRECT) != 0) + ((flags & ASX_IMPL_DIRECT_K) != 0) > 1) return ASX_ERR_INVALID_ARG;
+    if (flags & ~(ASX_ACT_RELU | ASX_RECOMPACT | ASX_IMPL_NAIVE | ASX_OUT_COMPACT | ASX_IN_COMPACT | ASX_ACT_SILU | ASX_F32 | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K | ASX_IMPL_ALL_ROWS)) return ASX_ERR_INVALID_ARG;
+    if (((flags & ASX_IMPL_ROW_GATHER) != 0) + ((flags & ASX_IMPL_WINDOW_PATCH) != 0) + ((flags & ASX_IMPL_DIRECT) != 0) + ((flags & ASX_IMPL_DIRECT_K) != 0) + ((flags & ASX_IMPL_ALL_ROWS) != 0) > 1) return ASX_ERR_INVALID_ARG;
     const bool f32 = (flags & ASX_F32) != 0;
     const int ES = f32 ? 4 : 2;                 // bytes per element of x, w and y
     const int EPC = 16 / ES;                    // elements per 16-byte chunk
@@ -505,34 +587,58 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     const int relu = (flags & ASX_ACT_SILU) ? 2 : (flags & ASX_ACT_RELU) ? 1 : 0;      // activation code: 0 identity, 1 ReLU, 2 SiLU
     // Small filter matrices take the direct form, which needs no list and rebuilds it beside the convolution when asked to;
     // few kept rows the direct form whose warps share the k range.
-    const int impl = flags & (ASX_IMPL_NAIVE | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K);
+    const int impl = flags & (ASX_IMPL_NAIVE | ASX_IMPL_ROW_GATHER | ASX_IMPL_WINDOW_PATCH | ASX_IMPL_DIRECT | ASX_IMPL_DIRECT_K | ASX_IMPL_ALL_ROWS);
     const int64_t known_rows = L->host_kept < 0 ? -1 : L->rows == P ? L->host_kept * Nb : L->host_kept;      // kept lowered rows, when the host knows
     const bool recompact = (flags & ASX_RECOMPACT) != 0, dense = !in_compact && !out_compact;
-    DirectPlan dplan;
-    DirectKPlan kplan;
-    // Its word form reads x in 4-byte words.  An x that lies between two words (allowed where the channels are no whole
-    // 16-byte chunks) takes the padded copy of the other forms.
-    const bool direct = dense && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) &&
-                        (dplan.words == 0 || (reinterpret_cast<uintptr_t>(x) & 3) == 0) &&
-                        (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, known_rows < 0 ? M : known_rows));
-    bool direct_k = dense && (impl == 0 || impl == ASX_IMPL_DIRECT_K) && plan_direct_k(g, ES, known_rows, L->num_sms, &kplan);
-    if (direct_k && impl == 0) {
-        // against what would run else: the estimates of a tensor-memory form leave out 4.5 us of a launch's set-up and ends
-        double other;
-        if (direct) {
-            other = direct_est_us(dplan, L->num_sms, known_rows, ES);
-        } else {
+    // The choice between the direct forms and the others depends on these values alone; it is kept for the next call with the same ones
+    // (working it out takes 0.6 us, a fifth of the smallest call).
+    const bool x_in_words = (reinterpret_cast<uintptr_t>(x) & 3) == 0;         // the direct form's words: see below
+    const int64_t choice_key[8] = {Nb, H, W, flags & (ASX_F32 | ASX_RECOMPACT | ASX_IN_COMPACT | ASX_OUT_COMPACT), impl, known_rows, L->rows, x_in_words};
+    asx_layer::Choice& choice = L->choice;
+    if (std::memcmp(choice.key, choice_key, sizeof(choice_key)) != 0) {
+        DirectPlan& dplan = choice.dplan;
+        DirectKPlan& kplan = choice.kplan;
+        // Its word form reads x in 4-byte words.  An x that lies between two words (allowed where the channels are no whole
+        // 16-byte chunks) takes the padded copy of the other forms.
+        bool direct = dense && (impl == 0 || impl == ASX_IMPL_DIRECT) && plan_direct(g, ES, &dplan) && (dplan.words == 0 || x_in_words) &&
+                      (impl == ASX_IMPL_DIRECT || direct_pays(dplan, L->num_sms, known_rows < 0 ? M : known_rows));
+        bool direct_k = dense && (impl == 0 || impl == ASX_IMPL_DIRECT_K) && plan_direct_k(g, ES, known_rows, L->num_sms, &kplan);
+        bool all_rows = impl == ASX_IMPL_ALL_ROWS;
+        if (impl == 0 && dense) {
+            // What the forms that compute every row and kept rows through tensor memory would take, where the call's own channels suit them.
+            // The estimates leave out 4.5 us of a launch's set-up and ends.  A mask that the host does not know may drop
+            // anything: no call for computing every row.
             FastPlan fp;
-            PatchPlan pp;
-            other = plan_fast(g, L->num_sms, known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp) ? fp.est_cost_us : 1e9;
-            if (!f32 && plan_patch(g, recompact && L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
-                plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, false, &pp);
-                other = std::min(other, pp.est_cost_us);
+            const bool fast = plan_fast(g, L->num_sms, known_rows < 0 ? M : known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp);
+            const double all_rows_us = fast && vec_in && known_rows >= 0 && fp.all.BN > 0 ? fp.all.est_cost_us + 4.5 : 1e9;
+            if (direct && all_rows_us < 0.9 * direct_est_us(dplan, L->num_sms, known_rows, ES)) {
+                direct = false;
+                all_rows = true;
             }
-            other += 4.5;
+            if (direct_k) {
+                double other;
+                if (direct) {
+                    other = direct_est_us(dplan, L->num_sms, known_rows, ES);
+                } else {
+                    PatchPlan pp;
+                    other = fast ? fp.est_cost_us : 1e9;
+                    if (!f32 && plan_patch(g, recompact && L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, 0, &pp)) {
+                        plan_patch_cost(g, L->num_sms, (known_rows + 127) / 128, false, &pp);
+                        other = std::min(other, pp.est_cost_us);
+                    }
+                    other = std::min(other + 4.5, all_rows_us);
+                }
+                direct_k = kplan.est_us < 0.95 * other;
+            }
         }
-        direct_k = kplan.est_us < 0.95 * other;
+        choice.direct = direct;
+        choice.direct_k = direct_k;
+        choice.all_rows = all_rows;
+        std::memcpy(choice.key, choice_key, sizeof(choice_key));
     }
+    const bool direct = choice.direct, direct_k = choice.direct_k, all_rows = choice.all_rows;
+    const DirectPlan& dplan = choice.dplan;
+    const DirectKPlan& kplan = choice.kplan;
     if (direct_k) {
         L->last_form = ASX_FORM_DIRECT_K;
         return launched(launch_direct_k(g, kplan, x, w, bias, y, L->d_mask, recompact ? L->d_kept : nullptr, L->d_small, L->host_kept, relu, L->residual,
@@ -773,6 +879,26 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             plan_patch_cost(gp, L->num_sms, (long long)(L->host_tiles.size() / 4), in_compact, &pplan);
             use_patch = pplan.est_cost_us <= plan.est_cost_us || (flags & ASX_IMPL_WINDOW_PATCH);
         }
+    }
+    // Every row, where that is estimated to be a good deal faster than the kept ones by either other way: it keeps the tensor cores busier, and
+    // under the power cap their clock falls (256 -> 256 channels 3x3 with 10 % dropped: 84 us in short runs against 82 gathered, 106 against 95 in long ones).
+    if (dense && plan.all.BN > 0 &&
+        (all_rows || (impl == 0 && known_rows >= 0 && plan.all.est_cost_us < 0.85 * (use_patch ? std::min(plan.est_cost_us, pplan.est_cost_us) : plan.est_cost_us)))) {
+        ConvGeom ga = g;
+        if (blocks2x2) {                                          // the window positions of the staged copy: runs of four blocks
+            ga.H = g.Ho + g.kh - 1;
+            ga.W = g.Wo;
+        }
+        const int64_t pixel = x_row_stride ? x_row_stride : (int64_t)g.C_in * ES;
+        s = map_all_rows(L, ga, xsrc, wsrc, ES, plan.all, pixel, pixel * g.W, pixel * g.W * g.H);
+        if (s != ASX_OK) return s;
+        plan.use_all = 1;
+        L->last_form = ASX_FORM_ALL_ROWS;
+        const bool write_list = fuse_compact && recompact, waits = mask_from_kernel == 2 && !write_list;
+        if (waits) launch_in_stream_order = false;
+        return launched(launch_fast(ga, plan, L->tmap_all_w, L->tmap_all_x, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
+                                    L->num_sms, 0, write_list ? 1 : 0, L->host_kept, nullptr, 0, nullptr, 0, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
+                                    waits ? 1 : 0, st), waits ? 1 : 0);
     }
     if (plan.ksplit > 1 && !use_patch) {
         const size_t ints = 2 * (size_t)(plan.items / plan.ksplit);

@@ -88,7 +88,30 @@ cudaError_t launch_naive(const ConvGeom& g, const void* x, const void* w, const 
                          const uint8_t* mask, const int32_t* kept, const int32_t* count, int relu, int f32,
                          cudaStream_t st);
 
-// ---- the tensor-core path (masked_conv_sm100.cu)
+// ---- the tensor-core path
+// Every row of the lowered matrix, dropped ones included (masked_conv_all_rows_sm100.cu): dense input and output
+struct AllRowsPlan {
+    int BN = 0, n_tiles = 0;   // BN 0: the geometry does not take this form
+    int pair = 0;              // two blocks share tiles of 256 rows and their filter slabs
+    int patch = 0;             // operand rows from patches of the input (stride 1), else from im2col loads
+    int rb = 128;              // bytes of a slice of the channels (128, 64 or 32)
+    int nc = 0, tail_steps = 0;      // slices, 32-byte steps of the last one
+    int a_bufs = 0, a_bytes = 0, b_slots = 0, G = 1, resident = 0;
+    int strips = 0, width = 0, pitch = 0, tiles = 0;      // patches: strips per image, their columns, positions per row in a patch, tiles per strip
+    int flat = 0;              // patches: a 1x1 layer, the strips are runs of positions
+    int items = 0;             // work items of a block or pair
+    int epi_groups = 2;        // groups of epilogue warps at work
+    int smem_bytes = 0;
+    double est_cost_us = 0;
+};
+bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* plan);
+// tmap_w: w as [C_out][taps][C_in], box (128 bytes of channels, 1, the filters of one slab load); tmap_x: x for im2col loads of 128
+// positions.  kept_out, count_out: where the kept-row list goes too, or null
+cudaError_t launch_all_rows(const ConvGeom& g, const AllRowsPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x, const float* bias,
+                            void* y, const uint8_t* mask, int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32,
+                            int* dev_status, int num_sms, int mask_from_kernel, int wait_limit_kcycles, cudaStream_t st);
+
+// Kept rows only, gathered (masked_conv_sm100.cu)
 struct FastPlan {
     int BN;           // UMMA N per tile (multiple of 16, <= 256)
     int n_tiles;      // ceil(C_out / BN)
@@ -101,6 +124,8 @@ struct FastPlan {
     int list_bytes;   // shared memory set aside for the fused compaction's list
     double est_cost_us;   // the planner's estimate of the launch's duration
     int pair = 0;         // a work item is a pair of blocks on 256 rows, each with its own 128 rows and half of every filter slab
+    AllRowsPlan all;      // the same call with every row computed
+    int use_all = 0;      // and whether it is run so (the caller's choice)
 };
 // elem_bytes: 2 (bf16 storage) or 4 (fp32 storage, TF32 contraction)
 bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fused_list_rows, bool allow_split, int elem_bytes,

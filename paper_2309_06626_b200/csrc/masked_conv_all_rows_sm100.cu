@@ -1,0 +1,740 @@
+// S2 + S3 + S4 with every row of the lowered matrix computed: the all-rows form of the masked convolution.
+//
+// The other forms build the operand rows of kept windows only, row by row: a gathered row of 128 bytes costs an SM's TMA unit about
+// five clocks, a row cut out of a window patch its share of the shared-memory port.  The windows of 128 CONSECUTIVE output
+// positions, dropped or not, need no such work, so where little is dropped this form computes the dropped rows too and writes zeros in their place:
+//
+//   patches (stride 1)  the input rows under 128 positions are loaded once per 64-channel slice, in whole rows, and every filter tap reads
+//                       its operand rows straight from the patch: position p's window lies (ky pitch + kx) positions further, and an operand
+//                       may start at any row of it.  Nothing is cut out or copied: four products of a 128 x 64 tile in 250 clocks.
+//   im2col (strides)    the im2col mode of the TMA unit loads one tap of 128 positions, over row and image ends, at the row gather's rate
+//                       (0.36 us a k-block); it has no use for the kept-row list and takes any channel count that is whole 16-byte chunks.
+//
+//   load threads     one for the input, one for the filter slabs, which stay in shared memory where they fit beside the patches
+//   issuing warps    two, which take the tiles in turn; with PAIR two blocks on two SMs share tiles of 256 positions, each with its own 128 and
+//                    half of the filter slab
+//   epilogue warps   two or four groups of four, which take the tiles in turn: bias, shortcut, activation, zeros for dropped rows; each warp passes
+//                    32 rows of 64 bytes through shared memory, so that every store is of whole neighbouring pieces, also where a row's
+//                    channels are no whole number of 16-byte chunks (the other tensor-memory forms store those value by value)
+//
+// Bound by the tensor core's reads of the operands and the issue (64 to 128 channels), the tensor core (256), the way out (1x1 layers).
+// Measured on layers inside a graph, before -> with this form: 64 -> 64 channels 3x3 at 56x56, batch 64, 10 % dropped 30.8 -> 22.3 us; 256 -> 256
+// at 14x14, 20 % 22.1 -> 18.5; fp32 128 -> 128 at 28x28, batch 16, 50 % 16.4 -> 14.4; 1x1 128 -> 128 at 80x80, batch 16, 40 % 18.2 -> 14.7;
+// 16 -> 286 3x3 at 80x80, batch 117, 60 % 1082 -> 256; 1x1 stride 2 272 -> 279, batch 97 330 -> 54.
+#include <algorithm>
+#include <atomic>
+#include <cuda_bf16.h>
+#include "asx_internal.h"
+#include "ptx_sm100.cuh"
+#include "conv_common.cuh"
+
+namespace asx {
+
+namespace {
+
+constexpr int BM = 128;                                 // output positions per block and tile (UMMA M of a block)
+constexpr int A_BYTES = BM * 128;                       // a stage: 128 rows of 128 swizzled bytes
+constexpr int MAX_STAGES = 8, MIN_STAGES = 3, MAX_ACC = 4;
+constexpr int WARP_LOAD = 0, WARP_MMA = 1, WARP_FILTERS = 2, WARP_MMA2 = 3, WARP_EPI0 = 4, EPI_GROUPS = 4;
+constexpr int LIST_WARPS = 4, WARP_LIST0 = WARP_EPI0 + 4 * EPI_GROUPS - LIST_WARPS;      // the last group
+constexpr int NUM_THREADS = 32 * (WARP_EPI0 + 4 * EPI_GROUPS);
+constexpr int STAGING_PITCH = 64 + 16;                  // bytes of a row in a warp's staging area: 16-byte accesses of neighbouring rows meet other banks
+constexpr int STAGING_GROUP = 4 * 32 * STAGING_PITCH;   // a group of epilogue warps
+
+struct AllRowsArgs {
+    FastDiv fdP, fdWo, fdNt;        // divisions by P, Wo and n_tiles
+    const float* bias;
+    void* y;
+    const uint8_t* mask;
+    const __nv_bfloat16* residual;
+    int* dev_status;
+    int32_t* kept_out;              // non-null: the kept-row list and its count are written too
+    int32_t* count_out;
+    int act;                        // 0 identity, 1 ReLU, 2 SiLU
+    int BN, n_tiles, items;
+    int a_bufs, a_bytes;            // operand buffers: a k-block's 128 rows, or (patches) a 64-channel slice of the tile's input rows
+    int b_slots, G, resident;       // groups of filter slabs, slabs a group (taps of one slice); resident: every k-block's, one a group, loaded once
+    int rb;                         // bytes of a slice of the channels: 128, or what fewer channels need
+    int nc, steps, tail_steps;      // slices; MMA steps (32 bytes of channels) of one, of the last one
+    FastDiv fdA, fdB;               // by a_bufs and b_slots
+    uint32_t a_uses, b_uses;        // operand buffers and groups of slabs that a tile takes
+    // patches: the output is cut into strips of `width` columns of an image, `strips` per image.  A strip's positions lie `pitch` to an output row in the
+    // patch, and `tiles` runs of 128 of them cover it.
+    FastDiv fdStrips, fdTiles, fdPitch;
+    int width, Ho, Wo, P, strips_all;
+    int acc_log2, tmem_cols;
+    int epi_groups;                 // groups of epilogue warps at work: four where a tile's products take less than its rows' way out, else two
+    int vec_out;                    // rows of y are whole 16-byte chunks
+    int y_half;                     // y (bf16) starts between two words
+    int mask_from_kernel;           // the mask was written by a kernel that may still be running
+    int wait_limit_kcycles;
+};
+
+struct alignas(16) Shared {
+    float bias[EPI_GROUPS * 4][32];        // of the columns that an epilogue warp is at
+    unsigned long long a_full[MAX_STAGES], a_empty[MAX_STAGES], b_full[MAX_STAGES], b_empty[MAX_STAGES];
+    unsigned long long acc_full[MAX_ACC], acc_empty[MAX_ACC];
+    unsigned long long turn[2];     // of the two issuing warps
+    unsigned int tmem_base;
+    WaitCtl ctl;
+    int list_total[2][LIST_WARPS];
+};
+
+// One work item of this block: 128 positions by BN columns.
+struct Item {
+    int n_tile;
+    int first;                      // im2col: the first output row; patches: the first position, counted in the strip
+    int image, x0;                  // patches: the strip's image and its first output column
+    bool any, other;                // this block has positions in it; (first block of a pair) the second block has
+};
+template <bool PATCH, bool PAIR>
+__device__ __forceinline__ Item item_of(int t, const ConvGeom& g, const AllRowsArgs& a, int rank)
+{
+    Item it;
+    const int u = (int)fd_div((uint32_t)t, a.fdNt);
+    it.n_tile = t - u * a.n_tiles;
+    it.image = it.x0 = 0;
+    if (PATCH) {
+        const int group = (int)fd_div((uint32_t)u, a.fdTiles), strip = PAIR ? 2 * group + rank : group;
+        it.first = (u - group * (int)a.fdTiles.d) * BM;
+        it.image = (int)fd_div((uint32_t)strip, a.fdStrips);
+        it.x0 = (strip - it.image * (int)a.fdStrips.d) * a.width;
+        it.any = strip < a.strips_all;
+        it.other = strip + 1 < a.strips_all;
+    } else {
+        it.first = (PAIR ? 2 * u + rank : u) * BM;
+        it.any = it.first < g.M;
+        it.other = it.first + BM < g.M;
+    }
+    return it;
+}
+
+// Where an issuing warp stands in the rings of operand buffers and of groups of filter slabs.
+struct Rings {
+    uint32_t a, a_phase, b, b_phase;
+};
+enum : int { RESIDENT = 0, FILTER_ROWS = 1, TAPS = 2 };      // slabs waited for once a launch, once a filter row, for every tap
+// The products of one slice of the channels.  One loop for each way the slabs come, without a condition in it: with the three in one
+// loop four products took 490 clocks, like this 250 (64 -> 64 channels 3x3 at 56x56, batch 64: 45.0 -> 25.2 us).
+template <bool F32, bool PAIR, bool PATCH, int GROUPS, int STEPS>
+__device__ __forceinline__ bool issue_slice(Rings& r, uint32_t lead, uint32_t d, uint32_t a0, uint32_t b0, uint32_t idesc, uint32_t started, int steps,
+                                            const ConvGeom& g, const AllRowsArgs& a, Shared* sh, volatile WaitCtl* ctl)
+{
+    const uint32_t rb16 = (uint32_t)a.rb >> 4, b_step = (uint32_t)(PAIR ? a.BN >> 1 : a.BN) * rb16, a_step = (uint32_t)a.a_bytes >> 4;
+    const uint32_t row_step = PATCH ? a.fdPitch.d * rb16 : 0u, hi = ptx::umma_desc_hi((uint32_t)a.rb);
+    auto wait = [&](unsigned long long* bars, uint32_t i, uint32_t phase) {
+        const bool ok = __all_sync(0xffffffffu, wait_bar<0>(ptx::smem_u32(&bars[i]), phase, ctl, a.dev_status));
+        ptx::tc_fence_after_sync();
+        return ok;
+    };
+    auto next_a = [&]() {
+        ptx::umma_commit<PAIR>(lead, ptx::smem_u32(&sh->a_empty[r.a]));
+        if (++r.a == (uint32_t)a.a_bufs) { r.a = 0; r.a_phase ^= 1u; }
+    };
+    auto next_b = [&]() {
+        ptx::umma_commit<PAIR>(lead, ptx::smem_u32(&sh->b_empty[r.b]));
+        if (++r.b == (uint32_t)a.b_slots) { r.b = 0; r.b_phase ^= 1u; }
+    };
+    if (PATCH && !wait(sh->a_full, r.a, r.a_phase)) return false;
+    // a position's window lies ky pitch + kx positions further for every tap: the rows that the tensor core reads may start
+    // anywhere, as the swizzle follows the address
+    uint32_t at = a0 + r.a * a_step;
+    uint32_t bl = GROUPS == RESIDENT ? b0 + r.b * b_step : 0u;
+    for (int ky = 0; ky < g.kh; ++ky, at += row_step) {
+        if (GROUPS == FILTER_ROWS) {
+            if (!wait(sh->b_full, r.b, r.b_phase)) return false;
+            bl = b0 + r.b * (uint32_t)a.G * b_step;
+        }
+        uint32_t ax = at;
+#pragma unroll 1
+        for (int kx = 0; kx < g.kw; ++kx, ax += rb16, bl += b_step) {
+            if (GROUPS == TAPS) {
+                if (!wait(sh->b_full, r.b, r.b_phase)) return false;
+                bl = b0 + r.b * b_step;
+            }
+            if (!PATCH) {
+                if (!wait(sh->a_full, r.a, r.a_phase)) return false;
+                ax = a0 + r.a * a_step;
+            }
+            if (STEPS > 0) {
+#pragma unroll
+                for (int k = 0; k < STEPS; ++k)    // 32 bytes of channels a step = 2 descriptor units
+                    ptx::umma<F32, PAIR>(lead, d, ax + 2 * k, bl + 2 * k, hi, idesc, k > 0 ? 1u : started);
+            } else {
+                for (int k = 0; k < steps; ++k) ptx::umma<F32, PAIR>(lead, d, ax + 2 * k, bl + 2 * k, hi, idesc, k > 0 ? 1u : started);
+            }
+            started = 1;
+            if (!PATCH) next_a();
+            if (GROUPS == TAPS) next_b();
+        }
+        if (GROUPS == FILTER_ROWS) next_b();
+    }
+    if (PATCH) next_a();
+    if (GROUPS == RESIDENT) r.b += (uint32_t)(g.kh * g.kw);
+    __syncwarp();
+    return true;
+}
+
+// PATCH: the operand rows are read from patches of the input, else from im2col loads.
+template <bool F32, bool RESIDUAL, bool PAIR, bool PATCH>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+masked_conv_all_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const ConvGeom g,
+                            const AllRowsArgs a)
+{
+    constexpr int ES = F32 ? 4 : 2, COLS = 64 / ES;      // columns that a warp takes at a time
+    extern __shared__ uint8_t smem_raw[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (the next kernel may read the mask before its own wait, so while a kernel is still writing that, not yet)
+    if (!a.mask_from_kernel) ptx::grid_launch_dependents();
+
+    const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+    const int BN = a.BN, BNB = PAIR ? BN >> 1 : BN;
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;               // of a pair: 0 issues the products
+    const int t_first = PAIR ? blockIdx.x >> 1 : blockIdx.x, t_step = PAIR ? gridDim.x >> 1 : gridDim.x;
+    const uint32_t b_bytes = (uint32_t)(BNB * a.rb), b_base = smem_base + (uint32_t)(a.a_bufs * a.a_bytes);
+    uint8_t* const after = smem_raw + (smem_base - ptx::smem_u32(smem_raw)) + a.a_bufs * a.a_bytes + a.b_slots * a.G * b_bytes;
+    Shared* sh = reinterpret_cast<Shared*>(after + a.epi_groups * STAGING_GROUP);
+    volatile WaitCtl* ctl = &sh->ctl;
+
+    {
+        constexpr int NB = 4 * MAX_STAGES + 2 * MAX_ACC + 2;
+        int i = tid - (NUM_THREADS - NB);
+        if (i >= 0) {
+            unsigned long long* bar;
+            uint32_t count = 1;
+            if (i < MAX_STAGES) bar = &sh->a_full[i];
+            else if ((i -= MAX_STAGES) < MAX_STAGES) bar = &sh->a_empty[i];
+            else if ((i -= MAX_STAGES) < MAX_STAGES) bar = &sh->b_full[i];
+            else if ((i -= MAX_STAGES) < MAX_STAGES) bar = &sh->b_empty[i];
+            else if ((i -= MAX_STAGES) < MAX_ACC) bar = &sh->acc_full[i];
+            else if ((i -= MAX_ACC) < MAX_ACC) { bar = &sh->acc_empty[i]; count = (PAIR ? 8u : 4u) * (uint32_t)(a.epi_groups > 1 << a.acc_log2 ? 2 : 1); }       // the warps that serve it, of both blocks
+            else bar = &sh->turn[i - MAX_ACC];
+            ptx::mbar_init(ptx::smem_u32(bar), count);
+            ptx::fence_mbar_init();
+        }
+        if (tid == 0) {
+            sh->ctl.abort = 0;
+            sh->ctl.limit_kcycles = a.wait_limit_kcycles;
+        }
+    }
+    if (warp == WARP_MMA) {
+        if (PAIR) {
+            ptx::tmem_alloc_pair(ptx::smem_u32(&sh->tmem_base), (uint32_t)a.tmem_cols);
+            ptx::tmem_relinquish_pair();
+        } else {
+            ptx::tmem_alloc(ptx::smem_u32(&sh->tmem_base), (uint32_t)a.tmem_cols);
+            ptx::tmem_relinquish();
+        }
+    }
+    if (warp == WARP_LOAD && lane == 0) {
+        ptx::prefetch_tensormap(&tmap_w);
+        ptx::prefetch_tensormap(&tmap_x);
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    const uint32_t tmem_base = sh->tmem_base;
+    if (PAIR) {
+        ptx::cluster_arrive();
+        ptx::cluster_wait();
+    }
+    const int acc_mask = (1 << a.acc_log2) - 1, bke = a.rb / ES;     // channels of a slice
+    ptx::grid_dependency_wait();
+    if (a.mask_from_kernel) ptx::grid_launch_dependents();
+
+    if (warp == WARP_LOAD) {
+        // ------------------------------------------------------------------ input by TMA
+        if (lane == 0) {
+            // both blocks of a pair report the bytes of a buffer to the first one
+            const uint32_t full0 = ptx::smem_u32(&sh->a_full[0]), to_full0 = PAIR ? ptx::cluster_map(full0, 0u) : full0;
+            int s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int t = t_first; t < a.items && ok; t += t_step) {
+                const Item it = item_of<PATCH, PAIR>(t, g, a, rank);
+                // (second block of a pair) none from here on: the buffers do not wait for this block any more, so it must not wait for them
+                if (!it.any) break;
+                if (PATCH) {
+                    const int pitch = (int)a.fdPitch.d, y0 = (int)fd_div((uint32_t)it.first, a.fdPitch);
+                    // input rows that the 128 positions' windows lie in; those past the strip are nobody's
+                    int rows = (int)fd_div((uint32_t)(it.first - y0 * pitch + BM - 1), a.fdPitch) + g.kh;
+                    if (rows > a.Ho + g.kh - 1 - y0) rows = a.Ho + g.kh - 1 - y0;
+                    const uint32_t row_bytes = (uint32_t)(pitch * a.rb), bytes = (uint32_t)rows * row_bytes * (PAIR && it.other ? 2u : 1u);
+                    for (int c = 0; c < a.nc; ++c) {
+                        if (!wait_bar<40>(ptx::smem_u32(&sh->a_empty[s]), ph ^ 1u, ctl, a.dev_status)) { ok = false; break; }
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(full0 + 8u * s, bytes);
+                        for (int r = 0; r < rows; ++r) {
+                            const uint32_t dst = smem_base + (uint32_t)(s * a.a_bytes) + (uint32_t)r * row_bytes;
+                            if (PAIR) ptx::tma_load_4d_pair(dst, &tmap_x, to_full0 + 8u * s, c * bke, it.x0 - g.pad_w, y0 + r - g.pad, it.image);
+                            else ptx::tma_load_4d(dst, &tmap_x, to_full0 + 8u * s, c * bke, it.x0 - g.pad_w, y0 + r - g.pad, it.image);
+                        }
+                        if (++s == a.a_bufs) { s = 0; ph ^= 1u; }
+                    }
+                } else {
+                    const int n = (int)fd_div((uint32_t)it.first, a.fdP), p = it.first - n * g.P;
+                    const int oy = (int)fd_div((uint32_t)p, a.fdWo), ox = p - oy * g.Wo;
+                    const int h0 = oy * g.stride - g.pad, w0 = ox * g.stride_w - g.pad_w;
+                    for (int c = 0; c < a.nc && ok; ++c)
+                        for (int ky = 0; ky < g.kh && ok; ++ky)
+                            for (int kx = 0; kx < g.kw; ++kx) {
+                                if (!wait_bar<40>(ptx::smem_u32(&sh->a_empty[s]), ph ^ 1u, ctl, a.dev_status)) { ok = false; break; }
+                                if (rank == 0) ptx::mbar_arrive_expect_tx(full0 + 8u * s, (uint32_t)(BM * a.rb) * (PAIR && it.other ? 2u : 1u));
+                                const uint32_t dst = smem_base + (uint32_t)(s * a.a_bytes);
+                                if (PAIR) ptx::tma_im2col_4d_pair(dst, &tmap_x, to_full0 + 8u * s, c * bke, w0, h0, n, kx, ky);
+                                else ptx::tma_im2col_4d(dst, &tmap_x, to_full0 + 8u * s, c * bke, w0, h0, n, kx, ky);
+                                if (++s == a.a_bufs) { s = 0; ph ^= 1u; }
+                            }
+                }
+            }
+            if (!ok)         // let loads already issued land before the block's shared memory goes away
+                for (int i = 0; i < 64; ++i) __nanosleep(1000);
+        }
+        __syncwarp();
+    } else if (warp == WARP_FILTERS) {
+        // ------------------------------------------------------------------ filters by TMA
+        if (lane == 0) {
+            const uint32_t full0 = ptx::smem_u32(&sh->b_full[0]), to_full0 = PAIR ? ptx::cluster_map(full0, 0u) : full0;
+            const int taps = g.kh * g.kw;
+            int s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            if (a.resident && rank == 0) ptx::mbar_arrive_expect_tx(full0, (uint32_t)(BN * a.rb) * (uint32_t)(a.b_slots * a.G));
+            for (int t = t_first; t < a.items && ok; t += t_step) {
+                const int n0 = (t - (int)fd_div((uint32_t)t, a.fdNt) * a.n_tiles) * BN + rank * BNB;
+                for (int c = 0; c < a.nc && ok; ++c)
+                    for (int tap0 = 0; tap0 < taps; tap0 += a.G) {
+                        const int gc = taps - tap0 < a.G ? taps - tap0 : a.G;
+                        const uint32_t bar = a.resident ? to_full0 : to_full0 + 8u * s;
+                        if (!a.resident) {
+                            if (!wait_bar<40>(ptx::smem_u32(&sh->b_empty[s]), ph ^ 1u, ctl, a.dev_status)) { ok = false; break; }
+                            if (rank == 0) ptx::mbar_arrive_expect_tx(full0 + 8u * s, (uint32_t)(gc * BN * a.rb));
+                        }
+                        uint32_t dst = b_base + (uint32_t)(s * a.G) * b_bytes;
+                        for (int i = 0; i < gc; ++i, dst += b_bytes) {
+                            if (PAIR) ptx::tma_load_3d_pair(dst, &tmap_w, bar, c * bke, tap0 + i, n0);
+                            else ptx::tma_load_3d(dst, &tmap_w, bar, c * bke, tap0 + i, n0);
+                        }
+                        if (++s == a.b_slots) { s = 0; ph ^= 1u; }
+                    }
+                if (a.resident) break;
+            }
+            if (!ok)
+                for (int i = 0; i < 64; ++i) __nanosleep(1000);
+        }
+        __syncwarp();
+    } else if ((warp == WARP_MMA || warp == WARP_MMA2) && rank == 0) {
+        // ------------------------------------------------------------------ MMA issue
+        // Two warps take the tiles in turn: one finds its tile, waits for its accumulator and sees the last products committed while the
+        // other issues (a warp alone spent 700 clocks a tile on that).  The rings are waited for in one's turn only: by then every earlier
+        // use of them has been seen, so that the phase before the one waited for is over.  The whole warp runs the loop in control flow that the compiler knows to be uniform, see
+        // the row gather's.
+        const uint32_t idesc = F32 ? ptx::umma_idesc_tf32(PAIR ? 2 * BM : BM, BN) : ptx::umma_idesc_bf16(PAIR ? 2 * BM : BM, BN);
+        const uint32_t a0 = ptx::umma_desc_lo(smem_base), b0 = ptx::umma_desc_lo(b_base), d0 = uniform(tmem_base);
+        const uint32_t lead = ptx::elect_one() ? 1u : 0u;
+        const int which = warp == WARP_MMA ? 0 : 1;
+        bool ok = true;
+        if (a.resident && t_first < a.items) ok = __all_sync(0xffffffffu, wait_bar<0>(ptx::smem_u32(&sh->b_full[0]), 0u, ctl, a.dev_status));
+        for (int ti = which, t = t_first + which * t_step; t < a.items && ok; t += 2 * t_step, ti += 2) {
+            const int buf = ti & acc_mask;
+            ok = __all_sync(0xffffffffu, wait_bar<0, PAIR>(ptx::smem_u32(&sh->acc_empty[buf]), ((uint32_t)(ti >> a.acc_log2) & 1u) ^ 1u, ctl, a.dev_status));
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            // the tile's first operand buffer and its first group of slabs, in rings that the other warp's tiles use too
+            Rings r;
+            {
+                const uint32_t na = (uint32_t)ti * a.a_uses, nb = (uint32_t)ti * a.b_uses, qa = fd_div(na, a.fdA), qb = fd_div(nb, a.fdB);
+                r.a = uniform(na - qa * a.fdA.d);
+                r.a_phase = uniform(qa & 1u);
+                r.b = a.resident ? 0u : uniform(nb - qb * a.fdB.d);
+                r.b_phase = uniform(qb & 1u);
+            }
+            uint32_t x0 = 0;
+            if (PATCH) {
+                const uint32_t first = (uint32_t)item_of<PATCH, PAIR>(t, g, a, rank).first;
+                x0 = uniform(first - fd_div(first, a.fdPitch) * a.fdPitch.d);
+            }
+            const uint32_t d = d0 + (uint32_t)(buf * BN), a_first = a0 + x0 * ((uint32_t)a.rb >> 4);
+            if (ti > 0) {
+                ok = __all_sync(0xffffffffu, wait_bar<0>(ptx::smem_u32(&sh->turn[which]), (uint32_t)((ti - 1) >> 1) & 1u, ctl, a.dev_status));
+                if (!ok) break;
+            }
+            uint32_t started = 0;
+            for (int c = 0; c < a.nc && ok; ++c) {
+                const int steps = c + 1 == a.nc ? a.tail_steps : a.steps;
+#define ASX_SLICE(B_GROUPS) \
+    (steps == 4   ? issue_slice<F32, PAIR, PATCH, B_GROUPS, 4>(r, lead, d, a_first, b0, idesc, started, steps, g, a, sh, ctl) \
+     : steps == 2 ? issue_slice<F32, PAIR, PATCH, B_GROUPS, 2>(r, lead, d, a_first, b0, idesc, started, steps, g, a, sh, ctl) \
+                  : issue_slice<F32, PAIR, PATCH, B_GROUPS, 0>(r, lead, d, a_first, b0, idesc, started, steps, g, a, sh, ctl))
+                if (a.resident) ok = ASX_SLICE(RESIDENT);
+                else if (a.G > 1) ok = ASX_SLICE(FILTER_ROWS);
+                else ok = ASX_SLICE(TAPS);
+#undef ASX_SLICE
+                started = 1;
+            }
+            if (!ok) break;
+            if (lead) ptx::mbar_arrive(ptx::smem_u32(&sh->turn[which ^ 1]));
+            ptx::umma_commit<PAIR>(lead, ptx::smem_u32(&sh->acc_full[buf]));
+            __syncwarp();
+        }
+    } else if (warp >= WARP_EPI0) {
+        // ------------------------------------------------------------------ epilogue
+        // Two or four groups of four warps take the tiles in turn, an accumulator always the same ones; of four groups for two accumulators
+        // two share a tile, each every other piece of 64 bytes of the columns.
+        const int grp = (warp - WARP_EPI0) >> 2, q = warp & 3, N = g.C_out;      // lanes 32 q .. of tensor memory belong to this warp
+        const int turns = a.epi_groups > acc_mask + 1 ? acc_mask + 1 : a.epi_groups, share = a.epi_groups > turns ? 2 : 1, part = grp / turns;
+        if (grp == EPI_GROUPS - 1 && a.kept_out != nullptr) {
+            // the kept-row list first, for whoever asks for it later
+            constexpr int PART = LIST_WARPS * 32 * 16;
+            for (int part_l = blockIdx.x; (long long)part_l * PART < g.rows; part_l += gridDim.x) {
+                write_kept_list<LIST_WARPS>(a.mask, g.rows, part_l, tid - 32 * WARP_LIST0, 3, sh->list_total, a.kept_out, a.count_out);
+                asm volatile("bar.sync 3, %0;" ::"n"(LIST_WARPS * 32) : "memory");        // the totals are free again
+            }
+        }
+        uint8_t* const stage = after + (warp - WARP_EPI0) * 32 * STAGING_PITCH;
+        uint8_t* const mine = stage + lane * STAGING_PITCH;
+        uint8_t* const yb = static_cast<uint8_t*>(a.y);
+        float* const sbias = sh->bias[warp - WARP_EPI0];
+        int ti = grp - part * turns;
+        for (int t = t_first + ti * t_step; t < a.items && grp < a.epi_groups; t += turns * t_step, ti += turns) {
+            const int buf = ti & acc_mask;
+            const Item it = item_of<PATCH, PAIR>(t, g, a, rank);
+            const int n0 = it.n_tile * BN;
+            int row = it.first + q * 32 + lane;                  // this thread's output row, or -1
+            if (PATCH) {
+                const int y = (int)fd_div((uint32_t)row, a.fdPitch), x = row - y * (int)a.fdPitch.d;
+                row = it.any && y < a.Ho && x < a.width && it.x0 + x < a.Wo ? it.image * a.P + y * a.Wo + it.x0 + x : -1;
+            } else if (row >= g.M) {
+                row = -1;
+            }
+            bool keep = false;                                   // (a position without an output row counts as dropped)
+            if (row >= 0) {
+                const int p = g.rows == g.P ? row - (int)fd_div((uint32_t)row, a.fdP) * g.P : row;
+                keep = __ldcg(a.mask + p) != 0;
+            }
+            const int cols = N - n0 < BN ? N - n0 : BN;
+            auto bias_of = [&](int c) { return a.bias != nullptr && lane < COLS && c + lane < cols ? __ldg(a.bias + n0 + c + lane) : 0.f; };
+            float next_bias = bias_of(part * COLS);              // of the first piece; the others' come a piece ahead
+            if (!warp_wait_bar<100>(ptx::smem_u32(&sh->acc_full[buf]), (uint32_t)(ti >> a.acc_log2) & 1u, ctl, a.dev_status)) break;
+            ptx::tc_fence_after_sync();
+            auto release = [&]() {
+                if (PAIR) ptx::mbar_arrive_cluster(ptx::cluster_map(ptx::smem_u32(&sh->acc_empty[buf]), 0u));
+                else ptx::mbar_arrive(ptx::smem_u32(&sh->acc_empty[buf]));
+            };
+            const uint32_t kept_bits = keep ? 0xffffffffu : 0u;
+            const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
+            // a piece: WORDS words of a row in shared memory, UNITS 16-byte units, which ROWS rows at a time leave again
+            constexpr int WORDS = 16, UNITS = 4, ROWS = 8;
+            int out_row[UNITS];                                  // output rows of ROWS i + lane / UNITS
+#pragma unroll
+            for (int i = 0; i < UNITS; ++i) out_row[i] = __shfl_sync(0xffffffffu, row, ROWS * i + lane / UNITS);
+            const long long pitch_y = (long long)N * ES;
+            if (part * COLS >= cols) {                           // (this tile has nothing for this group)
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) release();
+            }
+            for (int c0 = part * COLS; c0 < cols; c0 += share * COLS) {
+                sbias[lane] = next_bias;
+                next_bias = bias_of(c0 + share * COLS);
+                float v[COLS];
+                if (!F32 && c0 + 32 <= BN) {
+                    uint32_t r[32];
+                    ptx::tmem_ld_32(tacc + (uint32_t)c0, r);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < COLS; ++j) v[j] = __uint_as_float(r[j % 32]);
+                } else {
+                    uint32_t r[16];
+                    ptx::tmem_ld_16(tacc + (uint32_t)c0, r);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < COLS; ++j) v[j] = j < 16 ? __uint_as_float(r[j % 16]) : 0.f;
+                }
+                if (c0 + share * COLS >= cols) {                 // the accumulator is in registers now
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) release();
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < COLS; j += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(sbias + j);
+                    ptx::add2(v[j], v[j + 1], b4.x, b4.y);
+                    ptx::add2(v[j + 2], v[j + 3], b4.z, b4.w);
+                }
+                if (RESIDUAL && keep) {
+#pragma unroll
+                    for (int j = 0; j < COLS; j += 8) {
+                        if (c0 + j >= cols) break;
+                        float res[8];
+                        load_residual8(a.residual, (long long)row * N + n0 + c0 + j, cols - c0 - j, a.vec_out, res);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v[j + i] += res[i];
+                    }
+                }
+                if (a.act == 2) {
+#pragma unroll
+                    for (int j = 0; j < COLS; ++j) v[j] = silu(v[j]);
+                }
+                uint32_t word[WORDS];                            // pairs of bf16, or fp32 values
+#pragma unroll
+                for (int i = 0; i < WORDS; ++i) word[i] = F32 ? __float_as_uint(v[i]) : pack_bf16(v[2 * i % COLS], v[(2 * i + 1) % COLS]);
+                if (a.act == 1) {                                // rounding and ReLU change places without a change of the result
+#pragma unroll
+                    for (int i = 0; i < WORDS; ++i) word[i] = F32 ? __float_as_uint(fmaxf(__uint_as_float(word[i]), 0.f)) : ptx::max_bf16x2(word[i], 0u);
+                }
+#pragma unroll
+                for (int i = 0; i < WORDS; ++i) word[i] &= kept_bits;
+                const int ncols = cols - c0 < COLS ? cols - c0 : COLS;
+                int e = 0;
+                if (!F32 && !a.vec_out) {
+                    // Rows of bf16 whose channels are no whole 16-byte chunks start at any value: a row that starts between two words is staged half
+                    // a word on, so that its words lie in shared memory as they do in y, and its first and last halves are stored from here.
+                    e = row * N + n0 + c0 + a.y_half;
+                    unsigned short* const yh = static_cast<unsigned short*>(a.y) - a.y_half;
+                    const int odd = e & 1;
+                    if (row >= 0 && odd) yh[e] = (unsigned short)word[0];
+                    if (odd) {
+                        *reinterpret_cast<uint32_t*>(mine + 4 * WORDS) = word[WORDS - 1] >> 16;
+#pragma unroll
+                        for (int i = WORDS - 1; i > 0; --i) word[i] = __funnelshift_r(word[i - 1], word[i], 16);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < WORDS; i += 4) *reinterpret_cast<uint4*>(mine + 4 * i) = make_uint4(word[i], word[i + 1], word[i + 2], word[i + 3]);
+                if (!F32 && !a.vec_out && row >= 0 && ((ncols + e) & 1))
+                    (static_cast<unsigned short*>(a.y) - a.y_half)[e + ncols - 1] = *reinterpret_cast<const unsigned short*>(mine + 2 * (ncols - 1 + (e & 1)));
+                __syncwarp();
+                // The warp's 32 rows, from shared memory, neighbouring lanes on neighbouring pieces of a row.
+                if (a.vec_out) {
+                    const int u = 16 * (lane % UNITS);
+                    const uint8_t* const src = stage + (lane / UNITS) * STAGING_PITCH + u;
+                    uint8_t* const dst = yb + (long long)(n0 + c0) * ES + u;
+                    uint4 piece[UNITS];
+#pragma unroll
+                    for (int i = 0; i < UNITS; ++i) piece[i] = *reinterpret_cast<const uint4*>(src + i * ROWS * STAGING_PITCH);
+#pragma unroll
+                    for (int i = 0; i < UNITS; ++i)
+                        if (out_row[i] >= 0 && u < ncols * ES) *reinterpret_cast<uint4*>(dst + out_row[i] * pitch_y) = piece[i];
+                } else if (F32) {
+                    float* const yf = static_cast<float*>(a.y) + n0 + c0 + (lane & 15);
+#pragma unroll 8
+                    for (int rr = lane >> 4; rr < 32; rr += 2) {
+                        const int out = __shfl_sync(0xffffffffu, row, rr);
+                        const float w = *reinterpret_cast<const float*>(stage + rr * STAGING_PITCH + 4 * (lane & 15));
+                        if (out >= 0 && (lane & 15) < ncols) yf[(long long)out * N] = w;
+                    }
+                } else {
+                    // two rows at a time, a word a lane: the words that are the row's alone
+                    uint32_t* const yw = reinterpret_cast<uint32_t*>(yb - 2 * a.y_half) + (lane & 15);
+                    const int col2 = 2 * (lane & 15) + 2;
+                    if (row < 0) e = -1;
+#pragma unroll 8
+                    for (int rr = lane >> 4; rr < 32; rr += 2) {
+                        const int er = __shfl_sync(0xffffffffu, e, rr), odd = er & 1;
+                        const uint32_t w = *reinterpret_cast<const uint32_t*>(stage + rr * STAGING_PITCH + 4 * (lane & 15));
+                        if (er >= 0 && (lane & 15) >= odd && col2 - odd <= ncols) yw[er >> 1] = w;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+
+    ptx::tc_fence_before_sync();
+    if (PAIR) {                              // neither block gives up memory that the other still works in
+        ptx::cluster_arrive();
+        ptx::cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    if (warp == WARP_MMA) {
+        __syncwarp();
+        ptx::tc_fence_after_sync();
+        if (PAIR) ptx::tmem_dealloc_pair(tmem_base, (uint32_t)a.tmem_cols);
+        else ptx::tmem_dealloc(tmem_base, (uint32_t)a.tmem_cols);
+    }
+    if (PAIR) {
+        ptx::cluster_arrive_relaxed();
+        ptx::cluster_wait();
+    }
+}
+
+}  // namespace
+
+// The strips of a stride-1 layer: the cut that takes fewest tiles among those whose patch of 128 positions fits `patch_room` bytes.  False: none
+// does.
+static bool cut_strips(const ConvGeom& g, int rb, int patch_room, AllRowsPlan* plan)
+{
+    if (g.stride != 1 || g.stride_w != 1) return false;
+    long long best = 0;
+    const bool flat = g.kh == 1 && g.kw == 1 && g.pad == 0 && g.pad_w == 0;        // the image's shape does not matter: strips of 128 positions
+    for (int n = flat ? (g.M + BM - 1) / BM : 1, last = flat ? n : 64; n <= last; ++n) {
+        const int Wo = flat ? g.M : g.Wo, Ho = flat ? 1 : g.Ho;
+        const int width = flat ? BM : (Wo + n - 1) / n;
+        const int pitch = (width + g.kw - 1 + 7) / 8 * 8;
+        if (pitch > 256) continue;
+        if (width < 8 && best != 0) break;
+        int step = BM, x = pitch;                                                  // a tile's first column is a multiple of gcd(128, pitch)
+        while (x != 0) { const int r = step % x; step = x; x = r; }
+        const int rows = (pitch - step + BM - 1) / pitch + g.kh;                   // the most input rows of a tile
+        const long long bytes = ((long long)rows * pitch * rb + 1023) / 1024 * 1024;
+        if (bytes > patch_room) continue;
+        const long long tiles = ((long long)(Ho - 1) * pitch + width + BM - 1) / BM, strips = (Wo + width - 1) / width, all = tiles * strips;
+        if (best == 0 || all < best) {
+            best = all;
+            plan->strips = (int)strips;
+            plan->width = width;
+            plan->pitch = pitch;
+            plan->tiles = (int)tiles;
+            plan->a_bytes = (int)bytes;
+            plan->flat = flat ? 1 : 0;
+        }
+    }
+    return best != 0;
+}
+
+bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* plan)
+{
+    const int N = g.C_out;
+    const bool f32 = elem_bytes == 4;
+    if (g.C_in % (16 / elem_bytes) != 0 || g.stride > 8 || g.stride_w > 8 || num_sms < 2) return false;
+    // corners of the box of window positions are 8-bit, offsets of a tap in a window too
+    if (g.pad > 120 || g.pad_w > 120 || g.kh > 120 || g.kw > 120) return false;
+    // few channels take narrower slices: the rest of 128 bytes would be loaded as zeros
+    const int rb = g.C_in * elem_bytes <= 32 ? 32 : g.C_in * elem_bytes <= 64 ? 64 : 128, bke = rb / elem_bytes;
+    const int nc = (g.C_in + bke - 1) / bke, KB = g.kh * g.kw * nc;
+    const int tail = g.C_in - (nc - 1) * bke;
+    plan->nc = nc;
+    plan->rb = rb;
+    plan->tail_steps = (tail * elem_bytes + 31) / 32;
+    // Four groups of epilogue warps where the way out takes longer than a tile's products: few k-blocks, or rows at any address.
+    const bool whole = g.C_out % (16 / elem_bytes) == 0;
+    plan->epi_groups = KB <= (whole ? 4 : 24) ? 4 : 2;
+    const int fixed = 1024 + plan->epi_groups * STAGING_GROUP + (int)sizeof(Shared), avail = 227 * 1024 - fixed;
+    double best = 0.0;
+    AllRowsPlan best_plan;
+    for (int pair = 0; pair <= 1; ++pair) {
+        const int unit = pair ? 32 : 16;
+        const int slots = pair ? num_sms / 2 : num_sms;
+        for (int n_tiles = (N + 255) / 256; ; n_tiles *= 2) {
+            const int per = (N + n_tiles - 1) / n_tiles, BN = (per + unit - 1) / unit * unit, nt = (N + BN - 1) / BN, BNB = pair ? BN / 2 : BN;
+            for (int patch = 0; patch <= 1; ++patch) {
+                AllRowsPlan p = *plan;
+                p.patch = patch;
+                p.pair = pair;
+                p.BN = BN;
+                p.n_tiles = nt;
+                long long m_tiles;                                  // of this block or pair
+                const bool can_stay = nt == 1;
+                if (patch) {
+                    // two patches beside the filters if those can stay, else beside four slabs
+                    const long long all_b = (long long)KB * BNB * rb;
+                    p.resident = can_stay && all_b < avail && cut_strips(g, rb, (int)((avail - all_b) / 2), &p) ? 1 : 0;
+                    if (!p.resident && !cut_strips(g, rb, (avail - 4 * BNB * rb) / 2, &p)) continue;
+                    // a group of slabs, which is waited for once, is a filter row's where four such groups fit
+                    p.G = !p.resident && 4 * g.kw * BNB * rb <= avail - 2 * p.a_bytes ? g.kw : 1;
+                    const int room = avail - (p.resident ? KB : std::max(4, 2 * p.G)) * BNB * rb;
+                    p.a_bufs = std::max(2, std::min(4, room / p.a_bytes));
+                    p.b_slots = p.resident ? KB : std::min(MAX_STAGES, (avail - p.a_bufs * p.a_bytes) / (p.G * BNB * rb));
+                    const long long strips = (long long)(p.flat ? 1 : g.Nb) * p.strips;
+                    m_tiles = (pair ? (strips + 1) / 2 : strips) * p.tiles;
+                } else {
+                    p.a_bytes = A_BYTES;
+                    p.G = 1;
+                    p.resident = can_stay && (long long)KB * BNB * rb <= avail - 5 * A_BYTES ? 1 : 0;
+                    p.a_bufs = std::min(MAX_STAGES, p.resident ? (avail - KB * BNB * rb) / A_BYTES : avail / (A_BYTES + BNB * rb));
+                    p.b_slots = p.resident ? KB : p.a_bufs;
+                    if (p.a_bufs < MIN_STAGES) continue;
+                    m_tiles = pair ? (g.M + 2 * BM - 1) / (2 * BM) : (g.M + BM - 1) / BM;
+                }
+                if (m_tiles * nt >= (1ll << 30)) continue;
+                p.items = (int)(m_tiles * nt);
+                const long long waves = (p.items + slots - 1) / slots;
+                // microseconds: a k-block of the patch form waits for its slabs where they cannot stay; the way out of a tile's
+                // columns, of which four groups of warps take four tiles at a time
+                const double t_kb = !patch ? 0.36 : f32 ? 0.12 + 0.001 * BN : pair ? 0.085 + 0.001 * BN : p.resident ? 0.105 + 0.001 * BN : std::max(0.3, 0.105 + 0.001 * BN);
+                const double t_out = (whole ? 0.2 + 0.011 * BN : 0.3 + 0.02 * BN) * (f32 ? 2.0 : 1.0) * (p.epi_groups == 4 ? 1.0 : 1.7);
+                const double cost = (double)waves * std::max(KB * t_kb + 0.1, t_out) + 0.012 * BN + 2.0;
+                p.est_cost_us = cost;
+                p.smem_bytes = std::max(120 * 1024, fixed + p.a_bufs * p.a_bytes + p.b_slots * p.G * BNB * rb);      // one block per SM: tensor memory is not shared out
+                if (best_plan.BN == 0 || cost < best) { best = cost; best_plan = p; }
+            }
+            if (BN <= 64) break;
+        }
+    }
+    if (best_plan.BN == 0) return false;
+    *plan = best_plan;
+    return true;
+}
+
+cudaError_t launch_all_rows(const ConvGeom& g, const AllRowsPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x, const float* bias,
+                            void* y, const uint8_t* mask, int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32,
+                            int* dev_status, int num_sms, int mask_from_kernel, int wait_limit_kcycles, cudaStream_t st)
+{
+    AllRowsArgs a;
+    a.fdP = make_fastdiv((uint32_t)g.P);
+    a.fdWo = make_fastdiv((uint32_t)g.Wo);
+    a.fdNt = make_fastdiv((uint32_t)plan.n_tiles);
+    a.bias = bias;
+    a.y = y;
+    a.mask = mask;
+    a.residual = static_cast<const __nv_bfloat16*>(residual);
+    a.dev_status = dev_status;
+    a.kept_out = kept_out;
+    a.count_out = count_out;
+    a.act = relu;
+    a.BN = plan.BN;
+    a.n_tiles = plan.n_tiles;
+    const bool pair = plan.pair != 0;
+    const int blocks = pair ? 2 : 1, items = plan.items;
+    a.items = items;
+    a.a_bufs = plan.a_bufs;
+    a.a_bytes = plan.a_bytes;
+    a.fdStrips = make_fastdiv((uint32_t)std::max(1, plan.strips));
+    a.fdTiles = make_fastdiv((uint32_t)std::max(1, plan.tiles));
+    a.fdPitch = make_fastdiv((uint32_t)std::max(1, plan.pitch));
+    a.width = plan.width;
+    a.Ho = plan.flat ? 1 : g.Ho;
+    a.Wo = plan.flat ? g.M : g.Wo;
+    a.P = plan.flat ? g.M : g.P;
+    a.strips_all = plan.strips * (plan.flat ? 1 : g.Nb);
+    a.b_slots = plan.b_slots;
+    a.G = plan.G;
+    a.fdA = make_fastdiv((uint32_t)plan.a_bufs);
+    a.fdB = make_fastdiv((uint32_t)plan.b_slots);
+    a.a_uses = (uint32_t)(plan.patch ? plan.nc : plan.nc * g.kh * g.kw);
+    a.b_uses = (uint32_t)(plan.resident ? 0 : plan.nc * (plan.G > 1 ? g.kh : g.kh * g.kw));
+    a.resident = plan.resident;
+    a.nc = plan.nc;
+    a.rb = plan.rb;
+    a.steps = plan.rb / 32;
+    a.tail_steps = plan.tail_steps;
+    a.epi_groups = plan.epi_groups;
+    a.acc_log2 = plan.BN <= 128 ? 2 : 1;
+    int cols = 32;
+    while (cols < (plan.BN << a.acc_log2)) cols <<= 1;
+    a.tmem_cols = cols;
+    a.vec_out = (g.C_out % (f32 ? 4 : 8) == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0) ? 1 : 0;
+    a.y_half = (int)((reinterpret_cast<uintptr_t>(y) >> 1) & 1);
+    a.mask_from_kernel = mask_from_kernel;
+    a.wait_limit_kcycles = wait_limit_kcycles > 0 ? wait_limit_kcycles : WAIT_LIMIT_KCYCLES_DEFAULT;
+    const int slots = num_sms / blocks, grid = (items < slots ? items : slots) * blocks;
+    using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const AllRowsArgs);
+    const bool res = residual != nullptr;
+    if (f32 && res) return cudaErrorInvalidValue;
+    Kern kern;
+#define ASX_PICK(F32, RES) \
+    (plan.patch ? (pair ? masked_conv_all_rows_kernel<F32, RES, true, true> : masked_conv_all_rows_kernel<F32, RES, false, true>) \
+                : (pair ? masked_conv_all_rows_kernel<F32, RES, true, false> : masked_conv_all_rows_kernel<F32, RES, false, false>))
+    if (f32) kern = ASX_PICK(true, false);
+    else if (res) kern = ASX_PICK(false, true);
+    else kern = ASX_PICK(false, false);
+#undef ASX_PICK
+    static std::atomic<unsigned long long> smem_set[12];      // per instance
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), MAX_DYN_SMEM, smem_set[(f32 ? 8 : res ? 4 : 0) + (plan.patch ? 2 : 0) + (pair ? 1 : 0)]);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_cluster(kern, dim3((unsigned)grid), dim3(NUM_THREADS), blocks, (size_t)plan.smem_bytes, st, tmap_w, tmap_x, g, a);
+}
+
+}  // namespace asx

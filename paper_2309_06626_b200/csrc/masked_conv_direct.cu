@@ -35,6 +35,7 @@ namespace {
 
 constexpr int THREADS = 256, WARPS = THREADS / 32;
 constexpr int DIRECT_MAX_SMEM = 112 * 1024;
+constexpr int LIST_ROWS = THREADS * 16;  // mask entries that a list block takes
 constexpr int CHUNK = 32;               // output rows a warp scans at a time
 constexpr int QUEUE = 48;               // row queue of a warp: up to 15 left over and 32 new ones
 // The filter row (upper half) of a chunk or word past the window: no corner -255 .. 32767 puts it into an image of up to
@@ -101,45 +102,6 @@ __device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uin
     else
         asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// The list for asx_get_kept (S1): block `part` writes the positions of mask bytes 4096 part .. 4096 part + 4095, for which
-// it first counts the kept rows in front of them.  (One block for the whole list was the last to finish: 14 us for a
-// mask of 25 600 rows.)
-constexpr int LIST_ROWS = THREADS * 16;
-__device__ void write_kept_list(const uint8_t* __restrict__ mask, int rows, int part, int32_t* kept, int32_t* count)
-{
-    __shared__ int s_total[2][WARPS];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int first = part * LIST_ROWS + tid * 16;
-    const unsigned f = first < rows ? mask_flags16(mask, rows, first) : 0u;
-    int before = 0;
-#pragma unroll 4
-    for (int i = 0; i < part; ++i) before += __popc(mask_flags16(mask, rows, i * LIST_ROWS + tid * 16));
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
-    const int mine = __popc(f);
-    int incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += u;
-    }
-    if (lane == 31) {
-        s_total[0][warp] = before;
-        s_total[1][warp] = incl;
-    }
-    __syncthreads();
-    int at = incl - mine, all = 0;
-#pragma unroll
-    for (int i = 0; i < WARPS; ++i) {
-        at += s_total[0][i] + (i < warp ? s_total[1][i] : 0);
-        all += s_total[0][i] + s_total[1][i];
-    }
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-        if ((f >> q) & 1u) kept[at + __popc(f & ((1u << q) - 1u))] = first + q;
-    if (tid == 0 && (part + 1) * (long long)LIST_ROWS >= rows) *count = all;
 }
 
 // Shared memory: the filters in fragment order, the bias, one entry per chunk (or word) of a window, the warps' row
@@ -418,7 +380,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) masked_conv_direct_kernel(con
         if (block < a.list_blocks) {
             if (blockIdx.y != 0) return;
             ptx::grid_dependency_wait();           // an earlier kernel may still read the list
-            write_kept_list(a.mask, g.rows, block, a.kept_out, a.count_out);
+            __shared__ int totals[2][WARPS];
+            write_kept_list<WARPS>(a.mask, g.rows, block, tid, 0, totals, a.kept_out, a.count_out);
             return;
         }
         block -= a.list_blocks;

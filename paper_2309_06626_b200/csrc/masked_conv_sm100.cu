@@ -423,7 +423,7 @@ masked_conv_sm100_kernel(const __grid_constant__ CUtensorMap tmap_w, const __gri
                 const uint32_t al = a0 + (uint32_t)(s * (stage_bytes >> 4)), bl = al + (A_STAGE_BYTES >> 4);
 #pragma unroll
                 for (int i = 0; i < 4; ++i)                // 32 bytes of K a step: 16 bf16 or 8 fp32 elements, 2 descriptor units
-                    ptx::umma<F32, PAIR>(lead, d, al + 2 * i, bl + 2 * i, idesc, i > 0 || kb > 0 ? 1u : 0u);
+                    ptx::umma<F32, PAIR>(lead, d, al + 2 * i, bl + 2 * i, ptx::umma_desc_hi(128), idesc, i > 0 || kb > 0 ? 1u : 0u);
                 ptx::umma_commit<PAIR>(lead, ptx::smem_u32(&sh->empty[s]));
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
@@ -1013,6 +1013,8 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const int bke = 128 / elem_bytes;             // K elements per stage: 64 bf16 or 32 fp32
     const int KB = (g.K + bke - 1) / bke;
     if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
+    plan->use_all = 0;
+    if (!plan_all_rows(g, num_sms, elem_bytes, &plan->all)) plan->all.BN = 0;
     const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
     auto stage_bytes_of = [](int BN, int pair) { return A_STAGE_BYTES + (pair ? BN / 2 : BN) * BK * 2; };
     auto fixed_bytes = [&](int KS) { return 1024 + (int)(KS > 1 ? sizeof(SharedT<1>) : sizeof(SharedT<PLAIN_INFO_RING>)) + list_bytes; };
@@ -1029,6 +1031,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     // Pairs of blocks share tiles of 256 rows where the tiles are 256 wide and there is a wave of them: with narrower ones the row
     // requests, which a pair does not save, are all that counts (128 and 192 wide: 0-8 % slower than alone), and an item's hand-overs between the
     // two blocks take longer (1.2 us an item: a 256 -> 256 channel 1x1 layer, four k-blocks an item, 21.4 us alone, 25.0 in pairs).
+    const bool scalar_out = N % (16 / elem_bytes) != 0;
     int best_BN = 0, best_KS = 1, best_pair = 0;
     double best_cost = 0.0;
     const bool tma = g.C_in % bke == 0;
@@ -1055,7 +1058,9 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
                 const int kbi = (KB + KS - 1) / KS;
                 const double t_kb = 0.12 + 0.18 * fill + (pair ? 0.0005 : 0.001) * BN;                  // microseconds
                 // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
-                const double cost = (double)waves * (kbi * t_kb + (pair ? 1.5 : 0.3)) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
+                // rows of y that are no whole 16-byte chunks leave value by value
+                const double t_item = std::max(kbi * t_kb, scalar_out ? 0.2 * BN : 0.0);
+                const double cost = (double)waves * (t_item + (pair ? 1.5 : 0.3)) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
                 if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_pair = pair; best_cost = cost; }
             }
             if (BN <= 64 && whole) break;
@@ -1091,6 +1096,9 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
                         int mask_from_kernel, cudaStream_t st)
 {
     if (f32 && (in_rank != nullptr || residual != nullptr)) return cudaErrorInvalidValue;
+    if (plan.use_all)
+        return launch_all_rows(g, plan.all, tmap_w, tmap_x, bias, y, mask, write_list ? const_cast<int32_t*>(kept) : nullptr,
+                               const_cast<int32_t*>(count), relu, residual, f32, dev_status, num_sms, mask_from_kernel, wait_limit_kcycles, st);
     FastArgs a;
     a.fdcnt_host = make_fastdiv((uint32_t)(host_kept > 0 && host_kept < (1ll << 31) ? host_kept : 1));
     if (!(host_kept > 0 && host_kept < (1ll << 31))) a.fdcnt_host.d = 0;

@@ -133,6 +133,20 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t bar, uint3
                  : "memory");
 }
 
+// ---------------------------------------------------------------- pairs of values
+// (x, y) += (u, v), both sums rounded as two additions would
+__device__ __forceinline__ void add2(float& x, float& y, float u, float v)
+{
+    asm("{\n.reg .b64 a, b;\nmov.b64 a, {%0, %1};\nmov.b64 b, {%2, %3};\nadd.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}\n" : "+f"(x), "+f"(y) : "f"(u), "f"(v));
+}
+// The larger of two pairs of bf16, value by value; of a number and NaN the number.
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
 // ---------------------------------------------------------------- proxies, cp.async
 __device__ __forceinline__ void fence_proxy_async_smem()
 {
@@ -220,13 +234,53 @@ __device__ __forceinline__ void tma_gather4_2d(uint32_t dst, const void* tmap, u
         : "memory");
 }
 
-// Both loads for a block of a pair: into its own shared memory, the bytes counted on a barrier of either block (an address from
+// The same for a 3-D tensor.
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+// One filter tap's values of consecutive window positions (im2col mode): the map says how many positions and channels, (c0, c1, c2, c3) is the
+// first position's window corner (channel, column, row, image), (kx, ky) the tap; positions run over row and image ends, values outside
+// the image are zeros.
+__device__ __forceinline__ void tma_im2col_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3, int kx, int ky)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "h"((uint16_t)kx), "h"((uint16_t)ky)
+        : "memory");
+}
+
+// These loads for a block of a pair: into its own shared memory, the bytes counted on a barrier of either block (an address from
 // cluster_map).
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1)
 {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, %6}], [%2];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
+__device__ __forceinline__ void tma_im2col_4d_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3, int kx, int ky)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "h"((uint16_t)kx), "h"((uint16_t)ky)
         : "memory");
 }
 __device__ __forceinline__ void tma_gather4_2d_pair(uint32_t dst, const void* tmap, uint32_t bar, int c0,
@@ -280,14 +334,18 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 // The predicate stands on the instruction itself: in the warp's ordinary control flow, without a branch, every operand stays in uniform
 // registers.  In a branch of one lane, behind a wait that only one lane decides, they did not, and four products with their wait and
 // commit took 590 clocks whatever their width; as they are here, behind a wait decided by a vote, 340 (280 without the wait; 148 SMs,
-// 128 x 64 and 128 x 128 x 64, operands at rest).  An operand's descriptor is its lower word, the upper one is the same for all (UMMA_DESC_HI).
-constexpr uint32_t UMMA_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // of umma_desc_k_major_sw128
+// 128 x 64 and 128 x 128 x 64, operands at rest).  An operand's descriptor is its lower word; the upper one (desc_hi) is the same for all of a launch.
+// K-major operands whose rows are `row_bytes` (128, 64 or 32) with the swizzle of that width, 8-row groups one after the other.
+__device__ __forceinline__ uint32_t umma_desc_hi(uint32_t row_bytes)
+{
+    return (8u * row_bytes >> 4) | (1u << 14) | ((row_bytes == 128u ? 2u : row_bytes == 64u ? 4u : 6u) << 29);
+}
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t smem_addr) { return ((smem_addr & 0x3ffffu) >> 4) | (1u << 16); }
 // D[tmem] (+)= A[smem] * B[smem], fp32 accumulate; TF32: fp32 operands read as TF32 (sign, exponent and the upper 10 mantissa bits of
 // each value), 8 K-elements an instruction, else bf16, 16.  PAIR: 256 rows, of which each block of the pair holds 128 in its shared memory and gets those rows' results in
 // its tensor memory, by N filters, of which each block holds half; issued by the first block.
 template <bool TF32, bool PAIR>
-__device__ __forceinline__ void umma(uint32_t lead, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
+__device__ __forceinline__ void umma(uint32_t lead, uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate)
 {
 #define ASX_UMMA(GROUP, KIND)                                                                                               \
     asm volatile(                                                                                                           \
@@ -299,7 +357,7 @@ __device__ __forceinline__ void umma(uint32_t lead, uint32_t tmem_d, uint32_t a_
         "mov.b64 da, {%1, %3};\n"                                                                                          \
         "mov.b64 db, {%2, %3};\n"                                                                                          \
         "@q tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], da, db, %4, p;\n"                                        \
-        "}\n" ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(UMMA_DESC_HI), "r"(idesc), "r"(accumulate), "r"(lead)               \
+        "}\n" ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(lead)                    \
         : "memory")
     if (TF32) {
         if (PAIR) ASX_UMMA("2", "tf32");

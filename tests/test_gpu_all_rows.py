@@ -1,0 +1,89 @@
+"""The form that computes dropped rows too, against the library's plain kernel: tiles that end inside rows and images, channel counts that
+end inside a k-block, output rows at every alignment, strides, filters that reach over the image on all sides, masks per position and per row,
+everything and nothing dropped, residuals, the kept-row list."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2309_06626_b200 as asx
+
+pytestmark = pytest.mark.gpu
+
+
+def _values(gen, shape, f32, scale=1.0):
+    t = torch.randn(shape, generator=gen, device="cuda") * scale
+    return (t.view(torch.int32) & ~0x1fff).view(torch.float32) if f32 else t.to(torch.bfloat16)      # fp32: values that TF32 holds exactly
+
+
+CASES = [
+    # C_in, C_out, kh, kw, stride, pad, H, W, Nb, kept %, one mask entry per lowered row
+    (64, 64, 3, 3, 1, 1, 14, 14, 3, 60, False), (64, 64, 3, 3, 1, 1, 9, 13, 2, 50, True), (8, 16, 3, 3, 1, 1, 16, 16, 1, 80, False),
+    (40, 24, 5, 3, 2, 2, 23, 31, 2, 70, False), (96, 176, 3, 3, 2, 1, 29, 17, 3, 90, False), (72, 37, 1, 1, 1, 0, 20, 11, 2, 50, False),
+    (32, 255, 3, 3, 1, 1, 12, 12, 4, 50, True), (128, 256, 1, 1, 2, 0, 28, 28, 6, 75, False), (64, 513, 3, 3, 1, 1, 10, 10, 5, 50, False),
+    (16, 286, 3, 3, 1, 1, 11, 11, 3, 40, False), (64, 1, 3, 3, 1, 1, 8, 8, 1, 50, False), (200, 80, 7, 7, 1, 3, 9, 9, 2, 50, False),
+    (64, 64, 3, 3, 1, 1, 14, 14, 2, 0, False), (64, 48, 3, 3, 1, 1, 14, 14, 2, 100, False), (64, 64, 3, 3, 3, 0, 17, 17, 70, 50, False),
+    (64, 64, 3, 3, 1, 4, 5, 6, 2, 50, False), (512, 512, 3, 3, 1, 1, 7, 7, 9, 50, False), (64, 32, 1, 1, 1, 0, 160, 160, 2, 60, False),
+    (3, 64, 7, 7, 2, 3, 64, 64, 2, 60, False), (3, 48, 7, 7, 2, 3, 30, 48, 3, 60, False), (3, 32, 3, 3, 2, 1, 33, 40, 2, 60, False),
+    (5, 33, 3, 3, 1, 1, 12, 15, 2, 50, False), (130, 41, 1, 1, 2, 0, 15, 15, 4, 100, False),
+]
+
+
+@pytest.mark.parametrize("f32", [False, True], ids=["bf16", "f32"])
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(str(int(v)) for v in c))
+def test_every_row(case, f32):
+    cin, cout, kh, kw, stride, pad, H, W, Nb, percent, per_row = case
+    Ho, Wo = (H + 2 * pad - kh) // stride + 1, (W + 2 * pad - kw) // stride + 1
+    gen = torch.Generator(device="cuda").manual_seed(cin + 7 * cout)
+    x, w = _values(gen, (Nb, H, W, cin), f32), _values(gen, (cout, kh, kw, cin), f32, (kh * kw * cin) ** -0.5)
+    b = torch.randn((cout,), generator=gen, device="cuda")
+    rows = Ho * Wo * (Nb if per_row else 1)
+    mask = np.zeros(rows, np.uint8)
+    mask[np.random.default_rng(rows).permutation(rows)[:rows * percent // 100]] = 1
+    layer = asx.MaskedConvLayer(cin, cout, kh, kw, stride, pad)
+    layer.set_mask(mask)
+    base = asx.F32 if f32 else 0
+    dropped = torch.from_numpy(mask == 0).cuda()
+    for act in (0, asx.ACT_RELU, asx.ACT_SILU):
+        want = layer.run(x, w, b, flags=base | act | asx.IMPL_NAIVE).float().clone()
+        out = torch.full((Nb, Ho, Wo, cout), float("nan"), dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+        layer.run(x, w, b, out=out, flags=base | act | asx.IMPL_ALL_ROWS | asx.RECOMPACT)
+        torch.cuda.synchronize()
+        assert layer.device_status() == 0 and layer.last_run_form() == asx.FORM_ALL_ROWS
+        got = out.float()
+        # bf16: one rounding of the result; fp32: sums of up to 10,000 products in another order
+        assert (got - want).norm() <= (2e-5 if f32 else 5e-3) * want.norm()
+        assert not got.reshape(1 if per_row else Nb, rows, cout)[:, dropped].any()
+        assert np.array_equal(layer.kept(), np.flatnonzero(mask))
+    layer.close()
+
+
+@pytest.mark.parametrize("cout", [64, 72, 45])
+def test_residual(cout):
+    gen = torch.Generator(device="cuda").manual_seed(cout)
+    Nb, H = 3, 13
+    x, w, res = _values(gen, (Nb, H, H, 64), False), _values(gen, (cout, 3, 3, 64), False, 24 ** -1.0), _values(gen, (Nb, H, H, cout), False)
+    mask = (torch.rand(H * H, generator=gen, device="cuda") < 0.6)
+    layer = asx.MaskedConvLayer(64, cout, 3, 3, 1, 1)
+    layer.set_mask(mask.cpu().numpy().astype(np.uint8))
+    layer.set_residual(res)
+    got = layer.run(x, w, None, flags=asx.ACT_RELU | asx.IMPL_ALL_ROWS)
+    torch.cuda.synchronize()
+    assert layer.device_status() == 0 and layer.last_run_form() == asx.FORM_ALL_ROWS
+    z = torch.nn.functional.conv2d(x.permute(0, 3, 1, 2).double(), w.permute(0, 3, 1, 2).double(), padding=1).permute(0, 2, 3, 1) + res.double()
+    want = z.clamp(min=0) * mask.reshape(1, H, H, 1)
+    assert (got.double() - want).norm() <= 5e-3 * want.norm()
+    layer.close()
+
+
+def test_infinity_and_nan_stay_in_their_windows():
+    """Values past a window's channels, and of other rows, do not reach a result."""
+    layer = asx.MaskedConvLayer(40, 24, 3, 3, 1, 1)
+    x = torch.ones((2, 9, 9, 40), dtype=torch.bfloat16, device="cuda")
+    w = torch.ones((24, 3, 3, 40), dtype=torch.bfloat16, device="cuda")
+    w[3, 1, 1, 0] = float("inf")          # the channels of a tap are followed by the next tap's in memory
+    x[0, 4, 4] = float("nan")
+    layer.set_mask(np.ones(81, np.uint8))
+    want = layer.run(x, w, None, flags=asx.IMPL_NAIVE).clone()
+    got = layer.run(x, w, None, flags=asx.IMPL_ALL_ROWS)
+    assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.isinf(got), torch.isinf(want))
+    layer.close()
