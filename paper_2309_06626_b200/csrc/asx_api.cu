@@ -115,6 +115,11 @@ EncodeIm2colFn encode_im2col_fn()
     return fn;
 }
 
+bool can_all_rows(const ConvGeom& g, int num_sms, int ES, AllRowsPlan* plan)
+{
+    return plan_all_rows != nullptr && plan_all_rows(g, num_sms, ES, plan);
+}
+
 // The maps of the all-rows form: x (g.H x g.W pixels of g.C_in channels, `pixel_bytes` apart, `row_bytes` and `image_bytes` per row and
 // image) for loads of 128 window positions, w as [C_out][taps][C_in] with `slab` filters a load.  Channels past g.C_in read zeros
 // in both.
@@ -609,8 +614,9 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             // The estimates leave out 4.5 us of a launch's set-up and ends.  A mask that the host does not know may drop
             // anything: no call for computing every row.
             FastPlan fp;
+            AllRowsPlan ap;
             const bool fast = plan_fast(g, L->num_sms, known_rows < 0 ? M : known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp);
-            const double all_rows_us = fast && vec_in && known_rows >= 0 && fp.all.BN > 0 ? fp.all.est_cost_us + 4.5 : 1e9;
+            const double all_rows_us = vec_in && known_rows >= 0 && can_all_rows(g, L->num_sms, ES, &ap) ? ap.est_cost_us + 4.5 : 1e9;
             if (direct && all_rows_us < 0.9 * direct_est_us(dplan, L->num_sms, known_rows, ES)) {
                 direct = false;
                 all_rows = true;
@@ -882,23 +888,22 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     }
     // Every row, where that is estimated to be a good deal faster than the kept ones by either other way: it keeps the tensor cores busier, and
     // under the power cap their clock falls (256 -> 256 channels 3x3 with 10 % dropped: 84 us in short runs against 82 gathered, 106 against 95 in long ones).
-    if (dense && plan.all.BN > 0 &&
-        (all_rows || (impl == 0 && known_rows >= 0 && plan.all.est_cost_us < 0.85 * (use_patch ? std::min(plan.est_cost_us, pplan.est_cost_us) : plan.est_cost_us)))) {
+    AllRowsPlan aplan;
+    if (dense && (all_rows || (impl == 0 && known_rows >= 0)) && can_all_rows(g, L->num_sms, ES, &aplan) &&
+        (all_rows || aplan.est_cost_us < 0.85 * (use_patch ? std::min(plan.est_cost_us, pplan.est_cost_us) : plan.est_cost_us))) {
         ConvGeom ga = g;
         if (blocks2x2) {                                          // the window positions of the staged copy: runs of four blocks
             ga.H = g.Ho + g.kh - 1;
             ga.W = g.Wo;
         }
         const int64_t pixel = x_row_stride ? x_row_stride : (int64_t)g.C_in * ES;
-        s = map_all_rows(L, ga, xsrc, wsrc, ES, plan.all, pixel, pixel * g.W, pixel * g.W * g.H);
+        s = map_all_rows(L, ga, xsrc, wsrc, ES, aplan, pixel, pixel * g.W, pixel * g.W * g.H);
         if (s != ASX_OK) return s;
-        plan.use_all = 1;
         L->last_form = ASX_FORM_ALL_ROWS;
         const bool write_list = fuse_compact && recompact, waits = mask_from_kernel == 2 && !write_list;
         if (waits) launch_in_stream_order = false;
-        return launched(launch_fast(ga, plan, L->tmap_all_w, L->tmap_all_x, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
-                                    L->num_sms, 0, write_list ? 1 : 0, L->host_kept, nullptr, 0, nullptr, 0, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
-                                    waits ? 1 : 0, st), waits ? 1 : 0);
+        return launched(launch_all_rows(ga, aplan, L->tmap_all_w, L->tmap_all_x, bias, y, L->d_mask, write_list ? L->d_kept : nullptr, d_count, relu,
+                                        L->residual, f32 ? 1 : 0, d_status, L->num_sms, waits ? 1 : 0, L->wait_limit_kcycles, st), waits ? 1 : 0);
     }
     if (plan.ksplit > 1 && !use_patch) {
         const size_t ints = 2 * (size_t)(plan.items / plan.ksplit);
@@ -910,7 +915,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             if (cudaMemsetAsync(L->d_wscnt, 0, ints * sizeof(int), st) != cudaSuccess) return ASX_ERR_CUDA;
         }
     }
-    const int BNsel = use_patch ? pplan.BN : plan.pair ? plan.BN / 2 : plan.BN;      // filters of one slab load
+    const int BNsel = use_patch ? pplan.BN : plan.vec == 3 ? plan.BN / 2 : plan.BN;      // filters of one slab load
     const int Kw = g.K;
     const CUtensorMapDataType tm_type = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const cuuint32_t box_k = (cuuint32_t)(128 / ES);           // one 128-byte swizzled row of K elements
@@ -974,14 +979,14 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
                                      fuse_compact && recompact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->residual, L->d_tiles, (int)(L->host_tiles.size() / 4), L->tiles_rows,
                                      out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->wait_limit_kcycles, st));
     }
-    if (plan.vec == 2) {
+    if (plan.vec >= 2) {
         s = map_rows();
         if (s != ASX_OK) return s;
     }
-    L->last_form = plan.vec == 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
+    L->last_form = plan.vec >= 2 ? ASX_FORM_ROW_GATHER_TMA : ASX_FORM_ROW_GATHER_COPY;
     const bool waits_for_mask = mask_from_kernel == 2 && !fuse_compact;
     if (waits_for_mask) launch_in_stream_order = false;
-    return launched(launch_fast(g, plan, L->tmap, plan.vec == 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
+    return launched(launch_fast(g, plan, L->tmap, plan.vec >= 2 ? L->tmap_x : L->tmap, xsrc, bias, y, L->d_mask, L->d_kept, d_count, relu, d_status,
                                 L->num_sms, fuse_compact ? 1 : 0, recompact ? 1 : 0, L->host_kept, L->d_wscnt,
                                 out_compact ? 1 : 0, in_compact ? L->d_in_rank : nullptr, (int)L->in_kept, L->residual, f32 ? 1 : 0, L->wait_limit_kcycles,
                                 waits_for_mask ? 1 : 0, st), waits_for_mask ? 1 : 0);

@@ -104,12 +104,13 @@ struct AllRowsPlan {
     int smem_bytes = 0;
     double est_cost_us = 0;
 };
-bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* plan);
+// (weak: the host side also runs without this form's file, and then never takes it)
+bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* plan) __attribute__((weak));
 // tmap_w: w as [C_out][taps][C_in], box (128 bytes of channels, 1, the filters of one slab load); tmap_x: x for im2col loads of 128
 // positions.  kept_out, count_out: where the kept-row list goes too, or null
 cudaError_t launch_all_rows(const ConvGeom& g, const AllRowsPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x, const float* bias,
                             void* y, const uint8_t* mask, int32_t* kept_out, int32_t* count_out, int relu, const void* residual, int f32,
-                            int* dev_status, int num_sms, int mask_from_kernel, int wait_limit_kcycles, cudaStream_t st);
+                            int* dev_status, int num_sms, int mask_from_kernel, int wait_limit_kcycles, cudaStream_t st) __attribute__((weak));
 
 // Kept rows only, gathered (masked_conv_sm100.cu)
 struct FastPlan {
@@ -118,14 +119,12 @@ struct FastPlan {
     int stages;
     int smem_bytes;
     int vec;          // gather mode: 1 cp.async 16 B (a pixel's channels are whole 16-byte chunks), 2 TMA row
-                      // gather (they are whole 128-byte runs)
+                      // gather (they are whole 128-byte runs), 3 TMA row gather by pairs of blocks: a work item is 256 rows, each
+                      // block has its own 128 and half of every filter slab
     int ksplit;       // work items per output tile (shares of the k-blocks), which form a cluster
     long long items;  // m_tiles * n_tiles * ksplit for the estimated kept rows
     int list_bytes;   // shared memory set aside for the fused compaction's list
     double est_cost_us;   // the planner's estimate of the launch's duration
-    int pair = 0;         // a work item is a pair of blocks on 256 rows, each with its own 128 rows and half of every filter slab
-    AllRowsPlan all;      // the same call with every row computed
-    int use_all = 0;      // and whether it is run so (the caller's choice)
 };
 // elem_bytes: 2 (bf16 storage) or 4 (fp32 storage, TF32 contraction)
 bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fused_list_rows, bool allow_split, int elem_bytes,

@@ -104,7 +104,7 @@ struct alignas(16) SharedT {           // lives after the operand stages
     int scan_total[32];   // fused compaction: kept rows per warp
 };
 
-enum : int { GATHER_CPASYNC = 1, GATHER_TMA = 2 };
+enum : int { GATHER_CPASYNC = 1, GATHER_TMA = 2, GATHER_TMA_PAIR = 3 };
 
 // Work item t = (output tile, k share): tile = t / ksplit, share ks = t % ksplit covers k-blocks
 // [ks KB / ksplit, (ks + 1) KB / ksplit).  The shares of a tile are consecutive items, so they run
@@ -1013,8 +1013,6 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     const int bke = 128 / elem_bytes;             // K elements per stage: 64 bf16 or 32 fp32
     const int KB = (g.K + bke - 1) / bke;
     if (g.C_in % (16 / elem_bytes) != 0) return false;      // the caller pads the channels first
-    plan->use_all = 0;
-    if (!plan_all_rows(g, num_sms, elem_bytes, &plan->all)) plan->all.BN = 0;
     const int list_bytes = (fused_list_rows * 2 + 15) / 16 * 16;     // 16-bit kept list of the fused compaction
     auto stage_bytes_of = [](int BN, int pair) { return A_STAGE_BYTES + (pair ? BN / 2 : BN) * BK * 2; };
     auto fixed_bytes = [&](int KS) { return 1024 + (int)(KS > 1 ? sizeof(SharedT<1>) : sizeof(SharedT<PLAIN_INFO_RING>)) + list_bytes; };
@@ -1076,7 +1074,6 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     plan->BN = BN;
     plan->n_tiles = n_tiles;
     plan->ksplit = best_KS;
-    plan->pair = best_pair;
     plan->est_cost_us = best_cost;
     plan->items = (long long)m_tiles * n_tiles * best_KS;
     plan->stages = S;
@@ -1084,7 +1081,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     int smem = fixed_bytes(best_KS) + S * stage_bytes + split_bytes(BN, best_KS);
     if (smem < 120 * 1024) smem = 120 * 1024;      // one block per SM: tensor memory is not shared out
     plan->smem_bytes = smem;
-    plan->vec = (g.C_in % bke == 0) ? GATHER_TMA : GATHER_CPASYNC;
+    plan->vec = tma ? (best_pair ? GATHER_TMA_PAIR : GATHER_TMA) : GATHER_CPASYNC;
     return true;
 }
 
@@ -1096,9 +1093,6 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
                         int mask_from_kernel, cudaStream_t st)
 {
     if (f32 && (in_rank != nullptr || residual != nullptr)) return cudaErrorInvalidValue;
-    if (plan.use_all)
-        return launch_all_rows(g, plan.all, tmap_w, tmap_x, bias, y, mask, write_list ? const_cast<int32_t*>(kept) : nullptr,
-                               const_cast<int32_t*>(count), relu, residual, f32, dev_status, num_sms, mask_from_kernel, wait_limit_kcycles, st);
     FastArgs a;
     a.fdcnt_host = make_fastdiv((uint32_t)(host_kept > 0 && host_kept < (1ll << 31) ? host_kept : 1));
     if (!(host_kept > 0 && host_kept < (1ll << 31))) a.fdcnt_host.d = 0;
@@ -1146,14 +1140,14 @@ cudaError_t launch_fast(const ConvGeom& g, const FastPlan& plan, const CUtensorM
     // Shared k-blocks: one item per block (the host knows the count).  Else as many resident blocks as there may be items.
     const bool split = plan.ksplit > 1;
     const long long least = !split && plan.vec == GATHER_CPASYNC ? MIN_TILE_ROWS : BM;      // rows per tile
-    const bool pair = plan.pair != 0;
+    const bool pair = plan.vec == GATHER_TMA_PAIR;
     const int blocks = pair ? 2 : 1;              // of a work item
     const long long tiles = split ? plan.items : ((long long)g.M + blocks * least - 1) / (blocks * least) * plan.n_tiles;
     int grid = (split || tiles < num_sms / blocks ? (int)tiles : num_sms / blocks) * blocks;
     if (grid < blocks) grid = blocks;
     a.fdGrid = make_fastdiv((uint32_t)grid);
     a.mask_from_kernel = mask_from_kernel && !fuse_compact ? 1 : 0;
-    const int variant = plan.vec + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
+    const int variant = (pair ? GATHER_TMA : plan.vec) + (in_rank != nullptr ? 2 : 0);      // 1, 2: dense input; 3, 4: compact input
     const bool has_res = residual != nullptr, is_silu = relu == 2;
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const ConvGeom, const FastArgs);
     Kern kern = nullptr;
