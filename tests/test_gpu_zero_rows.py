@@ -1,0 +1,39 @@
+"""Zeros of dropped rows where a row's pieces do not divide the threads that write them: channel counts around 16-byte chunks and words, in both
+storage types, against the mask; kept rows stay what the plain kernel gives."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2309_06626_b200 as asx
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("f32", [False, True], ids=["bf16", "f32"])
+@pytest.mark.parametrize("cout", [1, 2, 3, 31, 33, 63, 72, 96, 129, 160, 192, 320, 1032])
+@pytest.mark.parametrize("per_row", [False, True])
+def test_general_zero_fill(cout, f32, per_row):
+    gen = torch.Generator(device="cuda").manual_seed(cout)
+    Nb, H, W = 3, 19, 23
+    x = torch.randn((Nb, H, W, 64), generator=gen, device="cuda")
+    w = torch.randn((cout, 3, 3, 64), generator=gen, device="cuda") / 24
+    x, w = (((t.view(torch.int32) & ~0x1fff).view(torch.float32)) if f32 else t.to(torch.bfloat16) for t in (x, w))
+    rows = H * W * (Nb if per_row else 1)
+    mask = (np.random.default_rng(rows + cout).random(rows) < 0.3).astype(np.uint8)
+    layer = asx.MaskedConvLayer(64, cout, 3, 3, 1, 1)
+    layer.set_mask(mask)
+    base = asx.F32 if f32 else 0
+    want = layer.run(x, w, None, flags=base | asx.IMPL_NAIVE).float().clone()
+    dt = torch.float32 if f32 else torch.bfloat16
+    # the rows before and behind the output hold what they held; an output that starts between two words where that is allowed
+    for shift in ((0, 1) if cout % (4 if f32 else 8) else (0,)):
+        buf = torch.full((want.numel() + 256,), 7.0, dtype=dt, device="cuda")
+        out = buf[64 + shift:64 + shift + want.numel()].view(want.shape)
+        layer.run(x, w, None, out=out, flags=base | asx.IMPL_ROW_GATHER)
+        torch.cuda.synchronize()
+        assert layer.device_status() == 0
+        got = out.float()
+        assert (got - want).norm() <= (2e-5 if f32 else 5e-3) * want.norm()
+        assert not got.reshape(-1, rows, cout)[:, torch.from_numpy(mask == 0).cuda()].any()
+        assert bool((buf[:64 + shift] == 7).all()) and bool((buf[64 + shift + want.numel():] == 7).all())
+    layer.close()
