@@ -617,7 +617,7 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             AllRowsPlan ap;
             const bool fast = plan_fast(g, L->num_sms, known_rows < 0 ? M : known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp);
             const double all_rows_us = vec_in && known_rows >= 0 && can_all_rows(g, L->num_sms, ES, &ap) ? ap.est_cost_us + 4.5 : 1e9;
-            if (direct && all_rows_us < 0.9 * direct_est_us(dplan, L->num_sms, known_rows, ES)) {
+            if (direct && all_rows_us < direct_est_us(dplan, L->num_sms, known_rows, ES)) {
                 direct = false;
                 all_rows = true;
             }

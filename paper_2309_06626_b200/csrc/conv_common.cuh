@@ -301,29 +301,32 @@ __device__ __forceinline__ void zero_fill_dropped_rows(void* y, const uint8_t* _
             dst += 4 * dstep;
         }
     } else {
-        // General path (channel counts whose chunks do not divide the threads, and rows at any address): a warp takes 32 rows at a time, a mask
+        // General path (channel counts whose chunks do not divide the threads, and rows at any address): a warp takes up to 32 rows at a time, a mask
         // byte a lane, the next rows' on its way, and walks over their units (16-byte chunks, or words) with a constant stride, storing
         // those of dropped rows; nothing in it divides but the mask's index once per 32 rows.  (One row a warp and turn, a mask byte and a 64-bit
         // division in front of each: 16,312 kept of 163,125 rows of 320 channels 96 us a launch, this 30.)
         const int zw = zt >> 5, nw = ZT / 32;
+        const long long share = (hi - lo + nw - 1) / nw;
+        const int take = share < 32 ? (int)share : 32;        // rows a warp takes at a time
         const bool bf16_rows = !F32 && !vec_out;
         const int units = vec_out ? cpr : F32 ? N : N / 2 + 1;
         const int dr = 32 / units, dc = 32 - dr * units, r_first = lane / units, c_first = lane - r_first * units;
         auto dropped = [&](long long row0) -> bool {
             const long long row = row0 + lane;
-            if (row >= hi) return false;
+            if (lane >= take || row >= hi) return false;
             return __ldg(mask + (shared_mask ? (uint32_t)row % (uint32_t)g.P : (uint32_t)row)) == 0;
         };
-        long long row0 = lo + zw * 32;
+        const int steps = (take * units + 31) / 32;
+        long long row0 = lo + zw * take;
         bool next = dropped(row0);
-        for (; row0 < hi; row0 += nw * 32) {
+        for (; row0 < hi; row0 += nw * take) {
             const unsigned drop = __ballot_sync(0xffffffffu, next);
-            next = dropped(row0 + nw * 32);
+            next = dropped(row0 + nw * take);
             if (drop == 0) continue;
             int r = r_first, c = c_first;
 #pragma unroll 4
-            for (int i = 0; i < units; ++i) {
-                if ((drop >> r) & 1u) {
+            for (int i = 0; i < steps; ++i) {
+                if (r < 32 && ((drop >> r) & 1u)) {
                     const long long el = (row0 + r) * N;
                     if (vec_out) {
                         *reinterpret_cast<uint4*>(yb + (el + c * EPC) * ES) = make_uint4(0, 0, 0, 0);

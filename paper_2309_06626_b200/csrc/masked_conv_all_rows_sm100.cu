@@ -20,7 +20,7 @@
 // Bound by the tensor core's reads of the operands and the issue (64 to 128 channels), the tensor core (256), the way out (1x1 layers).
 // Measured on layers inside a graph, before -> with this form: 64 -> 64 channels 3x3 at 56x56, batch 64, 10 % dropped 30.8 -> 22.3 us; 256 -> 256
 // at 14x14, 20 % 22.1 -> 18.5; fp32 128 -> 128 at 28x28, batch 16, 50 % 16.4 -> 14.4; 1x1 128 -> 128 at 80x80, batch 16, 40 % 18.2 -> 14.7;
-// 16 -> 286 3x3 at 80x80, batch 117, 60 % 1082 -> 256; 1x1 stride 2 272 -> 279, batch 97 330 -> 54.
+// 16 -> 286 3x3 at 80x80, batch 117, 60 % 1082 -> 296; 1x1 stride 2 272 -> 279, batch 97 330 -> 55.
 #include <algorithm>
 #include <atomic>
 #include <cuda_bf16.h>
@@ -516,24 +516,34 @@ masked_conv_all_rows_kernel(const __grid_constant__ CUtensorMap tmap_w, const __
 #pragma unroll
                     for (int i = 0; i < UNITS; ++i)
                         if (out_row[i] >= 0 && u < ncols * ES) *reinterpret_cast<uint4*>(dst + out_row[i] * pitch_y) = piece[i];
-                } else if (F32) {
-                    float* const yf = static_cast<float*>(a.y) + n0 + c0 + (lane & 15);
-#pragma unroll 8
-                    for (int rr = lane >> 4; rr < 32; rr += 2) {
-                        const int out = __shfl_sync(0xffffffffu, row, rr);
-                        const float w = *reinterpret_cast<const float*>(stage + rr * STAGING_PITCH + 4 * (lane & 15));
-                        if (out >= 0 && (lane & 15) < ncols) yf[(long long)out * N] = w;
-                    }
                 } else {
-                    // two rows at a time, a word a lane: the words that are the row's alone
-                    uint32_t* const yw = reinterpret_cast<uint32_t*>(yb - 2 * a.y_half) + (lane & 15);
-                    const int col2 = 2 * (lane & 15) + 2;
-                    if (row < 0) e = -1;
+                    // Two rows at a time, a word a lane: the words that are the row's alone.  In fp32 eight are read before the first is stored (for
+                    // all the compiler knows a store may change the next one: 18.0 -> 15.2 us for 3168 rows of 57 channels); in
+                    // bf16, where a row's first and last halves are on their way as well, that was slower (296 -> 307 us for 749,000 rows of 286).
+                    const int word_l = lane & 15, half = lane >> 4;
+                    const int at = row < 0 ? -1 : F32 ? row * N + n0 + c0 : e;          // in values (fp32), in half words from a whole word on (bf16)
+                    uint32_t* const yw = reinterpret_cast<uint32_t*>(yb - (F32 ? 0 : 2 * a.y_half)) + word_l;
+                    if (F32) {
+#pragma unroll
+                        for (int i0 = 0; i0 < 32; i0 += 16) {
+                            uint32_t w[8];
+                            int ar[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                ar[i] = __shfl_sync(0xffffffffu, at, i0 + 2 * i + half);
+                                w[i] = *reinterpret_cast<const uint32_t*>(stage + (i0 + 2 * i + half) * STAGING_PITCH + 4 * word_l);
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (ar[i] >= 0 && word_l < ncols) yw[ar[i]] = w[i];
+                        }
+                    } else {
 #pragma unroll 8
-                    for (int rr = lane >> 4; rr < 32; rr += 2) {
-                        const int er = __shfl_sync(0xffffffffu, e, rr), odd = er & 1;
-                        const uint32_t w = *reinterpret_cast<const uint32_t*>(stage + rr * STAGING_PITCH + 4 * (lane & 15));
-                        if (er >= 0 && (lane & 15) >= odd && col2 - odd <= ncols) yw[er >> 1] = w;
+                        for (int rr = half; rr < 32; rr += 2) {
+                            const int ar = __shfl_sync(0xffffffffu, at, rr), odd = ar & 1;
+                            const uint32_t w = *reinterpret_cast<const uint32_t*>(stage + rr * STAGING_PITCH + 4 * word_l);
+                            if (ar >= 0 && word_l >= odd && 2 * word_l + 2 - odd <= ncols) yw[ar >> 1] = w;
+                        }
                     }
                 }
                 __syncwarp();
@@ -619,7 +629,7 @@ bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* 
         const int slots = pair ? num_sms / 2 : num_sms;
         for (int n_tiles = (N + 255) / 256; ; n_tiles *= 2) {
             const int per = (N + n_tiles - 1) / n_tiles, BN = (per + unit - 1) / unit * unit, nt = (N + BN - 1) / BN, BNB = pair ? BN / 2 : BN;
-            for (int patch = 0; patch <= 1; ++patch) {
+            for (int patch = 1; patch >= 0; --patch) {
                 AllRowsPlan p = *plan;
                 p.patch = patch;
                 p.pair = pair;
@@ -653,9 +663,10 @@ bool plan_all_rows(const ConvGeom& g, int num_sms, int elem_bytes, AllRowsPlan* 
                 const long long waves = (p.items + slots - 1) / slots;
                 // microseconds: a k-block of the patch form waits for its slabs where they cannot stay; the way out of a tile's
                 // columns, of which four groups of warps take four tiles at a time
-                const double t_kb = !patch ? 0.36 : f32 ? 0.12 + 0.001 * BN : pair ? 0.085 + 0.001 * BN : p.resident ? 0.105 + 0.001 * BN : std::max(0.3, 0.105 + 0.001 * BN);
-                const double t_out = (whole ? 0.2 + 0.011 * BN : 0.3 + 0.02 * BN) * (f32 ? 2.0 : 1.0) * (p.epi_groups == 4 ? 1.0 : 1.7);
-                const double cost = (double)waves * std::max(KB * t_kb + 0.1, t_out) + 0.012 * BN + 2.0;
+                const double t_kb = !patch ? 0.36 : (f32 ? 0.03 : 0.0) + (pair ? 0.085 + 0.001 * BN : p.resident ? 0.105 + 0.001 * BN : std::max(0.3, 0.105 + 0.001 * BN));
+                const double t_out = (whole ? 0.15 + 0.0105 * BN : 0.3 + 0.02 * BN) * (f32 ? 2.0 : 1.0) * (p.epi_groups == 4 ? 1.0 : 1.7);
+                const double t_in = nc * p.a_bytes / 30e3;                  // every SM at once
+                const double cost = (double)waves * std::max(std::max(KB * t_kb + 0.1, t_out), patch ? t_in : 0.0) + t_out + (p.flat ? 0.5 : 1.2);
                 p.est_cost_us = cost;
                 p.smem_bytes = std::max(120 * 1024, fixed + p.a_bufs * p.a_bytes + p.b_slots * p.G * BNB * rb);      // one block per SM: tensor memory is not shared out
                 if (best_plan.BN == 0 || cost < best) { best = cost; best_plan = p; }

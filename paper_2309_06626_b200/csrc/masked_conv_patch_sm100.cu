@@ -731,7 +731,8 @@ void plan_patch_cost(const ConvGeom& g, int num_sms, long long n_mtiles, bool in
     const double t_tile = KB * (0.21 + 0.001 * plan->BN);
     // a compact input's patches come as 128-byte rows, four to a request of 13 clocks
     const double t_patch = in_compact ? (g.C_in / 64) * plan->cap_rows * plan->Wp / 4 * 13 / 1900.0 : 0.0;
-    plan->est_cost_us = (double)waves * (std::max(t_tile, t_patch) + 0.3) + 0.012 * plan->BN;
+    // more set-up than the row gather's: 64 -> 64 channels 3x3 at 56x56, one image, 7.5 us a launch against 6.7, a 7x7 stem in 2x2 blocks 9.9 against 7.5
+    plan->est_cost_us = (double)waves * (std::max(t_tile, t_patch) + 0.3) + 0.012 * plan->BN + (plan->px32 ? 2.4 : 0.7);
 }
 
 cudaError_t launch_patch(const ConvGeom& g, const PatchPlan& plan, const CUtensorMap& tmap_w, const CUtensorMap& tmap_x4,

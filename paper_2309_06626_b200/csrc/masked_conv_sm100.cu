@@ -1056,9 +1056,7 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
                 const int kbi = (KB + KS - 1) / KS;
                 const double t_kb = 0.12 + 0.18 * fill + (pair ? 0.0005 : 0.001) * BN;                  // microseconds
                 // sharing with more blocks than half the SMs: the next launch's clusters do not fit beside this one's
-                // rows of y that are no whole 16-byte chunks leave value by value
-                const double t_item = std::max(kbi * t_kb, scalar_out ? 0.2 * BN : 0.0);
-                const double cost = (double)waves * (t_item + (pair ? 1.5 : 0.3)) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
+                const double cost = (double)waves * (kbi * t_kb + (pair ? 1.5 : 0.3)) + 0.012 * BN + (KS > 1 ? (items > num_sms / 2 ? SPLIT_US + 2.0 : SPLIT_US) : 0.0);
                 if (best_BN == 0 || cost < best_cost * 0.97) { best_BN = BN; best_KS = KS; best_pair = pair; best_cost = cost; }
             }
             if (BN <= 64 && whole) break;
@@ -1074,7 +1072,8 @@ bool plan_fast(const ConvGeom& g, int num_sms, long long est_kept_rows, int fuse
     plan->BN = BN;
     plan->n_tiles = n_tiles;
     plan->ksplit = best_KS;
-    plan->est_cost_us = best_cost;
+    // rows of y that are no whole 16-byte chunks leave value by value, some 75 values a nanosecond from all SMs
+    plan->est_cost_us = scalar_out ? std::max(best_cost, (double)est_kept_rows * N / 75e3) : best_cost;
     plan->items = (long long)m_tiles * n_tiles * best_KS;
     plan->stages = S;
     plan->list_bytes = list_bytes;
