@@ -613,10 +613,11 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
             // What the forms that compute every row and kept rows through tensor memory would take, where the call's own channels suit them.
             // The estimates leave out 4.5 us of a launch's set-up and ends.  A mask that the host does not know may drop
             // anything: no call for computing every row.
+            const double list_us = recompact ? 4.5e-5 * (double)L->rows : 0.0;         // the list holds up a quarter of its epilogue warps
             FastPlan fp;
             AllRowsPlan ap;
             const bool fast = plan_fast(g, L->num_sms, known_rows < 0 ? M : known_rows, L->rows <= FUSED_COMPACT_MAX_ROWS ? (int)L->rows : 0, L->C_out % 8 == 0, ES, &fp);
-            const double all_rows_us = vec_in && known_rows >= 0 && can_all_rows(g, L->num_sms, ES, &ap) ? ap.est_cost_us + 4.5 : 1e9;
+            const double all_rows_us = vec_in && known_rows >= 0 && can_all_rows(g, L->num_sms, ES, &ap) ? ap.est_cost_us + 4.5 + list_us : 1e9;
             if (direct && all_rows_us < direct_est_us(dplan, L->num_sms, known_rows, ES)) {
                 direct = false;
                 all_rows = true;
@@ -665,7 +666,10 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
     // that as well (3-4 us).  The window-patch form has its row tiles from the host and reads the list late: building it
     // there costs 0.6 us for a mask of 3136 rows, 2 us for 15,000.
     bool fuse_compact = !(flags & ASX_IMPL_NAIVE) && L->rows <= FUSED_COMPACT_MAX_ROWS && (recompact || mask_from_kernel == 0);
-    if (recompact && !fuse_compact) {
+    // The form that computes every row builds lists of up to DIRECT_LIST_MAX_ROWS rows beside its tiles (a launch of its own takes its
+    // time in front).
+    bool list_inside = all_rows && recompact && !fuse_compact && L->rows <= DIRECT_LIST_MAX_ROWS;
+    if (recompact && !fuse_compact && !list_inside) {
         s = run_compaction(L, st);
         if (s != ASX_OK) return s;
     }
@@ -900,10 +904,14 @@ asx_status asx_run(asx_layer* L, const void* x, int Nb, int H, int W, const void
         s = map_all_rows(L, ga, xsrc, wsrc, ES, aplan, pixel, pixel * g.W, pixel * g.W * g.H);
         if (s != ASX_OK) return s;
         L->last_form = ASX_FORM_ALL_ROWS;
-        const bool write_list = fuse_compact && recompact, waits = mask_from_kernel == 2 && !write_list;
+        const bool write_list = recompact && (fuse_compact || list_inside), waits = mask_from_kernel == 2 && !write_list;
         if (waits) launch_in_stream_order = false;
         return launched(launch_all_rows(ga, aplan, L->tmap_all_w, L->tmap_all_x, bias, y, L->d_mask, write_list ? L->d_kept : nullptr, d_count, relu,
                                         L->residual, f32 ? 1 : 0, d_status, L->num_sms, waits ? 1 : 0, L->wait_limit_kcycles, st), waits ? 1 : 0);
+    }
+    if (list_inside) {                                            // another form after all
+        s = run_compaction(L, st);
+        if (s != ASX_OK) return s;
     }
     if (plan.ksplit > 1 && !use_patch) {
         const size_t ints = 2 * (size_t)(plan.items / plan.ksplit);

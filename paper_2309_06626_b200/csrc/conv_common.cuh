@@ -118,7 +118,7 @@ __device__ __forceinline__ void write_kept_list(const uint8_t* __restrict__ mask
     const int first = part * ROWS + tid * 16;
     const unsigned f = first < rows ? mask_flags16(mask, rows, first) : 0u;
     int before = 0;
-#pragma unroll 4
+#pragma unroll 8
     for (int i = 0; i < part; ++i) before += __popc(mask_flags16(mask, rows, i * ROWS + tid * 16));
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);

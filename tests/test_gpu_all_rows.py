@@ -75,6 +75,26 @@ def test_residual(cout):
     layer.close()
 
 
+@pytest.mark.parametrize("rows", [32768, 32769, 40000, 131072, 131073])
+def test_long_lists(rows):
+    """The kept-row list is built beside the tiles up to 131072 mask entries, by a launch of its own above."""
+    W = 8 if rows % 8 == 0 else 1
+    x = torch.randn((rows // W, 1, W, 8), device="cuda").to(torch.bfloat16)
+    w = torch.randn((16, 1, 1, 8), device="cuda").to(torch.bfloat16)
+    mask = (np.random.default_rng(rows).random(rows) < 0.5).astype(np.uint8)
+    layer = asx.MaskedConvLayer(8, 16, 1, 1, 1, 0)
+    layer.set_mask(mask)
+    layer.set_mask(1 - mask)
+    layer.set_mask(mask)
+    want = layer.run(x, w, None, flags=asx.IMPL_NAIVE).float().clone()
+    got = layer.run(x, w, None, flags=asx.IMPL_ALL_ROWS | asx.RECOMPACT).float()
+    torch.cuda.synchronize()
+    assert layer.device_status() == 0 and layer.last_run_form() == asx.FORM_ALL_ROWS
+    assert np.array_equal(layer.kept(), np.flatnonzero(mask))
+    assert (got - want).norm() <= 5e-3 * want.norm()
+    layer.close()
+
+
 def test_infinity_and_nan_stay_in_their_windows():
     """Values past a window's channels, and of other rows, do not reach a result."""
     layer = asx.MaskedConvLayer(40, 24, 3, 3, 1, 1)
