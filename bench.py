@@ -48,7 +48,8 @@ def csrc_digest() -> str:
     """Digest of the sources the fused kernels are compiled from."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("asx_internal.h", "conv_common.cuh", "masked_conv_direct.cu", "masked_conv_sm100.cu", "masked_conv_patch_sm100.cu", "ptx_sm100.cuh"):
+    for name in ("asx_internal.h", "conv_common.cuh", "masked_conv_direct.cu", "masked_conv_sm100.cu", "masked_conv_patch_sm100.cu",
+                 "masked_conv_all_rows_sm100.cu", "ptx_sm100.cuh"):
         h.update(name.encode())
         with open(os.path.join(ROOT, "paper_2309_06626_b200", "csrc", name), "rb") as fh:
             h.update(fh.read())
@@ -771,7 +772,7 @@ def run_ours(args):
                 "ms_per_step": e2e_ms},
         "gpu_launches": K * sum(L.launches for L in layers),
         "roofline": {
-            "bound": "tensor", "kernel": "masked_conv_sm100_kernel / masked_conv_patch_sm100_kernel / masked_conv_direct_kernel (one launch per layer)",
+            "bound": "tensor", "kernel": "masked_conv_sm100_kernel / masked_conv_patch_sm100_kernel / masked_conv_direct_kernel / masked_conv_all_rows_kernel (one launch per layer)",
             "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
             # frac is the spec quantity: per layer the slower of its kept-row FLOPs at the tensor peak and
             # its algorithmic bytes at the HBM peak, summed over the layers, over the measured step time
@@ -827,7 +828,7 @@ def run_ours(args):
                        "ms_serialised": per_layer_ms[i], "tflops": L.flops / (per_layer_ms[i] * 1e-3) / 1e12,
                        "gbs": L.bytes / (per_layer_ms[i] * 1e-3) / 1e9, "roof_ms": roofs[i],
                        "form": {0: "none", 1: "naive", 2: "row gather (copies)", 3: "row gather (TMA)", 4: "window patch",
-                                5: "direct", 6: "direct, shared k range"}[forms[i]]}
+                                5: "direct", 6: "direct, shared k range", 7: "all rows"}[forms[i]]}
                       for i, L in enumerate(layers)],
     }
     print(json.dumps(line), flush=True)
